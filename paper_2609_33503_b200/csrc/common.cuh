@@ -108,20 +108,29 @@ __device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.
 bool chained_launch_enabled();           // process-wide switch (relaxkv_set_chained_launch), on by default
 constexpr long long kChainedMaxRows = 8;
 
+// cluster > 1: the grid's x dimension is made of clusters of that many blocks (grid.x is a multiple of it).
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_chained(bool few_rows, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
-                                  Args&&... args) {
+inline cudaError_t launch_chained_clusters(bool few_rows, int cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block,
+                                           size_t smem, cudaStream_t stream, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = (few_rows && chained_launch_enabled()) ? 1 : 0;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_chained(bool few_rows, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                  Args&&... args) {
+  return launch_chained_clusters(few_rows, 1, kernel, grid, block, smem, stream, static_cast<Args&&>(args)...);
 }
 
 // Up to this many requests have their per-request scalars passed by value in kernel parameters.
