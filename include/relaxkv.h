@@ -207,7 +207,7 @@ relaxkv_status relaxkv_build_active_sets(
  *  - All calls on a device share the one array, and it keeps the previous call's contents.  Nothing
  *    in it needs to start at zero (each call overwrites every entry it later reads), but two calls
  *    that overlap on the GPU - different streams, no ordering between them - race on it: order them.
- *  - h_counts_pinned (optional) is filled from the array by a copy on `stream`, as above.
+ *  - h_counts_pinned (optional) is filled in `stream` order, as above.
  */
 relaxkv_status relaxkv_build_active_sets_static(
     const relaxkv_shape* shape, int32_t n_layers, const int32_t* h_k, const int32_t* anchors,

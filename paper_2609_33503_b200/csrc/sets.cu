@@ -1,19 +1,28 @@
 // Repair schedule: highest selected layer h_i, sorted union U, position->rank map and the per-layer
 // active targets R_l as ranks into U (Section 3.2; Algorithm 1, steps 6-12).  Integer work only.
 #include "common.cuh"
+#include "sm100_ptx.cuh"
 
 namespace relaxkv {
 
+// The four kernels of a schedule take a few microseconds each and depend on one another: they are launched chained, so
+// that each one's launch and ramp-up run under its predecessor.  Everything a predecessor writes is read through plain
+// pointers after griddep_wait().
 constexpr int kSetThreads = 1024;
+constexpr int kSetWarps = kSetThreads / 32;
+constexpr int kSetSlices = 8;                    // blocks of the cluster that writes one list
 
-__global__ void fill_i32_kernel(int* p, long long n, int v) {
+__global__ void __launch_bounds__(256) fill_i32_kernel(int* p, long long n, int v) {
+  griddep_launch();
+  griddep_wait();
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) p[i] = v;
 }
 
 // h[i] = max layer that selected position i.
-__global__ void highest_layer_kernel(ReqTable rt, int n_layers, const int* __restrict__ anchors,
-                                     int* __restrict__ h, DeviceStatus* st) {
+__global__ void __launch_bounds__(256) highest_layer_kernel(ReqTable rt, int n_layers, const int* anchors, int* h, DeviceStatus* st) {
+  griddep_launch();
+  griddep_wait();
   const int sum_k = rt.k_cu[rt.n_req];
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long long)n_layers * sum_k) return;
@@ -25,52 +34,19 @@ __global__ void highest_layer_kernel(ReqTable rt, int n_layers, const int* __res
   atomicMax(&h[rt.ctx_cu[b] + pos], l);
 }
 
-// Exclusive block scan of two counters (blockDim.x == kSetThreads); returns the totals too.
-__device__ __forceinline__ void block_scan2(int a, int b, int& a_excl, int& b_excl, int& a_tot, int& b_tot) {
-  __shared__ int wa[32], wb[32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int ia = a, ib = b;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    int ta = __shfl_up_sync(0xffffffffu, ia, o), tb = __shfl_up_sync(0xffffffffu, ib, o);
-    if (lane >= o) { ia += ta; ib += tb; }
-  }
-  if (lane == 31) { wa[warp] = ia; wb[warp] = ib; }
-  __syncthreads();
-  if (warp == 0) {
-    int va = wa[lane], vb = wb[lane];
-    int sa = va, sb = vb;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      int ta = __shfl_up_sync(0xffffffffu, sa, o), tb = __shfl_up_sync(0xffffffffu, sb, o);
-      if (lane >= o) { sa += ta; sb += tb; }
-    }
-    wa[lane] = sa - va; wb[lane] = sb - vb;          // exclusive warp offsets
-    if (lane == 31) { wa[31] = sa - va; wb[31] = sb - vb; }
-  }
-  __syncthreads();
-  a_excl = wa[warp] + ia - a;
-  b_excl = wb[warp] + ib - b;
-  __syncthreads();
-  // totals: last thread's inclusive value
-  __shared__ int ta_s, tb_s;
-  if (threadIdx.x == kSetThreads - 1) { ta_s = a_excl + a; tb_s = b_excl + b; }
-  __syncthreads();
-  a_tot = ta_s; b_tot = tb_s;
-  __syncthreads();
-}
-
 // Block (b, s): s == 0 counts |U_b|; s = l+1 counts |R_{l,b}|.  counts[b] and counts[B + l*B + b].
-__global__ void __launch_bounds__(kSetThreads)
-count_sets_kernel(ReqTable rt, int n_layers, const int* __restrict__ h, int* __restrict__ counts) {
+__global__ void __launch_bounds__(kSetThreads) count_sets_kernel(ReqTable rt, int n_layers, const int* h, int* counts) {
+  griddep_launch();
+  griddep_wait();
   const int B = rt.n_req;
   const int b = blockIdx.x % B, s = blockIdx.x / B;
   const int T = rt.ctx_len[b];
   const int* hb = h + rt.ctx_cu[b];
   const int thr = (s == 0) ? 0 : (s - 1);
   int n = 0;
+#pragma unroll 8
   for (int i = threadIdx.x; i < T; i += kSetThreads) n += (hb[i] >= thr) ? 1 : 0;
-  __shared__ int red[32];
+  __shared__ int red[kSetWarps];
   n = warp_reduce_sum(n);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = n;
   __syncthreads();
@@ -81,52 +57,79 @@ count_sets_kernel(ReqTable rt, int n_layers, const int* __restrict__ h, int* __r
   }
 }
 
-// u_cu[B+1] and r_cu[L*B+1] from the counts (one block; the arrays are short).
-__global__ void prefix_counts_kernel(int B, int n_layers, const int* __restrict__ counts,
-                                     int* __restrict__ u_cu, int* __restrict__ r_cu) {
-  if (threadIdx.x == 0) {
-    int a = 0;
-    for (int b = 0; b < B; ++b) { u_cu[b] = a; a += counts[b]; }
-    u_cu[B] = a;
-  }
-  if (threadIdx.x == 32) {
-    int a = 0;
-    const int n = n_layers * B;
-    for (int i = 0; i < n; ++i) { r_cu[i] = a; a += counts[B + i]; }
-    r_cu[n] = a;
-  }
-}
-
-// Block (b, 0) writes u_pos / u_rank; block (b, l+1) writes the ranks of R_{l,b}.
-__global__ void __launch_bounds__(kSetThreads)
-write_sets_kernel(ReqTable rt, int n_layers, const int* __restrict__ h, const int* __restrict__ u_cu,
-                  const int* __restrict__ r_cu, int* __restrict__ u_pos, int* __restrict__ u_rank,
-                  int* __restrict__ r_rank) {
+// Cluster (b, 0) writes u_pos / u_rank, cluster (b, l+1) the ranks of R_{l,b}; each block takes a contiguous slice of the
+// positions.  Where a list starts is the sum of the counts before it, which every block adds up for itself (u_cu and r_cu
+// are those sums).  One block per list took 20 / 77 / 149 us for segments of 16 K / 32 K / 64 K positions (a thread walked
+// 64 consecutive positions, one dependent uncoalesced load and store after the other), and a launch of its own for the
+// prefix of the counts another 4 us; now 7 / 20 / 24 us including what overlaps the kernels before it.
+__global__ void __launch_bounds__(kSetThreads) write_sets_kernel(ReqTable rt, int n_layers, const int* h, const int* counts,
+                                                                 int* u_pos, int* u_cu, int* u_rank, int* r_rank, int* r_cu,
+                                                                 int* host_counts) {
+  __shared__ int s_u[kSetWarps], s_r[kSetWarps], s_base[kSetWarps];
+  __shared__ int s_pub[2];                                    // this slice's totals, read by the cluster
   const int B = rt.n_req;
-  const int b = blockIdx.x % B, s = blockIdx.x / B;
+  const int slice = (int)blockIdx.x % kSetSlices, list = (int)blockIdx.x / kSetSlices;
+  const int b = list % B, s = list / B;
   const int T = rt.ctx_len[b];
   const int* hb = h + rt.ctx_cu[b];
   const int thr = (s == 0) ? 0 : (s - 1);
-  const int per = (T + kSetThreads - 1) / kSetThreads;
-  const int i0 = min(T, (int)threadIdx.x * per), i1 = min(T, i0 + per);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int per = ((T + kSetSlices - 1) / kSetSlices + 31) & ~31;
+  const int p0 = min(T, slice * per), p1 = min(T, p0 + per);
+  const int run = ((p1 - p0 + kSetWarps - 1) / kSetWarps + 31) & ~31;      // a contiguous run of positions per warp
+  const int i0 = min(p1, p0 + warp * run), i1 = min(p1, i0 + run);
+  griddep_launch();
+  griddep_wait();
   int nu = 0, nr = 0;
-  for (int i = i0; i < i1; ++i) { const int v = hb[i]; nu += (v >= 0); nr += (v >= thr); }
-  int eu, er, tu, tr;
-  block_scan2(nu, nr, eu, er, tu, tr);
-  if (s == 0) {
-    int* up = u_pos + u_cu[b];
-    int* ur = u_rank + rt.ctx_cu[b];
-    for (int i = i0; i < i1; ++i) {
-      if (hb[i] >= 0) { up[eu] = i; ur[i] = eu; ++eu; } else ur[i] = -1;
-    }
-  } else {
-    int* rr = r_rank + r_cu[(s - 1) * B + b];
-    for (int i = i0; i < i1; ++i) {
-      const int v = hb[i];
-      if (v >= thr) rr[er++] = eu;     // rank in U of this position = members of U before it
-      if (v >= 0) ++eu;
-    }
+#pragma unroll 8
+  for (int i = i0 + lane; i < i1; i += 32) { const int v = hb[i]; nu += (v >= 0); nr += (v >= thr); }
+  // the list's place: counts of the lists before it
+  const int* cnt = s == 0 ? counts : counts + B;
+  const int idx = s == 0 ? b : (s - 1) * B + b;
+  int base = 0;
+  for (int i = threadIdx.x; i < idx; i += kSetThreads) base += cnt[i];
+  nu = warp_reduce_sum(nu); nr = warp_reduce_sum(nr); base = warp_reduce_sum(base);
+  if (lane == 0) { s_u[warp] = nu; s_r[warp] = nr; s_base[warp] = base; }
+  __syncthreads();
+  const int wu = s_u[lane], wr = s_r[lane];
+  base = warp_reduce_sum(s_base[lane]);
+  int eu = warp_reduce_sum(lane < warp ? wu : 0), er = warp_reduce_sum(lane < warp ? wr : 0);
+  if (warp == 0) {
+    const int tu = warp_reduce_sum(wu), tr = warp_reduce_sum(wr);
+    if (lane == 0) { s_pub[0] = tu; s_pub[1] = tr; }
   }
+  ptx::cluster_sync();
+  int gu = 0, gr = 0;                                         // lane r fetches the totals of slice r
+  if (lane < slice) {
+    gu = ptx::ld_cluster_s32(ptx::mapa_shared(ptx::smem_u32(&s_pub[0]), (uint32_t)lane));
+    gr = ptx::ld_cluster_s32(ptx::mapa_shared(ptx::smem_u32(&s_pub[1]), (uint32_t)lane));
+  }
+  eu += warp_reduce_sum(gu); er += warp_reduce_sum(gr);
+
+  if (slice == 0 && threadIdx.x == 0) {
+    const int n = cnt[idx];
+    if (s == 0) { u_cu[b] = base; if (b == B - 1) u_cu[B] = base + n; }
+    else { r_cu[idx] = base; if (idx == n_layers * B - 1) r_cu[idx + 1] = base + n; }
+  }
+  if (host_counts != nullptr && blockIdx.x == 0)
+    for (int i = threadIdx.x; i < B + n_layers * B; i += kSetThreads) host_counts[i] = counts[i];
+  const uint32_t below = (1u << lane) - 1u;
+  int* ur = u_rank + rt.ctx_cu[b];
+  int* dst = s == 0 ? u_pos + base : r_rank + base;
+  for (int i = i0; i < i1; i += 32) {
+    const bool in = i + lane < i1;
+    const int v = in ? hb[i + lane] : -1;
+    const uint32_t mu = __ballot_sync(0xffffffffu, v >= 0), mr = __ballot_sync(0xffffffffu, in && v >= thr);
+    const int rank = eu + __popc(mu & below);                 // members of U before this position
+    if (s == 0) {
+      if (v >= 0) dst[rank] = i + lane;
+      if (in) ur[i + lane] = v >= 0 ? rank : -1;
+    } else if (in && v >= thr) {
+      dst[er + __popc(mr & below)] = rank;
+    }
+    eu += __popc(mu); er += __popc(mr);
+  }
+  ptx::cluster_sync();                                        // nobody leaves while a peer may still read its totals
 }
 
 }  // namespace relaxkv
@@ -144,20 +147,31 @@ static relaxkv_status build_sets(const relaxkv_shape* shape, int32_t n_layers, c
   fill_req_table(rt, shape, nullptr, h_k);
   const int B = shape->n_req;
   const long long sum_t = rt.ctx_cu[B];
-  // Nothing in `counts` has to start at zero: count_sets_kernel overwrites every entry that prefix_counts_kernel
-  // and the copy below read.
-  fill_i32_kernel<<<(unsigned)((sum_t + 255) / 256), 256, 0, stream>>>(highest_layer_out, sum_t, -1);
+  // The caller's counts are written by the last kernel where the device can reach them (pinned memory: a copy behind it
+  // would cost another 8 us of a schedule's 15), else by a copy.
+  int* host_counts = nullptr;
+  if (h_counts_pinned) {
+    cudaPointerAttributes attr;
+    if (cudaPointerGetAttributes(&attr, h_counts_pinned) != cudaSuccess) (void)cudaGetLastError();
+    else if (attr.type == cudaMemoryTypeHost) host_counts = static_cast<int*>(attr.devicePointer);
+  }
+  // Nothing in `counts` has to start at zero: count_sets_kernel overwrites every entry that write_sets_kernel and the
+  // copy below read.
   const long long n_anchor = (long long)n_layers * rt.k_cu[B];
-  highest_layer_kernel<<<(unsigned)((n_anchor + 255) / 256), 256, 0, stream>>>(rt, n_layers, anchors,
-                                                                              highest_layer_out, st);
-  const unsigned blocks = (unsigned)(B * (n_layers + 1));
-  count_sets_kernel<<<blocks, kSetThreads, 0, stream>>>(rt, n_layers, highest_layer_out, counts);
-  prefix_counts_kernel<<<1, 64, 0, stream>>>(B, n_layers, counts, u_cu_out, r_cu_out);
-  write_sets_kernel<<<blocks, kSetThreads, 0, stream>>>(rt, n_layers, highest_layer_out, u_cu_out, r_cu_out,
-                                                        u_pos_out, u_rank_out, r_rank_out);
-  relaxkv_status rc = launch_ok();
+  const unsigned lists = (unsigned)(B * (n_layers + 1));
+  cudaError_t e = launch_chained(true, fill_i32_kernel, dim3((unsigned)((sum_t + 255) / 256)), dim3(256), 0, stream,
+                                 highest_layer_out, sum_t, -1);
+  if (e == cudaSuccess)
+    e = launch_chained(true, highest_layer_kernel, dim3((unsigned)((n_anchor + 255) / 256)), dim3(256), 0, stream, rt, n_layers,
+                       anchors, highest_layer_out, st);
+  if (e == cudaSuccess)
+    e = launch_chained(true, count_sets_kernel, dim3(lists), dim3(kSetThreads), 0, stream, rt, n_layers, highest_layer_out, counts);
+  if (e == cudaSuccess)
+    e = launch_chained_clusters(true, kSetSlices, write_sets_kernel, dim3(lists * kSetSlices), dim3(kSetThreads), 0, stream, rt,
+                                n_layers, highest_layer_out, counts, u_pos_out, u_cu_out, u_rank_out, r_rank_out, r_cu_out, host_counts);
+  relaxkv_status rc = cuda_ok(e);
   if (rc != RELAXKV_OK) return rc;
-  if (h_counts_pinned)
+  if (h_counts_pinned && !host_counts)
     rc = cuda_ok(cudaMemcpyAsync(h_counts_pinned, counts, sizeof(int) * (size_t)(B + n_layers * B),
                                  cudaMemcpyDeviceToHost, stream));
   return rc;

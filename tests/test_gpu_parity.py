@@ -149,6 +149,50 @@ def test_active_sets_bitexact(case):
             prev = set(got.tolist())
 
 
+@pytest.mark.parametrize("ctx", [(1,), (31, 33), (4096,), (4097, 1, 640), (8193, 20000), (16385,), (40000, 7), (196609,)])
+def test_selection_and_schedule_at_slice_edges(ctx):
+    """Top-k, MinMax and the schedule where the slices of a segment (1, 2, 4 or 8 blocks), their warps' runs and the keys kept in
+    shared memory (196609 is past them) begin and end: bit-exact on scores with ties, both signs, zeros and infinities."""
+    from paper_2609_33503_b200.pipeline import RepairSession
+    rng = np.random.default_rng(sum(ctx))
+    L, nb = 3, len(ctx)
+    cu = np.concatenate([[0], np.cumsum(ctx)])
+    raw = np.empty((L, cu[-1]), dtype=np.float32)
+    raw[0] = np.exp(rng.standard_normal(cu[-1])) / cu[-1]
+    raw[1] = np.round(rng.standard_normal(cu[-1]) * 3) / 4                 # many ties, both signs and zeros
+    raw[2] = rng.standard_normal(cu[-1])
+    raw[2, ::3] = -np.inf
+    raw[2, ::5] = np.inf
+    for k in ([1] * nb, [max(1, round(0.15 * t)) for t in ctx], list(ctx)):
+        s = RepairSession(8, 2, 128, ctx, [1] * nb, L, k)
+        d_raw = torch.from_numpy(raw).cuda()
+        d_norm = torch.empty_like(d_raw)
+        B().relaxkv_select_topk(s.shape, L, s.k, d_raw, s.anchors, norm_scores_out=d_norm)
+        s.build_active_sets()
+        n_u, n_r = s.counts()
+        assert_status_ok()
+        anchors, norm = s.anchors.cpu().numpy(), d_norm.cpu().numpy()
+        k_cu = np.concatenate([[0], np.cumsum(k)])
+        u_cu, r_cu, r_rank = s.u_cu.cpu().numpy(), s.r_cu.cpu().numpy(), s.r_rank.cpu().numpy()
+        for b in range(nb):
+            seg = slice(cu[b], cu[b + 1])
+            want = [orc.topk(raw[l, seg].astype(np.float64), k[b]) for l in range(L)]
+            for l in range(L):
+                np.testing.assert_array_equal(anchors[l, k_cu[b]:k_cu[b + 1]], want[l])
+                if l < 2:                                                  # the same fp32 arithmetic: the same bits
+                    x = raw[l, seg]
+                    rng_x = x.max() - x.min()
+                    np.testing.assert_array_equal(norm[l, seg], (x - x.min()) / rng_x if rng_x > 0 else np.zeros_like(x))
+            ref = orc.active_sets(np.stack(want), ctx[b])
+            assert n_u[b] == len(ref.u_pos) == u_cu[b + 1] - u_cu[b]
+            np.testing.assert_array_equal(s.u_pos[u_cu[b]:u_cu[b + 1]].cpu().numpy(), ref.u_pos)
+            np.testing.assert_array_equal(s.u_rank[cu[b]:cu[b + 1]].cpu().numpy(), ref.u_rank)
+            for l in range(L):
+                got = r_rank[r_cu[l * nb + b]:r_cu[l * nb + b + 1]]
+                assert n_r[l][b] == len(got)
+                np.testing.assert_array_equal(got, ref.ranks(l))
+
+
 # --------------------------------------------------------------------- gather / scatter ----
 
 @pytest.mark.parametrize("head_major", [False, True])
