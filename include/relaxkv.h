@@ -348,10 +348,10 @@ relaxkv_status relaxkv_rmsnorm(const void* x, const void* weight, void* y, int64
 
 /* y = x weight^T (+ residual)      x [n_rows, n_in], weight [n_out, n_in] (the [out, in] layout),
  * residual NULL or [n_rows, n_out], y [n_rows, n_out] (may alias residual).  tcgen05 GEMM: 256-row tiles on SM pairs
- * for many rows; for 5 to 128 rows (the query's own tokens) 128 x 128 tiles whose K range is split over a
- * thread-block cluster and summed through distributed shared memory in a fixed order, so that all SMs stream
- * weights; calls of one to four rows (a decode token, the row that goes through the output head) stream the
- * weights once through a plain HBM-bound kernel instead. */
+ * for many rows; up to 128 rows (the query's own tokens, a decoded batch) 128 weight rows against all rows of x,
+ * K split over a thread-block cluster and summed through distributed shared memory in a fixed order, so that
+ * all SMs stream weights; one row (a decode token, the row that goes through the output head), and two to four
+ * with a short K, stream the weights once through a plain HBM-bound kernel instead. */
 relaxkv_status relaxkv_linear(const void* x, const void* weight, const void* residual, void* y,
                               int64_t n_rows, int32_t n_out, int32_t n_in, relaxkv_stream stream);
 
@@ -453,8 +453,8 @@ relaxkv_status relaxkv_debug_wait_timeout(relaxkv_stream stream);
 
 /*
  * Chained launches.  The short kernels of a decode step (RMSNorm, norm + rotary and the cache append
- * of at most 8 rows, the one- to four-row projections, the one-token attention and its merge) are
- * launched with CUDA's programmatic stream serialization: the next kernel's blocks become resident
+ * of at most 8 rows, the projections of up to 128 rows, the one-token attention and its merge), the
+ * top-k and the kernels of the schedule are launched with CUDA's programmatic stream serialization: the next kernel's blocks become resident
  * while the current kernel finishes, request the head of their weights into L2 (weights depend on
  * no earlier kernel) and then wait, inside the kernel, until every earlier kernel of the stream has
  * completed and its writes are visible.  Results are identical to plain

@@ -1,18 +1,28 @@
-// y = x W^T (+ residual) for at most 128 rows of x (the query's own tokens going through the block, Section 2 of the
-// paper: the query pass that yields the scores, and the query prefill that closes the time-to-first-token region).
-// With one row tile the 128 x 256 tiling of the large GEMM leaves most SMs without work (a 5120-wide projection is 20
-// tiles) and the time is the weight matrix streaming through those few SMs.  Here the tile is 128 x 128 and a
-// thread-block CLUSTER of S blocks (S = 1..8, chosen so that the launch is one wave of about all SMs) shares it and
-// splits K: block r multiplies K blocks [r n_k / S, (r + 1) n_k / S) into its own TMEM accumulator (six-stage TMA
-// ring, tcgen05.mma M=128 N=128 K=16), writes the partial tile into its own shared memory, and after a cluster
-// barrier every block sums, for the 8-column groups it owns (group g belongs to block g mod S), the S partials in rank
-// order - its own from local, the others' through distributed shared memory - adds the residual and writes bf16.
-// A fixed order: results do not depend on timing.  No scratch in global memory.
-// Up to three output segments (column ranges going to different buffers) serve the fused Q/K/V projection.
+// y = x W^T (+ residual) for at most 128 rows of x: the query's own tokens going through the block (Section 2 of the
+// paper: the query pass that yields the scores, and the query prefill that closes the time-to-first-token region) and the
+// decoded tokens of a batch.  The work is streaming the weight matrix once, so the weights are the M side of the MMA:
+// a tile is 128 weight rows (TMEM lanes = output features) against all rows of x (N = 16 ... 128 columns, the row count
+// rounded up to 16), and a thread block holds half an SM's shared memory as a TMA ring of 64-wide K blocks (a
+// whole SM's above 64 rows, where x takes as much of a stage as the weights).  128 to 192 KB of weights per SM are in
+// flight, and x rows that do not exist are neither multiplied nor, past the 16
+// granularity, staged.  A thread-block CLUSTER of S blocks shares a tile and splits K: block r multiplies K blocks
+// [r n_k / S, (r + 1) n_k / S) into its own TMEM accumulator, writes the partial tile into its own shared memory, and
+// after a cluster barrier every block sums, for the 128 / S features it owns, the S
+// partials in rank order - through distributed shared memory - adds the residual and writes bf16.  A fixed order: results
+// do not depend on timing.  No scratch in global memory.
+// Up to three output segments (feature ranges going to different buffers) serve the fused Q/K/V projection; the fused
+// gate/up projection takes 64 gate rows and their 64 up rows as one tile and applies the activation in the epilogue.
+// Bound by HBM (N K 2 bytes); with 128 rows of x as the M side, one block per SM and plain launches, four rows of a decode
+// step went through the FMA pipe (gate/up 34816 x 5120 77 us, 5120 x 17408 40 us, 6144 x 4096 13.6 us; now 56, 32 and 12.2:
+// 6.2, 5.6 and 4.1 TB/s), 57 rows took 65 / 36 / 16.2 us (now 59 / 34 / 13.8) and 128 rows 65 / 37.7 / 17.2 us (64 / 37.8 /
+// 17.4, and 2 to 3 us less behind a short kernel, where the start is hidden).
+// Launched chained: barriers, tensor memory and an L2 prefetch of the ring's first weight tiles come before the wait for
+// the kernels in front (a prefetch only: the weights are read after the wait, whoever wrote them).
 // The cluster barriers have no time limit, so every thread executes all of them whatever its (bounded) waits on the
 // mbarriers have returned, and no block leaves before its peers have read its partial tile.
 #include "common.cuh"
 #include "gemm_skinny.cuh"
+#include "gemv.cuh"
 #include "sm100_ptx.cuh"
 #include <algorithm>
 #include <atomic>
@@ -24,99 +34,126 @@ using namespace ptx;
 bool make_map_3d(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t stride1_bytes,
                  uint64_t stride2_bytes, uint32_t b1, uint32_t b2);          // attention_sm100.cu
 
-constexpr int kSkBM = 128, kSkBN = 128, kSkBK = 64, kSkStages = 6, kSkThreads = 192;
-constexpr int kSkABytes = kSkBM * kSkBK * 2, kSkBBytes = kSkBN * kSkBK * 2;
-constexpr int kSkStageBytes = kSkABytes + kSkBBytes;                       // 32 KB
-constexpr int kSkBars = 2 * kSkStages + 1;                                 // full, empty per stage; accumulator full
-constexpr int kSkSmem = kSkStages * kSkStageBytes + 8 * kSkBars + 16 + 1024;
-static_assert(kSkBM * kSkBN * 4 <= kSkStages * kSkStageBytes, "the partial tile reuses the TMA ring");
+constexpr int kSkFeat = 128, kSkBK = 64, kSkThreads = 192, kSkStagesMax = 7;
+constexpr int kSkWBytes = kSkFeat * kSkBK * 2;                             // weights of a stage: 16 KB, as two 64-row boxes
+constexpr int kSkRing2 = 108 * 1024, kSkRing1 = 192 * 1024;                // two blocks, one block per SM
+constexpr int kSkCols2 = 64;                                               // widest MMA that always takes the two-block form
+constexpr int kSkPitch = kSkFeat + 4;                                      // floats per staged row: 16-byte reads of 8 rows hit all banks
+constexpr int kSkDeepK = 8192;                                             // few rows: K from which eight blocks share a tile
+constexpr int kSkBars = 2 * kSkStagesMax + 1;                              // full, empty per stage; accumulator full
+constexpr int kSkTail = 8 * kSkBars + 16 + 1024;                           // barriers, slots, alignment
+constexpr int sk_stages(int n_cols, bool whole_sm) { return (whole_sm ? kSkRing1 : kSkRing2) / (kSkWBytes + n_cols * kSkBK * 2); }
+static_assert(sk_stages(16, false) <= kSkStagesMax && sk_stages(kSkCols2 + 16, true) <= kSkStagesMax, "barriers for every stage");
+static_assert(kSkinnyMaxRows * kSkPitch * 4 <= sk_stages(kSkinnyMaxRows, false) * (kSkWBytes + kSkinnyMaxRows * kSkBK * 2),
+              "the partial tile reuses the TMA ring");
 
-__device__ __forceinline__ float ld_cluster_f32(uint32_t cluster_addr) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr) : "memory");
+__device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t cluster_addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(cluster_addr));
   return v;
 }
 
 template <int S>
-__global__ void __launch_bounds__(kSkThreads, 1)
-gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
-                         int M, int N, int K, const __grid_constant__ SkinnyOut outs, DeviceStatus* st) {
+__global__ void __launch_bounds__(kSkThreads, 2)
+gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
+                         int M, int n_cols, int n_stages, int n_feat, int K, int swiglu, const __grid_constant__ SkinnyOut outs,
+                         DeviceStatus* st) {
   const uint32_t rank = (S > 1) ? cluster_ctarank() : 0u;
-  const int tn = (int)(blockIdx.x / S);
+  const int tile = (int)(blockIdx.x / S);
   const int n_k = (K + kSkBK - 1) / kSkBK;
   const int k0 = (int)((long long)rank * n_k / S), k1 = (int)((long long)(rank + 1) * n_k / S);
-  // after an expired wait elsewhere the tensor-core kernels move nothing until the status word has been read; here
-  // that means: run through the barriers (a block must not leave its cluster waiting), compute nothing
-  const bool drained = *reinterpret_cast<volatile int*>(&st->status) == RELAXKV_ERR_TIMEOUT;
+  // the weight rows of this tile: two boxes of 64
+  const int f0 = swiglu ? tile * (kSkFeat / 2) : tile * kSkFeat;            // first output feature
+  const int r0 = swiglu ? (f0 / 128) * 256 + f0 % 128 : f0, r1 = swiglu ? r0 + 128 : r0 + kSkFeat / 2;
 
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
-  const uint32_t bar0 = base + kSkStages * kSkStageBytes;
-  const uint32_t bar_full = bar0, bar_empty = bar0 + 8 * kSkStages, bar_acc = bar0 + 16 * kSkStages;
-  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + kSkStages * kSkStageBytes + 8 * kSkBars);
+  const uint32_t stage_bytes = (uint32_t)(kSkWBytes + n_cols * kSkBK * 2), ring = stage_bytes * (uint32_t)n_stages;
+  const uint32_t bar0 = base + ring;
+  const uint32_t bar_full = bar0, bar_empty = bar0 + 8 * kSkStagesMax, bar_acc = bar0 + 16 * kSkStagesMax;
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + ring + 8 * kSkBars);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(const_cast<uint32_t*>(tmem_slot) + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t tmem_cols = n_cols <= 32 ? 32u : (n_cols <= 64 ? 64u : 128u);
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kSkStages; ++s) { mbar_init(bar_full + 8 * s, 1); mbar_init(bar_empty + 8 * s, 1); }
+    for (int s = 0; s < n_stages; ++s) { mbar_init(bar_full + 8 * s, 1); mbar_init(bar_empty + 8 * s, 1); }
     mbar_init(bar_acc, 1);
-    *abort_flag = drained ? 1 : 0;
+    *abort_flag = 0;
     fence_barrier_init();
     fence_proxy_async_smem();
   }
-  if (warp == 5) { tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), kSkBN); tmem_relinquish(); }
+  if (warp == 4 && lane == 0) {
+    prefetch_tensormap(&tm_w); prefetch_tensormap(&tm_x);
+    for (int kt = k0; kt < min(k1, k0 + n_stages); ++kt) {
+      tma_prefetch_3d(&tm_w, kt * kSkBK, r0, 0);
+      if (swiglu || r1 < n_feat) tma_prefetch_3d(&tm_w, kt * kSkBK, r1, 0);
+    }
+  }
+  if (warp == 5) { tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), tmem_cols); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  // Only now that this block has its tensor memory may the next kernel's blocks come (they allocate some themselves).
+  // All blocks of a one-wave launch are resident by then, so the next kernel only takes room that is left over.
+  griddep_launch();
+  griddep_wait();
+  // after an expired wait elsewhere the tensor-core kernels move nothing until the status word has been read; here
+  // that means: run through the barriers (a block must not leave its cluster waiting), compute nothing
+  if (threadIdx.x == 0 && *reinterpret_cast<volatile int*>(&st->status) == RELAXKV_ERR_TIMEOUT) *abort_flag = 1;
+  __syncthreads();
+  const bool drained = *abort_flag != 0;
+  __syncthreads();
 
-  bool ok = !*abort_flag;
+  bool ok = !drained;
   if (warp == 4) {
     // ---- TMA producer ----
     if (lane == 0 && ok) {
-      prefetch_tensormap(&tm_a); prefetch_tensormap(&tm_b);
-      for (int kt = k0, it = 0; kt < k1; ++kt, ++it) {
-        const int s = it % kSkStages;
-        if (it >= kSkStages && !mbar_wait(bar_empty + 8 * s, (uint32_t)((it / kSkStages) - 1) & 1, abort_flag)) break;
-        mbar_expect_tx(bar_full + 8 * s, kSkStageBytes);
-        tma_load_3d(base + s * kSkStageBytes, &tm_a, bar_full + 8 * s, kt * kSkBK, 0, 0);
-        tma_load_3d(base + s * kSkStageBytes + kSkABytes, &tm_b, bar_full + 8 * s, kt * kSkBK, tn * kSkBN, 0);
+      for (int kt = k0, it = 0, s = 0, ph = 0; kt < k1; ++kt, ++it) {
+        if (it >= n_stages && !mbar_wait(bar_empty + 8 * s, (uint32_t)(ph ^ 1), abort_flag)) break;
+        const uint32_t dst = base + (uint32_t)s * stage_bytes;
+        mbar_expect_tx(bar_full + 8 * s, stage_bytes);
+        tma_load_3d(dst, &tm_w, bar_full + 8 * s, kt * kSkBK, r0, 0);
+        tma_load_3d(dst + kSkWBytes / 2, &tm_w, bar_full + 8 * s, kt * kSkBK, r1, 0);
+        tma_load_3d(dst + kSkWBytes, &tm_x, bar_full + 8 * s, kt * kSkBK, 0, 0);
+        if (++s == n_stages) { s = 0; ph ^= 1; }
       }
     }
   } else if (warp == 5) {
     // ---- MMA issuer ----
     if (lane == 0 && ok) {
-      constexpr uint32_t idesc = idesc_bf16_f32(kSkBM, kSkBN, 0);
+      const uint32_t idesc = idesc_bf16_f32(kSkFeat, n_cols, 0);
       bool go = true;
-      for (int kt = k0, it = 0; kt < k1; ++kt, ++it) {
-        const int s = it % kSkStages;
-        if (!(go = mbar_wait(bar_full + 8 * s, (uint32_t)(it / kSkStages) & 1, abort_flag))) break;
+      for (int kt = k0, it = 0, s = 0, ph = 0; kt < k1; ++kt, ++it) {
+        if (!(go = mbar_wait(bar_full + 8 * s, (uint32_t)ph, abort_flag))) break;
         tc_fence_after();
-        const uint32_t sa = base + s * kSkStageBytes;
-        mma_ss_4steps(tmem_base, desc_lo(sa, 16), desc_lo(sa + kSkABytes, 16), desc_hi_sw128(1024), idesc, it > 0 ? 1u : 0u);
+        const uint32_t sw = base + (uint32_t)s * stage_bytes;
+        mma_ss_4steps(tmem_base, desc_lo(sw, 16), desc_lo(sw + kSkWBytes, 16), desc_hi_sw128(1024), idesc, it > 0 ? 1u : 0u);
         mma_commit(bar_empty + 8 * s);
+        if (++s == n_stages) { s = 0; ph ^= 1; }
       }
       if (go) mma_commit(bar_acc);
     }
   } else {
-    // ---- epilogue warps (thread = row = TMEM lane): this block's partial tile -> its own shared memory, [column][row]
-    // fp32 (the lanes of a warp hold consecutive rows: every store below writes 128 consecutive bytes).  The MMAs have
-    // completed by then, so the TMA ring is free to hold it. ----
+    // ---- epilogue warps (thread = weight row = TMEM lane): this block's partial tile -> its own shared memory, [row of x]
+    // [feature] fp32 (the lanes of a warp hold consecutive features: every store below writes 128 consecutive bytes).
+    // The MMAs have completed by then, so the TMA ring is free to hold it. ----
     if (ok) ok = mbar_wait(bar_acc, 0, abort_flag);
     ok = __all_sync(0xffffffffu, ok);
     tc_fence_after();
     if (ok) {
-      const int row = warp * 32 + lane;
       const uint32_t t_lane = tmem_base + ((uint32_t)(warp * 32) << 16);
-      float* stage = reinterpret_cast<float*>(base_ptr);
+      float* stage = reinterpret_cast<float*>(base_ptr) + warp * 32 + lane;
 #pragma unroll 1
-      for (int c = 0; c < kSkBN / 32; ++c) {
+      for (int c = 0; c < M; c += 32) {
         uint32_t v[32];
-        tmem_ld32(t_lane + c * 32, v);
+        tmem_ld32(t_lane + c, v);
         tmem_wait_ld();
 #pragma unroll
-        for (int i = 0; i < 32; ++i) stage[(c * 32 + i) * kSkBM + row] = __uint_as_float(v[i]);
+        for (int i = 0; i < 32; ++i)
+          if (c + i < M) stage[(c + i) * kSkPitch] = __uint_as_float(v[i]);
       }
     }
   }
@@ -126,47 +163,64 @@ gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_
   ok = !*abort_flag;
 
   if (warp < 4 && ok) {
-    const int row = warp * 32 + lane;
-    const uint32_t stage_addr = base + (uint32_t)row * 4u;
     uint32_t peer[S];
 #pragma unroll
-    for (int src = 0; src < S; ++src) peer[src] = (S > 1) ? mapa_shared(stage_addr, (uint32_t)src) : stage_addr;
-    // 8-column groups g = rank, rank + S, ... of the tile
-#pragma unroll 1
-    for (int g = (int)rank; g < kSkBN / 8; g += S) {
-      const int col0 = tn * kSkBN + g * 8;
-      if (col0 >= N) break;
-      float f[8];
+    for (int src = 0; src < S; ++src) peer[src] = (S > 1) ? mapa_shared(base, (uint32_t)src) : base;
+    // this rank's run of the tile's features, four features of one row of x per thread and round: the lanes that share a
+    // row read up to 128 consecutive bytes of each peer (scattered 16-byte reads cost a tile of 128 rows another 8 us)
+    auto sum4 = [&](int m, int col) {
+      const uint32_t off = (uint32_t)(m * kSkPitch + col) * 4u;
+      float4 v[S];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) f[e] = 0.f;
+      for (int src = 0; src < S; ++src) v[src] = ld_cluster_f32x4(peer[src] + off);
+      float4 f = v[0];
 #pragma unroll
-      for (int src = 0; src < S; ++src) {                        // rank order: the same sum whatever the timing
-        float v[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = ld_cluster_f32(peer[src] + (uint32_t)((g * 8 + e) * kSkBM) * 4u);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) f[e] += v[e];
+      for (int src = 1; src < S; ++src) {                        // rank order: the same sum whatever the timing
+        f.x += v[src].x; f.y += v[src].y; f.z += v[src].z; f.w += v[src].w;
       }
-      if (row < M) {
-        // which output buffer these 8 columns go to (segment boundaries are multiples of 8 columns)
-        int sg = 0;
-        while (sg + 1 < outs.n && col0 >= outs.col0[sg + 1]) ++sg;
-        const int width = outs.col0[sg + 1] - outs.col0[sg];
-        const long long off = (long long)row * width + (col0 - outs.col0[sg]);
-        const uint16_t* res = outs.residual[sg];
-        if (res != nullptr) {
-          const uint4 r = __ldg(reinterpret_cast<const uint4*>(res + off));
-          const uint32_t rw[4] = {r.x, r.y, r.z, r.w};
+      return f;
+    };
+    const int all = (swiglu ? kSkFeat / 2 : kSkFeat) / 4, q0 = (int)rank * all / S, quads = ((int)rank + 1) * all / S - q0;
+    const int rows = 128 / quads, m0 = (int)threadIdx.x / quads;  // rows of x per round
+    const int col = (q0 + (int)threadIdx.x % quads) * 4, col0 = f0 + col;
+    // which output buffer these features go to (segment boundaries are multiples of 8)
+    int sg = 0;
+    while (sg + 1 < outs.n && col0 >= outs.col0[sg + 1]) ++sg;
+    const int width = outs.col0[sg + 1] - outs.col0[sg];
+    uint16_t* y = outs.y[sg] + (col0 - outs.col0[sg]);
+    const uint16_t* res = outs.residual[sg] ? outs.residual[sg] + (col0 - outs.col0[sg]) : nullptr;
+    if (m0 < rows && col0 < n_feat) {
+      constexpr int R = 4;                                       // rounds whose loads are in flight together
+      for (int mb = m0; mb < M; mb += R * rows) {
+        uint2 r[R];
+        float4 f[R], u[R];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) { f[2 * e] += __uint_as_float(rw[e] << 16); f[2 * e + 1] += __uint_as_float(rw[e] & 0xffff0000u); }
+        for (int j = 0; j < R; ++j) {
+          const int m = mb + j * rows;
+          r[j] = (res != nullptr && m < M) ? *reinterpret_cast<const uint2*>(res + (long long)m * width) : make_uint2(0u, 0u);
         }
-        uint32_t w[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          __nv_bfloat162 h2 = __floats2bfloat162_rn(f[2 * e], f[2 * e + 1]);
-          w[e] = *reinterpret_cast<uint32_t*>(&h2);
+        for (int j = 0; j < R; ++j) {
+          const int m = min(mb + j * rows, M - 1);
+          f[j] = sum4(m, col);
+          if (swiglu) u[j] = sum4(m, kSkFeat / 2 + col);
         }
-        *reinterpret_cast<uint4*>(outs.y[sg] + off) = make_uint4(w[0], w[1], w[2], w[3]);
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+          const int m = mb + j * rows;
+          if (m >= M) break;
+          float4 v = f[j];
+          if (swiglu) {                                          // one rounding, after the activation
+            v.x = v.x / (1.f + __expf(-v.x)) * u[j].x; v.y = v.y / (1.f + __expf(-v.y)) * u[j].y;
+            v.z = v.z / (1.f + __expf(-v.z)) * u[j].z; v.w = v.w / (1.f + __expf(-v.w)) * u[j].w;
+          }
+          if (res != nullptr) {
+            v.x += __uint_as_float(r[j].x << 16); v.y += __uint_as_float(r[j].x & 0xffff0000u);
+            v.z += __uint_as_float(r[j].y << 16); v.w += __uint_as_float(r[j].y & 0xffff0000u);
+          }
+          __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+          *reinterpret_cast<uint2*>(y + (long long)m * width) = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
+        }
       }
     }
   }
@@ -180,94 +234,98 @@ gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_
     while (global_timer_ns() - tw < 200000ull) __nanosleep(1000);
     __syncthreads();
   }
-  if (warp == 5) { tc_fence_after(); tmem_dealloc(tmem_base, kSkBN); }
+  if (warp == 5) { tc_fence_after(); tmem_dealloc(tmem_base, tmem_cols); }
 }
 
-// Largest number of S-block clusters of this kernel that can be resident at once (per device, looked up once).
+struct SkinnyPlan {
+  int n_rows, n_cols, n_stages, n_feat, n_in, swiglu, tiles, dev, sms;
+  bool whole_sm;                                                            // one block per SM, twice the stages
+  size_t smem;
+  DeviceStatus* st;
+  cudaStream_t stream;
+};
+
+template <int S>
+static bool opt_in_smem(int dev) {
+  static std::atomic<int> attr_done[kMaxDevices];
+  if (!attr_done[dev].load(std::memory_order_acquire)) {
+    if (cudaFuncSetAttribute(gemm_skinny_sm100_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSkRing1 + kSkTail) != cudaSuccess)
+      return false;
+    attr_done[dev].store(1, std::memory_order_release);
+  }
+  return true;
+}
+
+// Clusters of S blocks, one block per SM, that can be resident at once (per device, looked up once: a GPC's SMs are not a
+// multiple of every S).  0: error.
 template <int S>
 static int max_clusters(int dev, int sms) {
   static std::atomic<int> cached[kMaxDevices];
-  int n = cached[dev].load(std::memory_order_acquire);
+  int n = S == 1 ? sms : cached[dev].load(std::memory_order_acquire);
   if (n == 0) {
-    if (S == 1) {
-      n = sms;
-    } else {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)(sms / S * S));
-      cfg.blockDim = dim3(kSkThreads);
-      cfg.dynamicSmemBytes = kSkSmem;
-      cudaLaunchAttribute attr;
-      attr.id = cudaLaunchAttributeClusterDimension;
-      attr.val.clusterDim.x = (unsigned)S; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-      cfg.attrs = &attr;
-      cfg.numAttrs = 1;
-      if (cudaOccupancyMaxActiveClusters(&n, gemm_skinny_sm100_kernel<S>, &cfg) != cudaSuccess || n < 1) n = std::max(1, sms / S / 2);
-    }
+    if (!opt_in_smem<S>(dev)) return 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(sms / S * S));
+    cfg.blockDim = dim3(kSkThreads);
+    cfg.dynamicSmemBytes = kSkRing1 + kSkTail;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)S; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, gemm_skinny_sm100_kernel<S>, &cfg) != cudaSuccess || n < 1) n = std::max(1, sms / S / 2);
     cached[dev].store(n, std::memory_order_release);
   }
   return n;
 }
 
+// Launches with clusters of S blocks if that is one wave of resident blocks that have two K blocks each (or S is 1).
 template <int S>
-static bool prepare_s(int dev, int sms, int* n_clusters) {
-  static std::atomic<int> attr_done[kMaxDevices];
-  if (!attr_done[dev].load(std::memory_order_acquire)) {
-    if (cudaFuncSetAttribute(gemm_skinny_sm100_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSkSmem) != cudaSuccess)
-      return false;
-    attr_done[dev].store(1, std::memory_order_release);
-  }
-  *n_clusters = max_clusters<S>(dev, sms);
+static bool try_launch(const SkinnyPlan& p, const CUtensorMap& tm_w, const CUtensorMap& tm_x, const SkinnyOut& outs, relaxkv_status* rc) {
+  const int n_k = (p.n_in + kSkBK - 1) / kSkBK;
+  if (S > 1 && n_k < 2 * S) return false;
+  // with two blocks per SM an even cluster sits on S / 2 SMs (the occupancy query itself counts one block per SM)
+  const int resident = p.whole_sm ? max_clusters<S>(p.dev, p.sms) : (S % 2 ? 2 * max_clusters<S>(p.dev, p.sms) : max_clusters<(S + 1) / 2>(p.dev, p.sms));
+  if (resident < 1 || !opt_in_smem<S>(p.dev)) { *rc = RELAXKV_ERR_CUDA; return true; }
+  if (S > 1 && p.tiles > resident) return false;
+  *rc = cuda_ok(launch_chained_clusters(true, S, gemm_skinny_sm100_kernel<S>, dim3((unsigned)(p.tiles * S)), dim3(kSkThreads), p.smem,
+                                        p.stream, tm_w, tm_x, p.n_rows, p.n_cols, p.n_stages, p.n_feat, p.n_in, p.swiglu, outs, p.st));
   return true;
 }
 
-template <int S>
-static relaxkv_status launch_s(const CUtensorMap& tm_a, const CUtensorMap& tm_b, const SkinnyOut& outs, int n_rows, int n_out,
-                               int n_in, int tiles_n, DeviceStatus* st, cudaStream_t stream) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(tiles_n * S));
-  cfg.blockDim = dim3(kSkThreads);
-  cfg.dynamicSmemBytes = kSkSmem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = (unsigned)S; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, gemm_skinny_sm100_kernel<S>, tm_a, tm_b, n_rows, n_out, n_in, outs, st) != cudaSuccess)
-    return RELAXKV_ERR_CUDA;
-  return launch_ok();
-}
-
-int skinny_tiles(int n_out) { return (n_out + kSkBN - 1) / kSkBN; }
-
 relaxkv_status launch_gemm_skinny(const void* x, const void* weight, const SkinnyOut& outs, int n_rows, int n_out, int n_in,
-                                  cudaStream_t stream) {
+                                  int swiglu, cudaStream_t stream) {
   RELAXKV_RANGE("gemm_skinny_sm100_kernel");
-  CUtensorMap tm_a, tm_b;
-  if (!make_map_3d(&tm_a, x, (uint64_t)n_in, (uint64_t)n_rows, 1, (uint64_t)n_in * 2, (uint64_t)n_in * 2 * (uint64_t)n_rows, kSkBM, 1) ||
-      !make_map_3d(&tm_b, weight, (uint64_t)n_in, (uint64_t)n_out, 1, (uint64_t)n_in * 2, (uint64_t)n_in * 2 * (uint64_t)n_out, kSkBN, 1))
+  SkinnyPlan p = {};
+  p.n_rows = n_rows; p.n_in = n_in; p.swiglu = swiglu; p.stream = stream;
+  p.n_cols = (n_rows + 15) & ~15;                                            // N of the MMA
+  p.n_feat = swiglu ? n_out / 2 : n_out;
+  p.tiles = (n_out + kSkFeat - 1) / kSkFeat;                                 // also of the fused gate/up projection
+  CUtensorMap tm_w, tm_x;
+  if (!make_map_3d(&tm_w, weight, (uint64_t)n_in, (uint64_t)n_out, 1, (uint64_t)n_in * 2, (uint64_t)n_in * 2 * (uint64_t)n_out, kSkFeat / 2, 1) ||
+      !make_map_3d(&tm_x, x, (uint64_t)n_in, (uint64_t)n_rows, 1, (uint64_t)n_in * 2, (uint64_t)n_in * 2 * (uint64_t)n_rows, (uint32_t)p.n_cols, 1))
     return RELAXKV_ERR_CUDA;
-  DeviceStatus* st = status_word();
-  if (!st) return RELAXKV_ERR_CUDA;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return RELAXKV_ERR_CUDA;
-  const int sms = sm_count_of_current_device();
-  if (sms <= 0) return RELAXKV_ERR_CUDA;
-  const int tiles_n = skinny_tiles(n_out);
-  const int n_k = (n_in + kSkBK - 1) / kSkBK;
-  // the largest cluster whose launch is still one wave (all its clusters resident at once) and leaves every block at
-  // least two K blocks
-#define RELAXKV_TRY_S(SV)                                                                           \
-  if (n_k >= 2 * SV) {                                                                              \
-    int nc = 0;                                                                                     \
-    if (!prepare_s<SV>(dev, sms, &nc)) return RELAXKV_ERR_CUDA;                                      \
-    if (tiles_n <= nc) return launch_s<SV>(tm_a, tm_b, outs, n_rows, n_out, n_in, tiles_n, st, stream); \
-  }
-  RELAXKV_TRY_S(8) RELAXKV_TRY_S(7) RELAXKV_TRY_S(6) RELAXKV_TRY_S(5) RELAXKV_TRY_S(4) RELAXKV_TRY_S(3) RELAXKV_TRY_S(2)
-#undef RELAXKV_TRY_S
-  int nc = 0;
-  if (!prepare_s<1>(dev, sms, &nc)) return RELAXKV_ERR_CUDA;
-  return launch_s<1>(tm_a, tm_b, outs, n_rows, n_out, n_in, tiles_n, st, stream);
+  p.st = status_word();
+  if (!p.st || cudaGetDevice(&p.dev) != cudaSuccess || p.dev < 0 || p.dev >= kMaxDevices) return RELAXKV_ERR_CUDA;
+  p.sms = sm_count_of_current_device();
+  if (p.sms <= 0) return RELAXKV_ERR_CUDA;
+  // Above 64 rows two blocks of an SM would have three stages each; with no more tiles than SMs one block with six is
+  // faster (128 rows, 5120 x 17408: 38 against 43 us), with more tiles two (34816 x 5120: 63 against 73 us).
+  p.whole_sm = p.n_cols > kSkCols2 && p.tiles <= p.sms;
+  p.n_stages = sk_stages(p.n_cols, p.whole_sm);
+  p.smem = (size_t)p.n_stages * (kSkWBytes + p.n_cols * kSkBK * 2) + kSkTail;
+  relaxkv_status rc = RELAXKV_OK;
+  // the largest cluster that fits.  Up to four rows the choice goes by K alone, so that a projection has the same bits
+  // stacked with others and by itself.
+  const bool few = n_rows <= kGemvMaxRows, deep = n_in >= kSkDeepK;
+  if ((!few || deep) && try_launch<8>(p, tm_w, tm_x, outs, &rc)) return rc;
+  if (!few && (try_launch<7>(p, tm_w, tm_x, outs, &rc) || try_launch<6>(p, tm_w, tm_x, outs, &rc) || try_launch<5>(p, tm_w, tm_x, outs, &rc)))
+    return rc;
+  if (try_launch<4>(p, tm_w, tm_x, outs, &rc)) return rc;
+  if (!few && try_launch<3>(p, tm_w, tm_x, outs, &rc)) return rc;
+  if (try_launch<2>(p, tm_w, tm_x, outs, &rc)) return rc;
+  try_launch<1>(p, tm_w, tm_x, outs, &rc);
+  return rc;
 }
 
 }  // namespace relaxkv

@@ -417,6 +417,19 @@ gemm_pair_sm100_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
 
 using namespace relaxkv;
 
+// One to four rows: the plain streaming kernel or tensor-core tiles.  The streaming kernel has the shorter start but meets
+// every weight with a multiply-add per row on the FMA pipe, which is its bound from three rows on; the tiles' time hardly
+// depends on the rows.  By K alone, so that stacked and single projections take the same one.  Streaming / tiles, us:
+// one row 10.3 / 13.3 (5120 x 5120), 55 / 56 (gate/up 34816 x 5120); two rows 11.0 / 12.1 (6144 x 4096), 23 / 21 (4096 x
+// 14336), gate/up 9.4 / 8.7 (8192 x 2048), 44 / 40 (28672 x 4096); four rows 5.0 / 5.9 (2048 x 2048), 13.6 / 12.5
+// (6144 x 4096), 32 / 21 (4096 x 14336), gate/up 15.4 / 8.7 (8192 x 2048), 77 / 56 (34816 x 5120).
+static bool few_rows_stream(int64_t n_rows, int n_in, int swiglu) {
+  if (n_rows <= 1) return true;
+  if (n_rows > kGemvMaxRows) return false;
+  if (swiglu) return n_in < (n_rows == 2 ? 4096 : 2048);
+  return n_in < (n_rows == 2 ? 8192 : 4096);
+}
+
 static relaxkv_status launch_gemm(const void* x, const void* weight, const void* residual, void* y, int64_t n_rows,
                                   int32_t n_out, int32_t n_in, int swiglu, relaxkv_stream stream_,
                                   const GemmSegs* segs_in = nullptr) {
@@ -427,18 +440,15 @@ static relaxkv_status launch_gemm(const void* x, const void* weight, const void*
   if (n_rows < 0 || n_out < 8 || n_in < 8 || (n_out % 8) || (n_in % 8)) return RELAXKV_ERR_UNSUPPORTED_SHAPE;
   if (swiglu && ((n_out % 256) || residual)) return RELAXKV_ERR_UNSUPPORTED_SHAPE;
   if (n_rows == 0) return RELAXKV_OK;
-  if (n_rows <= kGemvMaxRows)       // a decode token: stream the weights once, no 128-row tiles
+  if (few_rows_stream(n_rows, n_in, swiglu))       // a decode token: stream the weights once, no tiles
     return launch_gemv(x, weight, residual, y, (int)n_rows, n_out, n_in, swiglu, static_cast<cudaStream_t>(stream_));
-  if (n_rows <= kSkinnyMaxRows && !swiglu && skinny_tiles(n_out) <= sm_count_of_current_device()) {
-    // one row tile and no more column tiles than SMs (the query's tokens through a 5120-wide projection): 128 x 128
-    // tiles, K split over a cluster so that about all SMs stream weights.  (The fused gate/up projection has 272 such
-    // tiles at the model shapes and keeps the large kernel.)
+  if (n_rows <= kSkinnyMaxRows) {   // the query's tokens, a decoded batch
     SkinnyOut outs = {};
     outs.y[0] = static_cast<uint16_t*>(y);
     outs.residual[0] = static_cast<const uint16_t*>(residual);
-    outs.col0[0] = 0; outs.col0[1] = n_out;
+    outs.col0[0] = 0; outs.col0[1] = swiglu ? n_out / 2 : n_out;
     outs.n = 1;
-    return launch_gemm_skinny(x, weight, outs, (int)n_rows, n_out, n_in, static_cast<cudaStream_t>(stream_));
+    return launch_gemm_skinny(x, weight, outs, (int)n_rows, n_out, n_in, swiglu, static_cast<cudaStream_t>(stream_));
   }
   // SM pairs (256-row tiles) unless that would leave a large share of the last tile row empty: with an odd number of
   // 128-row tiles, seven at most, the second block of the last pair would compute padding only (>= 1/8 of the work),
@@ -513,19 +523,19 @@ extern "C" relaxkv_status relaxkv_linear_qkv(const void* x, const void* w_qkv, v
   if (n_rows == 0) return RELAXKV_OK;
   const int n_out = n_q + 2 * n_kv;
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-  if (n_rows <= kGemvMaxRows) {
+  if (few_rows_stream(n_rows, n_in, 0)) {
     GemvOut outs = {};
     outs.y[0] = static_cast<uint16_t*>(q); outs.y[1] = static_cast<uint16_t*>(k); outs.y[2] = static_cast<uint16_t*>(v);
     outs.col0[0] = 0; outs.col0[1] = n_q; outs.col0[2] = n_q + n_kv; outs.col0[3] = n_out;
     outs.n = 3;
     return launch_gemv_segments(x, w_qkv, outs, (int)n_rows, n_out, n_in, stream);
   }
-  if (n_rows <= kSkinnyMaxRows && skinny_tiles(n_out) <= sm_count_of_current_device()) {
+  if (n_rows <= kSkinnyMaxRows) {
     SkinnyOut outs = {};
     outs.y[0] = static_cast<uint16_t*>(q); outs.y[1] = static_cast<uint16_t*>(k); outs.y[2] = static_cast<uint16_t*>(v);
     outs.col0[0] = 0; outs.col0[1] = n_q; outs.col0[2] = n_q + n_kv; outs.col0[3] = n_out;
     outs.n = 3;
-    return launch_gemm_skinny(x, w_qkv, outs, (int)n_rows, n_out, n_in, stream);
+    return launch_gemm_skinny(x, w_qkv, outs, (int)n_rows, n_out, n_in, 0, stream);
   }
   // many rows: one GEMM over the stacked matrix whose epilogue writes the three buffers (the K and V projections alone
   // have four 256-column tiles each and leave the last wave of SM pairs half empty) ...

@@ -1,5 +1,5 @@
-// Internal: the streaming kernel for projections of one to four rows (a decode token); relaxkv_linear and
-// relaxkv_linear_swiglu route there by the row count.
+// Internal: the streaming kernel for projections of one to four rows (a decode token); relaxkv_linear,
+// relaxkv_linear_qkv and relaxkv_linear_swiglu route there by the row count and K.
 #pragma once
 #include "common.cuh"
 

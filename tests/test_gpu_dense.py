@@ -100,6 +100,30 @@ def test_linear_of_a_few_rows(M, N, K, res):
     assert torch.equal(y, y2)
 
 
+@pytest.mark.parametrize("M,N,K,swiglu", [
+    (2, 264, 8200, False), (3, 1000, 4104, False), (4, 19208, 4096, False), (16, 136, 72, False), (64, 5128, 1032, False),
+    (65, 5128, 1032, False), (128, 37896, 136, False), (2, 256, 4104, True), (3, 512, 2056, True), (5, 256, 72, True),
+    (17, 1280, 520, True), (64, 512, 264, True), (65, 38144, 136, True), (128, 2048, 1032, True)])
+def test_weight_tiles_against_a_few_rows(M, N, K, swiglu):
+    """The 128-weight-row tiles at the edges of their choices: rows that fill and just pass an MMA width (16, 64), the two- and
+    the one-block form (64 / 65 rows), more tiles than blocks fit (150 and 297), one to eight blocks per tile (K from 72 to
+    8200), ragged last tiles and K blocks, and gate/up pairs; rows around the output stay untouched.  The fp32 sums of K
+    products of N(0,1) x N(0,1/K) err by less than 2e-3 absolute at these K in any order, a bf16 rounding on top."""
+    x, w = rnd(M, K, seed=51), rnd(N, K, scale=K ** -0.5, seed=52)
+    buf = torch.full((M + 2, N // 2 if swiglu else N), 7.0, dtype=torch.bfloat16, device="cuda")
+    y = buf[1:M + 1]
+    if swiglu:
+        B().relaxkv_linear_swiglu(x, B().tile_gate_up(w), y)
+        ref = blk.swiglu(blk.linear(blk.f64(bits(x)), blk.f64(bits(w)), None))
+    else:
+        B().relaxkv_linear(x, w, y)
+        ref = blk.linear(blk.f64(bits(x)), blk.f64(bits(w)), None)
+    st, detail = B().relaxkv_read_device_status()
+    assert st == 0, (st, detail)
+    close(y, ref, abs_floor=2e-3)
+    assert torch.all(buf[0] == 7.0) and torch.all(buf[M + 1] == 7.0)
+
+
 def test_linear_at_the_benchmark_shapes():
     """The projections at the sizes the repair loop runs them for the 32K Qwen3-14B-shaped stack: 18 000 active rows
     through a 5120 -> 5120 projection with residual (SM pairs) and the fused gate/up projection of 5120 -> 2 x 17408 on
