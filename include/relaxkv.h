@@ -452,9 +452,8 @@ relaxkv_status relaxkv_cache_attention(
 relaxkv_status relaxkv_debug_wait_timeout(relaxkv_stream stream);
 
 /*
- * Chained launches.  The short kernels of a decode step (RMSNorm, norm + rotary and the cache append
- * of at most 8 rows, the projections of up to 128 rows, the one-token attention and its merge), the
- * top-k and the kernels of the schedule are launched with CUDA's programmatic stream serialization: the next kernel's blocks become resident
+ * Chained launches.  The kernels of the calls above (all but the explicit-list maps and the score averages) are
+ * launched with CUDA's programmatic stream serialization: the next kernel's blocks become resident
  * while the current kernel finishes, request the head of their weights into L2 (weights depend on
  * no earlier kernel) and then wait, inside the kernel, until every earlier kernel of the stream has
  * completed and its writes are visible.  Results are identical to plain

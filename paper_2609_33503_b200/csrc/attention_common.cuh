@@ -12,7 +12,7 @@ struct AttnPlan {
   long long ctx_rows;     // rows the two buffers hold (tensor-map extent)
   long long sum_targets;  // sum of the host bounds on |R_{l,b}|
   float* split_o;         // workspace for a context split across blocks: [kSplitRowsCap, H, D] and [kSplitRowsCap, H]
-  float* split_lse;
+  float* split_lse;       // (its first word, zeroed by the gather, is the work counter of the persistent form)
   // what the attention kernel's K/V tensor maps cover: the materialised context, or the cache itself
   const void* k_base; const void* v_base;
   unsigned long long kv_token_stride_bytes, kv_head_stride_bytes;
@@ -67,7 +67,8 @@ inline relaxkv_status prepare_attention(
   plan.kv_token_stride_bytes = (unsigned long long)shape->n_kv_heads * shape->head_dim * 2;
   plan.dense_ctx = 0;
   return launch_gather(shape, mode, cache, k_new, v_new, u_pos, u_cu, r_rank, r_cu_layer, fresh_row,
-                       fresh_row ? need_ctx : 0, n_target_rows, need_ctx + kCtxPadRows, plan.kctx, plan.vctx, plan.ctx_rows, stream);
+                       fresh_row ? need_ctx : 0, n_target_rows, need_ctx + kCtxPadRows, plan.kctx, plan.vctx, plan.ctx_rows,
+                       reinterpret_cast<int*>(plan.split_lse), stream);
 }
 
 }  // namespace relaxkv

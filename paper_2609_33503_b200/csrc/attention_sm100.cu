@@ -147,8 +147,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                        const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ ReqTable rt,
                        int mode, int allow_empty, int head_inner, int dense_ctx, int H, int Hkv, int tile_targets, float scale_log2,
-                       const int* __restrict__ u_pos, const int* __restrict__ u_cu,
-                       const int* __restrict__ r_rank, const int* __restrict__ r_cu,
+                       const int* u_pos, const int* u_cu, const int* r_rank, const int* r_cu,
                        long long n_target_rows, uint16_t* __restrict__ out, float* __restrict__ lse_out,
                        float* __restrict__ part_o, float* __restrict__ part_lse, DeviceStatus* st) {
   using L = AttnSmem<D>;
@@ -161,6 +160,7 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const int B = rt.n_req;
   const int G = H / Hkv;
   const int n_pairs_total = rt.tile_cu[B];
+  griddep_wait();
   // Block order.  Large contexts: KV head outermost, so one head's K/V stays in L2 while its tiles run.
   // Contexts that fit L2 whole (head_inner): tile pair outermost, so the longest tiles of every head start first.
   const int hd = head_inner ? (int)(blockIdx.x % Hkv) : (int)(blockIdx.x / n_pairs_total);
@@ -478,6 +478,7 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   }
 
   // ---- teardown ------------------------------------------------------------------------------------
+  griddep_launch();
   tc_fence_before();
   __syncthreads();
   if (*abort_flag) {
@@ -547,8 +548,7 @@ __device__ __forceinline__ void item_load(const int4* rec, WorkItem& it) {
 }
 
 __device__ __forceinline__ WorkItem decode_item(int id, const ReqTable& rt, int head_inner, int Hkv, int mode, int tile_targets,
-                                                const int* __restrict__ u_pos, const int* __restrict__ u_cu,
-                                                const int* __restrict__ r_rank, const int* __restrict__ r_cu,
+                                                const int* u_pos, const int* u_cu, const int* r_rank, const int* r_cu,
                                                 long long n_target_rows, DeviceStatus* st) {
   WorkItem it;
   it.work = 0; it.pad = 0;
@@ -600,14 +600,14 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                          const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ ReqTable rt,
                          int mode, int allow_empty, int head_inner, int H, int Hkv, int tile_targets, float scale_log2,
-                         const int* __restrict__ u_pos, const int* __restrict__ u_cu,
-                         const int* __restrict__ r_rank, const int* __restrict__ r_cu,
+                         const int* u_pos, const int* u_cu, const int* r_rank, const int* r_cu,
                          long long n_target_rows, uint16_t* __restrict__ out, float* __restrict__ lse_out,
                          int total_items, int* __restrict__ work_counter, DeviceStatus* st) {
   using L = PersistSmem<D>;
   constexpr int kHalves = L::kHalves;
   constexpr uint32_t kTmemCols = 512;
   const int G = H / Hkv;
+  griddep_wait();
   if (*reinterpret_cast<volatile int*>(&st->status) == RELAXKV_ERR_TIMEOUT) return;
 
   extern __shared__ uint8_t smem_raw[];
@@ -971,6 +971,7 @@ attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
     }
   }
 
+  griddep_launch();
   tc_fence_before();
   __syncthreads();
   if (*abort_flag) {
@@ -1040,8 +1041,8 @@ constexpr int kMaxCombineSplits = 1024;       // four warps x 4 KB of weights
 // Merges the partial results of a context split: out = sum_s w_s O_s / sum_s w_s with w_s = exp(lse_s - max lse).
 // One warp per (target row, query head); rows past the true target count are left alone.
 __global__ void __launch_bounds__(kCombineThreads)
-combine_splits_kernel(const float* __restrict__ part_o, const float* __restrict__ part_lse, int n_splits,
-                      long long n_target_rows, int H, int D, const int* __restrict__ r_cu, int n_req,
+combine_splits_kernel(const float* part_o, const float* part_lse, int n_splits,
+                      long long n_target_rows, int H, int D, const int* r_cu, int n_req,
                       uint16_t* __restrict__ out, float* __restrict__ lse_out) {
   // the splits' weights of this warp's (row, head): the lanes fetch the log-sum-exps side by side (a serial walk over
   // the splits would pay one memory latency per split), the sums below still run in split order
@@ -1102,7 +1103,7 @@ relaxkv_status launch_combine_splits(const float* part_o, const float* part_lse,
   if (warps <= 0) return RELAXKV_OK;
   if (n_splits > kMaxCombineSplits) return RELAXKV_ERR_UNSUPPORTED_SHAPE;
   constexpr int wpb = kCombineThreads / 32;
-  return cuda_ok(launch_chained(n_target_rows <= kChainedMaxRows, combine_splits_kernel, (unsigned)((warps + wpb - 1) / wpb), kCombineThreads, 0, stream, part_o,
+  return cuda_ok(launch_chained(combine_splits_kernel, (unsigned)((warps + wpb - 1) / wpb), kCombineThreads, 0, stream, part_o,
                                 part_lse, n_splits, (long long)n_target_rows, H, D, r_cu, n_req, static_cast<uint16_t*>(out), lse_out));
 }
 
@@ -1205,21 +1206,18 @@ static relaxkv_status launch_attention(const relaxkv_shape* shape, int mode, Att
         return RELAXKV_ERR_CUDA;
       pattr_done[dev].store(1, std::memory_order_release);
     }
-    int* counter = reinterpret_cast<int*>(plan.split_lse);          // unused by a one-split call: the work counter
-    if (cudaMemsetAsync(counter, 0, sizeof(int), stream) != cudaSuccess) return RELAXKV_ERR_CUDA;
+    int* counter = reinterpret_cast<int*>(plan.split_lse);          // unused by a one-split call; zeroed by the gather
     long long pgrid = std::min<long long>(grid, sms);
     if (tun && tun->attention_grid_blocks > 0) pgrid = std::min<long long>(grid, tun->attention_grid_blocks);
     RELAXKV_RANGE("attention_persist_kernel");
-    pk<<<(unsigned)pgrid, kAttnThreads, PersistSmem<D>::kDynamic, stream>>>(
+    return cuda_ok(launch_chained(pk, (unsigned)pgrid, kAttnThreads, PersistSmem<D>::kDynamic, stream,
         tm_q, tm_k, tm_v, plan.rt, mode, allow_empty, head_inner, H, Hkv, tile_targets, shape->softmax_scale * kLog2eA,
-        u_pos, u_cu, r_rank, r_cu_layer, n_target_rows, static_cast<uint16_t*>(out), lse_out, (int)grid, counter, st);
-    return launch_ok();
+        u_pos, u_cu, r_rank, r_cu_layer, n_target_rows, static_cast<uint16_t*>(out), lse_out, (int)grid, counter, st));
   }
   RELAXKV_RANGE("attention_sm100_kernel");
-  kern<<<dim3((unsigned)grid, (unsigned)n_splits), kAttnThreads, AttnSmem<D>::kDynamic, stream>>>(
+  relaxkv_status rc = cuda_ok(launch_chained(kern, dim3((unsigned)grid, (unsigned)n_splits), kAttnThreads, AttnSmem<D>::kDynamic, stream,
       tm_q, tm_k, tm_v, plan.rt, mode, allow_empty, head_inner, plan.dense_ctx, H, Hkv, tile_targets, shape->softmax_scale * kLog2eA,
-      u_pos, u_cu, r_rank, r_cu_layer, n_target_rows, static_cast<uint16_t*>(out), lse_out, plan.split_o, plan.split_lse, st);
-  relaxkv_status rc = launch_ok();
+      u_pos, u_cu, r_rank, r_cu_layer, n_target_rows, static_cast<uint16_t*>(out), lse_out, plan.split_o, plan.split_lse, st));
   if (rc != RELAXKV_OK || n_splits == 1) return rc;
   return launch_combine_splits(plan.split_o, plan.split_lse, (int)n_splits, n_target_rows, H, D, r_cu_layer, B, plan.sum_targets,
                                out, lse_out, stream);

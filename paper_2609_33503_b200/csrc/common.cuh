@@ -91,26 +91,27 @@ inline relaxkv_status launch_ok() { return cuda_ok(cudaGetLastError()); }
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // ---- chained launches (programmatic dependent launch) ------------------------------------
-// The short kernels of a decode step or of the query's pass (norms, one-row projections, appends, the one-token
-// attention and its merge) follow one another on a stream, each a few microseconds long, and between two of them the
-// device drains, launches and ramps up again.  Launched with the programmatic-serialization attribute, the next
+// The kernels of this library follow one another on a stream, many of them a few microseconds long, and between two of
+// them the device drains, launches and ramps up again: 1.5 to 2.5 us each (8 layers of a query pass over 8K of context, 13
+// launches per layer: 1609 us with plain launches of more than eight rows, 1539 us chained; the schedule of a repair and
+// the loop around it 1 to 3 %).  Launched with the programmatic-serialization attribute, the next
 // kernel's blocks become resident as soon as every block of the current one has called griddep_launch(); they may do
-// whatever does not depend on earlier kernels (set-up, prefetching their weights) and then block in griddep_wait()
+// whatever does not depend on earlier kernels (set-up, prefetching their weights into L2) and then block in griddep_wait()
 // until the earlier kernels have completed and their writes are visible.  Rules kept by every kernel that is launched
-// this way: nothing written by another kernel is read, and nothing at all is written, before griddep_wait(); every
-// block executes griddep_wait() (so a kernel never completes before its predecessors).  Both instructions do nothing
-// in a kernel that was launched the plain way.  Only launches of a few rows are chained (`few_rows`: at most
-// kChainedMaxRows): the same kernels at the query's 64-128 rows sit between large tensor-core launches that are
-// launched the plain way, where the attribute measured 0.3 us per launch slower, not faster.
+// this way: nothing written by another kernel is read, and nothing at all is written, before griddep_wait(); index lists
+// that come from an earlier kernel are read through pointers without __restrict__ (a read-only load may not be moved up past the wait); every
+// block executes griddep_wait() (so a kernel never completes before its predecessors).  A kernel that takes tensor memory
+// calls griddep_launch() only after it has got it: every block then holds its share before a later kernel's block can ask
+// for some on the same SM.  Short kernels call griddep_launch() first thing, the tensor-core kernels of many blocks when
+// a block is through with its work.  Both instructions do nothing in a kernel that was launched the plain way.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 bool chained_launch_enabled();           // process-wide switch (relaxkv_set_chained_launch), on by default
-constexpr long long kChainedMaxRows = 8;
 
 // cluster > 1: the grid's x dimension is made of clusters of that many blocks (grid.x is a multiple of it).
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_chained_clusters(bool few_rows, int cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block,
+inline cudaError_t launch_chained_clusters(int cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block,
                                            size_t smem, cudaStream_t stream, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
@@ -119,7 +120,7 @@ inline cudaError_t launch_chained_clusters(bool few_rows, int cluster, void (*ke
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = (few_rows && chained_launch_enabled()) ? 1 : 0;
+  attr[0].val.programmaticStreamSerializationAllowed = chained_launch_enabled() ? 1 : 0;
   attr[1].id = cudaLaunchAttributeClusterDimension;
   attr[1].val.clusterDim.x = (unsigned)cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
@@ -128,9 +129,9 @@ inline cudaError_t launch_chained_clusters(bool few_rows, int cluster, void (*ke
 }
 
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_chained(bool few_rows, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                                   Args&&... args) {
-  return launch_chained_clusters(few_rows, 1, kernel, grid, block, smem, stream, static_cast<Args&&>(args)...);
+  return launch_chained_clusters(1, kernel, grid, block, smem, stream, static_cast<Args&&>(args)...);
 }
 
 // Up to this many requests have their per-request scalars passed by value in kernel parameters.

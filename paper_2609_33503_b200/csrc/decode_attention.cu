@@ -314,7 +314,7 @@ static relaxkv_status launch_g(const CUtensorMap& tm_k, const CUtensorMap& tm_v,
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, DecSmem<D>::kDynamic) != cudaSuccess) return RELAXKV_ERR_CUDA;
     attr_done[dev].store(1, std::memory_order_release);
   }
-  return cuda_ok(launch_chained(true, kern, grid, kDecThreads, DecSmem<D>::kDynamic, stream, tm_k, tm_v, plan.rt,
+  return cuda_ok(launch_chained(kern, grid, kDecThreads, DecSmem<D>::kDynamic, stream, tm_k, tm_v, plan.rt,
                                 static_cast<const uint16_t*>(q), tgt_pos, tgt_cu, (long long)n_target_rows, H, Hkv, scale_log2,
                                 static_cast<uint16_t*>(out), lse_out, plan.split_o, plan.split_lse, st));
 }

@@ -85,6 +85,8 @@ rmsnorm_short_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict_
 __global__ void rope_kernel(uint16_t* __restrict__ x, long long rows, int heads, int D, const int* __restrict__ positions,
                             double log2_theta) {
   const int half = D / 2, groups = half / 8;
+  griddep_launch();
+  griddep_wait();
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= rows * groups) return;
   const int gi = (int)(idx % groups);
@@ -237,6 +239,8 @@ rmsnorm_rows_bulk_kernel(const uint16_t* __restrict__ x, const uint16_t* __restr
   __shared__ volatile int gave_up[kRowWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long row = (long long)blockIdx.x * kRowWarps + warp;
+  griddep_launch();
+  griddep_wait();
   if (row >= n_rows) return;
   const uint32_t row_bytes = (uint32_t)C * 2;
   uint8_t* mine = row_stage + (size_t)warp * row_bytes;
@@ -293,6 +297,8 @@ head_norm_rope_rows_bulk_kernel(uint16_t* __restrict__ q, uint16_t* __restrict__
   __shared__ volatile int gave_up[kRowWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long row = (long long)blockIdx.x * kRowWarps + warp;
+  griddep_launch();
+  griddep_wait();
   if (row >= n_rows) return;
   const uint32_t q_bytes = (uint32_t)Hq * D * 2, k_bytes = (uint32_t)Hkv * D * 2;
   uint8_t* mine = row_stage + (size_t)warp * (q_bytes + k_bytes);
@@ -391,6 +397,8 @@ head_norm_rope_rows_bulk_kernel(uint16_t* __restrict__ q, uint16_t* __restrict__
 
 // out[r, i] = silu(gu[r, i]) * gu[r, I + i]
 __global__ void swiglu_kernel(const uint16_t* __restrict__ gu, uint16_t* __restrict__ out, long long rows, int I) {
+  griddep_launch();
+  griddep_wait();
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int per_row = I / 8;
   if (idx >= rows * per_row) return;
@@ -405,9 +413,10 @@ __global__ void swiglu_kernel(const uint16_t* __restrict__ gu, uint16_t* __restr
 }
 
 // positions of the layer's active targets: pos[row] = u_pos[u_cu[b] + r_rank[r_cu[b] + rho]]
-__global__ void target_positions_kernel(ReqTable rt, const int* __restrict__ u_pos, const int* __restrict__ u_cu,
-                                        const int* __restrict__ r_rank, const int* __restrict__ r_cu, int* __restrict__ pos,
+__global__ void target_positions_kernel(ReqTable rt, const int* u_pos, const int* u_cu, const int* r_rank, const int* r_cu, int* pos,
                                         DeviceStatus* st) {
+  griddep_launch();
+  griddep_wait();
   const int B = rt.n_req;
   const int y = blockIdx.x * blockDim.x + threadIdx.x;
   if (y >= rt.tile_cu[B]) return;
@@ -425,8 +434,9 @@ __global__ void target_positions_kernel(ReqTable rt, const int* __restrict__ u_p
 // One block copies one row (C a multiple of 8).
 __global__ void __launch_bounds__(128)
 carry_rows_kernel(ReqTable rt, const uint16_t* __restrict__ h_in, uint16_t* __restrict__ h_out, int C,
-                  const int* __restrict__ r_rank, const int* __restrict__ r_cu_l, const int* __restrict__ r_cu_next,
-                  DeviceStatus* st) {
+                  const int* r_rank, const int* r_cu_l, const int* r_cu_next, DeviceStatus* st) {
+  griddep_launch();
+  griddep_wait();
   const int B = rt.n_req;
   __shared__ long long src_row;
   const int y = blockIdx.x;
@@ -453,8 +463,9 @@ carry_rows_kernel(ReqTable rt, const uint16_t* __restrict__ h_in, uint16_t* __re
 // The same for many rows: one warp per row, the row travels through shared memory by bulk copies (see above).
 __global__ void __launch_bounds__(kRowWarps * 32)
 carry_rows_bulk_kernel(ReqTable rt, const uint16_t* __restrict__ h_in, uint16_t* __restrict__ h_out, int C,
-                       const int* __restrict__ r_rank, const int* __restrict__ r_cu_l, const int* __restrict__ r_cu_next,
-                       DeviceStatus* st) {
+                       const int* r_rank, const int* r_cu_l, const int* r_cu_next, DeviceStatus* st) {
+  griddep_launch();
+  griddep_wait();
   extern __shared__ __align__(128) uint8_t row_stage[];      // [warp][C] bf16
   __shared__ __align__(8) unsigned long long bars[kRowWarps];
   __shared__ volatile int gave_up[kRowWarps];
@@ -504,7 +515,7 @@ extern "C" relaxkv_status relaxkv_rmsnorm(const void* x, const void* weight, voi
   if (n_cols <= 256) {
     const long long blocks = (n_rows * 32 + 255) / 256;
     if (blocks > 0x7fffffffLL) return RELAXKV_ERR_UNSUPPORTED_SHAPE;
-    return cuda_ok(launch_chained(n_rows <= kChainedMaxRows, rmsnorm_short_kernel, (unsigned)blocks, 256, 0, static_cast<cudaStream_t>(stream),
+    return cuda_ok(launch_chained(rmsnorm_short_kernel, (unsigned)blocks, 256, 0, static_cast<cudaStream_t>(stream),
                                   static_cast<const uint16_t*>(x), static_cast<const uint16_t*>(weight),
                                   static_cast<uint16_t*>(y), (long long)n_rows, n_cols, eps));
   }
@@ -516,11 +527,10 @@ extern "C" relaxkv_status relaxkv_rmsnorm(const void* x, const void* weight, voi
     if (smem > 48 * 1024 - 256 &&
         cudaFuncSetAttribute(rmsnorm_rows_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return RELAXKV_ERR_CUDA;
-    rmsnorm_rows_bulk_kernel<<<(unsigned)((n_rows + kRowWarps - 1) / kRowWarps), kRowWarps * 32, smem, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const uint16_t*>(x), static_cast<const uint16_t*>(weight), static_cast<uint16_t*>(y), (long long)n_rows, n_cols, eps, st);
-    return launch_ok();
+    return cuda_ok(launch_chained(rmsnorm_rows_bulk_kernel, (unsigned)((n_rows + kRowWarps - 1) / kRowWarps), kRowWarps * 32, smem, static_cast<cudaStream_t>(stream),
+        static_cast<const uint16_t*>(x), static_cast<const uint16_t*>(weight), static_cast<uint16_t*>(y), (long long)n_rows, n_cols, eps, st));
   }
-  return cuda_ok(launch_chained(n_rows <= kChainedMaxRows, rmsnorm_kernel, (unsigned)n_rows, 256, 0, static_cast<cudaStream_t>(stream),
+  return cuda_ok(launch_chained(rmsnorm_kernel, (unsigned)n_rows, 256, 0, static_cast<cudaStream_t>(stream),
                                 static_cast<const uint16_t*>(x), static_cast<const uint16_t*>(weight),
                                 static_cast<uint16_t*>(y), n_cols, eps));
 }
@@ -532,9 +542,8 @@ extern "C" relaxkv_status relaxkv_rope(void* x, int64_t n_rows, int32_t n_heads,
   if (n_rows < 0 || n_heads < 1 || (head_dim != 64 && head_dim != 128)) return RELAXKV_ERR_UNSUPPORTED_SHAPE;
   if (n_rows == 0) return RELAXKV_OK;
   const long long n = n_rows * (head_dim / 16);
-  rope_kernel<<<(unsigned)((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-      static_cast<uint16_t*>(x), n_rows, n_heads, head_dim, positions, log2((double)theta));
-  return launch_ok();
+  return cuda_ok(launch_chained(rope_kernel, (unsigned)((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream),
+      static_cast<uint16_t*>(x), n_rows, n_heads, head_dim, positions, log2((double)theta)));
 }
 
 extern "C" relaxkv_status relaxkv_qk_norm_rope(void* q, void* k, int64_t n_rows, int32_t n_q_heads, int32_t n_kv_heads,
@@ -564,14 +573,13 @@ extern "C" relaxkv_status relaxkv_qk_norm_rope(void* q, void* k, int64_t n_rows,
     auto kern = head_dim == 128 ? head_norm_rope_rows_bulk_kernel<128> : head_norm_rope_rows_bulk_kernel<64>;
     if (smem > 48 * 1024 - 256 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return RELAXKV_ERR_CUDA;
-    kern<<<(unsigned)((n_rows + kRowWarps - 1) / kRowWarps), kRowWarps * 32, smem, st>>>(qp, kp, (long long)n_rows, n_q_heads, n_kv_heads,
-                                                                                       wq, wk, eps, positions, log2_theta, dst);
-    return launch_ok();
+    return cuda_ok(launch_chained(kern, (unsigned)((n_rows + kRowWarps - 1) / kRowWarps), kRowWarps * 32, smem, st,qp, kp, (long long)n_rows, n_q_heads, n_kv_heads,
+                                                                                       wq, wk, eps, positions, log2_theta, dst));
   }
   if (head_dim == 128)
-    return cuda_ok(launch_chained(n_rows <= kChainedMaxRows, head_norm_rope_kernel<128>, grid, 128, 0, st, qp, kp, n_q_heads, n_kv_heads, heads_per_block,
+    return cuda_ok(launch_chained(head_norm_rope_kernel<128>, grid, 128, 0, st, qp, kp, n_q_heads, n_kv_heads, heads_per_block,
                                   wq, wk, eps, positions, log2_theta));
-  return cuda_ok(launch_chained(n_rows <= kChainedMaxRows, head_norm_rope_kernel<64>, grid, 128, 0, st, qp, kp, n_q_heads, n_kv_heads, heads_per_block,
+  return cuda_ok(launch_chained(head_norm_rope_kernel<64>, grid, 128, 0, st, qp, kp, n_q_heads, n_kv_heads, heads_per_block,
                                 wq, wk, eps, positions, log2_theta));
 }
 
@@ -581,9 +589,8 @@ extern "C" relaxkv_status relaxkv_swiglu(const void* gate_up, void* out, int64_t
   if (n_rows < 0 || n_inter < 8 || (n_inter % 8)) return RELAXKV_ERR_UNSUPPORTED_SHAPE;
   if (n_rows == 0) return RELAXKV_OK;
   const long long n = n_rows * (n_inter / 8);
-  swiglu_kernel<<<(unsigned)((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-      static_cast<const uint16_t*>(gate_up), static_cast<uint16_t*>(out), n_rows, n_inter);
-  return launch_ok();
+  return cuda_ok(launch_chained(swiglu_kernel, (unsigned)((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream),
+      static_cast<const uint16_t*>(gate_up), static_cast<uint16_t*>(out), n_rows, n_inter));
 }
 
 extern "C" relaxkv_status relaxkv_target_positions(const relaxkv_shape* shape, const int32_t* u_pos, const int32_t* u_cu,
@@ -605,9 +612,8 @@ extern "C" relaxkv_status relaxkv_target_positions(const relaxkv_shape* shape, c
   if (total > 0x7fffffffLL) return RELAXKV_ERR_UNSUPPORTED_SHAPE;
   DeviceStatus* st = status_word();
   if (!st) return RELAXKV_ERR_CUDA;
-  target_positions_kernel<<<(unsigned)((total + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-      rt, u_pos, u_cu, r_rank, r_cu_layer, positions_out, st);
-  return launch_ok();
+  return cuda_ok(launch_chained(target_positions_kernel, (unsigned)((total + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream),
+      rt, u_pos, u_cu, r_rank, r_cu_layer, positions_out, st));
 }
 
 extern "C" relaxkv_status relaxkv_carry_rows(const relaxkv_shape* shape, const void* h_in, void* h_out, int32_t n_cols,
@@ -636,11 +642,9 @@ extern "C" relaxkv_status relaxkv_carry_rows(const relaxkv_shape* shape, const v
     if (smem > 48 * 1024 - 256 &&
         cudaFuncSetAttribute(carry_rows_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return RELAXKV_ERR_CUDA;
-    carry_rows_bulk_kernel<<<(unsigned)((total + kRowWarps - 1) / kRowWarps), kRowWarps * 32, smem, static_cast<cudaStream_t>(stream)>>>(
-        rt, static_cast<const uint16_t*>(h_in), static_cast<uint16_t*>(h_out), n_cols, r_rank, r_cu_layer, r_cu_next, st);
-    return launch_ok();
+    return cuda_ok(launch_chained(carry_rows_bulk_kernel, (unsigned)((total + kRowWarps - 1) / kRowWarps), kRowWarps * 32, smem, static_cast<cudaStream_t>(stream),
+        rt, static_cast<const uint16_t*>(h_in), static_cast<uint16_t*>(h_out), n_cols, r_rank, r_cu_layer, r_cu_next, st));
   }
-  carry_rows_kernel<<<(unsigned)total, 128, 0, static_cast<cudaStream_t>(stream)>>>(
-      rt, static_cast<const uint16_t*>(h_in), static_cast<uint16_t*>(h_out), n_cols, r_rank, r_cu_layer, r_cu_next, st);
-  return launch_ok();
+  return cuda_ok(launch_chained(carry_rows_kernel, (unsigned)total, 128, 0, static_cast<cudaStream_t>(stream),
+      rt, static_cast<const uint16_t*>(h_in), static_cast<uint16_t*>(h_out), n_cols, r_rank, r_cu_layer, r_cu_next, st));
 }

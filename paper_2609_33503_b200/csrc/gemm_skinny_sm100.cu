@@ -288,7 +288,7 @@ static bool try_launch(const SkinnyPlan& p, const CUtensorMap& tm_w, const CUten
   const int resident = p.whole_sm ? max_clusters<S>(p.dev, p.sms) : (S % 2 ? 2 * max_clusters<S>(p.dev, p.sms) : max_clusters<(S + 1) / 2>(p.dev, p.sms));
   if (resident < 1 || !opt_in_smem<S>(p.dev)) { *rc = RELAXKV_ERR_CUDA; return true; }
   if (S > 1 && p.tiles > resident) return false;
-  *rc = cuda_ok(launch_chained_clusters(true, S, gemm_skinny_sm100_kernel<S>, dim3((unsigned)(p.tiles * S)), dim3(kSkThreads), p.smem,
+  *rc = cuda_ok(launch_chained_clusters(S, gemm_skinny_sm100_kernel<S>, dim3((unsigned)(p.tiles * S)), dim3(kSkThreads), p.smem,
                                         p.stream, tm_w, tm_x, p.n_rows, p.n_cols, p.n_stages, p.n_feat, p.n_in, p.swiglu, outs, p.st));
   return true;
 }

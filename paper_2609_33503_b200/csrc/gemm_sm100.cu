@@ -46,6 +46,7 @@ gemm_sm100_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
                   int swiglu, const __grid_constant__ GemmSegs segs, DeviceStatus* st) {
   const int tiles_m = (int)((M + kGemmBM - 1) / kGemmBM), tiles_n = (N + kGemmBN - 1) / kGemmBN;
   const long long n_tiles = (long long)tiles_m * tiles_n;
+  griddep_wait();
   if (*reinterpret_cast<volatile int*>(&st->status) == RELAXKV_ERR_TIMEOUT) return;
   // tile t of the grouped order: kGemmGroupM row tiles x all column tiles at a time
   auto tile_of = [&](long long t, int& tm, int& tn) {
@@ -201,6 +202,7 @@ gemm_sm100_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
       mbar_arrive(bar_acc_empty + 8 * a);
     }
   }
+  griddep_launch();
   tc_fence_before();
   __syncthreads();
   if (*abort_flag) {
@@ -267,6 +269,7 @@ gemm_pair_sm100_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
   cluster_sync();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  griddep_wait();
   const int n_k = (K + kGemmBK - 1) / kGemmBK;
 
   if (warp == 4) {
@@ -401,6 +404,7 @@ gemm_pair_sm100_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
       mbar_arrive_remote(mapa_shared(bar_acc_empty + 8 * a, 0));
     }
   }
+  griddep_launch();
   tc_fence_before();
   __syncthreads();
   if (*abort_flag) {
@@ -496,16 +500,14 @@ static relaxkv_status launch_gemm(const void* x, const void* weight, const void*
       max_clusters[dev].store(n, std::memory_order_release);
     }
     const long long clusters = std::min<long long>(tiles_m2 * tiles_n, n_clusters);
-    gemm_pair_sm100_kernel<<<(unsigned)(2 * clusters), kGemmThreads, kPairSmem, static_cast<cudaStream_t>(stream_)>>>(
-        tm_a, tm_b, n_rows, n_out, n_in, static_cast<uint16_t*>(y), static_cast<const uint16_t*>(residual), swiglu, segs, st);
-    return launch_ok();
+    return cuda_ok(launch_chained(gemm_pair_sm100_kernel, (unsigned)(2 * clusters), kGemmThreads, kPairSmem, static_cast<cudaStream_t>(stream_),
+        tm_a, tm_b, n_rows, n_out, n_in, static_cast<uint16_t*>(y), static_cast<const uint16_t*>(residual), swiglu, segs, st));
   }
   const long long tiles_m = (n_rows + kGemmBM - 1) / kGemmBM;
   if (tiles_m * tiles_n > 0x7fffffffLL) return RELAXKV_ERR_UNSUPPORTED_SHAPE;
   const long long grid = std::min<long long>(tiles_m * tiles_n, sms);     // persistent: one CTA per SM
-  gemm_sm100_kernel<<<(unsigned)grid, kGemmThreads, kGemmSmem, static_cast<cudaStream_t>(stream_)>>>(
-      tm_a, tm_b, n_rows, n_out, n_in, static_cast<uint16_t*>(y), static_cast<const uint16_t*>(residual), swiglu, segs, st);
-  return launch_ok();
+  return cuda_ok(launch_chained(gemm_sm100_kernel, (unsigned)grid, kGemmThreads, kGemmSmem, static_cast<cudaStream_t>(stream_),
+      tm_a, tm_b, n_rows, n_out, n_in, static_cast<uint16_t*>(y), static_cast<const uint16_t*>(residual), swiglu, segs, st));
 }
 
 extern "C" relaxkv_status relaxkv_linear(const void* x, const void* weight, const void* residual, void* y,

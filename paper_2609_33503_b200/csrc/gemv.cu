@@ -148,10 +148,10 @@ static relaxkv_status launch_mk(const uint16_t* x, const uint16_t* w, const uint
   const unsigned blocks = (unsigned)((n_out + feat_per_block - 1) / feat_per_block);
   cudaError_t e = cudaSuccess;
   switch (n_rows) {
-    case 1: e = launch_chained(true, gemv_kernel<1, SWIGLU, SEG, KS>, blocks, kGemvThreads, 0, stream, x, w, residual, y, n_out, K, outs); break;
-    case 2: e = launch_chained(true, gemv_kernel<2, SWIGLU, SEG, KS>, blocks, kGemvThreads, 0, stream, x, w, residual, y, n_out, K, outs); break;
-    case 3: e = launch_chained(true, gemv_kernel<3, SWIGLU, SEG, KS>, blocks, kGemvThreads, 0, stream, x, w, residual, y, n_out, K, outs); break;
-    case 4: e = launch_chained(true, gemv_kernel<4, SWIGLU, SEG, KS>, blocks, kGemvThreads, 0, stream, x, w, residual, y, n_out, K, outs); break;
+    case 1: e = launch_chained(gemv_kernel<1, SWIGLU, SEG, KS>, blocks, kGemvThreads, 0, stream, x, w, residual, y, n_out, K, outs); break;
+    case 2: e = launch_chained(gemv_kernel<2, SWIGLU, SEG, KS>, blocks, kGemvThreads, 0, stream, x, w, residual, y, n_out, K, outs); break;
+    case 3: e = launch_chained(gemv_kernel<3, SWIGLU, SEG, KS>, blocks, kGemvThreads, 0, stream, x, w, residual, y, n_out, K, outs); break;
+    case 4: e = launch_chained(gemv_kernel<4, SWIGLU, SEG, KS>, blocks, kGemvThreads, 0, stream, x, w, residual, y, n_out, K, outs); break;
     default: return RELAXKV_ERR_INVALID_ARG;
   }
   return cuda_ok(e);

@@ -16,12 +16,12 @@ namespace relaxkv {
 
 // Warp-cooperative lower bound on an ascending list: 32 pivots per round instead of one.
 // Returns the first index with a[idx] >= key (n if none).  All lanes get the result.
-__device__ __forceinline__ int warp_lower_bound(const int* __restrict__ a, int n, int key, int lane) {
+__device__ __forceinline__ int warp_lower_bound(const int* a, int n, int key, int lane) {
   int lo = 0, hi = n;                     // the answer lies in [lo, hi]
   while (hi > lo) {
     const int step = (hi - lo + 31) / 32;
     const int idx = lo + lane * step;
-    const bool lt = (idx < hi) && (__ldg(a + idx) < key);
+    const bool lt = (idx < hi) && (a[idx] < key);
     const int n_lt = __popc(__ballot_sync(0xffffffffu, lt));   // pivots below the key: a prefix of the lanes
     if (n_lt == 0) {
       hi = lo;
@@ -101,10 +101,9 @@ gather_ctx_kernel(ReqTable rt, int mode, int n_kv_heads, int head_dim,
                   const uint16_t* __restrict__ cache_k, const uint16_t* __restrict__ cache_v,
                   long long tok_stride, long long head_stride,
                   const uint16_t* __restrict__ k_new, const uint16_t* __restrict__ v_new,
-                  const int* __restrict__ u_pos, const int* __restrict__ u_cu,
-                  const int* __restrict__ r_rank, const int* __restrict__ r_cu, const int* __restrict__ fresh_row,
+                  const int* u_pos, const int* u_cu, const int* r_rank, const int* r_cu, const int* fresh_row,
                   uint16_t* __restrict__ k_out, uint16_t* __restrict__ v_out, long long ctx_rows,
-                  long long fresh_map_rows, long long n_new_rows, int rows_per_warp, DeviceStatus* st) {
+                  long long fresh_map_rows, long long n_new_rows, int rows_per_warp, int* work_counter, DeviceStatus* st) {
   // fresh_map_rows: entries of fresh_row that were written (the host bound on the context rows of an explicit-list
   // call); n_new_rows: rows k_new / v_new hold.  An index past either is reported and the row zero-filled.
   extern __shared__ __align__(128) uint8_t stage[];          // [warp][row of the warp][K row | V row]
@@ -113,10 +112,13 @@ gather_ctx_kernel(ReqTable rt, int mode, int n_kv_heads, int head_dim,
   const int B = rt.n_req;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long x0 = ((long long)blockIdx.x * kMoveWarps + warp) * rows_per_warp;
+  griddep_launch();
+  griddep_wait();                              // the rows and the index lists come from earlier kernels
+  if (work_counter != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *work_counter = 0;
   if (x0 >= ctx_rows) return;
   const uint32_t bar = smem_u32(&bars[warp]);
   if (lane == 0) { gave_up[warp] = 0; mbar_init(bar, 1); fence_barrier_init(); }
-  const long long total = (mode == RELAXKV_CTX_UNION) ? (long long)__ldg(u_cu + B) : rt.ctx_cu[B];
+  const long long total = (mode == RELAXKV_CTX_UNION) ? (long long)u_cu[B] : rt.ctx_cu[B];
   const uint32_t row_bytes = (uint32_t)n_kv_heads * head_dim * 2;
   const uint32_t my_stage = smem_u32(stage) + (uint32_t)(warp * rows_per_warp + lane) * 2u * row_bytes;   // lanes < rows_per_warp
   int my_kind = 3;                             // lane rr keeps the source of row rr: 0 = cache, 1 = fresh, 2 = zero fill, 3 = skip
@@ -132,15 +134,15 @@ gather_ctx_kernel(ReqTable rt, int mode, int n_kv_heads, int head_dim,
       } else {
         int b = 0, c = -1, p;
         if (mode == RELAXKV_CTX_UNION) {
-          while (b + 1 < B && x >= __ldg(u_cu + b + 1)) ++b;
-          c = (int)(x - __ldg(u_cu + b));
-          p = __ldg(u_pos + x);
+          while (b + 1 < B && x >= u_cu[b + 1]) ++b;
+          c = (int)(x - u_cu[b]);
+          p = u_pos[x];
         } else {
           while (b + 1 < B && x >= rt.ctx_cu[b + 1]) ++b;
           p = (int)(x - rt.ctx_cu[b]);
-          const int ub = __ldg(u_cu + b), nu = __ldg(u_cu + b + 1) - ub;
+          const int ub = u_cu[b], nu = u_cu[b + 1] - ub;
           const int lb = warp_lower_bound(u_pos + ub, nu, p, lane);
-          if (lb < nu && __ldg(u_pos + ub + lb) == p) c = lb;
+          if (lb < nu && u_pos[ub + lb] == p) c = lb;
         }
         if (p < 0 || p >= rt.ctx_len[b]) {
           if (lane == 0) report(st, RELAXKV_ERR_BAD_INDEX, KID_GATHER, (int)x, p);
@@ -154,7 +156,7 @@ gather_ctx_kernel(ReqTable rt, int mode, int n_kv_heads, int head_dim,
               if (lane == 0) report(st, RELAXKV_ERR_BAD_INDEX, KID_GATHER, (int)x, (int)fresh_map_rows);
               kind = 2;
             } else {
-              const int fr = __ldg(fresh_row + x);
+              const int fr = fresh_row[x];
               if (fr >= n_new_rows) {
                 if (lane == 0) report(st, RELAXKV_ERR_BAD_INDEX, KID_GATHER, (int)x, fr);
                 kind = 2;
@@ -163,21 +165,21 @@ gather_ctx_kernel(ReqTable rt, int mode, int n_kv_heads, int head_dim,
               }
             }
           } else if (k_new != nullptr && c >= 0) {
-            const int rb = __ldg(r_cu + b), nr = __ldg(r_cu + b + 1) - rb;
+            const int rb = r_cu[b], nr = r_cu[b + 1] - rb;
             // first index of the R list with rank >= c: searched for the warp's first row of a request, then the
             // list is walked (consecutive context ranks: the answer moves by at most one entry per row)
             int rho;
             if (b == prev_b) {
               rho = rho_next;
-              while (rho < nr && __ldg(r_rank + rb + rho) < c) ++rho;     // only after a malformed (unsorted) list
+              while (rho < nr && r_rank[rb + rho] < c) ++rho;     // only after a malformed (unsorted) list
             } else {
               rho = warp_lower_bound(r_rank + rb, nr, c, lane);
             }
             prev_b = b;
             rho_next = rho;
-            if (rho < nr && __ldg(r_rank + rb + rho) == c) {
+            if (rho < nr && r_rank[rb + rho] == c) {
               rho_next = rho + 1;
-              const long long frow = (long long)(rb - __ldg(r_cu)) + rho;
+              const long long frow = (long long)(rb - r_cu[0]) + rho;
               if (frow >= n_new_rows) {
                 if (lane == 0) report(st, RELAXKV_ERR_BAD_INDEX, KID_GATHER, (int)x, (int)frow);
                 kind = 2;
@@ -235,8 +237,7 @@ scatter_kv_kernel(ReqTable rt, int n_kv_heads, int head_dim,
                   uint16_t* __restrict__ cache_k, uint16_t* __restrict__ cache_v,
                   long long tok_stride, long long head_stride,
                   const uint16_t* __restrict__ k_new, const uint16_t* __restrict__ v_new,
-                  const int* __restrict__ u_pos, const int* __restrict__ u_cu,
-                  const int* __restrict__ r_rank, const int* __restrict__ r_cu, int direct, int rows_per_warp,
+                  const int* u_pos, const int* u_cu, const int* r_rank, const int* r_cu, int direct, int rows_per_warp,
                   DeviceStatus* st) {
   // direct != 0: u_pos holds the targets' positions themselves (packed by r_cu); r_rank is not read
   extern __shared__ __align__(128) uint8_t stage[];          // [warp][row of the warp][K row | V row]
@@ -300,7 +301,8 @@ relaxkv_status launch_gather(const relaxkv_shape* shape, int mode, const relaxkv
                              const void* k_new, const void* v_new, const int32_t* u_pos, const int32_t* u_cu,
                              const int32_t* r_rank, const int32_t* r_cu_layer, const int32_t* fresh_row,
                              long long fresh_map_rows, long long n_new_rows,
-                             long long rows_to_cover, void* k_out, void* v_out, long long ctx_rows, cudaStream_t stream) {
+                             long long rows_to_cover, void* k_out, void* v_out, long long ctx_rows, int* work_counter,
+                             cudaStream_t stream) {
   ReqTable rt;
   fill_req_table(rt, shape, cache, nullptr);
   DeviceStatus* st = status_word();
@@ -317,14 +319,13 @@ relaxkv_status launch_gather(const relaxkv_shape* shape, int mode, const relaxkv
   const long long rows_per_block = (long long)kMoveWarps * rows_per_warp;
   const long long blocks = (rows_to_cover + rows_per_block - 1) / rows_per_block;
   RELAXKV_RANGE("gather_ctx_kernel");
-  gather_ctx_kernel<<<(unsigned)blocks, kMoveThreads, smem, stream>>>(
+  return cuda_ok(launch_chained(gather_ctx_kernel, (unsigned)blocks, kMoveThreads, smem, stream,
       rt, mode, shape->n_kv_heads, shape->head_dim,
       static_cast<const uint16_t*>(cache->k), static_cast<const uint16_t*>(cache->v),
-      cache->token_stride, cache->head_stride,
+      (long long)cache->token_stride, (long long)cache->head_stride,
       static_cast<const uint16_t*>(k_new), static_cast<const uint16_t*>(v_new),
       u_pos, u_cu, r_rank, r_cu_layer, fresh_row, static_cast<uint16_t*>(k_out), static_cast<uint16_t*>(v_out), ctx_rows,
-      fresh_map_rows, n_new_rows, rows_per_warp, st);
-  return launch_ok();
+      fresh_map_rows, n_new_rows, rows_per_warp, work_counter, st));
 }
 
 // Launches the cache update for `total` target rows (host bound); direct: see scatter_kv_kernel.
@@ -344,7 +345,7 @@ static relaxkv_status launch_scatter(const relaxkv_shape* shape, const ReqTable&
   const long long rows_per_block = (long long)kMoveWarps * rows_per_warp;
   const long long blocks = (total + rows_per_block - 1) / rows_per_block;
   RELAXKV_RANGE("scatter_kv_kernel");
-  return cuda_ok(launch_chained(total <= kChainedMaxRows, scatter_kv_kernel, (unsigned)blocks, kMoveThreads, smem, stream,
+  return cuda_ok(launch_chained(scatter_kv_kernel, (unsigned)blocks, kMoveThreads, smem, stream,
       rt, shape->n_kv_heads, shape->head_dim, static_cast<uint16_t*>(cache->k), static_cast<uint16_t*>(cache->v),
       (long long)cache->token_stride, (long long)cache->head_stride, static_cast<const uint16_t*>(k_new),
       static_cast<const uint16_t*>(v_new), u_pos, u_cu, r_rank, r_cu, direct, rows_per_warp, st));
@@ -384,7 +385,7 @@ extern "C" relaxkv_status relaxkv_gather_kv(
   if (ctx_rows < need) return RELAXKV_ERR_INVALID_ARG;
   // this entry point is not told how many rows k_new / v_new hold: the fresh-row index is bounded by the R list only
   return launch_gather(shape, mode, cache, k_new, v_new, u_pos, u_cu, r_rank, r_cu_layer, nullptr, 0, 0x7fffffffffffffffLL,
-                       need + kCtxPadRows, k_ctx_out, v_ctx_out, ctx_rows, static_cast<cudaStream_t>(stream));
+                       need + kCtxPadRows, k_ctx_out, v_ctx_out, ctx_rows, nullptr, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" relaxkv_status relaxkv_scatter_kv(

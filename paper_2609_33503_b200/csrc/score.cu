@@ -18,8 +18,9 @@ constexpr float kLn2 = 0.6931471805599453f;
 // One warp per row: the lanes walk the partials (fixed lane -> partial assignment, fixed shuffle tree, so
 // the result does not depend on scheduling).  part is [layer][n_part][H*sum_q].  Rows of layers whose
 // log-normalisers were supplied have only empty partials and are never read afterwards.
-__global__ void combine_lse_kernel(long long n_rows_total, long long n_rows, int n_part, const float2* __restrict__ part,
-                                   float* __restrict__ lse) {
+__global__ void combine_lse_kernel(long long n_rows_total, long long n_rows, int n_part, const float2* part, float* lse) {
+  griddep_launch();
+  griddep_wait();
   const int lane = threadIdx.x & 31;
   const long long gidx = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (gidx >= n_rows_total) return;
@@ -40,15 +41,17 @@ __global__ void combine_lse_kernel(long long n_rows_total, long long n_rows, int
   if (lane == 0) lse[gidx] = (M + log2f(z)) * kLn2;
 }
 
-void launch_combine_lse(int n_layers, int H, int sum_q, int n_part, const float2* part, float* lse, cudaStream_t stream) {
+cudaError_t launch_combine_lse(int n_layers, int H, int sum_q, int n_part, const float2* part, float* lse, cudaStream_t stream) {
   const long long n_rows = (long long)H * sum_q, total = n_rows * n_layers;
-  combine_lse_kernel<<<(unsigned)((total * 32 + 255) / 256), 256, 0, stream>>>(total, n_rows, n_part, part, lse);
+  return launch_chained(combine_lse_kernel, (unsigned)((total * 32 + 255) / 256), 256, 0, stream, total, n_rows, n_part, part, lse);
 }
 
 // raw[layer, i] = (sum of the partial column sums in a fixed order: KV head, query-row block, warpgroup) / (H * Q_b)
 // rt.tile_cu = prefix of the query-row blocks per request; colpart is [layer][2*Hkv*max_super][sum_t].
 __global__ void finalize_raw_kernel(ReqTable rt, int n_layers, int H, int Hkv, int max_super,
-                                    const float* __restrict__ colpart, float* __restrict__ raw) {
+                                    const float* colpart, float* raw) {
+  griddep_launch();
+  griddep_wait();
   const long long sum_t = rt.ctx_cu[rt.n_req];
   const long long gi = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (gi >= sum_t * n_layers) return;
@@ -78,13 +81,14 @@ static relaxkv_status score_layers(const relaxkv_shape* shape, ReqTable rt, cons
   if (rc != RELAXKV_OK) return rc;
   for (int b = 0; b < B; ++b) rt.tile_cu[b + 1] = rt.tile_cu[b] + plan.n_super[b];
   const long long total = rt.ctx_cu[B] * n_layers;
-  finalize_raw_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(rt, n_layers, H, Hkv, plan.max_super, colpart, raw);
-  return launch_ok();
+  return cuda_ok(launch_chained(finalize_raw_kernel, (unsigned)((total + 255) / 256), 256, 0, stream, rt, n_layers, H, Hkv, plan.max_super, colpart, raw));
 }
 
 // Positions of the query's own tokens (they follow the context: T_c, T_c + 1, ...) and their offsets, as the target
 // lists of the cache-only attention call.
 __global__ void query_positions_kernel(ReqTable rt, int* __restrict__ tgt_pos, int* __restrict__ tgt_cu) {
+  griddep_launch();
+  griddep_wait();
   const int B = rt.n_req;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i <= B) tgt_cu[i] = rt.q_cu[i];
@@ -189,8 +193,8 @@ extern "C" relaxkv_status relaxkv_query_prefill_attention(
   ReqTable rt;
   fill_req_table(rt, shape, cache, nullptr);
   const long long n = std::max<long long>(sum_q, B + 1);
-  query_positions_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(rt, tgt_pos, tgt_cu);
-  if ((rc = launch_ok()) != RELAXKV_OK) return rc;
+  rc = cuda_ok(launch_chained(query_positions_kernel, (unsigned)((n + 255) / 256), 256, 0, stream, rt, tgt_pos, tgt_cu));
+  if (rc != RELAXKV_OK) return rc;
   rc = relaxkv_cache_attention(&ext, cache, q, tgt_pos, tgt_cu, sum_q, q_len, out, lse_out, workspace, workspace_bytes, stream_);
   if (rc != RELAXKV_OK || !raw_scores_out) return rc;
   // column sums over the CONTEXT keys with the rows' normalisers from the attention above

@@ -47,12 +47,13 @@ struct ScoreLayers {
 template <int D, bool PASS2>
 __global__ void __launch_bounds__(kScThreads, 1)
 score_sm100_kernel(const __grid_constant__ ScoreLayers layers, const __grid_constant__ ReqTable rt, int H, int Hkv,
-                   float scale_log2, int n_splits, int max_super, const float* __restrict__ lse_ws,
-                   float2* __restrict__ part_all, float* __restrict__ colpart_all, DeviceStatus* st) {
+                   float scale_log2, int n_splits, int max_super, const float* lse_ws,
+                   float2* part_all, float* colpart_all, DeviceStatus* st) {
   using L = ScoreSmem<D>;
   constexpr int kHalves = L::kHalves;
   constexpr float kLog2e = 1.4426950408889634f;
 
+  griddep_wait();
   // ---- which unit ---------------------------------------------------------------------------------
   const int B = rt.n_req;
   const int G = H / Hkv;
@@ -283,6 +284,7 @@ score_sm100_kernel(const __grid_constant__ ScoreLayers layers, const __grid_cons
   }
 
   // ---- teardown --------------------------------------------------------------------------------------
+  griddep_launch();
   tc_fence_before();
   __syncthreads();
   if (*abort_flag) {
@@ -365,11 +367,13 @@ relaxkv_status launch_score_sm100(const relaxkv_shape* shape, ReqTable rt, const
     attr_done[dev].store(1, std::memory_order_release);
   }
   if (need_pass1) {
-    k1<<<grid, kScThreads, smem, stream>>>(layers, rt, H, Hkv, scale_log2, n_splits, plan.max_super, lse_ws, part, colpart, st);
-    launch_combine_lse(n_layers, H, sum_q, n_splits * 2, part, lse_ws, stream);
+    if (launch_chained(k1, grid, kScThreads, smem, stream, layers, rt, H, Hkv, scale_log2, n_splits, plan.max_super, lse_ws, part,
+                       colpart, st) != cudaSuccess ||
+        launch_combine_lse(n_layers, H, sum_q, n_splits * 2, part, lse_ws, stream) != cudaSuccess)
+      return RELAXKV_ERR_CUDA;
   }
-  k2<<<grid, kScThreads, smem, stream>>>(layers, rt, H, Hkv, scale_log2, n_splits, plan.max_super, lse_ws, part, colpart, st);
-  return launch_ok();
+  return cuda_ok(launch_chained(k2, grid, kScThreads, smem, stream, layers, rt, H, Hkv, scale_log2, n_splits, plan.max_super, lse_ws,
+                                part, colpart, st));
 }
 
 template relaxkv_status launch_score_sm100<64>(const relaxkv_shape*, ReqTable, const ScorePlan&, int, const void* const*,

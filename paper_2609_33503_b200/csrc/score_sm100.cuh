@@ -13,7 +13,7 @@ struct ScorePlan {
 ScorePlan plan_score(const relaxkv_shape* shape);
 
 // lse[layer, h, row] = natural-log sum over n_part partial (max, sum) pairs in log2 units (score.cu).
-void launch_combine_lse(int n_layers, int H, int sum_q, int n_part, const float2* part, float* lse, cudaStream_t stream);
+cudaError_t launch_combine_lse(int n_layers, int H, int sum_q, int n_part, const float2* part, float* lse, cudaStream_t stream);
 
 // Scores n_layers (<= kScoreLayersPerLaunch) layers with ONE launch per pass: pass 1 for the layers without
 // supplied log-normalisers + combine, then pass 2.  Fills colpart[layer][(g*max_super + super)*2 + wg][sum_t].

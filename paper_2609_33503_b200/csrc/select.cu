@@ -233,7 +233,7 @@ static relaxkv_status launch_select_slices(const ReqTable& rt, int n_layers, con
     const int per = ((rt.ctx_len[b] + NS - 1) / NS + 31) & ~31;
     if (per <= kSelKeysMax) cap = std::max(cap, per);
   }
-  return cuda_ok(launch_chained_clusters(true, NS, select_topk_kernel<NS>, dim3((unsigned)(n_layers * rt.n_req * NS)),
+  return cuda_ok(launch_chained_clusters(NS, select_topk_kernel<NS>, dim3((unsigned)(n_layers * rt.n_req * NS)),
                                          dim3(kSelThreads), (size_t)cap * 4, stream, rt, n_layers, cap, raw, norm, anchors, st));
 }
 

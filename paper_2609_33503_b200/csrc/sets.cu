@@ -159,15 +159,15 @@ static relaxkv_status build_sets(const relaxkv_shape* shape, int32_t n_layers, c
   // copy below read.
   const long long n_anchor = (long long)n_layers * rt.k_cu[B];
   const unsigned lists = (unsigned)(B * (n_layers + 1));
-  cudaError_t e = launch_chained(true, fill_i32_kernel, dim3((unsigned)((sum_t + 255) / 256)), dim3(256), 0, stream,
+  cudaError_t e = launch_chained(fill_i32_kernel, dim3((unsigned)((sum_t + 255) / 256)), dim3(256), 0, stream,
                                  highest_layer_out, sum_t, -1);
   if (e == cudaSuccess)
-    e = launch_chained(true, highest_layer_kernel, dim3((unsigned)((n_anchor + 255) / 256)), dim3(256), 0, stream, rt, n_layers,
+    e = launch_chained(highest_layer_kernel, dim3((unsigned)((n_anchor + 255) / 256)), dim3(256), 0, stream, rt, n_layers,
                        anchors, highest_layer_out, st);
   if (e == cudaSuccess)
-    e = launch_chained(true, count_sets_kernel, dim3(lists), dim3(kSetThreads), 0, stream, rt, n_layers, highest_layer_out, counts);
+    e = launch_chained(count_sets_kernel, dim3(lists), dim3(kSetThreads), 0, stream, rt, n_layers, highest_layer_out, counts);
   if (e == cudaSuccess)
-    e = launch_chained_clusters(true, kSetSlices, write_sets_kernel, dim3(lists * kSetSlices), dim3(kSetThreads), 0, stream, rt,
+    e = launch_chained_clusters(kSetSlices, write_sets_kernel, dim3(lists * kSetSlices), dim3(kSetThreads), 0, stream, rt,
                                 n_layers, highest_layer_out, counts, u_pos_out, u_cu_out, u_rank_out, r_rank_out, r_cu_out, host_counts);
   relaxkv_status rc = cuda_ok(e);
   if (rc != RELAXKV_OK) return rc;
