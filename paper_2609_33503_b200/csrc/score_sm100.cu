@@ -8,7 +8,7 @@
 //   pass 2 (column sums):     S^T = K_tile Q_chunk^T   lanes = keys,       columns = query rows
 // so that in both passes the reduction a thread needs runs along its own TMEM lane.  Two softmax
 // warpgroups take the buffers alternately; the exponentials (one per 2*D MMA flops) bound the
-// kernel, not the tensor pipe and not HBM.  Partial results are combined in a fixed order by the
+// kernel first, the tensor pipe (1.05 of the 1.96 ms of a 32K x 40-layer pass at the GEMM peak) next, not HBM.  Partial results are combined in a fixed order by the
 // small kernels of score.cu, so scores are bit-reproducible.
 #include "score_sm100.cuh"
 #include "sm100_ptx.cuh"
@@ -35,6 +35,22 @@ struct ScoreSmem {
   static constexpr int kMisc = kBar + 8 * kNumBars;
   static constexpr int kTotal = kMisc + 16;
 };
+
+// a0 + a1 + a2 + a3 += sum over 16 values of 2^(s * scale + c), running sum e taking every fourth value from e; PER: c differs per value (c[0..15]), else it is c[0]
+// for all.  Scaling and sums use packed fp32 pairs: the scores of a 32K x 40-layer call took 2319 + 2093 us with one
+// instruction per value, 2149 + 1957 us with pairs.  (With a fourth or more of the exponentials as a polynomial on the FMA
+// pipe the two passes took 2.6 ms each and longer: that pipe's pairs cost two clocks, and the tensor pipe and the power cap
+// are close as well.)
+template <bool PER>
+__device__ __forceinline__ void exp2_sum16(const uint32_t* s, float scale, const float* c, float& a0, float& a1, float& a2, float& a3) {
+#pragma unroll
+  for (int i = 0; i < 16; i += 2) {
+    float x0, x1;
+    fma2(x0, x1, __uint_as_float(s[i]), __uint_as_float(s[i + 1]), scale, scale, c[PER ? i : 0], c[PER ? i + 1 : 0]);
+    if (i & 2) add2(a2, a3, fast_exp2(x0), fast_exp2(x1));
+    else add2(a0, a1, fast_exp2(x0), fast_exp2(x1));
+  }
+}
 
 // Per-layer arguments of one launch: tensor maps of the layer's Q rows and K cache, its supplied
 // log-normalisers (NULL: computed by pass 1) - by value in the kernel parameters.
@@ -137,16 +153,15 @@ score_sm100_kernel(const __grid_constant__ ScoreLayers layers, const __grid_cons
     *reinterpret_cast<uint4*>(smem_raw + L::kQ + hf * L::kQHalfBytes + (rows_loaded + r) * 128 + piece * 16) = make_uint4(0, 0, 0, 0);
   }
   if (PASS2) {
-    // log-normalisers of the resident rows in log2 units; rows past the block's end can never contribute
+    // negated log-normalisers of the resident rows in log2 units; rows past the block's end can never contribute
     for (int r = threadIdx.x; r < n_chunks * 128; r += kScThreads)
-      lse2s[r] = (r < rows) ? lse[(long long)(g * G + r % G) * sum_q + rt.q_cu[b] + t0 + r / G] * kLog2e : INFINITY;
+      lse2s[r] = (r < rows) ? -(lse[(long long)(g * G + r % G) * sum_q + rt.q_cu[b] + t0 + r / G] * kLog2e) : -INFINITY;
   }
   fence_proxy_async_smem();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  const int n_items = (kt1 - kt0) * n_chunks;
 
   if (warp == 8) {
     // ================= TMA producer =================
@@ -171,26 +186,30 @@ score_sm100_kernel(const __grid_constant__ ScoreLayers layers, const __grid_cons
     if (lane == 0) {
       constexpr uint32_t idesc = idesc_bf16_f32(128, 128, 0);
       bool ok = mbar_wait(bar_q, 0, abort_flag);
-      int it = 0;
+      // Every instruction of this lane between two MMAs delays the next one, so the operands' descriptors are carried as
+      // their low words and the four K steps of a 64-dim half are one batch.
+      constexpr uint32_t hi = desc_hi_sw128(1024);
+      const uint32_t q_lo = desc_lo(q_smem, 16), k_lo = desc_lo(k_smem, 16);
+      uint32_t buf = 0, buf_ph = 1, s = 0, k_ph = 0;                     // buf_ph: parity of the buffer's previous round
       for (int kt = kt0; ok && kt < kt1; ++kt) {
-        const int u = kt - kt0, s = u % kScKStages;
-        if (!(ok = mbar_wait(bar_kfull + 8 * s, (u / kScKStages) & 1, abort_flag))) break;
-        for (int c = 0; c < n_chunks; ++c, ++it) {
-          const int buf = it % kScBufs;
-          if (it >= kScBufs && !(ok = mbar_wait(bar_sempty + 8 * buf, ((it / kScBufs) - 1) & 1, abort_flag))) break;
+        if (!(ok = mbar_wait(bar_kfull + 8 * s, k_ph, abort_flag))) break;
+        const uint32_t kl = k_lo + s * (kHalves * L::kKHalfBytes / 16);
+        uint32_t ql = q_lo;
+        for (int c = 0; c < n_chunks; ++c, ql += 128 * 128 / 16) {
+          // a fresh barrier counts as having completed the phase before its first: the first round waits for nothing
+          if (!(ok = mbar_wait(bar_sempty + 8 * buf, buf_ph, abort_flag))) break;
           tc_fence_after();
 #pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) {
-            const uint32_t hf = kk >> 2, off = (kk & 3) * 32;
-            const uint64_t dq = smem_desc_sw128(q_smem + hf * L::kQHalfBytes + c * 128 * 128 + off, 16, 1024);
-            const uint64_t dk = smem_desc_sw128(k_smem + (s * kHalves + hf) * L::kKHalfBytes + off, 16, 1024);
-            if (PASS2) mma_ss(tmem_base + buf * 128, dk, dq, idesc, kk > 0);
-            else       mma_ss(tmem_base + buf * 128, dq, dk, idesc, kk > 0);
+          for (int hf = 0; hf < kHalves; ++hf) {
+            const uint32_t q = ql + hf * (L::kQHalfBytes / 16), k = kl + hf * (L::kKHalfBytes / 16);
+            mma_ss_4steps(tmem_base + buf * 128, PASS2 ? k : q, PASS2 ? q : k, hi, idesc, hf > 0 ? 1u : 0u);
           }
           mma_commit(bar_sfull + 8 * buf);
+          if (++buf == kScBufs) { buf = 0; buf_ph ^= 1u; }
         }
         if (!ok) break;
         mma_commit(bar_kempty + 8 * s);
+        if (++s == kScKStages) { s = 0; k_ph ^= 1u; }
       }
     }
   } else {
@@ -225,12 +244,11 @@ score_sm100_kernel(const __grid_constant__ ScoreLayers layers, const __grid_cons
               const float4* l4 = reinterpret_cast<const float4*>(lse2s + c * 128);
               float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll
-              for (int i = 0; i < 32; ++i) {
-                const float4 lv = l4[i];
-                a0 += fast_exp2(fmaf(__uint_as_float(s[4 * i]), scale_log2, -lv.x));
-                a1 += fast_exp2(fmaf(__uint_as_float(s[4 * i + 1]), scale_log2, -lv.y));
-                a2 += fast_exp2(fmaf(__uint_as_float(s[4 * i + 2]), scale_log2, -lv.z));
-                a3 += fast_exp2(fmaf(__uint_as_float(s[4 * i + 3]), scale_log2, -lv.w));
+              for (int i = 0; i < 128; i += 16) {
+                float nl[16];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) *reinterpret_cast<float4*>(nl + 4 * e) = l4[i / 4 + e];
+                exp2_sum16<true>(s + i, scale_log2, nl, a0, a1, a2, a3);
               }
               acc += (a0 + a1) + (a2 + a3);
             } else {
@@ -250,13 +268,9 @@ score_sm100_kernel(const __grid_constant__ ScoreLayers layers, const __grid_cons
               const float m_new = fmaxf(m_row[c], mx * scale_log2);
               if (m_new > -INFINITY) {
                 float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+                const float neg_m = -m_new;
 #pragma unroll
-                for (int i = 0; i < 128; i += 4) {
-                  a0 += fast_exp2(fmaf(__uint_as_float(s[i]), scale_log2, -m_new));
-                  a1 += fast_exp2(fmaf(__uint_as_float(s[i + 1]), scale_log2, -m_new));
-                  a2 += fast_exp2(fmaf(__uint_as_float(s[i + 2]), scale_log2, -m_new));
-                  a3 += fast_exp2(fmaf(__uint_as_float(s[i + 3]), scale_log2, -m_new));
-                }
+                for (int i = 0; i < 128; i += 16) exp2_sum16<false>(s + i, scale_log2, &neg_m, a0, a1, a2, a3);
                 z_row[c] = z_row[c] * fast_exp2(m_row[c] - m_new) + ((a0 + a1) + (a2 + a3));
                 m_row[c] = m_new;
               }
@@ -297,7 +311,6 @@ score_sm100_kernel(const __grid_constant__ ScoreLayers layers, const __grid_cons
     tc_fence_after();
     tmem_dealloc(tmem_base, 512);
   }
-  (void)n_items;
 }
 
 // ---- host side ------------------------------------------------------------------------------------------
