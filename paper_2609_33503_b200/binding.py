@@ -53,6 +53,29 @@ class _CacheView(ctypes.Structure):
                 ("head_stride", ctypes.c_int64), ("h_req_token_offset", ctypes.POINTER(ctypes.c_int64))]
 
 
+# Argument types of the entry points, declared once so that a call passes plain integers and floats (p pointer or stream,
+# i int32, l int64, z size_t, f float, d double): a ctypes object per argument and a stream object per call were most of
+# the 15 us that a call of a decode step took on the host.
+_CTYPE = {"p": ctypes.c_void_p, "i": ctypes.c_int32, "l": ctypes.c_int64, "z": ctypes.c_size_t, "f": ctypes.c_float, "d": ctypes.c_double}
+_ST = ctypes.c_int32
+_SIGNATURES = {
+    "relaxkv_status_string": (ctypes.c_char_p, "i"), "relaxkv_anchor_count": (ctypes.c_int32, "id"),
+    "relaxkv_workspace_bytes": (ctypes.c_size_t, "pip"), "relaxkv_set_chained_launch": (ctypes.c_int32, "i"),
+    "relaxkv_score_select": (_ST, "pi pp pp ppp pzp"), "relaxkv_select_topk": (_ST, "pip ppp p"),
+    "relaxkv_build_active_sets": (_ST, "pipp pppppp p pzp"), "relaxkv_build_active_sets_static": (_ST, "pipp pppppp p p"),
+    "relaxkv_sparse_ctx_attention": (_ST, "pip ppp pppp lpp pp pzp"),
+    "relaxkv_sparse_ctx_attention_simt": (_ST, "pip ppp pppp lpp pp pzp"),
+    "relaxkv_scatter_kv": (_ST, "pp pp pppp p p"), "relaxkv_gather_kv": (_ST, "pip pp pppp p pp lp"),
+    "relaxkv_list_attention": (_ST, "pp ppp pppp lpp pp pzp"), "relaxkv_cache_attention": (_ST, "pp p pp lp pp pzp"),
+    "relaxkv_scatter_kv_lists": (_ST, "pp pp pp p p"), "relaxkv_mean_scores": (_ST, "pi pp p"),
+    "relaxkv_scale_scores": (_ST, "pi pf p"), "relaxkv_query_prefill_attention": (_ST, "pp ppp p pzp"),
+    "relaxkv_rmsnorm": (_ST, "ppp li f p"), "relaxkv_linear": (_ST, "pppp lii p"), "relaxkv_linear_qkv": (_ST, "pp ppp liii p"),
+    "relaxkv_linear_swiglu": (_ST, "ppp lii p"), "relaxkv_rope": (_ST, "p lii p f p"),
+    "relaxkv_qk_norm_rope": (_ST, "pp liii pp f p f p"), "relaxkv_swiglu": (_ST, "pp li p"),
+    "relaxkv_target_positions": (_ST, "p pppp p p p"), "relaxkv_carry_rows": (_ST, "p pp i ppp p p"),
+    "relaxkv_debug_wait_timeout": (_ST, "p"), "relaxkv_read_device_status": (_ST, "pp p"),
+}
+
 _lib = None
 
 
@@ -64,14 +87,9 @@ def lib() -> ctypes.CDLL:
             raise RuntimeError(f"{LIB_PATH} is missing: build it with `python -m paper_2609_33503_b200.build` "
                                "(nvcc, sm_100a). There is no CPU fallback.")
         l = ctypes.CDLL(LIB_PATH)
-        l.relaxkv_status_string.restype = ctypes.c_char_p
-        l.relaxkv_status_string.argtypes = [ctypes.c_int32]
-        l.relaxkv_anchor_count.restype = ctypes.c_int32
-        l.relaxkv_anchor_count.argtypes = [ctypes.c_int32, ctypes.c_double]
-        l.relaxkv_workspace_bytes.restype = ctypes.c_size_t
-        l.relaxkv_workspace_bytes.argtypes = [ctypes.c_void_p, ctypes.c_int32, ctypes.c_void_p]
-        for name in ENTRY_POINTS[3:]:
-            getattr(l, name).restype = ctypes.c_int32
+        for name, (restype, args) in _SIGNATURES.items():
+            fn = getattr(l, name)
+            fn.restype, fn.argtypes = restype, [_CTYPE[c] for c in args.replace(" ", "")]
         _lib = l
     return _lib
 
@@ -94,17 +112,23 @@ def _check(status: int, where: str) -> None:
 def _i32(xs: Optional[Sequence[int]]):
     if xs is None:
         return None
-    return (ctypes.c_int32 * len(xs))(*[int(x) for x in xs])
+    return (ctypes.c_int32 * len(xs))(*map(int, xs))
 
 
-def _ptr(t: Optional[torch.Tensor]):
-    return ctypes.c_void_p(None) if t is None else ctypes.c_void_p(t.data_ptr())
+def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)     # the handle without a Stream object around it
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
+def _stream(stream) -> int:
     if stream is None:
+        if _raw_stream is not None and _current_device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_current_device())
         stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 class Shape:
@@ -183,7 +207,7 @@ def relaxkv_score_select(shape: Shape, q_layers: List[torch.Tensor], cache_layer
         lses = (ctypes.c_void_p * n_layers)(*[(t.data_ptr() if t is not None else None) for t in row_lse_layers])
     _check(lib().relaxkv_score_select(shape.ref(), n_layers, qs, caches, lses, _i32(k), _ptr(raw_scores_out),
                                       _ptr(norm_scores_out), _ptr(anchors_out), _ptr(workspace),
-                                      ctypes.c_size_t(workspace.numel() * workspace.element_size()), _stream(stream)),
+                                      workspace.nbytes, _stream(stream)),
            "relaxkv_score_select")
 
 
@@ -203,7 +227,7 @@ def relaxkv_build_active_sets(shape: Shape, n_layers: int, k: Sequence[int], anc
                                            _ptr(highest_layer_out), _ptr(u_pos_out), _ptr(u_cu_out),
                                            _ptr(u_rank_out), _ptr(r_rank_out), _ptr(r_cu_out), _ptr(counts_pinned),
                                            _ptr(workspace),
-                                           ctypes.c_size_t(workspace.numel() * workspace.element_size()),
+                                           workspace.nbytes,
                                            _stream(stream)),
            "relaxkv_build_active_sets")
 
@@ -226,9 +250,9 @@ def _attention(fn_name, shape, mode, cache, q_new, k_new, v_new, u_pos, u_cu, r_
                max_ctx, out, lse_out, workspace, stream):
     fn = getattr(lib(), fn_name)
     _check(fn(shape.ref(), int(mode), cache.ref(), _ptr(q_new), _ptr(k_new), _ptr(v_new), _ptr(u_pos), _ptr(u_cu),
-              _ptr(r_rank), _ptr(r_cu_layer), ctypes.c_int64(q_new.shape[0]), _i32(max_targets), _i32(max_ctx),
+              _ptr(r_rank), _ptr(r_cu_layer), q_new.shape[0], _i32(max_targets), _i32(max_ctx),
               _ptr(out), _ptr(lse_out), _ptr(workspace),
-              ctypes.c_size_t(workspace.numel() * workspace.element_size()), _stream(stream)), fn_name)
+              workspace.nbytes, _stream(stream)), fn_name)
 
 
 def relaxkv_sparse_ctx_attention(shape: Shape, mode: int, cache: CacheView, q_new: torch.Tensor,
@@ -262,7 +286,7 @@ def relaxkv_gather_kv(shape: Shape, mode: int, cache: CacheView, k_new: Optional
                       v_ctx_out: torch.Tensor, stream=None) -> None:
     _check(lib().relaxkv_gather_kv(shape.ref(), int(mode), cache.ref(), _ptr(k_new), _ptr(v_new), _ptr(u_pos),
                                    _ptr(u_cu), _ptr(r_rank), _ptr(r_cu_layer), _i32(max_ctx), _ptr(k_ctx_out),
-                                   _ptr(v_ctx_out), ctypes.c_int64(k_ctx_out.shape[0]), _stream(stream)),
+                                   _ptr(v_ctx_out), k_ctx_out.shape[0], _stream(stream)),
            "relaxkv_gather_kv")
 
 
@@ -272,9 +296,9 @@ def relaxkv_list_attention(shape: Shape, cache: CacheView, q_new: torch.Tensor, 
                            max_ctx: Sequence[int], out: torch.Tensor, workspace: torch.Tensor,
                            lse_out: Optional[torch.Tensor] = None, stream=None) -> None:
     _check(lib().relaxkv_list_attention(shape.ref(), cache.ref(), _ptr(q_new), _ptr(k_new), _ptr(v_new), _ptr(ctx_pos),
-                                        _ptr(ctx_cu), _ptr(tgt_pos), _ptr(tgt_cu), ctypes.c_int64(q_new.shape[0]),
+                                        _ptr(ctx_cu), _ptr(tgt_pos), _ptr(tgt_cu), q_new.shape[0],
                                         _i32(max_targets), _i32(max_ctx), _ptr(out), _ptr(lse_out), _ptr(workspace),
-                                        ctypes.c_size_t(workspace.numel() * workspace.element_size()), _stream(stream)),
+                                        workspace.nbytes, _stream(stream)),
            "relaxkv_list_attention")
 
 
@@ -282,8 +306,8 @@ def relaxkv_cache_attention(shape: Shape, cache: CacheView, q_new: torch.Tensor,
                             max_targets: Sequence[int], out: torch.Tensor, workspace: torch.Tensor,
                             lse_out: Optional[torch.Tensor] = None, stream=None) -> None:
     _check(lib().relaxkv_cache_attention(shape.ref(), cache.ref(), _ptr(q_new), _ptr(tgt_pos), _ptr(tgt_cu),
-                                         ctypes.c_int64(q_new.shape[0]), _i32(max_targets), _ptr(out), _ptr(lse_out),
-                                         _ptr(workspace), ctypes.c_size_t(workspace.numel() * workspace.element_size()),
+                                         q_new.shape[0], _i32(max_targets), _ptr(out), _ptr(lse_out),
+                                         _ptr(workspace), workspace.nbytes,
                                          _stream(stream)),
            "relaxkv_cache_attention")
 
@@ -293,7 +317,7 @@ def relaxkv_query_prefill_attention(shape: Shape, cache: CacheView, q: torch.Ten
     """shape.ctx_lens = context tokens, shape.q_lens = query tokens; the cache holds both (context rows first)."""
     _check(lib().relaxkv_query_prefill_attention(shape.ref(), cache.ref(), _ptr(q), _ptr(out), _ptr(lse_out),
                                                  _ptr(raw_scores_out), _ptr(workspace),
-                                                 ctypes.c_size_t(workspace.numel() * workspace.element_size()),
+                                                 workspace.nbytes,
                                                  _stream(stream)),
            "relaxkv_query_prefill_attention")
 
@@ -311,19 +335,19 @@ def relaxkv_mean_scores(shape: Shape, n_layers: int, scores: torch.Tensor, mean_
 
 def relaxkv_scale_scores(shape: Shape, n_layers: int, scores: torch.Tensor, factor: float, stream=None) -> None:
     """scores *= factor in place (fp32 [n_layers, sum T_c] on the device)."""
-    _check(lib().relaxkv_scale_scores(shape.ref(), int(n_layers), _ptr(scores), ctypes.c_float(factor), _stream(stream)),
+    _check(lib().relaxkv_scale_scores(shape.ref(), int(n_layers), _ptr(scores), float(factor), _stream(stream)),
            "relaxkv_scale_scores")
 
 
 def relaxkv_rmsnorm(x: torch.Tensor, weight: torch.Tensor, y: torch.Tensor, eps: float, stream=None) -> None:
-    _check(lib().relaxkv_rmsnorm(_ptr(x), _ptr(weight), _ptr(y), ctypes.c_int64(x.shape[0]), int(x.shape[1]),
-                                 ctypes.c_float(eps), _stream(stream)), "relaxkv_rmsnorm")
+    _check(lib().relaxkv_rmsnorm(_ptr(x), _ptr(weight), _ptr(y), x.shape[0], int(x.shape[1]),
+                                 float(eps), _stream(stream)), "relaxkv_rmsnorm")
 
 
 def relaxkv_linear(x: torch.Tensor, weight: torch.Tensor, y: torch.Tensor, residual: Optional[torch.Tensor] = None,
                    stream=None) -> None:
     """y = x weight^T (+ residual); weight is [n_out, n_in]."""
-    _check(lib().relaxkv_linear(_ptr(x), _ptr(weight), _ptr(residual), _ptr(y), ctypes.c_int64(x.shape[0]),
+    _check(lib().relaxkv_linear(_ptr(x), _ptr(weight), _ptr(residual), _ptr(y), x.shape[0],
                                 int(weight.shape[0]), int(weight.shape[1]), _stream(stream)), "relaxkv_linear")
 
 
@@ -339,7 +363,7 @@ def relaxkv_linear_qkv(x: torch.Tensor, w_qkv: torch.Tensor, q: torch.Tensor, k:
     n = x.shape[0]
     n_q, n_kv = q.numel() // max(n, 1), k.numel() // max(n, 1)
     assert w_qkv.shape[0] == n_q + 2 * n_kv and v.numel() == k.numel()
-    _check(lib().relaxkv_linear_qkv(_ptr(x), _ptr(w_qkv), _ptr(q), _ptr(k), _ptr(v), ctypes.c_int64(n), int(n_q), int(n_kv),
+    _check(lib().relaxkv_linear_qkv(_ptr(x), _ptr(w_qkv), _ptr(q), _ptr(k), _ptr(v), n, int(n_q), int(n_kv),
                                     int(w_qkv.shape[1]), _stream(stream)), "relaxkv_linear_qkv")
 
 
@@ -355,28 +379,28 @@ def tile_gate_up(w_gate_up: torch.Tensor) -> torch.Tensor:
 
 
 def relaxkv_linear_swiglu(x: torch.Tensor, weight_tiled: torch.Tensor, out: torch.Tensor, stream=None) -> None:
-    _check(lib().relaxkv_linear_swiglu(_ptr(x), _ptr(weight_tiled), _ptr(out), ctypes.c_int64(x.shape[0]),
+    _check(lib().relaxkv_linear_swiglu(_ptr(x), _ptr(weight_tiled), _ptr(out), x.shape[0],
                                        int(weight_tiled.shape[0] // 2), int(weight_tiled.shape[1]), _stream(stream)),
            "relaxkv_linear_swiglu")
 
 
 def relaxkv_rope(x: torch.Tensor, positions: torch.Tensor, theta: float, stream=None) -> None:
     """In place on x [rows, heads, D]; positions int32 [rows]."""
-    _check(lib().relaxkv_rope(_ptr(x), ctypes.c_int64(x.shape[0]), int(x.shape[1]), int(x.shape[2]), _ptr(positions),
-                              ctypes.c_float(theta), _stream(stream)), "relaxkv_rope")
+    _check(lib().relaxkv_rope(_ptr(x), x.shape[0], int(x.shape[1]), int(x.shape[2]), _ptr(positions),
+                              float(theta), _stream(stream)), "relaxkv_rope")
 
 
 def relaxkv_qk_norm_rope(q: torch.Tensor, k: torch.Tensor, positions: torch.Tensor, theta: float,
                          w_q_norm: Optional[torch.Tensor] = None, w_k_norm: Optional[torch.Tensor] = None, eps: float = 1e-6,
                          stream=None) -> None:
     """Per-head RMSNorm (when weights are given) and rotary embedding of q [n, H, D] and k [n, H_kv, D], in place."""
-    _check(lib().relaxkv_qk_norm_rope(_ptr(q), _ptr(k), ctypes.c_int64(q.shape[0]), int(q.shape[1]), int(k.shape[1]),
-                                      int(q.shape[2]), _ptr(w_q_norm), _ptr(w_k_norm), ctypes.c_float(eps), _ptr(positions),
-                                      ctypes.c_float(theta), _stream(stream)), "relaxkv_qk_norm_rope")
+    _check(lib().relaxkv_qk_norm_rope(_ptr(q), _ptr(k), q.shape[0], int(q.shape[1]), int(k.shape[1]),
+                                      int(q.shape[2]), _ptr(w_q_norm), _ptr(w_k_norm), float(eps), _ptr(positions),
+                                      float(theta), _stream(stream)), "relaxkv_qk_norm_rope")
 
 
 def relaxkv_swiglu(gate_up: torch.Tensor, out: torch.Tensor, stream=None) -> None:
-    _check(lib().relaxkv_swiglu(_ptr(gate_up), _ptr(out), ctypes.c_int64(gate_up.shape[0]), int(out.shape[1]),
+    _check(lib().relaxkv_swiglu(_ptr(gate_up), _ptr(out), gate_up.shape[0], int(out.shape[1]),
                                 _stream(stream)), "relaxkv_swiglu")
 
 

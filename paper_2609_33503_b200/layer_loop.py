@@ -58,14 +58,14 @@ class LayerLoop:
             rec("norm", lambda: B.relaxkv_rmsnorm(h, w["w_in_norm"], x, blk.eps))
             if "w_qkv" not in w:                            # weight-loading step, once per layer: [Wq; Wk; Wv] stacked
                 w["w_qkv"] = B.stack_qkv(w["wq"], w["wk"], w["wv"])
-            rec("qkv_proj", lambda: B.relaxkv_linear_qkv(x, w["w_qkv"], q.view(n, -1), k.view(n, -1), v.view(n, -1)))
+            rec("qkv_proj", lambda: B.relaxkv_linear_qkv(x, w["w_qkv"], q, k, v))
             # per-head RMSNorm of the projected queries and keys (models that have one) and the rotary embedding at the
             # targets' original positions: one pass over q and k
             rec("rope", lambda: (B.relaxkv_target_positions(s.shape, s.u_pos, s.u_cu, s.r_rank, s.r_cu_layer(l), n_r[l], pos),
                                  B.relaxkv_qk_norm_rope(q, k, pos, blk.rope_theta, w.get("w_q_norm"), w.get("w_k_norm"), blk.eps)))
             rec("attention", lambda: s.attention(l, caches[l], q, k, v, o, n_r[l], n_u))
             rec("scatter", lambda: s.scatter(l, caches[l], k, v, n_r[l]))
-            rec("o_proj", lambda: B.relaxkv_linear(o.view(n, -1), w["wo"], a, residual=h))
+            rec("o_proj", lambda: B.relaxkv_linear(o, w["wo"], a, residual=h))
             rec("norm", lambda: B.relaxkv_rmsnorm(a, w["w_post_norm"], x, blk.eps))
             if blk.inter % 128 == 0:
                 if "w_gate_up_tiled" not in w:          # weight-loading step, once per layer

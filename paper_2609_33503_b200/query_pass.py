@@ -77,11 +77,11 @@ class QueryPass:
         rec("norm", lambda: B.relaxkv_rmsnorm(h, w["w_in_norm"], x, blk.eps))
         if "w_qkv" not in w:                            # weight-loading step, once per layer: [Wq; Wk; Wv] stacked
             w["w_qkv"] = B.stack_qkv(w["wq"], w["wk"], w["wv"])
-        rec("qkv_proj", lambda: B.relaxkv_linear_qkv(x, w["w_qkv"], q.view(n, -1), k.view(n, -1), v.view(n, -1)))
+        rec("qkv_proj", lambda: B.relaxkv_linear_qkv(x, w["w_qkv"], q, k, v))
         rec("rope", lambda: B.relaxkv_qk_norm_rope(q, k, pos, blk.rope_theta, w.get("w_q_norm"), w.get("w_k_norm"), blk.eps))
         rec("append_kv", lambda: B.relaxkv_scatter_kv_lists(shape, cache, k, v, pos, cu, counts))
         rec("attention", attend)
-        rec("o_proj", lambda: B.relaxkv_linear(o.view(n, -1), w["wo"], a, residual=h))
+        rec("o_proj", lambda: B.relaxkv_linear(o, w["wo"], a, residual=h))
         rec("norm", lambda: B.relaxkv_rmsnorm(a, w["w_post_norm"], x, blk.eps))
         if blk.inter % 128 == 0:
             if "w_gate_up_tiled" not in w:              # weight-loading step, once per layer
