@@ -1049,18 +1049,35 @@ combine_splits_kernel(const float* part_o, const float* part_lse, int n_splits,
   __shared__ float wgt_s[kCombineThreads / 32][kMaxCombineSplits];
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long w = (long long)blockIdx.x * (kCombineThreads / 32) + wib;
-  griddep_launch();
-  griddep_wait();                               // the partial results come from the kernel before
-  const long long rows_true = min((long long)(r_cu[n_req] - r_cu[0]), n_target_rows);
-  if (w >= rows_true * H) return;
   const long long row = w / H;
   const int h = (int)(w - row * H);
+  const bool mine = row < n_target_rows;
+  const int per = D / 32;                       // 2 or 4 consecutive floats per lane
+  const float* o = part_o + (row * H + h) * D + lane * per;
+  const long long sp_stride = n_target_rows * H * D;
+  auto load = [&](int sp) -> float4 {
+    if (per == 4) return *reinterpret_cast<const float4*>(o + sp * sp_stride);
+    const float2 v = *reinterpret_cast<const float2*>(o + sp * sp_stride);
+    return make_float4(v.x, v.y, 0.f, 0.f);
+  };
+  griddep_launch();
+  griddep_wait();                               // the partial results come from the kernel before
+  if (!mine) return;
+  // A launch of a few rows is a chain of memory latencies, so the first partial results, the log-sum-exps and the row
+  // count are fetched side by side (what rows past the true count or empty splits hold is not used), and each further
+  // group of partial results while the one before is added up.
+  constexpr int U = 8;
+  float4 v[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) v[u] = u < n_splits ? load(u) : make_float4(0.f, 0.f, 0.f, 0.f);
+  const long long rows_true = min((long long)(r_cu[n_req] - r_cu[0]), n_target_rows);
   float mx = -INFINITY;
   for (int sp = lane; sp < n_splits; sp += 32) {
     const float l = part_lse[((long long)sp * n_target_rows + row) * H + h];
     wgt_s[wib][sp] = l;
     mx = fmaxf(mx, l);
   }
+  if (row >= rows_true) return;
   mx = warp_reduce_max(mx);
   __syncwarp();
   for (int sp = lane; sp < n_splits; sp += 32) {
@@ -1068,30 +1085,29 @@ combine_splits_kernel(const float* part_o, const float* part_lse, int n_splits,
     wgt_s[wib][sp] = (l == -INFINITY || mx == -INFINITY) ? 0.f : __expf(l - mx);
   }
   __syncwarp();
-  const int per = D / 32;                       // 2 or 4 consecutive floats per lane
   float acc[4] = {0.f, 0.f, 0.f, 0.f};
   float den = 0.f;
-  const float* o = part_o + (row * H + h) * D + lane * per;
-  const long long sp_stride = n_target_rows * H * D;
-#pragma unroll 8
-  for (int sp = 0; sp < n_splits; ++sp) {       // fixed order: reproducible
-    const float wgt = wgt_s[wib][sp];
-    den += wgt;
-    const bool live = wgt > 0.f;                  // an empty split wrote no partial output: whatever is there is ignored
-    if (per == 4) {
-      const float4 v = *reinterpret_cast<const float4*>(o + sp * sp_stride);
-      acc[0] = fmaf(wgt, live ? v.x : 0.f, acc[0]); acc[1] = fmaf(wgt, live ? v.y : 0.f, acc[1]);
-      acc[2] = fmaf(wgt, live ? v.z : 0.f, acc[2]); acc[3] = fmaf(wgt, live ? v.w : 0.f, acc[3]);
-    } else {
-      const float2 v = *reinterpret_cast<const float2*>(o + sp * sp_stride);
-      acc[0] = fmaf(wgt, live ? v.x : 0.f, acc[0]); acc[1] = fmaf(wgt, live ? v.y : 0.f, acc[1]);
+  for (int s0 = 0; s0 < n_splits; s0 += U) {    // fixed order: reproducible
+    float4 nx[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) nx[u] = s0 + U + u < n_splits ? load(s0 + U + u) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const float wgt = s0 + u < n_splits ? wgt_s[wib][s0 + u] : 0.f;
+      const bool live = wgt > 0.f;                // an empty split wrote no partial output: whatever is there is ignored
+      den += wgt;
+      acc[0] = fmaf(wgt, live ? v[u].x : 0.f, acc[0]); acc[1] = fmaf(wgt, live ? v[u].y : 0.f, acc[1]);
+      acc[2] = fmaf(wgt, live ? v[u].z : 0.f, acc[2]); acc[3] = fmaf(wgt, live ? v[u].w : 0.f, acc[3]);
+      v[u] = nx[u];
     }
   }
   const float inv = den > 0.f ? 1.f / den : 0.f;
   uint16_t* optr = out + (row * H + h) * D + lane * per;
-  for (int e = 0; e < per; e += 2) {
-    __nv_bfloat162 h2 = __floats2bfloat162_rn(acc[e] * inv, acc[e + 1] * inv);
-    *reinterpret_cast<uint32_t*>(optr + e) = *reinterpret_cast<uint32_t*>(&h2);
+  __nv_bfloat162 h01 = __floats2bfloat162_rn(acc[0] * inv, acc[1] * inv);
+  *reinterpret_cast<uint32_t*>(optr) = *reinterpret_cast<uint32_t*>(&h01);
+  if (per == 4) {
+    __nv_bfloat162 h23 = __floats2bfloat162_rn(acc[2] * inv, acc[3] * inv);
+    *reinterpret_cast<uint32_t*>(optr + 2) = *reinterpret_cast<uint32_t*>(&h23);
   }
   if (lane == 0 && lse_out) lse_out[(long long)h * n_target_rows + row] = den > 0.f ? mx + logf(den) : -INFINITY;
 }

@@ -60,34 +60,28 @@ __device__ __forceinline__ void mma_bf16_16816(float* d, const uint32_t* a, uint
 template <int D, int GMAX>
 __global__ void __launch_bounds__(kDecThreads, 1)
 decode_attention_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
-                        const __grid_constant__ ReqTable rt, const uint16_t* __restrict__ q,
-                        const int* __restrict__ tgt_pos, const int* __restrict__ tgt_cu, long long n_target_rows, int H, int Hkv,
+                        const __grid_constant__ ReqTable rt, int max_splits, const uint16_t* q,
+                        const int* tgt_pos, const int* tgt_cu, long long n_target_rows, int H, int Hkv,
                         float scale_log2, uint16_t* __restrict__ out, float* __restrict__ lse_out, float* __restrict__ part_o,
                         float* __restrict__ part_lse, DeviceStatus* st) {
   using L = DecSmem<D>;
   const int G = H / Hkv;
-  const int b = blockIdx.z, hd = blockIdx.y, split = blockIdx.x, n_splits = gridDim.x;
+  // rt.tile_cu: prefix of the splits per request
+  const int b = find_segment(rt.tile_cu, rt.n_req, (int)blockIdx.x), hd = blockIdx.y;
+  const int split = (int)blockIdx.x - rt.tile_cu[b], n_splits = rt.tile_cu[b + 1] - rt.tile_cu[b];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   griddep_launch();
-  griddep_wait();                          // q, the lists and the newest cache row come from the kernels before
-  const int nr = tgt_cu[b + 1] - tgt_cu[b];
-  if (nr <= 0) return;
-  const long long row = (long long)tgt_cu[b] - tgt_cu[0];
-  if (nr > rt.bound_a[b] || nr > 1 || row >= n_target_rows) {      // more targets than the host bound (one): touch nothing
-    if (threadIdx.x == 0) report(st, RELAXKV_ERR_BAD_INDEX, KID_ATTN_SIMT, nr, (int)row);
-    return;
+  if (threadIdx.x == kDecConsumers * 32) {
+    // The kernels in front are short and leave HBM idle: the ring's first tiles are requested into L2 meanwhile (their
+    // place by the host's bound on the context; a prefetch only, the rows are read after the wait).
+    prefetch_tensormap(&tm_k); prefetch_tensormap(&tm_v);
+    const int n_all = (rt.ctx_len[b] + kDecTile - 1) / kDecTile, share = (n_all + n_splits - 1) / n_splits;
+    for (int t = split * share; t < min(n_all, split * share + min(share, kDecStages)); ++t)
+      for (int hf = 0; hf < L::kHalves; ++hf) {
+        tma_prefetch_3d(&tm_k, hf * 64, hd, (int)rt.tok_off[b] + t * kDecTile);
+        tma_prefetch_3d(&tm_v, hf * 64, hd, (int)rt.tok_off[b] + t * kDecTile);
+      }
   }
-  const int pos = tgt_pos[tgt_cu[b]];
-  if (pos < 0 || pos >= rt.ctx_len[b]) {
-    if (threadIdx.x == 0) report(st, RELAXKV_ERR_BAD_INDEX, KID_ATTN_SIMT, pos, rt.ctx_len[b]);
-    return;
-  }
-  if (*reinterpret_cast<volatile int*>(&st->status) == RELAXKV_ERR_TIMEOUT) return;   // drain after a timeout
-  const int n_keys = pos + 1;
-  const int n_tiles = (n_keys + kDecTile - 1) / kDecTile;
-  const int per = (n_tiles + n_splits - 1) / n_splits;
-  const int t0 = split * per, t1 = min(n_tiles, t0 + per);            // this block's tiles
-
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
@@ -104,6 +98,29 @@ decode_attention_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
     fence_barrier_init();
     fence_proxy_async_smem();
   }
+  griddep_wait();                          // q, the lists and the newest cache row come from the kernels before
+  const int c0 = tgt_cu[0], cb = tgt_cu[b], nr = tgt_cu[b + 1] - cb;
+  if (nr <= 0) return;
+  const long long row = (long long)cb - c0;
+  if (nr > rt.bound_a[b] || nr > 1 || row >= n_target_rows) {      // more targets than the host bound (one): touch nothing
+    if (threadIdx.x == 0) report(st, RELAXKV_ERR_BAD_INDEX, KID_ATTN_SIMT, nr, (int)row);
+    return;
+  }
+  const int pos = tgt_pos[cb];
+  if (pos < 0 || pos >= rt.ctx_len[b]) {
+    if (threadIdx.x == 0) report(st, RELAXKV_ERR_BAD_INDEX, KID_ATTN_SIMT, pos, rt.ctx_len[b]);
+    return;
+  }
+  if (*reinterpret_cast<volatile int*>(&st->status) == RELAXKV_ERR_TIMEOUT) return;   // drain after a timeout
+  // the merge walks max_splits partial results of every row: those that no block of this request computes are empty
+  if (split == 0)
+    for (int i = threadIdx.x; i < (max_splits - n_splits) * G; i += kDecThreads)
+      part_lse[((long long)(n_splits + i / G) * n_target_rows + row) * H + hd * G + i % G] = -INFINITY;
+  const int n_keys = pos + 1;
+  const int n_tiles = (n_keys + kDecTile - 1) / kDecTile;
+  const int per = (n_tiles + n_splits - 1) / n_splits;
+  const int t0 = split * per, t1 = min(n_tiles, t0 + per);            // this block's tiles
+
   for (int i = threadIdx.x; i < GMAX * D; i += kDecThreads) {
     const int g = i / D, d = i - g * D;
     q_s[g][d] = (g < G) ? bf16_bits_to_float(q[(row * H + hd * G + g) * D + d]) : 0.f;     // exact; the scale goes on S
@@ -116,7 +133,6 @@ decode_attention_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
   if (warp == kDecConsumers) {
     // ================= producer =================
     if (lane == 0) {
-      prefetch_tensormap(&tm_k); prefetch_tensormap(&tm_v);
       const int row0 = (int)rt.tok_off[b];
       for (int t = t0, it = 0; t < t1; ++t, ++it) {
         const int s = it % kDecStages;
@@ -290,7 +306,7 @@ decode_attention_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
     const float val = none ? 0.f : acc / zb;
     const float lse = none ? -INFINITY : (mb + log2f(zb)) * kLn2D;
     const int h = hd * G + g;
-    if (n_splits == 1) {
+    if (max_splits == 1) {
       const __nv_bfloat16 hv = __float2bfloat16(val);
       out[(row * H + h) * D + d] = *reinterpret_cast<const uint16_t*>(&hv);
       if (d == 0 && lse_out) lse_out[(long long)h * n_target_rows + row] = lse;
@@ -303,7 +319,7 @@ decode_attention_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
 }
 
 template <int D, int GMAX>
-static relaxkv_status launch_g(const CUtensorMap& tm_k, const CUtensorMap& tm_v, const AttnPlan& plan, dim3 grid, const void* q,
+static relaxkv_status launch_g(const CUtensorMap& tm_k, const CUtensorMap& tm_v, const AttnPlan& plan, int max_splits, const void* q,
                                const int32_t* tgt_pos, const int32_t* tgt_cu, int64_t n_target_rows, int H, int Hkv, float scale_log2,
                                void* out, float* lse_out, DeviceStatus* st, cudaStream_t stream) {
   static std::atomic<int> attr_done[kMaxDevices];
@@ -314,13 +330,14 @@ static relaxkv_status launch_g(const CUtensorMap& tm_k, const CUtensorMap& tm_v,
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, DecSmem<D>::kDynamic) != cudaSuccess) return RELAXKV_ERR_CUDA;
     attr_done[dev].store(1, std::memory_order_release);
   }
-  return cuda_ok(launch_chained(kern, grid, kDecThreads, DecSmem<D>::kDynamic, stream, tm_k, tm_v, plan.rt,
+  const dim3 grid((unsigned)plan.rt.tile_cu[plan.rt.n_req], (unsigned)Hkv);
+  return cuda_ok(launch_chained(kern, grid, kDecThreads, DecSmem<D>::kDynamic, stream, tm_k, tm_v, plan.rt, max_splits,
                                 static_cast<const uint16_t*>(q), tgt_pos, tgt_cu, (long long)n_target_rows, H, Hkv, scale_log2,
                                 static_cast<uint16_t*>(out), lse_out, plan.split_o, plan.split_lse, st));
 }
 
 template <int D>
-static relaxkv_status launch_d(const relaxkv_shape* shape, const AttnPlan& plan, const void* q, const int32_t* tgt_pos,
+static relaxkv_status launch_d(const relaxkv_shape* shape, AttnPlan plan, const void* q, const int32_t* tgt_pos,
                                const int32_t* tgt_cu, int64_t n_target_rows, void* out, float* lse_out, cudaStream_t stream) {
   const int H = shape->n_q_heads, Hkv = shape->n_kv_heads, G = H / Hkv, B = shape->n_req;
   const int sms = sm_count_of_current_device();
@@ -333,25 +350,33 @@ static relaxkv_status launch_d(const relaxkv_shape* shape, const AttnPlan& plan,
       !make_map_3d(&tm_v, plan.v_base, D, Hkv, (uint64_t)plan.ctx_rows, plan.kv_head_stride_bytes, plan.kv_token_stride_bytes, 1u,
                    (uint32_t)kDecTile))
     return RELAXKV_ERR_CUDA;
-  int max_ctx = 1;
-  for (int b = 0; b < B; ++b) max_ctx = std::max(max_ctx, shape->h_ctx_len[b]);
-  const int max_tiles = (max_ctx + kDecTile - 1) / kDecTile;
-  // one block per SM (the ring takes its shared memory): one wave of blocks, at least two tiles each, as many
-  // splits as the split workspace has slots for
-  long long n_splits = std::max<long long>(1, sms / std::max(1, B * Hkv));
-  n_splits = std::min<long long>(n_splits, std::max(1, max_tiles / 2));
-  if (shape->h_tuning && shape->h_tuning->attention_ctx_splits > 0) n_splits = shape->h_tuning->attention_ctx_splits;
-  n_splits = std::min<long long>(n_splits, kSplitRowsCap / std::max<long long>(1, n_target_rows));
-  n_splits = std::max<long long>(1, std::min<long long>(n_splits, 1024));
+  // One block per SM (the ring takes its shared memory), one wave of blocks.  All blocks get about the same number of
+  // tiles, at least two: the fewest per block for which the requests' blocks fit the wave.  (The same number of splits for
+  // every request gave contexts of 8257, 4141, 6014 and 2049 tokens four each: 17 tiles in the longest block against 8.8
+  // on average; BEFORE_AFTER.)
+  int n_tiles[kMaxReqInline];
+  long long all_tiles = 0;
+  for (int b = 0; b < B; ++b) { n_tiles[b] = (shape->h_ctx_len[b] + kDecTile - 1) / kDecTile; all_tiles += n_tiles[b]; }
+  const long long slots = std::max(1, sms / Hkv);                            // blocks per KV head
+  const long long cap = std::max<long long>(1, std::min<long long>(kSplitRowsCap / std::max<long long>(1, n_target_rows), 1024));
+  const int forced = (shape->h_tuning && shape->h_tuning->attention_ctx_splits > 0) ? shape->h_tuning->attention_ctx_splits : 0;
+  long long per = std::max<long long>(2, (all_tiles + slots - 1) / slots);
+  auto blocks_with = [&](long long p) { long long n = 0; for (int b = 0; b < B; ++b) n += (n_tiles[b] + p - 1) / p; return n; };
+  while (blocks_with(per) > std::max<long long>(slots, B)) ++per;
+  int max_splits = 1;
+  for (int b = 0; b < B; ++b) {
+    const int ns = (int)std::min<long long>(cap, forced ? forced : (n_tiles[b] + per - 1) / per);
+    plan.rt.tile_cu[b + 1] = plan.rt.tile_cu[b] + ns;
+    max_splits = std::max(max_splits, ns);
+  }
   RELAXKV_RANGE("decode_attention_kernel");
-  const dim3 grid((unsigned)n_splits, (unsigned)Hkv, (unsigned)B);
   const float scale_log2 = shape->softmax_scale * kLog2eD;
   relaxkv_status rc;
-  if (G <= 4) rc = launch_g<D, 4>(tm_k, tm_v, plan, grid, q, tgt_pos, tgt_cu, n_target_rows, H, Hkv, scale_log2, out, lse_out, st, stream);
-  else if (G <= 8) rc = launch_g<D, 8>(tm_k, tm_v, plan, grid, q, tgt_pos, tgt_cu, n_target_rows, H, Hkv, scale_log2, out, lse_out, st, stream);
-  else rc = launch_g<D, 16>(tm_k, tm_v, plan, grid, q, tgt_pos, tgt_cu, n_target_rows, H, Hkv, scale_log2, out, lse_out, st, stream);
-  if (rc != RELAXKV_OK || n_splits == 1) return rc;
-  return launch_combine_splits(plan.split_o, plan.split_lse, (int)n_splits, n_target_rows, H, shape->head_dim, tgt_cu, B,
+  if (G <= 4) rc = launch_g<D, 4>(tm_k, tm_v, plan, max_splits, q, tgt_pos, tgt_cu, n_target_rows, H, Hkv, scale_log2, out, lse_out, st, stream);
+  else if (G <= 8) rc = launch_g<D, 8>(tm_k, tm_v, plan, max_splits, q, tgt_pos, tgt_cu, n_target_rows, H, Hkv, scale_log2, out, lse_out, st, stream);
+  else rc = launch_g<D, 16>(tm_k, tm_v, plan, max_splits, q, tgt_pos, tgt_cu, n_target_rows, H, Hkv, scale_log2, out, lse_out, st, stream);
+  if (rc != RELAXKV_OK || max_splits == 1) return rc;
+  return launch_combine_splits(plan.split_o, plan.split_lse, max_splits, n_target_rows, H, shape->head_dim, tgt_cu, B,
                                plan.sum_targets, out, lse_out, stream);
 }
 
