@@ -160,6 +160,7 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const int B = rt.n_req;
   const int G = H / Hkv;
   const int n_pairs_total = rt.tile_cu[B];
+  if (threadIdx.x == 256) { prefetch_tensormap(&tm_q); prefetch_tensormap(&tm_k); prefetch_tensormap(&tm_v); }
   griddep_wait();
   // Block order.  Large contexts: KV head outermost, so one head's K/V stays in L2 while its tiles run.
   // Contexts that fit L2 whole (head_inner): tile pair outermost, so the longest tiles of every head start first.
@@ -282,7 +283,6 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   if (warp == 8) {
     // ================= TMA producer =================
     if (lane == 0) {
-      prefetch_tensormap(&tm_q); prefetch_tensormap(&tm_k); prefetch_tensormap(&tm_v);
       mbar_expect_tx(bar_q, (uint32_t)(2 * kHalves * tile_targets * G * 128));
       for (int x = 0; x < 2; ++x)
         for (int hf = 0; hf < kHalves; ++hf)
@@ -607,6 +607,7 @@ attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
   constexpr int kHalves = L::kHalves;
   constexpr uint32_t kTmemCols = 512;
   const int G = H / Hkv;
+  if (threadIdx.x == 256) { prefetch_tensormap(&tm_q); prefetch_tensormap(&tm_k); prefetch_tensormap(&tm_v); }
   griddep_wait();
   if (*reinterpret_cast<volatile int*>(&st->status) == RELAXKV_ERR_TIMEOUT) return;
 
@@ -666,7 +667,6 @@ attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
   if (warp == 8) {
     // ================= producer: work items, Q tiles, K/V tiles =================
     if (lane == 0) {
-      prefetch_tensormap(&tm_q); prefetch_tensormap(&tm_k); prefetch_tensormap(&tm_v);
       int n_fetched = 0, n_pub = 0;
       bool ok = true;
       auto fetch_work = [&](WorkItem& it) -> bool {          // next item that has work; false when the list is exhausted

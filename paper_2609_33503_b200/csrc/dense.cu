@@ -21,17 +21,36 @@ __device__ __forceinline__ uint4 pack8(const float* f) {
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// y = x / sqrt(mean(x^2) + eps) * w ; one block per row, C a multiple of 8.
+// y = x / sqrt(mean(x^2) + eps) * w ; one block per row, C a multiple of 8.  A launch of a few rows is a chain of memory
+// latencies, so the row and the weights are fetched side by side and kept in registers (up to kNormHeld columns; wider rows
+// are read again), and the weights are requested into L2 before the wait for the kernel in front.
+constexpr int kNormChunks = 4, kNormHeld = kNormChunks * 256 * 8;
 __global__ void __launch_bounds__(256)
-rmsnorm_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ w, uint16_t* __restrict__ y, int C, float eps) {
+rmsnorm_kernel(const uint16_t* x, const uint16_t* w, uint16_t* y, int C, float eps) {
   const long long row = blockIdx.x;
   const uint16_t* xr = x + row * C;
   float ss = 0.f;
   griddep_launch();
+  if ((threadIdx.x & 7) == 0)                                  // one 128-byte line per eight threads
+    for (int i = threadIdx.x * 8; i < C; i += 256 * 8) asm volatile("prefetch.global.L2 [%0];" ::"l"(w + i));
   griddep_wait();
-  for (int i = threadIdx.x * 8; i < C; i += 256 * 8) {
+  uint4 xv[kNormChunks], wv[kNormChunks];
+#pragma unroll
+  for (int c = 0; c < kNormChunks; ++c) {
+    const int i = threadIdx.x * 8 + c * 256 * 8;
+    xv[c] = i < C ? *reinterpret_cast<const uint4*>(xr + i) : make_uint4(0u, 0u, 0u, 0u);
+    wv[c] = i < C ? *reinterpret_cast<const uint4*>(w + i) : make_uint4(0u, 0u, 0u, 0u);
+  }
+#pragma unroll
+  for (int c = 0; c < kNormChunks; ++c) {
     float f[8];
-    unpack8(__ldg(reinterpret_cast<const uint4*>(xr + i)), f);
+    unpack8(xv[c], f);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) ss = fmaf(f[e], f[e], ss);
+  }
+  for (int i = threadIdx.x * 8 + kNormHeld; i < C; i += 256 * 8) {
+    float f[8];
+    unpack8(*reinterpret_cast<const uint4*>(xr + i), f);
 #pragma unroll
     for (int e = 0; e < 8; ++e) ss = fmaf(f[e], f[e], ss);
   }
@@ -43,14 +62,21 @@ rmsnorm_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ w, u
 #pragma unroll
   for (int i = 0; i < 8; ++i) tot += red[i];                 // fixed order: reproducible
   const float inv = rsqrtf(tot / (float)C + eps);
-  for (int i = threadIdx.x * 8; i < C; i += 256 * 8) {
+  auto put = [&](int i, const uint4& xi, const uint4& wi) {
     float f[8], g[8];
-    unpack8(__ldg(reinterpret_cast<const uint4*>(xr + i)), f);
-    unpack8(__ldg(reinterpret_cast<const uint4*>(w + i)), g);
+    unpack8(xi, f);
+    unpack8(wi, g);
 #pragma unroll
     for (int e = 0; e < 8; ++e) f[e] = f[e] * inv * g[e];
     *reinterpret_cast<uint4*>(y + row * C + i) = pack8(f);
+  };
+#pragma unroll
+  for (int c = 0; c < kNormChunks; ++c) {
+    const int i = threadIdx.x * 8 + c * 256 * 8;
+    if (i < C) put(i, xv[c], wv[c]);
   }
+  for (int i = threadIdx.x * 8 + kNormHeld; i < C; i += 256 * 8)
+    put(i, *reinterpret_cast<const uint4*>(xr + i), *reinterpret_cast<const uint4*>(w + i));
 }
 
 // Short rows (a head vector: C <= 256): one warp per row, each lane 8 elements, so the per-head Q/K norm of a
@@ -129,7 +155,7 @@ __global__ void rope_kernel(uint16_t* __restrict__ x, long long rows, int heads,
 template <int D>
 __global__ void __launch_bounds__(128)
 head_norm_rope_kernel(uint16_t* __restrict__ q, uint16_t* __restrict__ k, int Hq, int Hkv, int heads_per_block, const uint16_t* __restrict__ wq,
-                      const uint16_t* __restrict__ wk, float eps, const int* __restrict__ positions, double log2_theta) {
+                      const uint16_t* __restrict__ wk, float eps, const int* positions, double log2_theta) {
   constexpr int DPL = D / 32, half = D / 2;
   constexpr int U = 4;                                        // heads a warp has in flight at once
   __shared__ float cs_s[half], sn_s[half];
@@ -190,12 +216,13 @@ head_norm_rope_kernel(uint16_t* __restrict__ q, uint16_t* __restrict__ k, int Hq
     }
   };
   griddep_launch();
+  double inv_freq = 0.0;                                      // (does not depend on the kernels before)
+  if (threadIdx.x < half) inv_freq = exp2(-log2_theta * (2.0 * threadIdx.x / D));
   griddep_wait();                                             // q, k and the positions may come from the kernels before
   uint2 raw[U];
   load_batch(h_first, raw);
   if (threadIdx.x < half) {
     const int i = threadIdx.x;
-    const double inv_freq = exp2(-log2_theta * (2.0 * i / D));
     double ang = (double)positions[row] * inv_freq;
     ang -= 6.283185307179586 * floor(ang * 0.15915494309189535);
     sincosf((float)ang, &sn_s[i], &cs_s[i]);

@@ -112,12 +112,12 @@ gather_ctx_kernel(ReqTable rt, int mode, int n_kv_heads, int head_dim,
   const int B = rt.n_req;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long x0 = ((long long)blockIdx.x * kMoveWarps + warp) * rows_per_warp;
+  const uint32_t bar = smem_u32(&bars[warp]);
   griddep_launch();
+  if (lane == 0) { gave_up[warp] = 0; mbar_init(bar, 1); fence_barrier_init(); }
   griddep_wait();                              // the rows and the index lists come from earlier kernels
   if (work_counter != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *work_counter = 0;
   if (x0 >= ctx_rows) return;
-  const uint32_t bar = smem_u32(&bars[warp]);
-  if (lane == 0) { gave_up[warp] = 0; mbar_init(bar, 1); fence_barrier_init(); }
   const long long total = (mode == RELAXKV_CTX_UNION) ? (long long)u_cu[B] : rt.ctx_cu[B];
   const uint32_t row_bytes = (uint32_t)n_kv_heads * head_dim * 2;
   const uint32_t my_stage = smem_u32(stage) + (uint32_t)(warp * rows_per_warp + lane) * 2u * row_bytes;   // lanes < rows_per_warp
@@ -246,11 +246,11 @@ scatter_kv_kernel(ReqTable rt, int n_kv_heads, int head_dim,
   const int B = rt.n_req;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long y0 = ((long long)blockIdx.x * kMoveWarps + warp) * rows_per_warp;
+  const uint32_t bar = smem_u32(&bars[warp]);
   griddep_launch();
+  if (lane == 0) { gave_up[warp] = 0; mbar_init(bar, 1); fence_barrier_init(); }
   griddep_wait();                              // the rows and the index lists come from earlier kernels
   if (y0 >= rt.tile_cu[B]) return;             // rt.tile_cu = prefix of the host bounds on |R_{l,b}|
-  const uint32_t bar = smem_u32(&bars[warp]);
-  if (lane == 0) { gave_up[warp] = 0; mbar_init(bar, 1); fence_barrier_init(); }
   const uint32_t row_bytes = (uint32_t)n_kv_heads * head_dim * 2;
   const uint32_t my_stage = smem_u32(stage) + (uint32_t)(warp * rows_per_warp + lane) * 2u * row_bytes;   // lanes < rows_per_warp
   long long d = -1, s = 0;

@@ -69,6 +69,10 @@ score_sm100_kernel(const __grid_constant__ ScoreLayers layers, const __grid_cons
   constexpr int kHalves = L::kHalves;
   constexpr float kLog2e = 1.4426950408889634f;
 
+  {
+    const int layer0 = blockIdx.z / n_splits;
+    if (threadIdx.x == 0) { prefetch_tensormap(&layers.tm_q[layer0]); prefetch_tensormap(&layers.tm_k[layer0]); }
+  }
   griddep_wait();
   // ---- which unit ---------------------------------------------------------------------------------
   const int B = rt.n_req;
@@ -166,7 +170,6 @@ score_sm100_kernel(const __grid_constant__ ScoreLayers layers, const __grid_cons
   if (warp == 8) {
     // ================= TMA producer =================
     if (lane == 0) {
-      prefetch_tensormap(&tm_q); prefetch_tensormap(&tm_k);
       mbar_expect_tx(bar_q, (uint32_t)(n_box * kHalves * kScTokBox * G * 128));
       for (int i = 0; i < n_box; ++i)
         for (int hf = 0; hf < kHalves; ++hf)
