@@ -162,6 +162,7 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const int n_pairs_total = rt.tile_cu[B];
   if (threadIdx.x == 256) { prefetch_tensormap(&tm_q); prefetch_tensormap(&tm_k); prefetch_tensormap(&tm_v); }
   griddep_wait();
+  const int status = *reinterpret_cast<volatile int*>(&st->status);       // (fetched beside the lists)
   // Block order.  Large contexts: KV head outermost, so one head's K/V stays in L2 while its tiles run.
   // Contexts that fit L2 whole (head_inner): tile pair outermost, so the longest tiles of every head start first.
   const int hd = head_inner ? (int)(blockIdx.x % Hkv) : (int)(blockIdx.x / n_pairs_total);
@@ -180,7 +181,7 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     if (threadIdx.x == 0) report(st, RELAXKV_ERR_BAD_INDEX, KID_ATTN_SM100, nr, nu);
     return;
   }
-  if (*reinterpret_cast<volatile int*>(&st->status) == RELAXKV_ERR_TIMEOUT) return;   // drain after a timeout
+  if (status == RELAXKV_ERR_TIMEOUT) return;                  // drain after a timeout
   const int pair = n_pairs_true - 1 - p_rev;
   const int rho0 = pair * pair_targets;                       // first target of tile A
   const int ctx_len_b = (mode == RELAXKV_CTX_UNION) ? nu : rt.ctx_len[b];

@@ -98,7 +98,9 @@ decode_attention_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
     fence_barrier_init();
     fence_proxy_async_smem();
   }
+  __syncthreads();                         // the barriers are ready: the producer starts as soon as it knows the position
   griddep_wait();                          // q, the lists and the newest cache row come from the kernels before
+  const int status = *reinterpret_cast<volatile int*>(&st->status);
   const int c0 = tgt_cu[0], cb = tgt_cu[b], nr = tgt_cu[b + 1] - cb;
   if (nr <= 0) return;
   const long long row = (long long)cb - c0;
@@ -111,7 +113,7 @@ decode_attention_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
     if (threadIdx.x == 0) report(st, RELAXKV_ERR_BAD_INDEX, KID_ATTN_SIMT, pos, rt.ctx_len[b]);
     return;
   }
-  if (*reinterpret_cast<volatile int*>(&st->status) == RELAXKV_ERR_TIMEOUT) return;   // drain after a timeout
+  if (status == RELAXKV_ERR_TIMEOUT) return;                         // drain after a timeout
   // the merge walks max_splits partial results of every row: those that no block of this request computes are empty
   if (split == 0)
     for (int i = threadIdx.x; i < (max_splits - n_splits) * G; i += kDecThreads)
@@ -120,12 +122,6 @@ decode_attention_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
   const int n_tiles = (n_keys + kDecTile - 1) / kDecTile;
   const int per = (n_tiles + n_splits - 1) / n_splits;
   const int t0 = split * per, t1 = min(n_tiles, t0 + per);            // this block's tiles
-
-  for (int i = threadIdx.x; i < GMAX * D; i += kDecThreads) {
-    const int g = i / D, d = i - g * D;
-    q_s[g][d] = (g < G) ? bf16_bits_to_float(q[(row * H + hd * G + g) * D + d]) : 0.f;     // exact; the scale goes on S
-  }
-  __syncthreads();
 
   float frag_m[2] = {-INFINITY, -INFINITY}, frag_z[2] = {0.f, 0.f}, frag_o[D / 8][4];     // a consumer warp's result (fragment layout)
 #pragma unroll
@@ -147,6 +143,12 @@ decode_attention_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
     }
   } else {
     // ================= consumers =================
+    // the query heads (the producer is on its way already: the consumers' own barrier)
+    for (int i = threadIdx.x; i < GMAX * D; i += kDecConsumers * 32) {
+      const int g = i / D, d = i - g * D;
+      q_s[g][d] = (g < G) ? bf16_bits_to_float(q[(row * H + hd * G + g) * D + d]) : 0.f;     // exact; the scale goes on S
+    }
+    asm volatile("bar.sync 1, %0;" ::"n"(kDecConsumers * 32) : "memory");
     const int gid = lane >> 2, tig = lane & 3;                        // fragment coordinates: row gid (and gid + 8), column pair tig
     // Q as A fragments, one per 16 dims: rows = the G query heads (zero beyond)
     uint32_t qa[D / 16][4];
