@@ -179,28 +179,40 @@ constexpr int kMaxCtxSplits = 32;
 
 constexpr int kScoreLayersPerLaunch = 48;   // layers scored by one launch (their tensor maps travel as parameters)
 
-// Key-range splits for a launch that scores `layers` layers at once: at least two waves of CTAs on the 148
-// SMs (one CTA per SM), and a count that fills its last wave (every CTA of a launch does the same work).
-inline int score_splits(long long units_times_heads, int layers) {
-  const long long per = units_times_heads * layers;
-  if (per <= 0) return 1;
-  int best = 1;
-  double best_eff = 0.0;
-  for (int ns = 1; ns <= kScoreSplitsMax; ++ns) {
-    const long long ctas = per * ns;
-    if (ctas < 2 * 148 && ns < kScoreSplitsMax) continue;
-    const long long waves = (ctas + 147) / 148;
-    const double eff = (double)ctas / (double)(waves * 148);
-    if (eff > best_eff + 0.02) { best_eff = eff; best = ns; }      // prefer fewer, longer CTAs unless clearly better
-    if (ctas >= 16 * 148) break;
-  }
-  return best;
-}
-
 // Query-row blocks a request needs so that each block's rows fit resident (scoring kernel).
 inline int score_blocks(int q_len, int group) {
   const int max_tok = kScoreMaxRows / group / kScoreTokBox * kScoreTokBox;
   return q_len > 0 ? (q_len + max_tok - 1) / max_tok : 0;
+}
+
+// Key-range splits for a launch that scores `layers` layers at once (one CTA per SM, every CTA of a launch about the same
+// work): the count with the least waves x (start + 128-key tiles of a CTA x 128-row chunks of a tile x item).  Start and item
+// are what a CTA takes before its first product and per product of 128 x 128 (about 4 and 0.75 us).  With at least two
+// waves whatever the size, a 16K layer of 256 rows ran in 1.7 waves of four tiles per CTA: its scoring and schedule took 76 us,
+// 70 in one wave; the 32K pass of a query of 128 rows 60 us per layer, now 57.
+inline int score_splits(const relaxkv_shape* s, int layers) {
+  const int group = s->n_q_heads / s->n_kv_heads;
+  long long units = 0;
+  int tiles = 1, chunks = 1;
+  for (int b = 0; b < s->n_req; ++b) {
+    const int q = s->h_q_len ? s->h_q_len[b] : 0, nb = score_blocks(q, group);
+    if (nb == 0) continue;
+    units += nb;
+    const int tok = ((q + nb - 1) / nb + kScoreTokBox - 1) / kScoreTokBox * kScoreTokBox;
+    const int c = ((tok < q ? tok : q) * group + 127) / 128, t = (s->h_ctx_len[b] + 127) / 128;
+    if (c > chunks) chunks = c;
+    if (t > tiles) tiles = t;
+  }
+  const long long per = units * s->n_kv_heads * layers;
+  if (per <= 0) return 1;
+  int best = 1;
+  double best_cost = 0.0;
+  for (int ns = 1; ns <= kScoreSplitsMax && ns <= tiles; ++ns) {
+    const double waves = (double)((per * ns + 147) / 148);
+    const double cost = waves * (4.0 + 0.75 * chunks * ((tiles + ns - 1) / ns));
+    if (ns == 1 || cost < best_cost) { best_cost = cost; best = ns; }
+  }
+  return best;
 }
 
 struct WsLayout {
@@ -240,11 +252,9 @@ inline WsLayout ws_layout(const relaxkv_shape* s, int n_layers) {
     const int nb = score_blocks(s->h_q_len ? s->h_q_len[b] : 0, s->n_q_heads / s->n_kv_heads);
     if (nb > max_blocks) max_blocks = nb;
   }
-  long long units = 0;
-  for (int b = 0; b < s->n_req; ++b) units += score_blocks(s->h_q_len ? s->h_q_len[b] : 0, s->n_q_heads / s->n_kv_heads);
   long long part_slots = 1;                 // max over launch sizes of layers x 2 x splits
   for (int lc = 1; lc <= lc_max; ++lc) {
-    const long long v = (long long)lc * 2 * score_splits(units * s->n_kv_heads, lc);
+    const long long v = (long long)lc * 2 * score_splits(s, lc);
     if (v > part_slots) part_slots = v;
   }
   w.part = a; a = align_up(a + (size_t)part_slots * s->n_q_heads * sum_q * 8, 256);

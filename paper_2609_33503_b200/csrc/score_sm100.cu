@@ -367,7 +367,7 @@ relaxkv_status launch_score_sm100(const relaxkv_shape* shape, ReqTable rt, const
   DeviceStatus* st = status_word();
   if (!st) return RELAXKV_ERR_CUDA;
   const float scale_log2 = shape->softmax_scale * 1.4426950408889634f;
-  const int n_splits = score_splits((long long)plan.units * Hkv, n_layers);
+  const int n_splits = score_splits(shape, n_layers);
   const dim3 grid((unsigned)rt.tile_cu[B], (unsigned)Hkv, (unsigned)(n_splits * n_layers));
   if (grid.x == 0) return RELAXKV_OK;
   constexpr int smem = ScoreSmem<D>::kTotal;
