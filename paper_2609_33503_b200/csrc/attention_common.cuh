@@ -19,6 +19,11 @@ struct AttnPlan {
   int dense_ctx;          // 1: context = the cache's own rows (request b starts at rt.tok_off[b]), limits are positions
 };
 
+// relaxkv_cache_attention; without lists the targets are the last shape->h_q_len[b] tokens of every request.
+relaxkv_status cache_attention(const relaxkv_shape* shape, const relaxkv_cache_view* cache, const void* q_new, const int32_t* tgt_pos,
+                               const int32_t* tgt_cu, int64_t n_target_rows, const int32_t* h_max_targets, void* out, float* lse_out,
+                               void* workspace, size_t workspace_bytes, cudaStream_t stream);
+
 // Validates the arguments of an attention call and enqueues the gather of the mixed context into
 // the workspace.  On success `plan` describes what the attention kernel reads.
 inline relaxkv_status prepare_attention(

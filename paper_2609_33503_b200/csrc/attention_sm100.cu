@@ -169,7 +169,11 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const int tt = head_inner ? (int)(blockIdx.x / Hkv) : (int)(blockIdx.x - hd * n_pairs_total);
   const int b = find_segment(rt.tile_cu, B, tt);
   const int p_rev = tt - rt.tile_cu[b];
-  const int nr = r_cu[b + 1] - r_cu[b];
+  // no lists (r_cu == NULL): the targets are the last q_len tokens of every request
+  const int row_b = r_cu ? r_cu[b] : rt.q_cu[b];
+  const int nr = r_cu ? r_cu[b + 1] - row_b : rt.q_len[b];
+  const long long row0 = r_cu ? (long long)row_b - r_cu[0] : row_b;
+  const int first_pos = rt.ctx_len[b] - nr;
   // dense_ctx: the context is the cache itself (every position of the request), a target's limit is its position
   const int nu = dense_ctx ? rt.ctx_len[b] : (u_cu[b + 1] - u_cu[b]);
   const int pair_targets = 2 * tile_targets;
@@ -177,7 +181,7 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   if (p_rev >= n_pairs_true) return;
   // a true count above its host bound, or more target rows than q_new / out hold: report, touch nothing
   if (nr > rt.bound_a[b] || (mode == RELAXKV_CTX_UNION && nu > rt.bound_b[b]) ||
-      (long long)(r_cu[b + 1] - r_cu[0]) > n_target_rows) {
+      row0 + nr > n_target_rows) {
     if (threadIdx.x == 0) report(st, RELAXKV_ERR_BAD_INDEX, KID_ATTN_SM100, nr, nu);
     return;
   }
@@ -186,7 +190,7 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const int rho0 = pair * pair_targets;                       // first target of tile A
   const int ctx_len_b = (mode == RELAXKV_CTX_UNION) ? nu : rt.ctx_len[b];
   const long long ctx_base = dense_ctx ? rt.tok_off[b] : ((mode == RELAXKV_CTX_UNION) ? (long long)u_cu[b] : rt.ctx_cu[b]);
-  const long long q_row_base = (long long)(r_cu[b] - r_cu[0]) + rho0;
+  const long long q_row_base = row0 + rho0;
   // valid targets and context tiles of each query tile
   int n_valid[2], n_kv[2];
 #pragma unroll
@@ -194,7 +198,8 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     n_valid[x] = max(0, min(tile_targets, nr - rho0 - x * tile_targets));
     n_kv[x] = 0;
     if (n_valid[x] > 0) {
-      const int c = r_rank[r_cu[b] + rho0 + x * tile_targets + n_valid[x] - 1];
+      const int rho_last = rho0 + x * tile_targets + n_valid[x] - 1;
+      const int c = r_cu ? r_rank[row_b + rho_last] : first_pos + rho_last;
       const int cc = min(max(c, 0), max(nu - 1, 0));
       int lim_last = (mode == RELAXKV_CTX_UNION) ? cc : u_pos[u_cu[b] + cc];
       lim_last = min(max(lim_last, 0), ctx_len_b - 1);
@@ -397,7 +402,7 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     int limit = 0;
     bool row_empty = false;                                     // explicit lists: a target that sees no context entry
     if (row_valid) {
-      const int c = r_rank[r_cu[b] + rho_t];
+      const int c = r_cu ? r_rank[row_b + rho_t] : first_pos + rho_t;
       if (c == -1 && allow_empty) {
         row_empty = true;
       } else if (c < 0 || c >= nu) {
@@ -1071,7 +1076,7 @@ combine_splits_kernel(const float* part_o, const float* part_lse, int n_splits,
   float4 v[U];
 #pragma unroll
   for (int u = 0; u < U; ++u) v[u] = u < n_splits ? load(u) : make_float4(0.f, 0.f, 0.f, 0.f);
-  const long long rows_true = min((long long)(r_cu[n_req] - r_cu[0]), n_target_rows);
+  const long long rows_true = r_cu ? min((long long)(r_cu[n_req] - r_cu[0]), n_target_rows) : n_target_rows;
   float mx = -INFINITY;
   for (int sp = lane; sp < n_splits; sp += 32) {
     const float l = part_lse[((long long)sp * n_target_rows + row) * H + h];
@@ -1327,13 +1332,23 @@ extern "C" relaxkv_status relaxkv_list_attention(
 extern "C" relaxkv_status relaxkv_cache_attention(
     const relaxkv_shape* shape, const relaxkv_cache_view* cache, const void* q_new,
     const int32_t* tgt_pos, const int32_t* tgt_cu, int64_t n_target_rows, const int32_t* h_max_targets,
-    void* out, float* lse_out, void* workspace, size_t workspace_bytes, relaxkv_stream stream_) {
+    void* out, float* lse_out, void* workspace, size_t workspace_bytes, relaxkv_stream stream) {
   RELAXKV_RANGE("relaxkv_cache_attention");
-  cudaStream_t stream = static_cast<cudaStream_t>(stream_);
+  if (!tgt_pos || !tgt_cu) return RELAXKV_ERR_INVALID_ARG;
+  return relaxkv::cache_attention(shape, cache, q_new, tgt_pos, tgt_cu, n_target_rows, h_max_targets, out, lse_out, workspace,
+                                  workspace_bytes, static_cast<cudaStream_t>(stream));
+}
+
+// No lists (both NULL): the targets are the last shape->h_q_len[b] tokens of every request, known to the kernels without a
+// launch that writes them down.
+relaxkv_status relaxkv::cache_attention(
+    const relaxkv_shape* shape, const relaxkv_cache_view* cache, const void* q_new,
+    const int32_t* tgt_pos, const int32_t* tgt_cu, int64_t n_target_rows, const int32_t* h_max_targets,
+    void* out, float* lse_out, void* workspace, size_t workspace_bytes, cudaStream_t stream) {
   relaxkv_status rc = check_shape(shape);
   if (rc != RELAXKV_OK) return rc;
   if ((rc = check_cache(shape, cache, true)) != RELAXKV_OK) return rc;
-  if (!q_new || !out || !tgt_pos || !tgt_cu || !h_max_targets || !workspace) return RELAXKV_ERR_INVALID_ARG;
+  if (!q_new || !out || !h_max_targets || !workspace) return RELAXKV_ERR_INVALID_ARG;
   if (!aligned16(q_new) || !aligned16(out) || n_target_rows < 1) return RELAXKV_ERR_INVALID_ARG;
   if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return RELAXKV_ERR_INVALID_ARG;
   const WsLayout ws = ws_layout(shape, 1);

@@ -101,14 +101,15 @@ decode_attention_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
   __syncthreads();                         // the barriers are ready: the producer starts as soon as it knows the position
   griddep_wait();                          // q, the lists and the newest cache row come from the kernels before
   const int status = *reinterpret_cast<volatile int*>(&st->status);
-  const int c0 = tgt_cu[0], cb = tgt_cu[b], nr = tgt_cu[b + 1] - cb;
+  // no lists: the target is the last token of every request that has one
+  const int c0 = tgt_cu ? tgt_cu[0] : 0, cb = tgt_cu ? tgt_cu[b] : rt.q_cu[b], nr = tgt_cu ? tgt_cu[b + 1] - cb : rt.q_len[b];
   if (nr <= 0) return;
   const long long row = (long long)cb - c0;
   if (nr > rt.bound_a[b] || nr > 1 || row >= n_target_rows) {      // more targets than the host bound (one): touch nothing
     if (threadIdx.x == 0) report(st, RELAXKV_ERR_BAD_INDEX, KID_ATTN_SIMT, nr, (int)row);
     return;
   }
-  const int pos = tgt_pos[cb];
+  const int pos = tgt_cu ? tgt_pos[cb] : rt.ctx_len[b] - 1;
   if (pos < 0 || pos >= rt.ctx_len[b]) {
     if (threadIdx.x == 0) report(st, RELAXKV_ERR_BAD_INDEX, KID_ATTN_SIMT, pos, rt.ctx_len[b]);
     return;

@@ -4,6 +4,7 @@
 // followed by the segmented top-k (select.cu).  The two passes run on the tensor cores
 // (score_sm100.cu); this file holds the entry point and the small kernels that combine their partial
 // results in a fixed order, so results are bit-reproducible from run to run.
+#include "attention_common.cuh"
 #include "common.cuh"
 #include "score_sm100.cuh"
 #include "select.cuh"
@@ -102,20 +103,6 @@ static relaxkv_status score_layers(const relaxkv_shape* shape, ReqTable rt, cons
   return cuda_ok(launch_chained(finalize_raw_kernel, (unsigned)((total + 255) / 256), 256, 0, stream, rt, n_layers, H, Hkv, plan.max_super, colpart, raw));
 }
 
-// Positions of the query's own tokens (they follow the context: T_c, T_c + 1, ...) and their offsets, as the target
-// lists of the cache-only attention call.
-__global__ void query_positions_kernel(ReqTable rt, int* __restrict__ tgt_pos, int* __restrict__ tgt_cu) {
-  griddep_launch();
-  griddep_wait();
-  const int B = rt.n_req;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i <= B) tgt_cu[i] = rt.q_cu[i];
-  if (i < rt.q_cu[B]) {
-    const int b = find_segment(rt.q_cu, B, i);
-    tgt_pos[i] = rt.ctx_len[b] + (i - rt.q_cu[b]);
-  }
-}
-
 }  // namespace relaxkv
 
 using namespace relaxkv;
@@ -206,14 +193,9 @@ extern "C" relaxkv_status relaxkv_query_prefill_attention(
   if (workspace_bytes < ws.total) return RELAXKV_ERR_WORKSPACE_TOO_SMALL;
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
   char* base = static_cast<char*>(workspace);
-  int* tgt_pos = reinterpret_cast<int*>(base + ws.list_limit);        // regions the cache-only attention does not use
-  int* tgt_cu = reinterpret_cast<int*>(base + ws.list_fresh);
   ReqTable rt;
   fill_req_table(rt, shape, cache, nullptr);
-  const long long n = std::max<long long>(sum_q, B + 1);
-  rc = cuda_ok(launch_chained(query_positions_kernel, (unsigned)((n + 255) / 256), 256, 0, stream, rt, tgt_pos, tgt_cu));
-  if (rc != RELAXKV_OK) return rc;
-  rc = relaxkv_cache_attention(&ext, cache, q, tgt_pos, tgt_cu, sum_q, q_len, out, lse_out, workspace, workspace_bytes, stream_);
+  rc = cache_attention(&ext, cache, q, nullptr, nullptr, sum_q, q_len, out, lse_out, workspace, workspace_bytes, stream);
   if (rc != RELAXKV_OK || !raw_scores_out) return rc;
   // column sums over the CONTEXT keys with the rows' normalisers from the attention above
   const ScorePlan plan = plan_score(shape);
