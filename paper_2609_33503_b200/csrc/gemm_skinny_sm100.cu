@@ -100,17 +100,14 @@ gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_
   // All blocks of a one-wave launch are resident by then, so the next kernel only takes room that is left over.
   griddep_launch();
   griddep_wait();
-  // after an expired wait elsewhere the tensor-core kernels move nothing until the status word has been read; here
-  // that means: run through the barriers (a block must not leave its cluster waiting), compute nothing
-  if (threadIdx.x == 0 && *reinterpret_cast<volatile int*>(&st->status) == RELAXKV_ERR_TIMEOUT) *abort_flag = 1;
-  __syncthreads();
-  const bool drained = *abort_flag != 0;
-  __syncthreads();
-
-  bool ok = !drained;
+  // After an expired wait elsewhere the tensor-core kernels write nothing until the status word has been read.  The word is
+  // fetched here and looked at before the outputs are written: waiting for it first would cost a memory latency, and
+  // everything up to there stays inside the block and its cluster.
+  const int status = *reinterpret_cast<volatile int*>(&st->status);
+  bool ok = true;
   if (warp == 4) {
     // ---- TMA producer ----
-    if (lane == 0 && ok) {
+    if (lane == 0) {
       for (int kt = k0, it = 0, s = 0, ph = 0; kt < k1; ++kt, ++it) {
         if (it >= n_stages && !mbar_wait(bar_empty + 8 * s, (uint32_t)(ph ^ 1), abort_flag)) break;
         const uint32_t dst = base + (uint32_t)s * stage_bytes;
@@ -123,7 +120,7 @@ gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_
     }
   } else if (warp == 5) {
     // ---- MMA issuer ----
-    if (lane == 0 && ok) {
+    if (lane == 0) {
       const uint32_t idesc = idesc_bf16_f32(kSkFeat, n_cols, 0);
       bool go = true;
       for (int kt = k0, it = 0, s = 0, ph = 0; kt < k1; ++kt, ++it) {
@@ -140,7 +137,7 @@ gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_
     // ---- epilogue warps (thread = weight row = TMEM lane): this block's partial tile -> its own shared memory, [row of x]
     // [feature] fp32 (the lanes of a warp hold consecutive features: every store below writes 128 consecutive bytes).
     // The MMAs have completed by then, so the TMA ring is free to hold it. ----
-    if (ok) ok = mbar_wait(bar_acc, 0, abort_flag);
+    ok = mbar_wait(bar_acc, 0, abort_flag);
     ok = __all_sync(0xffffffffu, ok);
     tc_fence_after();
     if (ok) {
@@ -189,7 +186,7 @@ gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_
     const int width = outs.col0[sg + 1] - outs.col0[sg];
     uint16_t* y = outs.y[sg] + (col0 - outs.col0[sg]);
     const uint16_t* res = outs.residual[sg] ? outs.residual[sg] + (col0 - outs.col0[sg]) : nullptr;
-    if (m0 < rows && col0 < n_feat) {
+    if (m0 < rows && col0 < n_feat && status != RELAXKV_ERR_TIMEOUT) {
       constexpr int R = 4;                                       // rounds whose loads are in flight together
       for (int mb = m0; mb < M; mb += R * rows) {
         uint2 r[R];
@@ -228,7 +225,7 @@ gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_
   tc_fence_before();
   __syncthreads();
   if (S > 1) cluster_sync();
-  if (*abort_flag && !drained) {
+  if (*abort_flag) {
     if (threadIdx.x == 0) report(st, RELAXKV_ERR_TIMEOUT, KID_GEMM_SM100, (int)blockIdx.x, 1);
     const uint64_t tw = global_timer_ns();
     while (global_timer_ns() - tw < 200000ull) __nanosleep(1000);
