@@ -1,7 +1,7 @@
 // Projections of a handful of rows (a decode token, the last query row going through the output head): y = x W^T with
 // one row of x, or two to four where K is short (more rows or a longer K take the tensor-core tiles of
-// gemm_skinny_sm100.cu: a weight byte then meets more multiply-adds than the FMA pipe does in its HBM time).  The work is reading W once (HBM-bound: every weight byte meets one to four
-// multiply-adds), so this is a plain streaming kernel, not the 128-row tensor-core GEMM: each warp owns two output
+// gemm_skinny_sm100.cu: a weight byte then meets more multiply-adds than the FMA pipe does in its HBM time).  The work is
+// reading W once (HBM-bound), so this is a plain streaming kernel without tiles: each warp owns two output
 // features (16 per block: a 5120-wide projection is 320 blocks, all resident at once), its lanes stride over K in
 // 16-byte pieces with eight independent weight loads in flight per lane, x stays in L1, and a shuffle tree sums the
 // lanes' partial dot products in a fixed order.  (Algorithm 1 runs the model's
