@@ -2,6 +2,8 @@
 // active targets R_l as ranks into U (Section 3.2; Algorithm 1, steps 6-12).  Integer work only.
 #include "common.cuh"
 #include "sm100_ptx.cuh"
+#include <algorithm>
+#include <atomic>
 
 namespace relaxkv {
 
@@ -132,6 +134,111 @@ __global__ void __launch_bounds__(kSetThreads) write_sets_kernel(ReqTable rt, in
   ptx::cluster_sync();                                        // nobody leaves while a peer may still read its totals
 }
 
+// The whole schedule of ONE request in one launch: a cluster whose blocks each hold a contiguous slice of the positions in
+// shared memory.  Every block reads all anchors and keeps the layers of its own positions; the blocks' counts per layer meet
+// through distributed shared memory, which gives every list's place; a warp then writes one list of its block's slice, or a run
+// of it.  Four dependent launches become one, for work that is mostly their latency: positions of a slice times lists up to
+// kOneWorkMax.  Four launches / one, us on the GPU: 1 K positions and 1 layer 6.9 / 4.5, 32 layers 10.1 / 6.5; 8 K and 1 layer
+// 8.0 / 5.3, 6 layers 8.3 / 9.4; 16 K and 1 layer 9.0 / 6.3; past the line 16 K and 12 layers 10.6 / 18.0.  On the host 16 / 8.
+constexpr int kOneWorkMax = 8192;
+constexpr int kOneLayersMax = kOneWorkMax / 32;  // a slice is at least 32 positions
+
+__global__ void __launch_bounds__(kSetThreads) schedule_one_kernel(int T, int k, int n_layers, const int* anchors, int* h, int* u_pos,
+                                                                   int* u_cu, int* u_rank, int* r_rank, int* r_cu, int* counts,
+                                                                   int* host_counts, DeviceStatus* st) {
+  extern __shared__ int s_h[];                                // highest layer of the slice's positions
+  __shared__ int s_hist[kOneLayersMax], s_cnt[kOneLayersMax]; // positions whose highest layer is / is at least l; s_cnt is read by the cluster
+  __shared__ int s_run_u[kSetWarps], s_run_r[kSetWarps];
+  __shared__ int s_tot[kOneLayersMax], s_before[kOneLayersMax], s_base[kOneLayersMax];
+  const int slice = (int)blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int per = ((T + kSetSlices - 1) / kSetSlices + 31) & ~31;
+  const int p0 = min(T, slice * per), n = min(T, p0 + per) - p0;
+  for (int i = tid; i < n; i += kSetThreads) s_h[i] = -1;
+  for (int l = tid; l < n_layers; l += kSetThreads) s_hist[l] = 0;
+  griddep_launch();
+  griddep_wait();
+  __syncthreads();
+  const int n_anchors = n_layers * k;
+#pragma unroll 8
+  for (int idx = tid; idx < n_anchors; idx += kSetThreads) {
+    const int pos = anchors[idx];
+    if ((unsigned)(pos - p0) < (unsigned)n) atomicMax(&s_h[pos - p0], idx / k);
+    else if (slice == 0 && (pos < 0 || pos >= T)) report(st, RELAXKV_ERR_BAD_INDEX, KID_SETS, idx, pos);
+  }
+  __syncthreads();
+  for (int i0 = warp * 32; i0 < n; i0 += kSetThreads) {
+    const int v = i0 + lane < n ? s_h[i0 + lane] : -1;
+    if (i0 + lane < n) h[p0 + i0 + lane] = v;
+    const unsigned same = __match_any_sync(0xffffffffu, v);   // few layers: many lanes count into one word
+    if (v >= 0 && lane == __ffs(same) - 1) atomicAdd(&s_hist[v], __popc(same));
+  }
+  __syncthreads();
+  if (tid < n_layers) {
+    int c = 0;
+    for (int l = tid; l < n_layers; ++l) c += s_hist[l];
+    s_cnt[tid] = c;
+  }
+  ptx::cluster_sync();
+  if (tid < n_layers) {
+    int tot = 0, before = 0;
+#pragma unroll
+    for (int r = 0; r < kSetSlices; ++r) {
+      const int c = ptx::ld_cluster_s32(ptx::mapa_shared(ptx::smem_u32(&s_cnt[tid]), (uint32_t)r));
+      tot += c;
+      if (r < slice) before += c;
+    }
+    s_tot[tid] = tot; s_before[tid] = before;
+  }
+  __syncthreads();
+  if (tid < n_layers) {
+    int base = 0;
+    for (int l = 0; l < tid; ++l) base += s_tot[l];
+    s_base[tid] = base + s_before[tid];
+    if (slice == 0) {
+      r_cu[tid] = base;
+      counts[1 + tid] = s_tot[tid];
+      if (host_counts) host_counts[1 + tid] = s_tot[tid];
+      if (tid == n_layers - 1) r_cu[n_layers] = base + s_tot[tid];
+      if (tid == 0) { u_cu[0] = 0; u_cu[1] = s_tot[0]; counts[0] = s_tot[0]; if (host_counts) host_counts[0] = s_tot[0]; }
+    }
+  }
+  __syncthreads();
+  // with few lists several warps share one: a run of the slice each, behind the counts of the runs before it
+  int share = 1;
+  while (2 * share * (n_layers + 1) <= kSetWarps) share *= 2;
+  const int run = ((n + share - 1) / share + 31) & ~31;
+  const int i0 = min(n, (warp % share) * run), i1 = min(n, i0 + run);
+  int du = 0, dr = 0;
+  if (share > 1) {
+    const int thr = max(0, warp / share - 1);
+    for (int i = i0 + lane; i < i1; i += 32) { const int v = s_h[i]; du += (v >= 0); dr += (v >= thr); }
+    du = warp_reduce_sum(du); dr = warp_reduce_sum(dr);
+    if (lane == 0) { s_run_u[warp] = du; s_run_r[warp] = dr; }
+    __syncthreads();
+    du = 0; dr = 0;
+    for (int w = warp - warp % share; w < warp; ++w) { du += s_run_u[w]; dr += s_run_r[w]; }
+  }
+  const uint32_t below = (1u << lane) - 1u;
+  for (int list = warp / share; list <= n_layers; list += kSetWarps / share) {      // 0: U, l + 1: R_l
+    const int thr = list == 0 ? 0 : list - 1;
+    int eu = s_before[0] + du, er = list == 0 ? 0 : s_base[thr] + dr;
+#pragma unroll 4
+    for (int i = i0 + lane; i - lane < i1; i += 32) {
+      const int v = i < i1 ? s_h[i] : -1;
+      const uint32_t mu = __ballot_sync(0xffffffffu, v >= 0), mr = __ballot_sync(0xffffffffu, v >= thr);
+      const int rank = eu + __popc(mu & below);
+      if (list == 0) {
+        if (v >= 0) u_pos[rank] = p0 + i;
+        if (i < i1) u_rank[p0 + i] = v >= 0 ? rank : -1;
+      } else if (v >= thr) {
+        r_rank[er + __popc(mr & below)] = rank;
+      }
+      eu += __popc(mu); er += __popc(mr);
+    }
+  }
+  ptx::cluster_sync();                                        // nobody leaves while a peer may still read its counts
+}
+
 }  // namespace relaxkv
 
 using namespace relaxkv;
@@ -155,9 +262,17 @@ static relaxkv_status build_sets(const relaxkv_shape* shape, int32_t n_layers, c
     if (cudaPointerGetAttributes(&attr, h_counts_pinned) != cudaSuccess) (void)cudaGetLastError();
     else if (attr.type == cudaMemoryTypeHost) host_counts = static_cast<int*>(attr.devicePointer);
   }
+  const long long n_anchor = (long long)n_layers * rt.k_cu[B];
+  const long long slice_len = ((sum_t + kSetSlices - 1) / kSetSlices + 31) & ~31ll;
+  if (B == 1 && slice_len * (n_layers + 1) <= kOneWorkMax) {           // one request, little work: everything in one launch
+    const relaxkv_status rc1 = cuda_ok(launch_chained_clusters(
+        kSetSlices, schedule_one_kernel, dim3(kSetSlices), dim3(kSetThreads), (size_t)slice_len * 4, stream, rt.ctx_len[0], rt.k[0], n_layers,
+        anchors, highest_layer_out, u_pos_out, u_cu_out, u_rank_out, r_rank_out, r_cu_out, counts, host_counts, st));
+    if (rc1 != RELAXKV_OK || !h_counts_pinned || host_counts) return rc1;
+    return cuda_ok(cudaMemcpyAsync(h_counts_pinned, counts, sizeof(int) * (size_t)(1 + n_layers), cudaMemcpyDeviceToHost, stream));
+  }
   // Nothing in `counts` has to start at zero: count_sets_kernel overwrites every entry that write_sets_kernel and the
   // copy below read.
-  const long long n_anchor = (long long)n_layers * rt.k_cu[B];
   const unsigned lists = (unsigned)(B * (n_layers + 1));
   cudaError_t e = launch_chained(fill_i32_kernel, dim3((unsigned)((sum_t + 255) / 256)), dim3(256), 0, stream,
                                  highest_layer_out, sum_t, -1);
