@@ -98,8 +98,9 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // kernel's blocks become resident as soon as every block of the current one has called griddep_launch(); they may do
 // whatever does not depend on earlier kernels (set-up, prefetching their weights into L2) and then block in griddep_wait()
 // until the earlier kernels have completed and their writes are visible.  Rules kept by every kernel that is launched
-// this way: nothing written by another kernel is read, and nothing at all is written, before griddep_wait(); index lists
-// that come from an earlier kernel are read through pointers without __restrict__ (a read-only load may not be moved up past the wait); every
+// this way: nothing written by another kernel is read, and nothing at all is written, before griddep_wait(); everything
+// read from global memory, index lists and data alike, is read through plain pointers (no const __restrict__, no __ldg: the
+// compiler may move a read-only load up past the wait, which orders ordinary memory accesses alone); every
 // block executes griddep_wait() (so a kernel never completes before its predecessors).  A kernel that takes tensor memory
 // calls griddep_launch() only after it has got it: every block then holds its share before a later kernel's block can ask
 // for some on the same SM.  Short kernels call griddep_launch() first thing, the tensor-core kernels of many blocks when

@@ -82,7 +82,7 @@ rmsnorm_kernel(const uint16_t* x, const uint16_t* w, uint16_t* y, int C, float e
 // Short rows (a head vector: C <= 256): one warp per row, each lane 8 elements, so the per-head Q/K norm of a
 // [rows, heads, D] tensor is one pass over it.  In place (y == x) is fine: a lane writes what it alone read.
 __global__ void __launch_bounds__(256)
-rmsnorm_short_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ w, uint16_t* __restrict__ y, long long rows,
+rmsnorm_short_kernel(const uint16_t* x, const uint16_t* w, uint16_t* __restrict__ y, long long rows,
                      int C, float eps) {
   const long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -99,7 +99,7 @@ rmsnorm_short_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict_
   const float inv = rsqrtf(ss / (float)C + eps);
   if (mine) {
     float g[8];
-    unpack8(__ldg(reinterpret_cast<const uint4*>(w + lane * 8)), g);
+    unpack8(*reinterpret_cast<const uint4*>(w + lane * 8), g);
 #pragma unroll
     for (int e = 0; e < 8; ++e) f[e] = f[e] * inv * g[e];
     *reinterpret_cast<uint4*>(y + row * C + lane * 8) = pack8(f);
@@ -108,7 +108,7 @@ rmsnorm_short_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict_
 
 // Rotate-half rotary embedding in place on x [rows, heads, D]; one thread per (row, 8 pairs): the eight
 // (cos, sin) pairs are computed once and applied to every head of the row.
-__global__ void rope_kernel(uint16_t* __restrict__ x, long long rows, int heads, int D, const int* __restrict__ positions,
+__global__ void rope_kernel(uint16_t* __restrict__ x, long long rows, int heads, int D, const int* positions,
                             double log2_theta) {
   const int half = D / 2, groups = half / 8;
   griddep_launch();
@@ -154,8 +154,8 @@ __global__ void rope_kernel(uint16_t* __restrict__ x, long long rows, int heads,
 // values are rounded to bf16, as they would be if the normalised heads had been stored and read back.
 template <int D>
 __global__ void __launch_bounds__(128)
-head_norm_rope_kernel(uint16_t* __restrict__ q, uint16_t* __restrict__ k, int Hq, int Hkv, int heads_per_block, const uint16_t* __restrict__ wq,
-                      const uint16_t* __restrict__ wk, float eps, const int* positions, double log2_theta) {
+head_norm_rope_kernel(uint16_t* __restrict__ q, uint16_t* __restrict__ k, int Hq, int Hkv, int heads_per_block, const uint16_t* wq,
+                      const uint16_t* wk, float eps, const int* positions, double log2_theta) {
   constexpr int DPL = D / 32, half = D / 2;
   constexpr int U = 4;                                        // heads a warp has in flight at once
   __shared__ float cs_s[half], sn_s[half];
@@ -259,7 +259,7 @@ __device__ __forceinline__ void row_wait_failed(DeviceStatus* st, long long row)
 
 // y = x / sqrt(mean(x^2) + eps) * w, one warp per row of C columns (C * 2 bytes a multiple of 16).
 __global__ void __launch_bounds__(kRowWarps * 32)
-rmsnorm_rows_bulk_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ w, uint16_t* __restrict__ y, long long n_rows,
+rmsnorm_rows_bulk_kernel(const uint16_t* x, const uint16_t* w, uint16_t* __restrict__ y, long long n_rows,
                          int C, float eps, DeviceStatus* st) {
   extern __shared__ __align__(128) uint8_t row_stage[];      // [warp][C] bf16
   __shared__ __align__(8) unsigned long long bars[kRowWarps];
@@ -296,7 +296,7 @@ rmsnorm_rows_bulk_kernel(const uint16_t* __restrict__ x, const uint16_t* __restr
   for (int i = lane * 8; i < C; i += 32 * 8) {
     float f[8], g[8];
     unpack8(*reinterpret_cast<const uint4*>(mine + i * 2), f);
-    unpack8(__ldg(reinterpret_cast<const uint4*>(w + i)), g);
+    unpack8(*reinterpret_cast<const uint4*>(w + i), g);
 #pragma unroll
     for (int e = 0; e < 8; ++e) f[e] = f[e] * inv * g[e];
     *reinterpret_cast<uint4*>(mine + i * 2) = pack8(f);
@@ -316,8 +316,8 @@ rmsnorm_rows_bulk_kernel(const uint16_t* __restrict__ x, const uint16_t* __restr
 template <int D>
 __global__ void __launch_bounds__(kRowWarps * 32)
 head_norm_rope_rows_bulk_kernel(uint16_t* __restrict__ q, uint16_t* __restrict__ k, long long n_rows, int Hq, int Hkv,
-                                const uint16_t* __restrict__ wq, const uint16_t* __restrict__ wk, float eps,
-                                const int* __restrict__ positions, double log2_theta, DeviceStatus* st) {
+                                const uint16_t* wq, const uint16_t* wk, float eps,
+                                const int* positions, double log2_theta, DeviceStatus* st) {
   constexpr int P = D / 32, half = D / 2;
   extern __shared__ __align__(128) uint8_t row_stage[];      // [warp][Hq + Hkv][D] bf16
   __shared__ __align__(8) unsigned long long bars[kRowWarps];
@@ -423,7 +423,7 @@ head_norm_rope_rows_bulk_kernel(uint16_t* __restrict__ q, uint16_t* __restrict__
 }
 
 // out[r, i] = silu(gu[r, i]) * gu[r, I + i]
-__global__ void swiglu_kernel(const uint16_t* __restrict__ gu, uint16_t* __restrict__ out, long long rows, int I) {
+__global__ void swiglu_kernel(const uint16_t* gu, uint16_t* __restrict__ out, long long rows, int I) {
   griddep_launch();
   griddep_wait();
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -432,8 +432,8 @@ __global__ void swiglu_kernel(const uint16_t* __restrict__ gu, uint16_t* __restr
   const long long r = idx / per_row;
   const int i = (int)(idx - r * per_row) * 8;
   float g[8], u[8];
-  unpack8(__ldg(reinterpret_cast<const uint4*>(gu + r * 2 * I + i)), g);
-  unpack8(__ldg(reinterpret_cast<const uint4*>(gu + r * 2 * I + I + i)), u);
+  unpack8(*reinterpret_cast<const uint4*>(gu + r * 2 * I + i), g);
+  unpack8(*reinterpret_cast<const uint4*>(gu + r * 2 * I + I + i), u);
 #pragma unroll
   for (int e = 0; e < 8; ++e) g[e] = g[e] / (1.f + __expf(-g[e])) * u[e];
   *reinterpret_cast<uint4*>(out + r * I + i) = pack8(g);
@@ -460,7 +460,7 @@ __global__ void target_positions_kernel(ReqTable rt, const int* u_pos, const int
 // Hidden rows that stay active: for each target of layer l+1 (rank c), its row among layer l's targets.
 // One block copies one row (C a multiple of 8).
 __global__ void __launch_bounds__(128)
-carry_rows_kernel(ReqTable rt, const uint16_t* __restrict__ h_in, uint16_t* __restrict__ h_out, int C,
+carry_rows_kernel(ReqTable rt, const uint16_t* h_in, uint16_t* __restrict__ h_out, int C,
                   const int* r_rank, const int* r_cu_l, const int* r_cu_next, DeviceStatus* st) {
   griddep_launch();
   griddep_wait();
@@ -484,12 +484,12 @@ carry_rows_kernel(ReqTable rt, const uint16_t* __restrict__ h_in, uint16_t* __re
   if (src_row < 0) return;
   const long long dst_row = (long long)(r_cu_next[b] - r_cu_next[0]) + rho;
   for (int i = threadIdx.x * 8; i < C; i += 128 * 8)
-    *reinterpret_cast<uint4*>(h_out + dst_row * C + i) = __ldg(reinterpret_cast<const uint4*>(h_in + src_row * C + i));
+    *reinterpret_cast<uint4*>(h_out + dst_row * C + i) = *reinterpret_cast<const uint4*>(h_in + src_row * C + i);
 }
 
 // The same for many rows: one warp per row, the row travels through shared memory by bulk copies (see above).
 __global__ void __launch_bounds__(kRowWarps * 32)
-carry_rows_bulk_kernel(ReqTable rt, const uint16_t* __restrict__ h_in, uint16_t* __restrict__ h_out, int C,
+carry_rows_bulk_kernel(ReqTable rt, const uint16_t* h_in, uint16_t* __restrict__ h_out, int C,
                        const int* r_rank, const int* r_cu_l, const int* r_cu_next, DeviceStatus* st) {
   griddep_launch();
   griddep_wait();

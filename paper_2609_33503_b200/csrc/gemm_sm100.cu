@@ -42,7 +42,7 @@ __device__ __forceinline__ uint16_t* chunk_ptr(const GemmSegs& segs, uint16_t* y
 
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_sm100_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
-                  long long M, int N, int K, uint16_t* __restrict__ y, const uint16_t* __restrict__ residual,
+                  long long M, int N, int K, uint16_t* __restrict__ y, const uint16_t* residual,
                   int swiglu, const __grid_constant__ GemmSegs segs, DeviceStatus* st) {
   const int tiles_m = (int)((M + kGemmBM - 1) / kGemmBM), tiles_n = (N + kGemmBN - 1) / kGemmBN;
   const long long n_tiles = (long long)tiles_m * tiles_n;
@@ -181,7 +181,7 @@ gemm_sm100_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
 #pragma unroll
               for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[i8 + e]);
               if (residual != nullptr) {
-                const uint4 r = __ldg(reinterpret_cast<const uint4*>(residual + off + i8));
+                const uint4 r = *reinterpret_cast<const uint4*>(residual + off + i8);
                 const uint32_t rw[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) { f[2 * e] += __uint_as_float(rw[e] << 16); f[2 * e + 1] += __uint_as_float(rw[e] & 0xffff0000u); }
@@ -223,7 +223,7 @@ constexpr int kPairSmem = kPairStages * kPairStageBytes + 8 * kPairBarsTotal + 1
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
 gemm_pair_sm100_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
-                  long long M, int N, int K, uint16_t* __restrict__ y, const uint16_t* __restrict__ residual,
+                  long long M, int N, int K, uint16_t* __restrict__ y, const uint16_t* residual,
                   int swiglu, const __grid_constant__ GemmSegs segs, DeviceStatus* st) {
   // a cluster of two CTAs computes 256 x 256 output tiles: CTA rank r holds rows [128 r, 128 r + 128) of the tile's A
   // rows and of its B rows (= output columns), the leader's MMA thread drives both SMs (M = 256), every CTA drains
@@ -383,7 +383,7 @@ gemm_pair_sm100_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
 #pragma unroll
               for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[i8 + e]);
               if (residual != nullptr) {
-                const uint4 r = __ldg(reinterpret_cast<const uint4*>(residual + off + i8));
+                const uint4 r = *reinterpret_cast<const uint4*>(residual + off + i8);
                 const uint32_t rw[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) { f[2 * e] += __uint_as_float(rw[e] << 16); f[2 * e + 1] += __uint_as_float(rw[e] & 0xffff0000u); }

@@ -32,7 +32,7 @@ __device__ __forceinline__ void unpack8_gemv(const uint4& v, float* f) {
 //         chains, which is what bounds such a launch (not bandwidth).
 template <int M, int SWIGLU, int SEG, int KS>
 __global__ void __launch_bounds__(kGemvThreads)
-gemv_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ w, const uint16_t* __restrict__ residual,
+gemv_kernel(const uint16_t* x, const uint16_t* w, const uint16_t* residual,
             uint16_t* __restrict__ y, int n_out, int K, const GemvOut outs) {
   constexpr int kWarps = kGemvThreads / 32, kGroups = kWarps / KS;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -67,10 +67,10 @@ gemv_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ w, cons
   for (int k = k_lo + lane * 8; k < k_hi; k += 32 * 8) {
     uint4 wv[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) wv[r] = __ldg(reinterpret_cast<const uint4*>(wr[r] + k));     // all loads first
+    for (int r = 0; r < R; ++r) wv[r] = *reinterpret_cast<const uint4*>(wr[r] + k);     // all loads first
     float xf[M][8];
 #pragma unroll
-    for (int m = 0; m < M; ++m) unpack8_gemv(__ldg(reinterpret_cast<const uint4*>(x + (long long)m * K + k)), xf[m]);
+    for (int m = 0; m < M; ++m) unpack8_gemv(*reinterpret_cast<const uint4*>(x + (long long)m * K + k), xf[m]);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       float wf[8];

@@ -98,9 +98,9 @@ __device__ __forceinline__ void issue_row_stores(uint16_t* k_dst, uint16_t* v_ds
 // staging area, and once they have landed the same lanes issue the copies to the materialised context.
 __global__ void __launch_bounds__(kMoveThreads)
 gather_ctx_kernel(ReqTable rt, int mode, int n_kv_heads, int head_dim,
-                  const uint16_t* __restrict__ cache_k, const uint16_t* __restrict__ cache_v,
+                  const uint16_t* cache_k, const uint16_t* cache_v,
                   long long tok_stride, long long head_stride,
-                  const uint16_t* __restrict__ k_new, const uint16_t* __restrict__ v_new,
+                  const uint16_t* k_new, const uint16_t* v_new,
                   const int* u_pos, const int* u_cu, const int* r_rank, const int* r_cu, const int* fresh_row,
                   uint16_t* __restrict__ k_out, uint16_t* __restrict__ v_out, long long ctx_rows,
                   long long fresh_map_rows, long long n_new_rows, int rows_per_warp, int* work_counter, DeviceStatus* st) {
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kMoveThreads)
 scatter_kv_kernel(ReqTable rt, int n_kv_heads, int head_dim,
                   uint16_t* __restrict__ cache_k, uint16_t* __restrict__ cache_v,
                   long long tok_stride, long long head_stride,
-                  const uint16_t* __restrict__ k_new, const uint16_t* __restrict__ v_new,
+                  const uint16_t* k_new, const uint16_t* v_new,
                   const int* u_pos, const int* u_cu, const int* r_rank, const int* r_cu, int direct, int rows_per_warp,
                   DeviceStatus* st) {
   // direct != 0: u_pos holds the targets' positions themselves (packed by r_cu); r_rank is not read
