@@ -172,6 +172,8 @@ inline void fill_req_table(ReqTable& t, const relaxkv_shape* s, const relaxkv_ca
 // ---- workspace layout -------------------------------------------------------------------
 // Calls are stream-ordered, so the regions of different calls overlap.
 constexpr int kScoreSplitsMax = 64;   // key-range splits of the scoring passes (grid.z), at most
+constexpr int kScoreSms = 148;        // SMs the splits are chosen for (a workspace size does not depend on the device asked)
+constexpr int kScoreCtasMax = 32 * kScoreSms;   // CTAs of a scoring pass up to which its key range is split further
 constexpr int kScoreMaxRows = 640;    // query rows (token x head-in-group) resident per scoring CTA
 constexpr int kScoreTokBox = 8;       // query tokens per TMA box of the scoring kernel
 constexpr int kCtxPadRows = 128;      // zero rows after the materialised context
@@ -184,6 +186,13 @@ constexpr int kScoreLayersPerLaunch = 48;   // layers scored by one launch (thei
 inline int score_blocks(int q_len, int group) {
   const int max_tok = kScoreMaxRows / group / kScoreTokBox * kScoreTokBox;
   return q_len > 0 ? (q_len + max_tok - 1) / max_tok : 0;
+}
+
+// Most key-range splits a launch of `layers` layers may take, by the query rows alone (the choice itself is not monotone in
+// the context).  A workspace has room for that many, so a shorter context never needs more workspace than a longer one.
+inline int score_splits_most(long long units_times_heads, int layers) {
+  const long long per = units_times_heads * layers, most = per > 0 ? kScoreCtasMax / per : 1;
+  return most < 1 ? 1 : (most > kScoreSplitsMax ? kScoreSplitsMax : (int)most);
 }
 
 // Key-range splits for a launch that scores `layers` layers at once (one CTA per SM, every CTA of a launch about the same
@@ -208,8 +217,9 @@ inline int score_splits(const relaxkv_shape* s, int layers) {
   if (per <= 0) return 1;
   int best = 1;
   double best_cost = 0.0;
-  for (int ns = 1; ns <= kScoreSplitsMax && ns <= tiles; ++ns) {
-    const double waves = (double)((per * ns + 147) / 148);
+  const int most = score_splits_most(units * s->n_kv_heads, layers);
+  for (int ns = 1; ns <= most && ns <= tiles; ++ns) {
+    const double waves = (double)((per * ns + kScoreSms - 1) / kScoreSms);
     const double cost = waves * (4.0 + 0.75 * chunks * ((tiles + ns - 1) / ns));
     if (ns == 1 || cost < best_cost) { best_cost = cost; best = ns; }
   }
@@ -248,16 +258,19 @@ inline WsLayout ws_layout(const relaxkv_shape* s, int n_layers) {
   a = 0;
   const int lc_max = n_layers < kScoreLayersPerLaunch ? n_layers : kScoreLayersPerLaunch;
   w.lse = a; a = align_up(a + (size_t)lc_max * s->n_q_heads * sum_q * 4, 256);
-  int max_blocks = 1;
+  int max_blocks = 1, tiles = 1;
+  long long units = 0;
   for (int b = 0; b < s->n_req; ++b) {
     const int nb = score_blocks(s->h_q_len ? s->h_q_len[b] : 0, s->n_q_heads / s->n_kv_heads);
+    units += nb;
     if (nb > max_blocks) max_blocks = nb;
+    if ((s->h_ctx_len[b] + 127) / 128 > tiles) tiles = (s->h_ctx_len[b] + 127) / 128;
   }
-  long long part_slots = 1;                 // max over launch sizes of layers x 2 x splits
-  for (int lc = 1; lc <= lc_max; ++lc) {
-    const long long v = (long long)lc * 2 * score_splits(s, lc);
-    if (v > part_slots) part_slots = v;
-  }
+  // layers x splits of a launch, at most, over the launches of 1 to lc_max layers: min(splits x lc, max(lc, CTAs / units))
+  const long long by_ctas = kScoreCtasMax / (units > 0 ? units * s->n_kv_heads : 1);
+  const long long by_splits = (long long)(tiles < kScoreSplitsMax ? tiles : kScoreSplitsMax) * lc_max;
+  const long long fit = by_ctas < by_splits ? by_ctas : by_splits;
+  const long long part_slots = 2 * (fit > lc_max ? fit : lc_max);
   w.part = a; a = align_up(a + (size_t)part_slots * s->n_q_heads * sum_q * 8, 256);
   w.colpart = a; a = align_up(a + (size_t)lc_max * 2 * s->n_kv_heads * max_blocks * sum_t * 4, 256);
   size_t score_total = a;

@@ -189,8 +189,9 @@ extern "C" relaxkv_status relaxkv_query_prefill_attention(
   if (sum_q > 0x7fffffffLL) return RELAXKV_ERR_UNSUPPORTED_SHAPE;
   relaxkv_shape ext = *shape;                       // the same batch with the query's tokens counted into the cache rows
   ext.h_ctx_len = ext_len;
-  const WsLayout ws = ws_layout(&ext, 1);
-  if (workspace_bytes < ws.total) return RELAXKV_ERR_WORKSPACE_TOO_SMALL;
+  // the context's own layout, which the scores take, needs no more than the one of context and query
+  const WsLayout ws = ws_layout(&ext, 1), ws_sc = ws_layout(shape, 1);
+  if (workspace_bytes < ws.total || workspace_bytes < ws_sc.total) return RELAXKV_ERR_WORKSPACE_TOO_SMALL;
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
   char* base = static_cast<char*>(workspace);
   ReqTable rt;
@@ -199,8 +200,6 @@ extern "C" relaxkv_status relaxkv_query_prefill_attention(
   if (rc != RELAXKV_OK || !raw_scores_out) return rc;
   // column sums over the CONTEXT keys with the rows' normalisers from the attention above
   const ScorePlan plan = plan_score(shape);
-  const WsLayout ws_sc = ws_layout(shape, 1);
-  if (workspace_bytes < ws_sc.total) return RELAXKV_ERR_WORKSPACE_TOO_SMALL;
   const void* q_arr[1] = {q};
   const float* lse_arr[1] = {lse_out};
   if (shape->head_dim == 128)

@@ -2,6 +2,7 @@
 header declares, and rejects bad arguments before any launch."""
 import ctypes
 import os
+import random
 import re
 
 import pytest
@@ -45,6 +46,24 @@ def test_status_strings_and_workspace():
     assert ws >= 2 * 32768 * 8 * 128 * 2          # room for the materialised K~ and V~
     assert B.relaxkv_workspace_bytes(B.Shape(40, 8, 96, [128], [8]), 1) == 0     # unsupported head_dim
     assert B.relaxkv_workspace_bytes(B.Shape(40, 7, 128, [128], [8]), 1) == 0    # H % H_kv != 0
+
+
+def test_a_shorter_context_never_needs_more_workspace():
+    """relaxkv_query_prefill_attention takes the workspace of the shape whose contexts count the query's tokens too, and scores in
+    the layout of the context alone: that one must fit, whatever the lengths (four shapes where it once did not come first)."""
+    rng = random.Random(3)
+    shapes = [(64, 4, 64, [61, 32597], [2003, 164]), (32, 2, 64, [31929, 988], [1442, 11]), (4, 1, 64, [68161], [3879]),
+              (64, 4, 64, [58235, 1994, 115, 2179], [1657, 1029, 699, 3])]
+    for _ in range(4000):
+        h, hkv, d = rng.choice([(4, 1, 64), (8, 2, 128), (32, 8, 128), (40, 8, 128), (64, 4, 64), (32, 2, 64), (16, 16, 128)])
+        nb = rng.choice([1, 1, 2, 3, 4, 8, 64])
+        shapes.append((h, hkv, d, [int(2 ** rng.uniform(0, 17)) for _ in range(nb)], [int(2 ** rng.uniform(0, 12)) for _ in range(nb)]))
+    for h, hkv, d, ctx, q in shapes:
+        layers = rng.choice([1, 1, 2, 8, 40, 64])
+        ext = B.relaxkv_workspace_bytes(B.Shape(h, hkv, d, [t + n for t, n in zip(ctx, q)], q), layers)
+        own = B.relaxkv_workspace_bytes(B.Shape(h, hkv, d, ctx, q), layers)
+        less = B.relaxkv_workspace_bytes(B.Shape(h, hkv, d, [rng.randint(1, t) for t in ctx], q), layers)
+        assert less <= own <= ext, (h, hkv, d, ctx, q, layers, less, own, ext)
 
 
 FAKE = ctypes.c_void_p(0x10000)      # aligned, never dereferenced: calls must fail before any launch
