@@ -12,7 +12,7 @@ namespace relaxkv {
 // pointers after griddep_wait().
 constexpr int kSetThreads = 1024;
 constexpr int kSetWarps = kSetThreads / 32;
-constexpr int kSetSlices = 8;                    // blocks of the cluster that writes one list
+constexpr int kSetSlices = 8;                    // blocks of a cluster that writes one list, at most
 
 __global__ void __launch_bounds__(256) fill_i32_kernel(int* p, long long n, int v) {
   griddep_launch();
@@ -59,24 +59,25 @@ __global__ void __launch_bounds__(kSetThreads) count_sets_kernel(ReqTable rt, in
   }
 }
 
-// Cluster (b, 0) writes u_pos / u_rank, cluster (b, l+1) the ranks of R_{l,b}; each block takes a contiguous slice of the
-// positions.  Where a list starts is the sum of the counts before it, which every block adds up for itself (u_cu and r_cu
+// Cluster (b, 0) writes u_pos / u_rank, cluster (b, l+1) the ranks of R_{l,b}; each of its NS blocks takes a contiguous slice of the
+// positions (set_slices).  Where a list starts is the sum of the counts before it, which every block adds up for itself (u_cu and r_cu
 // are those sums).  One block per list took 20 / 77 / 149 us for segments of 16 K / 32 K / 64 K positions (a thread walked
 // 64 consecutive positions, one dependent uncoalesced load and store after the other), and a launch of its own for the
 // prefix of the counts another 4 us; now 7 / 20 / 24 us including what overlaps the kernels before it.
+template <int NS>                                 // slices = blocks of a cluster
 __global__ void __launch_bounds__(kSetThreads) write_sets_kernel(ReqTable rt, int n_layers, const int* h, const int* counts,
                                                                  int* u_pos, int* u_cu, int* u_rank, int* r_rank, int* r_cu,
                                                                  int* host_counts) {
   __shared__ int s_u[kSetWarps], s_r[kSetWarps], s_base[kSetWarps];
   __shared__ int s_pub[2];                                    // this slice's totals, read by the cluster
   const int B = rt.n_req;
-  const int slice = (int)blockIdx.x % kSetSlices, list = (int)blockIdx.x / kSetSlices;
+  const int slice = (int)blockIdx.x % NS, list = (int)blockIdx.x / NS;
   const int b = list % B, s = list / B;
   const int T = rt.ctx_len[b];
   const int* hb = h + rt.ctx_cu[b];
   const int thr = (s == 0) ? 0 : (s - 1);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int per = ((T + kSetSlices - 1) / kSetSlices + 31) & ~31;
+  const int per = ((T + NS - 1) / NS + 31) & ~31;
   const int p0 = min(T, slice * per), p1 = min(T, p0 + per);
   const int run = ((p1 - p0 + kSetWarps - 1) / kSetWarps + 31) & ~31;      // a contiguous run of positions per warp
   const int i0 = min(p1, p0 + warp * run), i1 = min(p1, i0 + run);
@@ -96,17 +97,19 @@ __global__ void __launch_bounds__(kSetThreads) write_sets_kernel(ReqTable rt, in
   const int wu = s_u[lane], wr = s_r[lane];
   base = warp_reduce_sum(s_base[lane]);
   int eu = warp_reduce_sum(lane < warp ? wu : 0), er = warp_reduce_sum(lane < warp ? wr : 0);
-  if (warp == 0) {
-    const int tu = warp_reduce_sum(wu), tr = warp_reduce_sum(wr);
-    if (lane == 0) { s_pub[0] = tu; s_pub[1] = tr; }
+  if (NS > 1) {
+    if (warp == 0) {
+      const int tu = warp_reduce_sum(wu), tr = warp_reduce_sum(wr);
+      if (lane == 0) { s_pub[0] = tu; s_pub[1] = tr; }
+    }
+    ptx::cluster_sync();
+    int gu = 0, gr = 0;                                       // lane r fetches the totals of slice r
+    if (lane < slice) {
+      gu = ptx::ld_cluster_s32(ptx::mapa_shared(ptx::smem_u32(&s_pub[0]), (uint32_t)lane));
+      gr = ptx::ld_cluster_s32(ptx::mapa_shared(ptx::smem_u32(&s_pub[1]), (uint32_t)lane));
+    }
+    eu += warp_reduce_sum(gu); er += warp_reduce_sum(gr);
   }
-  ptx::cluster_sync();
-  int gu = 0, gr = 0;                                         // lane r fetches the totals of slice r
-  if (lane < slice) {
-    gu = ptx::ld_cluster_s32(ptx::mapa_shared(ptx::smem_u32(&s_pub[0]), (uint32_t)lane));
-    gr = ptx::ld_cluster_s32(ptx::mapa_shared(ptx::smem_u32(&s_pub[1]), (uint32_t)lane));
-  }
-  eu += warp_reduce_sum(gu); er += warp_reduce_sum(gr);
 
   if (slice == 0 && threadIdx.x == 0) {
     const int n = cnt[idx];
@@ -131,7 +134,7 @@ __global__ void __launch_bounds__(kSetThreads) write_sets_kernel(ReqTable rt, in
     }
     eu += __popc(mu); er += __popc(mr);
   }
-  ptx::cluster_sync();                                        // nobody leaves while a peer may still read its totals
+  if (NS > 1) ptx::cluster_sync();                            // nobody leaves while a peer may still read its totals
 }
 
 // The whole schedule of ONE request in one launch: a cluster whose blocks each hold a contiguous slice of the positions in
@@ -243,13 +246,31 @@ __global__ void __launch_bounds__(kSetThreads) schedule_one_kernel(int T, int k,
 
 using namespace relaxkv;
 
+// Blocks that share one list (1, 2, 4 or 8): the count with the least waves x (wave + slice).  A wave of two blocks of 1024 threads
+// per SM takes about 3 us, 4 / 4.5 / 5.5 as clusters of 2 / 4 / 8, and a block about 0.3 us per 1 K positions of its slice.  Long
+// lists want many blocks: 9 lists of 200 K positions 86 / 57 / 38 / 30 us with 1 / 2 / 4 / 8, one request of 64 K x 40 layers 31 / 23 / 21 / 24.
+// Many lists want one each: 64 requests of 1 K x 40 layers 48 / 101 / 188 / 432 us, 8 of 8 K x 40 17 / 24 / 35 / 63, 8 of 32 K x 40 42 / 46 / 56 / 89
+// (the whole schedule; eight blocks for every list took 2.6 M threads for 2624 lists).
+static int set_slices(const ReqTable& rt, long long lists, int sms) {
+  int t_max = 1, best = 1;
+  for (int b = 0; b < rt.n_req; ++b) t_max = std::max(t_max, rt.ctx_len[b]);
+  const double wave_us[4] = {3.0, 4.0, 4.5, 5.5};
+  double best_cost = 0.0;
+  for (int i = 0, ns = 1; ns <= kSetSlices; ++i, ns *= 2) {
+    const double cost = (double)((lists * ns + 2 * sms - 1) / (2 * sms)) * (wave_us[i] + 3e-4 * t_max / ns);
+    if (ns == 1 || cost < best_cost) { best_cost = cost; best = ns; }
+  }
+  return best;
+}
+
 // The launch sequence both entry points share: `counts` (device int32 [B + n_layers*B]) is the only scratch.
 static relaxkv_status build_sets(const relaxkv_shape* shape, int32_t n_layers, const int32_t* h_k, const int32_t* anchors,
                                  int32_t* highest_layer_out, int32_t* u_pos_out, int32_t* u_cu_out, int32_t* u_rank_out,
                                  int32_t* r_rank_out, int32_t* r_cu_out, int32_t* h_counts_pinned, int* counts,
                                  cudaStream_t stream) {
   DeviceStatus* st = status_word();
-  if (!st) return RELAXKV_ERR_CUDA;
+  const int sms = sm_count_of_current_device();
+  if (!st || sms <= 0) return RELAXKV_ERR_CUDA;
   ReqTable rt;
   fill_req_table(rt, shape, nullptr, h_k);
   const int B = shape->n_req;
@@ -281,9 +302,18 @@ static relaxkv_status build_sets(const relaxkv_shape* shape, int32_t n_layers, c
                        anchors, highest_layer_out, st);
   if (e == cudaSuccess)
     e = launch_chained(count_sets_kernel, dim3(lists), dim3(kSetThreads), 0, stream, rt, n_layers, highest_layer_out, counts);
-  if (e == cudaSuccess)
-    e = launch_chained_clusters(kSetSlices, write_sets_kernel, dim3(lists * kSetSlices), dim3(kSetThreads), 0, stream, rt,
-                                n_layers, highest_layer_out, counts, u_pos_out, u_cu_out, u_rank_out, r_rank_out, r_cu_out, host_counts);
+  if (e == cudaSuccess) {
+    auto write = [&](auto* kernel, int slices) {
+      return launch_chained_clusters(slices, kernel, dim3(lists * (unsigned)slices), dim3(kSetThreads), 0, stream, rt, n_layers,
+                                     highest_layer_out, counts, u_pos_out, u_cu_out, u_rank_out, r_rank_out, r_cu_out, host_counts);
+    };
+    switch (set_slices(rt, lists, sms)) {
+      case 1: e = write(write_sets_kernel<1>, 1); break;
+      case 2: e = write(write_sets_kernel<2>, 2); break;
+      case 4: e = write(write_sets_kernel<4>, 4); break;
+      default: e = write(write_sets_kernel<8>, 8);
+    }
+  }
   relaxkv_status rc = cuda_ok(e);
   if (rc != RELAXKV_OK) return rc;
   if (h_counts_pinned && !host_counts)

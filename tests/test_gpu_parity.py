@@ -193,6 +193,35 @@ def test_selection_and_schedule_at_slice_edges(ctx):
                 np.testing.assert_array_equal(got, ref.ranks(l))
 
 
+@pytest.mark.parametrize("ctx,L", [((1,) + tuple(range(33, 96)), 6), ((1024,) * 64, 40), ((4097,) * 3 + (31, 32, 1), 40), ((65536, 640), 60),
+                                   ((32768,), 40), ((32769, 5), 12), ((100001,), 6), ((70000, 4096, 1, 16385), 3)])
+def test_schedule_by_the_blocks_per_list(ctx, L):
+    """Schedules of few long lists to many short ones (one to eight blocks share a list): every output bit-exact against the oracle,
+    with a sixth of the positions never selected and the anchors of a request's layers overlapping."""
+    from paper_2609_33503_b200.pipeline import RepairSession
+    rng = np.random.default_rng(len(ctx) * 1000 + L)
+    nb, k = len(ctx), [max(1, t // 9) for t in ctx]
+    cu = np.concatenate([[0], np.cumsum(ctx)])
+    want = [np.stack([np.sort(rng.choice(max(1, t - t // 6), size=kb, replace=False)) for _ in range(L)]).astype(np.int32) for t, kb in zip(ctx, k)]
+    s = RepairSession(8, 2, 128, ctx, [1] * nb, L, k)
+    for t in (s.highest_layer, s.u_pos, s.u_cu, s.u_rank, s.r_rank, s.r_cu, s.counts_pinned):
+        t.fill_(-7)
+    s.build_active_sets(torch.from_numpy(np.concatenate(want, axis=1)).cuda())
+    n_u, n_r = s.counts()
+    assert_status_ok()
+    u_cu, r_cu, u_pos, u_rank, r_rank = (t.cpu().numpy() for t in (s.u_cu, s.r_cu, s.u_pos, s.u_rank, s.r_rank))
+    assert u_cu[0] == r_cu[0] == 0
+    for b in range(nb):
+        ref = orc.active_sets(want[b], ctx[b])
+        assert n_u[b] == len(ref.u_pos) == u_cu[b + 1] - u_cu[b]
+        np.testing.assert_array_equal(u_pos[u_cu[b]:u_cu[b + 1]], ref.u_pos)
+        np.testing.assert_array_equal(u_rank[cu[b]:cu[b + 1]], ref.u_rank)
+        for l in range(L):
+            got = r_rank[r_cu[l * nb + b]:r_cu[l * nb + b + 1]]
+            assert n_r[l][b] == len(got)
+            np.testing.assert_array_equal(got, ref.ranks(l))
+
+
 # --------------------------------------------------------------------- gather / scatter ----
 
 @pytest.mark.parametrize("head_major", [False, True])
