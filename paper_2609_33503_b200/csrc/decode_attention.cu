@@ -12,6 +12,7 @@
 // adds them in a fixed order.  Every wait is bounded.
 #include "attention_common.cuh"
 #include "decode_attention.cuh"
+#include "decode_splits.cuh"
 #include "sm100_ptx.cuh"
 #include <algorithm>
 #include <atomic>
@@ -353,22 +354,17 @@ static relaxkv_status launch_d(const relaxkv_shape* shape, AttnPlan plan, const 
       !make_map_3d(&tm_v, plan.v_base, D, Hkv, (uint64_t)plan.ctx_rows, plan.kv_head_stride_bytes, plan.kv_token_stride_bytes, 1u,
                    (uint32_t)kDecTile))
     return RELAXKV_ERR_CUDA;
-  // One block per SM (the ring takes its shared memory), one wave of blocks.  All blocks get about the same number of
-  // tiles, at least two: the fewest per block for which the requests' blocks fit the wave.  (The same number of splits for
-  // every request gave contexts of 8257, 4141, 6014 and 2049 tokens four each: 17 tiles in the longest block against 8.8
-  // on average: 23.5 us a call with the merge, now 20.5.)
+  // One block per SM (the ring takes its shared memory).  (The same number of splits for every request gave contexts of 8257,
+  // 4141, 6014 and 2049 tokens four each: 17 tiles in the longest block against 8.8 on average: 23.5 us a call with the
+  // merge, now 20.5.)
   int n_tiles[kMaxReqInline];
-  long long all_tiles = 0;
-  for (int b = 0; b < B; ++b) { n_tiles[b] = (shape->h_ctx_len[b] + kDecTile - 1) / kDecTile; all_tiles += n_tiles[b]; }
-  const long long slots = std::max(1, sms / Hkv);                            // blocks per KV head
+  for (int b = 0; b < B; ++b) n_tiles[b] = (shape->h_ctx_len[b] + kDecTile - 1) / kDecTile;
+  const int per = decode_tiles_per_block(n_tiles, B, std::max(1, sms / Hkv));      // room per KV head
   const long long cap = std::max<long long>(1, std::min<long long>(kSplitRowsCap / std::max<long long>(1, n_target_rows), 1024));
   const int forced = (shape->h_tuning && shape->h_tuning->attention_ctx_splits > 0) ? shape->h_tuning->attention_ctx_splits : 0;
-  long long per = std::max<long long>(2, (all_tiles + slots - 1) / slots);
-  auto blocks_with = [&](long long p) { long long n = 0; for (int b = 0; b < B; ++b) n += (n_tiles[b] + p - 1) / p; return n; };
-  while (blocks_with(per) > std::max<long long>(slots, B)) ++per;
   int max_splits = 1;
   for (int b = 0; b < B; ++b) {
-    const int ns = (int)std::min<long long>(cap, forced ? forced : (n_tiles[b] + per - 1) / per);
+    const int ns = (int)std::min<long long>(cap, forced ? forced : decode_blocks(n_tiles[b], per));
     plan.rt.tile_cu[b + 1] = plan.rt.tile_cu[b] + ns;
     max_splits = std::max(max_splits, ns);
   }

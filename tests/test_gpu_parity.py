@@ -871,6 +871,40 @@ def test_decode_attention_one_token_per_request(H, Hkv, D, n_splits, head_major)
     assert st == B().ERR_BAD_INDEX
 
 
+@pytest.mark.parametrize("H,Hkv,D,lens", [
+    (8, 8, 64, [12000] + [200 + 37 * i for i in range(23)]), (16, 8, 128, [130 * i + 1 for i in range(1, 12)] + [9001]),
+    (5, 1, 128, [257, 385, 1, 128, 511, 4000]), (64, 64, 64, [1500, 40, 700])], ids=["24_one_long", "12_long_last", "few_tiles", "heads_fill_the_sms"])
+def test_decode_attention_of_ragged_batches(H, Hkv, D, lens):
+    """One token per request where the requests nearly fill the GPU or more: a long context is split beside short ones that are not,
+    three tiles stay one block.  Against the oracle, and the same token without lists (a query of one token) bit for bit."""
+    offs = np.concatenate([[0], np.cumsum(lens)[:-1]]).tolist()
+    g = torch.Generator(device="cpu").manual_seed(12)
+    k_all = torch.randn(sum(lens), Hkv, D, generator=g).to(torch.bfloat16).cuda()
+    v_all = torch.randn(sum(lens), Hkv, D, generator=g).to(torch.bfloat16).cuda()
+    nb = len(lens)
+    q = torch.randn(nb, H, D, generator=g).to(torch.bfloat16).cuda()
+    shape = B().Shape(H, Hkv, D, lens, [1] * nb, D ** -0.5)
+    ws = torch.empty(B().relaxkv_workspace_bytes(shape, 1) + 256, dtype=torch.uint8, device="cuda")
+    ws = ws[(-ws.data_ptr()) % 256:]
+    out, lse = torch.full_like(q, 3.0), torch.zeros(H, nb, dtype=torch.float32, device="cuda")
+    view = B().CacheView(k_all, v_all, offs)
+    tgt_pos = torch.tensor([t - 1 for t in lens], dtype=torch.int32).cuda()
+    B().relaxkv_cache_attention(shape, view, q, tgt_pos, torch.arange(nb + 1, dtype=torch.int32).cuda(), [1] * nb, out, ws, lse_out=lse)
+    assert_status_ok()
+    for b, (o, t) in enumerate(zip(offs, lens)):
+        kb, vb = inputs.bf16_bits(k_all[o:o + t].contiguous()), inputs.bf16_bits(v_all[o:o + t].contiguous())
+        ref, ref_lse = orc.list_attention(kb, vb, inputs.bf16_bits(q[b:b + 1]), None, None, np.arange(t), np.array([t - 1], dtype=np.int32), D ** -0.5)
+        mx, mean = attention_errors(out[b:b + 1], ref)
+        assert mx <= MAX_ABS and mean <= MEAN_ABS, (b, mx, mean)
+        np.testing.assert_allclose(lse[:, b:b + 1].cpu().numpy().T, ref_lse, atol=2e-3, rtol=1e-4)
+    if min(lens) > 1:
+        own = B().Shape(H, Hkv, D, [t - 1 for t in lens], [1] * nb, D ** -0.5)
+        out2, lse2 = torch.full_like(q, 3.0), torch.zeros_like(lse)
+        B().relaxkv_query_prefill_attention(own, view, q, out2, lse2, None, ws)
+        assert_status_ok()
+        assert torch.equal(out, out2) and torch.equal(lse, lse2)
+
+
 def _one_rank_group():
     """A process group of this one process on the GPU (NCCL): the all-reduce of the sharded path runs for real,
     over a single rank."""
