@@ -67,9 +67,11 @@ decode_attention_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
                         float* __restrict__ part_lse, DeviceStatus* st) {
   using L = DecSmem<D>;
   const int G = H / Hkv;
-  // rt.tile_cu: prefix of the splits per request
-  const int b = find_segment(rt.tile_cu, rt.n_req, (int)blockIdx.x), hd = blockIdx.y;
-  const int split = (int)blockIdx.x - rt.tile_cu[b], n_splits = rt.tile_cu[b + 1] - rt.tile_cu[b];
+  // rt.tile_cu: prefix of the splits per request.  KV heads fastest: the blocks of a long request start one behind the other in
+  // request order (heads slowest, its last head waited for all other requests' blocks: 64 requests, one of 128 K, 699 us, 678 so)
+  const int hd = (int)blockIdx.x % Hkv, at = (int)blockIdx.x / Hkv;
+  const int b = find_segment(rt.tile_cu, rt.n_req, at);
+  const int split = at - rt.tile_cu[b], n_splits = rt.tile_cu[b + 1] - rt.tile_cu[b];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   griddep_launch();
   if (threadIdx.x == kDecConsumers * 32) {
@@ -334,7 +336,7 @@ static relaxkv_status launch_g(const CUtensorMap& tm_k, const CUtensorMap& tm_v,
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, DecSmem<D>::kDynamic) != cudaSuccess) return RELAXKV_ERR_CUDA;
     attr_done[dev].store(1, std::memory_order_release);
   }
-  const dim3 grid((unsigned)plan.rt.tile_cu[plan.rt.n_req], (unsigned)Hkv);
+  const dim3 grid((unsigned)(plan.rt.tile_cu[plan.rt.n_req] * Hkv));
   return cuda_ok(launch_chained(kern, grid, kDecThreads, DecSmem<D>::kDynamic, stream, tm_k, tm_v, plan.rt, max_splits,
                                 static_cast<const uint16_t*>(q), tgt_pos, tgt_cu, (long long)n_target_rows, H, Hkv, scale_log2,
                                 static_cast<uint16_t*>(out), lse_out, plan.split_o, plan.split_lse, st));
