@@ -21,34 +21,43 @@ __device__ __forceinline__ uint4 pack8(const float* f) {
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// y = x / sqrt(mean(x^2) + eps) * w ; one block per row, C a multiple of 8.  A launch of a few rows is a chain of memory
-// latencies, so the row and the weights are fetched side by side and kept in registers (up to kNormHeld columns; wider rows
-// are read again), and the weights are requested into L2 before the wait for the kernel in front.
+// y = x / sqrt(mean(x^2) + eps) * w ; one block per row, C a multiple of 8.  HELD (a launch of a few rows, a chain of memory
+// latencies): the row and the weights are fetched side by side and kept in registers (up to kNormHeld columns; wider rows
+// are read again), and the weights are requested into L2 before the wait for the kernel in front.  Otherwise (more rows than are
+// resident at once, bandwidth counts) the row is read twice and few registers are held, and the next kernel's blocks come when a
+// block is through: with registers held and blocks of later launches in between, 2000 rows of 512 / 2048 / 12288 columns
+// took 5.5 / 6.5 / 20.9 us, 20000 of 12288 204; so 3.2 / 4.2 / 13.4 and 147.
 constexpr int kNormChunks = 4, kNormHeld = kNormChunks * 256 * 8;
+constexpr int kNormHeldRows = 296;                              // two blocks per SM
+template <bool HELD>
 __global__ void __launch_bounds__(256)
-rmsnorm_kernel(const uint16_t* x, const uint16_t* w, uint16_t* y, int C, float eps) {
+rmsnorm_kernel(const uint16_t* x, const uint16_t* w, uint16_t* __restrict__ y, int C, float eps) {
+  constexpr int kChunks = HELD ? kNormChunks : 0;
+  constexpr int kFrom = kChunks * 256 * 8;                     // columns from here on are read a second time
   const long long row = blockIdx.x;
   const uint16_t* xr = x + row * C;
   float ss = 0.f;
-  griddep_launch();
-  if ((threadIdx.x & 7) == 0)                                  // one 128-byte line per eight threads
-    for (int i = threadIdx.x * 8; i < C; i += 256 * 8) asm volatile("prefetch.global.L2 [%0];" ::"l"(w + i));
+  if (HELD) {
+    griddep_launch();
+    if ((threadIdx.x & 7) == 0)                                // one 128-byte line per eight threads
+      for (int i = threadIdx.x * 8; i < C; i += 256 * 8) asm volatile("prefetch.global.L2 [%0];" ::"l"(w + i));
+  }
   griddep_wait();
-  uint4 xv[kNormChunks], wv[kNormChunks];
+  uint4 xv[HELD ? kNormChunks : 1], wv[HELD ? kNormChunks : 1];
 #pragma unroll
-  for (int c = 0; c < kNormChunks; ++c) {
+  for (int c = 0; c < kChunks; ++c) {
     const int i = threadIdx.x * 8 + c * 256 * 8;
     xv[c] = i < C ? *reinterpret_cast<const uint4*>(xr + i) : make_uint4(0u, 0u, 0u, 0u);
     wv[c] = i < C ? *reinterpret_cast<const uint4*>(w + i) : make_uint4(0u, 0u, 0u, 0u);
   }
 #pragma unroll
-  for (int c = 0; c < kNormChunks; ++c) {
+  for (int c = 0; c < kChunks; ++c) {
     float f[8];
     unpack8(xv[c], f);
 #pragma unroll
     for (int e = 0; e < 8; ++e) ss = fmaf(f[e], f[e], ss);
   }
-  for (int i = threadIdx.x * 8 + kNormHeld; i < C; i += 256 * 8) {
+  for (int i = threadIdx.x * 8 + kFrom; i < C; i += 256 * 8) {
     float f[8];
     unpack8(*reinterpret_cast<const uint4*>(xr + i), f);
 #pragma unroll
@@ -71,12 +80,13 @@ rmsnorm_kernel(const uint16_t* x, const uint16_t* w, uint16_t* y, int C, float e
     *reinterpret_cast<uint4*>(y + row * C + i) = pack8(f);
   };
 #pragma unroll
-  for (int c = 0; c < kNormChunks; ++c) {
+  for (int c = 0; c < kChunks; ++c) {
     const int i = threadIdx.x * 8 + c * 256 * 8;
     if (i < C) put(i, xv[c], wv[c]);
   }
-  for (int i = threadIdx.x * 8 + kNormHeld; i < C; i += 256 * 8)
+  for (int i = threadIdx.x * 8 + kFrom; i < C; i += 256 * 8)
     put(i, *reinterpret_cast<const uint4*>(xr + i), *reinterpret_cast<const uint4*>(w + i));
+  if (!HELD) griddep_launch();
 }
 
 // Short rows (a head vector: C <= 256): one warp per row, each lane 8 elements, so the per-head Q/K norm of a
@@ -557,7 +567,8 @@ extern "C" relaxkv_status relaxkv_rmsnorm(const void* x, const void* weight, voi
     return cuda_ok(launch_chained(rmsnorm_rows_bulk_kernel, (unsigned)((n_rows + kRowWarps - 1) / kRowWarps), kRowWarps * 32, smem, static_cast<cudaStream_t>(stream),
         static_cast<const uint16_t*>(x), static_cast<const uint16_t*>(weight), static_cast<uint16_t*>(y), (long long)n_rows, n_cols, eps, st));
   }
-  return cuda_ok(launch_chained(rmsnorm_kernel, (unsigned)n_rows, 256, 0, static_cast<cudaStream_t>(stream),
+  auto kern = n_rows <= kNormHeldRows ? rmsnorm_kernel<true> : rmsnorm_kernel<false>;
+  return cuda_ok(launch_chained(kern, (unsigned)n_rows, 256, 0, static_cast<cudaStream_t>(stream),
                                 static_cast<const uint16_t*>(x), static_cast<const uint16_t*>(weight),
                                 static_cast<uint16_t*>(y), n_cols, eps));
 }

@@ -187,6 +187,26 @@ def test_rmsnorm_rope_swiglu():
     close(out, blk.swiglu(blk.f64(bits(gu))), abs_floor=1e-3)
 
 
+@pytest.mark.parametrize("C", [264, 2048, 8192, 8200, 12288])
+def test_rmsnorm_forms_at_their_line(C):
+    """One block per row with the row in registers (up to 296 rows, 8192 columns held) and without (297): against the oracle, the same
+    bits for a row in both, in place too."""
+    x, w = rnd(297, C, seed=14, scale=2.0), rnd(C, seed=15)
+    ys = []
+    for rows in (297, 296):
+        y = torch.full((298, C), 7.0, dtype=torch.bfloat16, device="cuda")
+        B().relaxkv_rmsnorm(x[:rows], w, y[:rows], 1e-6)
+        assert torch.all(y[rows:] == 7.0)
+        z = x[:rows].clone()
+        B().relaxkv_rmsnorm(z, w, z, 1e-6)
+        assert torch.equal(z, y[:rows])
+        ys.append(y)
+    st, detail = B().relaxkv_read_device_status()
+    assert st == 0, (st, detail)
+    assert torch.equal(ys[0][:296], ys[1][:296])
+    close(ys[0][:297], blk.rmsnorm(blk.f64(bits(x)), blk.f64(bits(w)), 1e-6), abs_floor=1e-3)
+
+
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("with_norm", [True, False])
 @pytest.mark.parametrize("n,H,Hkv", [(37, 5, 2), (2100, 40, 8), (2050, 18, 3), (4100, 40, 8), (4097, 18, 3)],
