@@ -452,7 +452,7 @@ relaxkv_status relaxkv_cache_attention(
 relaxkv_status relaxkv_debug_wait_timeout(relaxkv_stream stream);
 
 /*
- * Chained launches.  The kernels of the calls above (all but the explicit-list maps and the score averages) are
+ * Chained launches.  The kernels of the calls above (all but the explicit-list maps, the score averages and relaxkv_rope) are
  * launched with CUDA's programmatic stream serialization: the next kernel's blocks become resident
  * while the current kernel finishes, request the head of their weights into L2 (weights depend on
  * no earlier kernel) and then wait, inside the kernel, until every earlier kernel of the stream has

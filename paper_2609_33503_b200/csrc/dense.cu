@@ -117,12 +117,12 @@ rmsnorm_short_kernel(const uint16_t* x, const uint16_t* w, uint16_t* __restrict_
 }
 
 // Rotate-half rotary embedding in place on x [rows, heads, D]; one thread per (row, 8 pairs): the eight
-// (cos, sin) pairs are computed once and applied to every head of the row.
+// (cos, sin) pairs are computed once and applied to every head of the row.  Launched the plain way: a launch is a wave of
+// long-running blocks or less, and chained ones crowd onto the SMs that have room beside their predecessor's blocks (40 heads of 128,
+// 57 / 500 / 5000 rows 18.4 / 20.2 / 30.4 us chained, 16.1 / 16.1 / 19.0 plain).
 __global__ void rope_kernel(uint16_t* __restrict__ x, long long rows, int heads, int D, const int* positions,
                             double log2_theta) {
   const int half = D / 2, groups = half / 8;
-  griddep_launch();
-  griddep_wait();
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= rows * groups) return;
   const int gi = (int)(idx % groups);
@@ -580,8 +580,9 @@ extern "C" relaxkv_status relaxkv_rope(void* x, int64_t n_rows, int32_t n_heads,
   if (n_rows < 0 || n_heads < 1 || (head_dim != 64 && head_dim != 128)) return RELAXKV_ERR_UNSUPPORTED_SHAPE;
   if (n_rows == 0) return RELAXKV_OK;
   const long long n = n_rows * (head_dim / 16);
-  return cuda_ok(launch_chained(rope_kernel, (unsigned)((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream),
-      static_cast<uint16_t*>(x), n_rows, n_heads, head_dim, positions, log2((double)theta)));
+  rope_kernel<<<(unsigned)((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+      static_cast<uint16_t*>(x), n_rows, n_heads, head_dim, positions, log2((double)theta));
+  return launch_ok();
 }
 
 extern "C" relaxkv_status relaxkv_qk_norm_rope(void* q, void* k, int64_t n_rows, int32_t n_q_heads, int32_t n_kv_heads,
