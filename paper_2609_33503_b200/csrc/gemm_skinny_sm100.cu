@@ -9,7 +9,9 @@
 // [r n_k / S, (r + 1) n_k / S) into its own TMEM accumulator, writes the partial tile into its own shared memory, and
 // after a cluster barrier every block sums, for the 128 / S features it owns, the S
 // partials in rank order - through distributed shared memory - adds the residual and writes bf16.  A fixed order: results
-// do not depend on timing.  No scratch in global memory.
+// do not depend on timing.  No scratch in global memory.  Up to four rows (a decoded batch) K is always summed in eight parts, each
+// in TMEM columns of its own where a block has several: the bits then depend on K alone, not on how many blocks share a tile, so a
+// projection gives the same bits stacked with others and by itself.
 // Up to three output segments (feature ranges going to different buffers) serve the fused Q/K/V projection; the fused
 // gate/up projection takes 64 gate rows and their 64 up rows as one tile and applies the activation in the epilogue.
 // Bound by HBM (N K 2 bytes); with 128 rows of x as the M side, one block per SM and plain launches, four rows of a decode
@@ -39,7 +41,7 @@ constexpr int kSkWBytes = kSkFeat * kSkBK * 2;                             // we
 constexpr int kSkRing2 = 108 * 1024, kSkRing1 = 192 * 1024;                // two blocks, one block per SM
 constexpr int kSkCols2 = 64;                                               // widest MMA that always takes the two-block form
 constexpr int kSkPitch = kSkFeat + 4;                                      // floats per staged row: 16-byte reads of 8 rows hit all banks
-constexpr int kSkDeepK = 8192;                                             // few rows: K from which eight blocks share a tile
+constexpr int kSkParts = 8, kSkPartCols = 16;                               // few rows: parts of K, MMA columns of each
 constexpr int kSkBars = 2 * kSkStagesMax + 1;                              // full, empty per stage; accumulator full
 constexpr int kSkTail = 8 * kSkBars + 16 + 1024;                           // barriers, slots, alignment
 constexpr int sk_stages(int n_cols, bool whole_sm) { return (whole_sm ? kSkRing1 : kSkRing2) / (kSkWBytes + n_cols * kSkBK * 2); }
@@ -53,7 +55,8 @@ __device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t cluster_addr) {
   return v;
 }
 
-template <int S>
+// S blocks per tile; a block's share of K is PL parts, each summed in an accumulator of its own (PL > 1: n_cols is kSkPartCols).
+template <int S, int PL>
 __global__ void __launch_bounds__(kSkThreads, 2)
 gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
                          int M, int n_cols, int n_stages, int n_feat, int K, int swiglu, const __grid_constant__ SkinnyOut outs,
@@ -61,7 +64,8 @@ gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_
   const uint32_t rank = (S > 1) ? cluster_ctarank() : 0u;
   const int tile = (int)(blockIdx.x / S);
   const int n_k = (K + kSkBK - 1) / kSkBK;
-  const int k0 = (int)((long long)rank * n_k / S), k1 = (int)((long long)(rank + 1) * n_k / S);
+  auto part_begin = [&](int j) { return (int)((long long)j * n_k / (S * PL)); };       // first K block of part j (of all ranks)
+  const int k0 = part_begin((int)rank * PL), k1 = part_begin(((int)rank + 1) * PL);
   // the weight rows of this tile: two boxes of 64
   const int f0 = swiglu ? tile * (kSkFeat / 2) : tile * kSkFeat;            // first output feature
   const int r0 = swiglu ? (f0 / 128) * 256 + f0 % 128 : f0, r1 = swiglu ? r0 + 128 : r0 + kSkFeat / 2;
@@ -75,7 +79,7 @@ gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + ring + 8 * kSkBars);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(const_cast<uint32_t*>(tmem_slot) + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t tmem_cols = n_cols <= 32 ? 32u : (n_cols <= 64 ? 64u : 128u);
+  const uint32_t tmem_cols = n_cols * PL <= 32 ? 32u : (n_cols * PL <= 64 ? 64u : 128u);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < n_stages; ++s) { mbar_init(bar_full + 8 * s, 1); mbar_init(bar_empty + 8 * s, 1); }
@@ -123,13 +127,18 @@ gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_
     if (lane == 0) {
       const uint32_t idesc = idesc_bf16_f32(kSkFeat, n_cols, 0);
       bool go = true;
-      for (int kt = k0, it = 0, s = 0, ph = 0; kt < k1; ++kt, ++it) {
-        if (!(go = mbar_wait(bar_full + 8 * s, (uint32_t)ph, abort_flag))) break;
-        tc_fence_after();
-        const uint32_t sw = base + (uint32_t)s * stage_bytes;
-        mma_ss_4steps(tmem_base, desc_lo(sw, 16), desc_lo(sw + kSkWBytes, 16), desc_hi_sw128(1024), idesc, it > 0 ? 1u : 0u);
-        mma_commit(bar_empty + 8 * s);
-        if (++s == n_stages) { s = 0; ph ^= 1; }
+      int s = 0, ph = 0;
+      for (int i = 0; go && i < PL; ++i) {
+        const int kb = part_begin((int)rank * PL + i), ke = part_begin((int)rank * PL + i + 1);
+        for (int kt = kb; kt < ke; ++kt) {
+          if (!(go = mbar_wait(bar_full + 8 * s, (uint32_t)ph, abort_flag))) break;
+          tc_fence_after();
+          const uint32_t sw = base + (uint32_t)s * stage_bytes;
+          mma_ss_4steps(tmem_base + (uint32_t)(i * n_cols), desc_lo(sw, 16), desc_lo(sw + kSkWBytes, 16), desc_hi_sw128(1024), idesc,
+                        kt > kb ? 1u : 0u);
+          mma_commit(bar_empty + 8 * s);
+          if (++s == n_stages) { s = 0; ph ^= 1; }
+        }
       }
       if (go) mma_commit(bar_acc);
     }
@@ -144,13 +153,15 @@ gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_
       const uint32_t t_lane = tmem_base + ((uint32_t)(warp * 32) << 16);
       float* stage = reinterpret_cast<float*>(base_ptr) + warp * 32 + lane;
 #pragma unroll 1
-      for (int c = 0; c < M; c += 32) {
+      for (int c = 0; c < (PL > 1 ? PL * kSkPartCols : M); c += 32) {
         uint32_t v[32];
         tmem_ld32(t_lane + c, v);
         tmem_wait_ld();
 #pragma unroll
-        for (int i = 0; i < 32; ++i)
-          if (c + i < M) stage[(c + i) * kSkPitch] = __uint_as_float(v[i]);
+        for (int i = 0; i < 32; ++i) {                           // staged: the rows of x of one part behind the other
+          const int m = PL > 1 ? i % kSkPartCols : c + i, part = PL > 1 ? c / kSkPartCols + i / kSkPartCols : 0;
+          if (m < M) stage[(part * M + m) * kSkPitch] = __uint_as_float(v[i]);
+        }
       }
     }
   }
@@ -166,13 +177,13 @@ gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_
     // this rank's run of the tile's features, four features of one row of x per thread and round: the lanes that share a
     // row read up to 128 consecutive bytes of each peer (scattered 16-byte reads cost a tile of 128 rows another 8 us)
     auto sum4 = [&](int m, int col) {
-      const uint32_t off = (uint32_t)(m * kSkPitch + col) * 4u;
-      float4 v[S];
+      float4 v[S * PL];
 #pragma unroll
-      for (int src = 0; src < S; ++src) v[src] = ld_cluster_f32x4(peer[src] + off);
+      for (int src = 0; src < S * PL; ++src)
+        v[src] = ld_cluster_f32x4(peer[src / PL] + (uint32_t)((src % PL * M + m) * kSkPitch + col) * 4u);
       float4 f = v[0];
 #pragma unroll
-      for (int src = 1; src < S; ++src) {                        // rank order: the same sum whatever the timing
+      for (int src = 1; src < S * PL; ++src) {                   // order of K: the same sum whatever the timing
         f.x += v[src].x; f.y += v[src].y; f.z += v[src].z; f.w += v[src].w;
       }
       return f;
@@ -242,11 +253,11 @@ struct SkinnyPlan {
   cudaStream_t stream;
 };
 
-template <int S>
+template <int S, int PL>
 static bool opt_in_smem(int dev) {
   static std::atomic<int> attr_done[kMaxDevices];
   if (!attr_done[dev].load(std::memory_order_acquire)) {
-    if (cudaFuncSetAttribute(gemm_skinny_sm100_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSkRing1 + kSkTail) != cudaSuccess)
+    if (cudaFuncSetAttribute(gemm_skinny_sm100_kernel<S, PL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSkRing1 + kSkTail) != cudaSuccess)
       return false;
     attr_done[dev].store(1, std::memory_order_release);
   }
@@ -260,7 +271,7 @@ static int max_clusters(int dev, int sms) {
   static std::atomic<int> cached[kMaxDevices];
   int n = S == 1 ? sms : cached[dev].load(std::memory_order_acquire);
   if (n == 0) {
-    if (!opt_in_smem<S>(dev)) return 0;
+    if (!opt_in_smem<S, 1>(dev)) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(sms / S * S));
     cfg.blockDim = dim3(kSkThreads);
@@ -270,22 +281,22 @@ static int max_clusters(int dev, int sms) {
     attr.val.clusterDim.x = (unsigned)S; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm_skinny_sm100_kernel<S>, &cfg) != cudaSuccess || n < 1) n = std::max(1, sms / S / 2);
+    if (cudaOccupancyMaxActiveClusters(&n, gemm_skinny_sm100_kernel<S, 1>, &cfg) != cudaSuccess || n < 1) n = std::max(1, sms / S / 2);
     cached[dev].store(n, std::memory_order_release);
   }
   return n;
 }
 
 // Launches with clusters of S blocks if that is one wave of resident blocks that have two K blocks each (or S is 1).
-template <int S>
+template <int S, int PL = 1>
 static bool try_launch(const SkinnyPlan& p, const CUtensorMap& tm_w, const CUtensorMap& tm_x, const SkinnyOut& outs, relaxkv_status* rc) {
   const int n_k = (p.n_in + kSkBK - 1) / kSkBK;
   if (S > 1 && n_k < 2 * S) return false;
   // with two blocks per SM an even cluster sits on S / 2 SMs (the occupancy query itself counts one block per SM)
   const int resident = p.whole_sm ? max_clusters<S>(p.dev, p.sms) : (S % 2 ? 2 * max_clusters<S>(p.dev, p.sms) : max_clusters<(S + 1) / 2>(p.dev, p.sms));
-  if (resident < 1 || !opt_in_smem<S>(p.dev)) { *rc = RELAXKV_ERR_CUDA; return true; }
+  if (resident < 1 || !opt_in_smem<S, PL>(p.dev)) { *rc = RELAXKV_ERR_CUDA; return true; }
   if (S > 1 && p.tiles > resident) return false;
-  *rc = cuda_ok(launch_chained_clusters(S, gemm_skinny_sm100_kernel<S>, dim3((unsigned)(p.tiles * S)), dim3(kSkThreads), p.smem,
+  *rc = cuda_ok(launch_chained_clusters(S, gemm_skinny_sm100_kernel<S, PL>, dim3((unsigned)(p.tiles * S)), dim3(kSkThreads), p.smem,
                                         p.stream, tm_w, tm_x, p.n_rows, p.n_cols, p.n_stages, p.n_feat, p.n_in, p.swiglu, outs, p.st));
   return true;
 }
@@ -312,15 +323,18 @@ relaxkv_status launch_gemm_skinny(const void* x, const void* weight, const Skinn
   p.n_stages = sk_stages(p.n_cols, p.whole_sm);
   p.smem = (size_t)p.n_stages * (kSkWBytes + p.n_cols * kSkBK * 2) + kSkTail;
   relaxkv_status rc = RELAXKV_OK;
-  // the largest cluster that fits.  Up to four rows the choice goes by K alone, so that a projection has the same bits
-  // stacked with others and by itself.
-  const bool few = n_rows <= kGemvMaxRows, deep = n_in >= kSkDeepK;
-  if ((!few || deep) && try_launch<8>(p, tm_w, tm_x, outs, &rc)) return rc;
-  if (!few && (try_launch<7>(p, tm_w, tm_x, outs, &rc) || try_launch<6>(p, tm_w, tm_x, outs, &rc) || try_launch<5>(p, tm_w, tm_x, outs, &rc)))
+  // The largest cluster that fits.  Up to four rows K is always summed in kSkParts parts, however many blocks share them, so that a
+  // projection has the same bits stacked with others and by itself.
+  if (n_rows <= kGemvMaxRows && (n_in + kSkBK - 1) / kSkBK >= kSkParts) {
+    if (try_launch<8, 1>(p, tm_w, tm_x, outs, &rc) || try_launch<4, 2>(p, tm_w, tm_x, outs, &rc) || try_launch<2, 4>(p, tm_w, tm_x, outs, &rc))
+      return rc;
+    try_launch<1, 8>(p, tm_w, tm_x, outs, &rc);
     return rc;
-  if (try_launch<4>(p, tm_w, tm_x, outs, &rc)) return rc;
-  if (!few && try_launch<3>(p, tm_w, tm_x, outs, &rc)) return rc;
-  if (try_launch<2>(p, tm_w, tm_x, outs, &rc)) return rc;
+  }
+  if (try_launch<8>(p, tm_w, tm_x, outs, &rc) || try_launch<7>(p, tm_w, tm_x, outs, &rc) || try_launch<6>(p, tm_w, tm_x, outs, &rc) ||
+      try_launch<5>(p, tm_w, tm_x, outs, &rc) || try_launch<4>(p, tm_w, tm_x, outs, &rc) || try_launch<3>(p, tm_w, tm_x, outs, &rc) ||
+      try_launch<2>(p, tm_w, tm_x, outs, &rc))
+    return rc;
   try_launch<1>(p, tm_w, tm_x, outs, &rc);
   return rc;
 }

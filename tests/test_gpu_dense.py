@@ -124,6 +124,24 @@ def test_weight_tiles_against_a_few_rows(M, N, K, swiglu):
     assert torch.all(buf[0] == 7.0) and torch.all(buf[M + 1] == 7.0)
 
 
+@pytest.mark.parametrize("M", [2, 3, 4])
+@pytest.mark.parametrize("n_q,n_kv,K", [(8192, 1024, 5120), (8192, 1024, 8192), (5120, 1024, 4104), (1024, 128, 4096), (20480, 4096, 8200), (2048, 264, 2056)])
+def test_stacked_projections_give_the_bits_of_single_ones(M, n_q, n_kv, K):
+    """Two to four rows: the stacked matrix has more tiles than its parts and is shared by other numbers of blocks (8, 4, 2 and 1 for
+    these), the sums over K have the same order: equal bits, and both against the oracle."""
+    x = rnd(M, K, seed=61)
+    ws = [rnd(n, K, scale=K ** -0.5, seed=62 + i) for i, n in enumerate((n_q, n_kv, n_kv))]
+    outs = [torch.full((M, n), 7.0, dtype=torch.bfloat16, device="cuda") for n in (n_q, n_kv, n_kv)]
+    B().relaxkv_linear_qkv(x, B().stack_qkv(*ws), *outs)
+    for w, out in zip(ws, outs):
+        one = torch.full_like(out, 7.0)
+        B().relaxkv_linear(x, w, one)
+        assert torch.equal(one, out)
+        close(out[:, -200:], blk.linear(blk.f64(bits(x)), blk.f64(bits(w[-200:].contiguous())), None), abs_floor=2e-3)
+    st, detail = B().relaxkv_read_device_status()
+    assert st == 0, (st, detail)
+
+
 def test_linear_at_the_benchmark_shapes():
     """The projections at the sizes the repair loop runs them for the 32K Qwen3-14B-shaped stack: 18 000 active rows
     through a 5120 -> 5120 projection with residual (SM pairs) and the fused gate/up projection of 5120 -> 2 x 17408 on
