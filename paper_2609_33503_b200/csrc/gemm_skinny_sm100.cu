@@ -3,7 +3,7 @@
 // decoded tokens of a batch.  The work is streaming the weight matrix once, so the weights are the M side of the MMA:
 // a tile is 128 weight rows (TMEM lanes = output features) against all rows of x (N = 16 ... 128 columns, the row count
 // rounded up to 16), and a thread block holds half an SM's shared memory as a TMA ring of 64-wide K blocks (a
-// whole SM's above 64 rows, where x takes as much of a stage as the weights).  128 to 192 KB of weights per SM are in
+// whole SM's above 64 rows, where x takes as much of a stage as the weights, and from 33 rows on for few tiles).  128 to 192 KB of weights per SM are in
 // flight, and x rows that do not exist are neither multiplied nor, past the 16
 // granularity, staged.  A thread-block CLUSTER of S blocks shares a tile and splits K: block r multiplies K blocks
 // [r n_k / S, (r + 1) n_k / S) into its own TMEM accumulator, writes the partial tile into its own shared memory, and
@@ -45,7 +45,7 @@ constexpr int kSkParts = 8, kSkPartCols = 16;                               // f
 constexpr int kSkBars = 2 * kSkStagesMax + 1;                              // full, empty per stage; accumulator full
 constexpr int kSkTail = 8 * kSkBars + 16 + 1024;                           // barriers, slots, alignment
 constexpr int sk_stages(int n_cols, bool whole_sm) { return (whole_sm ? kSkRing1 : kSkRing2) / (kSkWBytes + n_cols * kSkBK * 2); }
-static_assert(sk_stages(16, false) <= kSkStagesMax && sk_stages(kSkCols2 + 16, true) <= kSkStagesMax, "barriers for every stage");
+static_assert(sk_stages(16, false) <= kSkStagesMax, "barriers for every stage");
 static_assert(kSkinnyMaxRows * kSkPitch * 4 <= sk_stages(kSkinnyMaxRows, false) * (kSkWBytes + kSkinnyMaxRows * kSkBK * 2),
               "the partial tile reuses the TMA ring");
 
@@ -318,9 +318,12 @@ relaxkv_status launch_gemm_skinny(const void* x, const void* weight, const Skinn
   p.sms = sm_count_of_current_device();
   if (p.sms <= 0) return RELAXKV_ERR_CUDA;
   // Above 64 rows two blocks of an SM would have three stages each; with no more tiles than SMs one block with six is
-  // faster (128 rows, 5120 x 17408: 38 against 43 us), with more tiles two (34816 x 5120: 63 against 73 us).
-  p.whole_sm = p.n_cols > kSkCols2 && p.tiles <= p.sms;
-  p.n_stages = sk_stages(p.n_cols, p.whole_sm);
+  // faster (128 rows, 5120 x 17408: 38 against 43 us), with more tiles two (34816 x 5120: 63 against 73 us).  From 33 rows on
+  // clusters of at least four blocks also want an SM per block, which all of them get where the tiles are a quarter of the SMs
+  // (64 rows, two blocks / one: 2048 x 2048 8.4 / 6.9 us, 3072 x 2048 9.8 / 7.6, 4096 x 4096 12.9 / 10.7, 4096 x 14336 25.9 / 24.1; 33 rows 6.8 / 6.2,
+  // 7.8 / 7.1, 11.0 / 10.2, 24.0 / 23.5; 40 tiles of 5120 x 5120 14.4 / 13.8 and 13.2 / 13.1; 17 rows, 2048 x 4096 7.4 / 7.8).
+  p.whole_sm = (p.n_cols > kSkCols2 && p.tiles <= p.sms) || (p.n_cols > 32 && p.tiles * 4 <= p.sms);
+  p.n_stages = std::min(kSkStagesMax, sk_stages(p.n_cols, p.whole_sm));
   p.smem = (size_t)p.n_stages * (kSkWBytes + p.n_cols * kSkBK * 2) + kSkTail;
   relaxkv_status rc = RELAXKV_OK;
   // The largest cluster that fits.  Up to four rows K is always summed in kSkParts parts, however many blocks share them, so that a

@@ -142,6 +142,19 @@ def test_stacked_projections_give_the_bits_of_single_ones(M, n_q, n_kv, K):
     assert st == 0, (st, detail)
 
 
+@pytest.mark.parametrize("M,N,K", [(32, 4736, 520), (33, 4736, 520), (33, 4744, 520), (49, 4096, 4104), (64, 4736, 1032), (64, 128, 8), (48, 2048, 1000)])
+def test_one_block_per_sm_from_33_rows(M, N, K):
+    """Both sides of the line where few tiles (37 of 128 weight rows) take a whole SM's shared memory per block: against the oracle,
+    rows around the output untouched."""
+    x, w = rnd(M, K, seed=55), rnd(N, K, scale=K ** -0.5, seed=56)
+    buf = torch.full((M + 2, N), 7.0, dtype=torch.bfloat16, device="cuda")
+    B().relaxkv_linear(x, w, buf[1:M + 1])
+    st, detail = B().relaxkv_read_device_status()
+    assert st == 0, (st, detail)
+    close(buf[1:M + 1], blk.linear(blk.f64(bits(x)), blk.f64(bits(w)), None), abs_floor=2e-3)
+    assert torch.all(buf[0] == 7.0) and torch.all(buf[M + 1] == 7.0)
+
+
 def test_linear_at_the_benchmark_shapes():
     """The projections at the sizes the repair loop runs them for the 32K Qwen3-14B-shaped stack: 18 000 active rows
     through a 5120 -> 5120 projection with residual (SM pairs) and the fused gate/up projection of 5120 -> 2 x 17408 on
