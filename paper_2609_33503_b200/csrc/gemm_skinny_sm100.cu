@@ -326,9 +326,9 @@ relaxkv_status launch_gemm_skinny(const void* x, const void* weight, const Skinn
   p.n_stages = std::min(kSkStagesMax, sk_stages(p.n_cols, p.whole_sm));
   p.smem = (size_t)p.n_stages * (kSkWBytes + p.n_cols * kSkBK * 2) + kSkTail;
   relaxkv_status rc = RELAXKV_OK;
-  // The largest cluster that fits.  Up to four rows K is always summed in kSkParts parts, however many blocks share them, so that a
-  // projection has the same bits stacked with others and by itself.
-  if (n_rows <= kGemvMaxRows && (n_in + kSkBK - 1) / kSkBK >= kSkParts) {
+  // The largest cluster that fits.  A projection of up to four rows is always summed over K in kSkParts parts, however many blocks
+  // share them, so that it has the same bits stacked with others and by itself.
+  if (n_rows <= kGemvMaxRows && !swiglu && (n_in + kSkBK - 1) / kSkBK >= kSkParts) {
     if (try_launch<8, 1>(p, tm_w, tm_x, outs, &rc) || try_launch<4, 2>(p, tm_w, tm_x, outs, &rc) || try_launch<2, 4>(p, tm_w, tm_x, outs, &rc))
       return rc;
     try_launch<1, 8>(p, tm_w, tm_x, outs, &rc);

@@ -423,14 +423,19 @@ using namespace relaxkv;
 
 // One to four rows: the plain streaming kernel or tensor-core tiles.  The streaming kernel has the shorter start but meets
 // every weight with a multiply-add per row on the FMA pipe, which is its bound from three rows on; the tiles' time hardly
-// depends on the rows.  By K alone, so that stacked and single projections take the same one.  Streaming / tiles, us:
-// one row 10.3 / 13.3 (5120 x 5120), 55 / 56 (gate/up 34816 x 5120); two rows 11.0 / 12.1 (6144 x 4096), 23 / 21 (4096 x
-// 14336), gate/up 9.4 / 8.7 (8192 x 2048), 44 / 40 (28672 x 4096); four rows 5.0 / 5.9 (2048 x 2048), 13.6 / 12.5
-// (6144 x 4096), 32 / 21 (4096 x 14336), gate/up 15.4 / 8.7 (8192 x 2048), 77 / 56 (34816 x 5120).
-static bool few_rows_stream(int64_t n_rows, int n_in, int swiglu) {
+// depends on the rows.  Projections go by K alone, so that stacked and single ones take the same.  Streaming / tiles, us:
+// one row 10.3 / 13.3 (5120 x 5120), 55 / 56 (gate/up 34816 x 5120); two rows 11.0 / 12.1 (6144 x 4096), 24 / 22 (4096 x
+// 14336), three rows 6.1 / 6.7 (2048 x 4096), 12.5 / 12.5 (6144 x 4096), 48 / 40 (28672 x 4096), four rows 5.0 / 5.9
+// (2048 x 2048), 14.2 / 12.5 (6144 x 4096), 31 / 22 (4096 x 14336).  Gate/up matrices are nobody's part: there small ones stream, up to
+// kSwigluStream2 weights for two rows, 2048 x 4096 for three and four.  Two rows 6.1 / 7.6 (2048 x 4096), 12.8 / 13.8 (6144 x 4096),
+// 12.8 / 14.4 (5120 x 5120), 17.2 / 15.5 (7168 x 5120), 43 / 40 (28672 x 4096); four rows 4.6 / 6.0 (2048 x 2048), 6.1 / 7.9 (2048 x
+// 4096), 7.5 / 7.0 (3072 x 2048), 11.8 / 10.7 (4096 x 4096), 15.4 / 9.4 (8192 x 2048), 77 / 56 (34816 x 5120).
+constexpr long long kSwigluStream2 = 28ll << 20;
+static bool few_rows_stream(int64_t n_rows, int n_out, int n_in, int swiglu) {
   if (n_rows <= 1) return true;
   if (n_rows > kGemvMaxRows) return false;
-  if (swiglu) return n_in < (n_rows == 2 ? 4096 : 2048);
+  if (swiglu && n_rows == 2) return n_in < 4096 || (long long)n_out * n_in <= kSwigluStream2;
+  if (swiglu) return n_in < 2048 || (n_out <= 2048 && n_in <= 4096);
   return n_in < (n_rows == 2 ? 8192 : 4096);
 }
 
@@ -444,7 +449,7 @@ static relaxkv_status launch_gemm(const void* x, const void* weight, const void*
   if (n_rows < 0 || n_out < 8 || n_in < 8 || (n_out % 8) || (n_in % 8)) return RELAXKV_ERR_UNSUPPORTED_SHAPE;
   if (swiglu && ((n_out % 256) || residual)) return RELAXKV_ERR_UNSUPPORTED_SHAPE;
   if (n_rows == 0) return RELAXKV_OK;
-  if (few_rows_stream(n_rows, n_in, swiglu))       // a decode token: stream the weights once, no tiles
+  if (few_rows_stream(n_rows, n_out, n_in, swiglu))       // a decode token: stream the weights once, no tiles
     return launch_gemv(x, weight, residual, y, (int)n_rows, n_out, n_in, swiglu, static_cast<cudaStream_t>(stream_));
   if (n_rows <= kSkinnyMaxRows) {   // the query's tokens, a decoded batch
     SkinnyOut outs = {};
@@ -525,7 +530,7 @@ extern "C" relaxkv_status relaxkv_linear_qkv(const void* x, const void* w_qkv, v
   if (n_rows == 0) return RELAXKV_OK;
   const int n_out = n_q + 2 * n_kv;
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-  if (few_rows_stream(n_rows, n_in, 0)) {
+  if (few_rows_stream(n_rows, n_out, n_in, 0)) {
     GemvOut outs = {};
     outs.y[0] = static_cast<uint16_t*>(q); outs.y[1] = static_cast<uint16_t*>(k); outs.y[2] = static_cast<uint16_t*>(v);
     outs.col0[0] = 0; outs.col0[1] = n_q; outs.col0[2] = n_q + n_kv; outs.col0[3] = n_out;
