@@ -195,32 +195,42 @@ inline int score_splits_most(long long units_times_heads, int layers) {
   return most < 1 ? 1 : (most > kScoreSplitsMax ? kScoreSplitsMax : (int)most);
 }
 
-// Key-range splits for a launch that scores `layers` layers at once (one CTA per SM, every CTA of a launch about the same
-// work): the count with the least waves x (start + 128-key tiles of a CTA x 128-row chunks of a tile x item).  Start and item
-// are what a CTA takes before its first product and per product of 128 x 128 (about 4 and 0.75 us).  With at least two
+// Key-range splits for a launch that scores `layers` layers at once (one CTA per SM): the count with the least rounds x longest
+// CTA.  A CTA takes start + 128-key tiles x 128-row chunks of a tile x item, start and item being what it spends before its first
+// product and per product of 128 x 128 (about 4 and 0.75 us, here in quarters of a us); a round is the time of the longest CTA on
+// all SMs, and the rounds are those that all CTAs' time fills.  With at least two
 // waves whatever the size, a 16K layer of 256 rows ran in 1.7 waves of four tiles per CTA: its scoring and schedule took 76 us,
 // 70 in one wave; the 32K pass of a query of 128 rows 60 us per layer, now 57.
 inline int score_splits(const relaxkv_shape* s, int layers) {
   const int group = s->n_q_heads / s->n_kv_heads;
+  struct { int blocks, tiles, chunks; } req[kMaxReqInline];
+  int n = 0, tiles = 1;
   long long units = 0;
-  int tiles = 1, chunks = 1;
   for (int b = 0; b < s->n_req; ++b) {
     const int q = s->h_q_len ? s->h_q_len[b] : 0, nb = score_blocks(q, group);
     if (nb == 0) continue;
     units += nb;
     const int tok = ((q + nb - 1) / nb + kScoreTokBox - 1) / kScoreTokBox * kScoreTokBox;
-    const int c = ((tok < q ? tok : q) * group + 127) / 128, t = (s->h_ctx_len[b] + 127) / 128;
-    if (c > chunks) chunks = c;
-    if (t > tiles) tiles = t;
+    req[n].blocks = nb;
+    req[n].chunks = ((tok < q ? tok : q) * group + 127) / 128;
+    req[n].tiles = (s->h_ctx_len[b] + 127) / 128;
+    if (req[n].tiles > tiles) tiles = req[n].tiles;
+    ++n;
   }
-  const long long per = units * s->n_kv_heads * layers;
-  if (per <= 0) return 1;
+  const long long copies = (long long)s->n_kv_heads * layers;
   int best = 1;
-  double best_cost = 0.0;
-  const int most = score_splits_most(units * s->n_kv_heads, layers);
+  long long best_cost = 0;
+  const int most = units > 0 ? score_splits_most(units * s->n_kv_heads, layers) : 1;
   for (int ns = 1; ns <= most && ns <= tiles; ++ns) {
-    const double waves = (double)((per * ns + kScoreSms - 1) / kScoreSms);
-    const double cost = waves * (4.0 + 0.75 * chunks * ((tiles + ns - 1) / ns));
+    long long all = 0, longest = 1;
+    const double inv = 1.0 / ns;                             // (a division per request and count was most of this function's time)
+    for (int i = 0; i < n; ++i) {
+      const int per = (int)((req[i].tiles + ns - 1) * inv + 1e-6);
+      const long long cta = 16 + 3ll * req[i].chunks * per;
+      all += cta * (req[i].tiles < ns ? req[i].tiles : ns) * req[i].blocks;      // the other splits of a short request are empty
+      if (cta > longest) longest = cta;
+    }
+    const long long round = kScoreSms * longest, cost = (all * copies + round - 1) / round * longest;
     if (ns == 1 || cost < best_cost) { best_cost = cost; best = ns; }
   }
   return best;
