@@ -58,8 +58,8 @@ def _check_linear(M, N, K, res):
 @pytest.mark.parametrize("n_q,n_kv,K", [(512, 128, 512), (5120, 1024, 5120), (320, 72, 264), (352, 96, 520)])
 def test_linear_qkv_writes_the_three_projections(M, n_q, n_kv, K):
     """The fused Q/K/V projection (stacked weight, three output buffers) through its three routes - the streaming
-    kernel (1-4 rows), the cluster split-K kernel (5-128 rows: segment boundaries inside a tile at the odd shape), one
-    large GEMM whose epilogue writes the three buffers (300 rows: the single-block kernel, 1000 rows: SM pairs; widths
+    kernel (one row, three with a K below 4096), the cluster split-K kernel (up to 128 rows: segment boundaries inside a tile at the odd
+    shape), one large GEMM whose epilogue writes the three buffers (300 rows: the single-block kernel, 1000 rows: SM pairs; widths
     that are multiples of 32, also with boundaries inside a 256-column tile) or three large GEMMs (other widths) -
     against the oracle's linear per projection; bytes around the outputs stay untouched."""
     x = rnd(M, K, seed=11)
@@ -74,7 +74,7 @@ def test_linear_qkv_writes_the_three_projections(M, n_q, n_kv, K):
         ref = blk.linear(blk.f64(bits(x)), blk.f64(bits(w)), None)
         close(out, ref, abs_floor=2e-3)
         assert torch.all(buf[0] == 7.0) and torch.all(buf[M + 1] == 7.0)
-        if M <= 4:                                   # the streaming kernel: same arithmetic as the single projection
+        if M <= 4:                                   # the order of the sums goes by K alone: the bits of the single projection
             one = torch.empty_like(out)
             B().relaxkv_linear(x, w, one)
             assert torch.equal(one, out)
@@ -83,10 +83,10 @@ def test_linear_qkv_writes_the_three_projections(M, n_q, n_kv, K):
 @pytest.mark.parametrize("M,N,K,res", [(5, 8, 8, False), (17, 136, 72, True), (100, 1000, 520, True), (128, 5120, 1032, False),
                                        (64, 264, 5120, True), (128, 19200, 64, False), (33, 2048, 17408, True)])
 def test_linear_of_a_few_rows(M, N, K, res):
-    """5 to 128 rows: 128 x 128 tiles whose K range is split over a thread-block cluster (1 to 8 blocks, by the
-    number of column tiles and K blocks) and summed through distributed shared memory; ragged N and K tails, a residual
-    that aliases the output, K shorter than two blocks per cluster member, more column tiles than SMs (19200 / 128 =
-    150: the large kernel takes that one); run twice: bit-identical (the partial sums are added in rank order)."""
+    """5 to 128 rows: tiles of 128 weight rows whose K range is split over a thread-block cluster (1 to 8 blocks, by the
+    number of tiles and K blocks) and summed through distributed shared memory; ragged N and K tails, a residual
+    that aliases the output, K shorter than two blocks per cluster member, more tiles than SMs (19200 / 128 =
+    150: one block each, two per SM); run twice: bit-identical (the partial sums are added in rank order)."""
     x, w = rnd(M, K, seed=41), rnd(N, K, scale=K ** -0.5, seed=42)
     r = rnd(M, N, seed=43) if res else None
     y = r.clone() if res else torch.full((M, N), 7.0, dtype=torch.bfloat16, device="cuda")
