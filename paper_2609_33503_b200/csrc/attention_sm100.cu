@@ -484,9 +484,9 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   }
 
   // ---- teardown ------------------------------------------------------------------------------------
-  griddep_launch();
   tc_fence_before();
   __syncthreads();
+  griddep_launch();                         // behind the barrier: one thread that calls it early speaks for its block
   if (*abort_flag) {
     if (threadIdx.x == 0) report(st, RELAXKV_ERR_TIMEOUT, KID_ATTN_SM100, pair, hd);
     // give copies and MMAs still in flight time to land before shared memory and TMEM are released
@@ -977,9 +977,9 @@ attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
     }
   }
 
-  griddep_launch();
   tc_fence_before();
   __syncthreads();
+  griddep_launch();                         // behind the barrier: one thread that calls it early speaks for its block
   if (*abort_flag) {
     if (threadIdx.x == 0) report(st, RELAXKV_ERR_TIMEOUT, KID_ATTN_SM100, (int)blockIdx.x, -2);
     const uint64_t t0 = global_timer_ns();

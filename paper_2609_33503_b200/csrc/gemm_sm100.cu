@@ -202,9 +202,9 @@ gemm_sm100_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
       mbar_arrive(bar_acc_empty + 8 * a);
     }
   }
-  griddep_launch();
   tc_fence_before();
   __syncthreads();
+  griddep_launch();                         // behind the barrier: one thread that calls it early speaks for its block
   if (*abort_flag) {
     if (threadIdx.x == 0) report(st, RELAXKV_ERR_TIMEOUT, KID_GEMM_SM100, (int)blockIdx.x, 0);
     const uint64_t tw = global_timer_ns();
@@ -404,9 +404,9 @@ gemm_pair_sm100_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
       mbar_arrive_remote(mapa_shared(bar_acc_empty + 8 * a, 0));
     }
   }
-  griddep_launch();
   tc_fence_before();
   __syncthreads();
+  griddep_launch();                         // behind the barrier: one thread that calls it early speaks for its block
   if (*abort_flag) {
     if (threadIdx.x == 0) report(st, RELAXKV_ERR_TIMEOUT, KID_GEMM_SM100, (int)blockIdx.x, 0);
     const uint64_t tw = global_timer_ns();

@@ -301,9 +301,9 @@ score_sm100_kernel(const __grid_constant__ ScoreLayers layers, const __grid_cons
   }
 
   // ---- teardown --------------------------------------------------------------------------------------
-  griddep_launch();
   tc_fence_before();
   __syncthreads();
+  griddep_launch();                         // behind the barrier: one thread that calls it early speaks for its block
   if (*abort_flag) {
     if (threadIdx.x == 0) report(st, RELAXKV_ERR_TIMEOUT, KID_SCORE_SM100, (int)blockIdx.x, split);
     const uint64_t tw = global_timer_ns();
