@@ -258,6 +258,12 @@ constexpr int kRowWarps = 4;
 constexpr int kRowBulkMinRows = 4096;        // fewer rows: the latency-oriented kernels above (equal at 2048 rows)
 constexpr int kRowBulkMaxBytes = 16 * 1024;  // per row (and warp) of shared memory
 
+// A launch of more bytes than this lets the next kernel's blocks come first thing (20000 rows of 2048 / 8192 columns 27.2 / 104.5 us,
+// 28.4 / 106.8 when they come as its own end); one of fewer, which the L2 holds, as its blocks end (5000 rows of 512 / 2048 / 4096 columns 3.1 /
+// 6.6 / 12.9 us against 3.8 / 8.0 / 13.7).
+constexpr long long kRowEarlyBytes = 48ll << 20;
+static inline int rows_early(long long n_rows, long long row_bytes) { return n_rows * row_bytes > kRowEarlyBytes ? 1 : 0; }
+
 __device__ __forceinline__ void row_wait_failed(DeviceStatus* st, long long row) {
   if ((threadIdx.x & 31) == 0) {
     report(st, RELAXKV_ERR_TIMEOUT, KID_DENSE, (int)row, -1);
@@ -270,13 +276,13 @@ __device__ __forceinline__ void row_wait_failed(DeviceStatus* st, long long row)
 // y = x / sqrt(mean(x^2) + eps) * w, one warp per row of C columns (C * 2 bytes a multiple of 16).
 __global__ void __launch_bounds__(kRowWarps * 32)
 rmsnorm_rows_bulk_kernel(const uint16_t* x, const uint16_t* w, uint16_t* __restrict__ y, long long n_rows,
-                         int C, float eps, DeviceStatus* st) {
+                         int C, float eps, int early, DeviceStatus* st) {
   extern __shared__ __align__(128) uint8_t row_stage[];      // [warp][C] bf16
   __shared__ __align__(8) unsigned long long bars[kRowWarps];
   __shared__ volatile int gave_up[kRowWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long row = (long long)blockIdx.x * kRowWarps + warp;
-  griddep_launch();
+  if (early) griddep_launch();
   griddep_wait();
   if (row >= n_rows) return;
   const uint32_t row_bytes = (uint32_t)C * 2;
@@ -327,14 +333,14 @@ template <int D>
 __global__ void __launch_bounds__(kRowWarps * 32)
 head_norm_rope_rows_bulk_kernel(uint16_t* __restrict__ q, uint16_t* __restrict__ k, long long n_rows, int Hq, int Hkv,
                                 const uint16_t* wq, const uint16_t* wk, float eps,
-                                const int* positions, double log2_theta, DeviceStatus* st) {
+                                const int* positions, double log2_theta, int early, DeviceStatus* st) {
   constexpr int P = D / 32, half = D / 2;
   extern __shared__ __align__(128) uint8_t row_stage[];      // [warp][Hq + Hkv][D] bf16
   __shared__ __align__(8) unsigned long long bars[kRowWarps];
   __shared__ volatile int gave_up[kRowWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long row = (long long)blockIdx.x * kRowWarps + warp;
-  griddep_launch();
+  if (early) griddep_launch();
   griddep_wait();
   if (row >= n_rows) return;
   const uint32_t q_bytes = (uint32_t)Hq * D * 2, k_bytes = (uint32_t)Hkv * D * 2;
@@ -565,7 +571,8 @@ extern "C" relaxkv_status relaxkv_rmsnorm(const void* x, const void* weight, voi
         cudaFuncSetAttribute(rmsnorm_rows_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return RELAXKV_ERR_CUDA;
     return cuda_ok(launch_chained(rmsnorm_rows_bulk_kernel, (unsigned)((n_rows + kRowWarps - 1) / kRowWarps), kRowWarps * 32, smem, static_cast<cudaStream_t>(stream),
-        static_cast<const uint16_t*>(x), static_cast<const uint16_t*>(weight), static_cast<uint16_t*>(y), (long long)n_rows, n_cols, eps, st));
+        static_cast<const uint16_t*>(x), static_cast<const uint16_t*>(weight), static_cast<uint16_t*>(y), (long long)n_rows, n_cols, eps,
+        rows_early(n_rows, (long long)n_cols * 2), st));
   }
   auto kern = n_rows <= kNormHeldRows ? rmsnorm_kernel<true> : rmsnorm_kernel<false>;
   return cuda_ok(launch_chained(kern, (unsigned)n_rows, 256, 0, static_cast<cudaStream_t>(stream),
@@ -613,7 +620,7 @@ extern "C" relaxkv_status relaxkv_qk_norm_rope(void* q, void* k, int64_t n_rows,
     if (smem > 48 * 1024 - 256 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return RELAXKV_ERR_CUDA;
     return cuda_ok(launch_chained(kern, (unsigned)((n_rows + kRowWarps - 1) / kRowWarps), kRowWarps * 32, smem, st,qp, kp, (long long)n_rows, n_q_heads, n_kv_heads,
-                                                                                       wq, wk, eps, positions, log2_theta, dst));
+                                                                                       wq, wk, eps, positions, log2_theta, rows_early(n_rows, (long long)(n_q_heads + n_kv_heads) * head_dim * 2), dst));
   }
   if (head_dim == 128)
     return cuda_ok(launch_chained(head_norm_rope_kernel<128>, grid, 128, 0, st, qp, kp, n_q_heads, n_kv_heads, heads_per_block,
