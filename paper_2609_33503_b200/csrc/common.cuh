@@ -130,7 +130,9 @@ inline cudaError_t launch_chained_clusters(int cluster, void (*kernel)(KArgs...)
   attr[1].val.clusterDim.x = (unsigned)cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = cluster > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+  if (e != cudaSuccess) (void)cudaGetLastError();      // reported by the return value: not a second time by a later call's launch_ok()
+  return e;
 }
 
 template <typename... KArgs, typename... Args>

@@ -155,6 +155,17 @@ def test_one_block_per_sm_from_33_rows(M, N, K):
     assert torch.all(buf[0] == 7.0) and torch.all(buf[M + 1] == 7.0)
 
 
+def test_a_refused_launch_is_reported_once():
+    """2^40 rows make a grid of no blocks (2^32 cut to 32 bits), which the runtime refuses: that call says so, the next one, which looks at the
+    runtime's last error behind its own launch, does not."""
+    x, out = rnd(8, 16, seed=91), torch.empty(8, 8, dtype=torch.bfloat16, device="cuda")
+    st = B().lib().relaxkv_swiglu(x.data_ptr(), out.data_ptr(), 1 << 40, 8, torch.cuda.current_stream().cuda_stream)
+    assert st == B().ERR_CUDA
+    scores = torch.ones(1, 64, device="cuda")
+    B().relaxkv_scale_scores(B().Shape(8, 2, 128, [64], [1]), 1, scores, 0.5)
+    assert torch.all(scores == 0.5)
+
+
 def test_linear_at_the_benchmark_shapes():
     """The projections at the sizes the repair loop runs them for the 32K Qwen3-14B-shaped stack: 18 000 active rows
     through a 5120 -> 5120 projection with residual (SM pairs) and the fused gate/up projection of 5120 -> 2 x 17408 on
