@@ -151,6 +151,13 @@ class ClockSampler:
 # the CUDA arm
 # --------------------------------------------------------------------------------------------------
 
+def schedule_launches(w):
+    """Kernels of relaxkv_build_active_sets: one for one request with little work (an eighth of the positions, rounded up to 32, times the
+    lists), else four (sets.cu)."""
+    share = ((sum(w.ctx_lens) + 7) // 8 + 31) // 32 * 32
+    return 1 if len(w.ctx_lens) == 1 and share * (w.n_layers + 1) <= 8192 else 4
+
+
 class GpuJob:
     """Device-resident inputs of one workload.  The per-layer caches do not depend on the anchor ratio;
     `prepare(ratio)` runs one untimed selection pass and builds the "freshly recomputed" rows of the active
@@ -224,9 +231,9 @@ class GpuJob:
             f = self.fresh[l]
             rec("attention", lambda: s.attention(l, self.views[l], f[0], f[1], f[2], self.outs[l], n_r[l], n_u, mode=mode))
             rec("scatter", lambda: s.scatter(l, self.views[l], f[1], f[2], n_r[l]))
-        # kernels per step: 4 scoring launches per group of <= 48 layers, 1 select, 4 for the sets, and per layer
+        # kernels per step: 4 scoring launches per group of <= 48 layers, 1 select, those of the sets, and per layer
         # gather + attention + scatter
-        self.launches_per_step = 4 * ((L + 47) // 48) + 1 + 4 + 3 * L
+        self.launches_per_step = 4 * ((L + 47) // 48) + 1 + schedule_launches(w) + 3 * L
 
     kv_reps = 10          # timed replays of the gather / scatter graphs (--kv-reps)
 
@@ -690,7 +697,7 @@ class ListJob:
                                                               tgt_cu, mt, mc, self.outs[l], s.workspace))
             rec("scatter", lambda: B.relaxkv_scatter_kv_lists(s.shape, job.views[l], f[1], f[2], tgt_pos, tgt_cu, mt))
         n_lists = (1 if self.config == "layerwise_sparse" else 2) + (0 if self.global_targets else L)
-        self.launches_per_step = 4 * ((L + 47) // 48) + 1 + 4 + n_lists + 4 * L      # per layer: maps, gather, attention, scatter
+        self.launches_per_step = 4 * ((L + 47) // 48) + 1 + schedule_launches(job.w) + n_lists + 4 * L      # per layer: maps, gather, attention, scatter
 
 
 def run_list_config(args):

@@ -315,11 +315,6 @@ __device__ __forceinline__ float warp_reduce_max(float v) {
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
-__device__ __forceinline__ float warp_reduce_min(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
 
 // Find the request that owns global tile/row index x given an inclusive-exclusive prefix array.
 __device__ __forceinline__ int find_segment(const int* cu, int n, int x) {

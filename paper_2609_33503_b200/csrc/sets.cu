@@ -141,8 +141,11 @@ __global__ void __launch_bounds__(kSetThreads) write_sets_kernel(ReqTable rt, in
 // shared memory.  Every block reads all anchors and keeps the layers of its own positions; the blocks' counts per layer meet
 // through distributed shared memory, which gives every list's place; a warp then writes one list of its block's slice, or a run
 // of it.  Four dependent launches become one, for work that is mostly their latency: positions of a slice times lists up to
-// kOneWorkMax.  Four launches / one, us on the GPU: 1 K positions and 1 layer 6.9 / 4.5, 32 layers 10.1 / 6.5; 8 K and 1 layer
-// 8.0 / 5.3, 6 layers 8.3 / 9.4; 16 K and 1 layer 9.0 / 6.3; past the line 16 K and 12 layers 10.6 / 18.0.  On the host 16 / 8.
+// kOneWorkMax.  Launched call by call the host's time decides (16 us for four launches, 8 for one), replayed from a graph the GPU's.
+// Four launches / one, us, call by call and (from a graph): 1 K positions and 1 layer 14.1 / 6.5 (6.1 / 4.2), 32 layers 14.7 / 7.4
+// (6.7 / 6.2); 8 K and 1 layer 14.0 / 6.7 (7.9 / 5.1), 5 layers 14.6 / 8.8 (8.6 / 7.3), 6 layers, work 7168, 14.7 / 10.6 (8.2 / 9.1); 16 K and 3
+// layers, the line, 14.4 / 11.0 (9.3 / 9.5); past it 16 K and 12 layers 10.6 / 18.0 on the GPU.  The line is drawn for calls (the counts are
+// read by the host behind this one); from 6144 to it a replay loses up to 1 us, with a hundred lists and more up to 3.
 constexpr int kOneWorkMax = 8192;
 constexpr int kOneLayersMax = kOneWorkMax / 32;  // a slice is at least 32 positions
 
