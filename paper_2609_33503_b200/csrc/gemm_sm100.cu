@@ -451,7 +451,11 @@ static relaxkv_status launch_gemm(const void* x, const void* weight, const void*
   if (n_rows == 0) return RELAXKV_OK;
   if (few_rows_stream(n_rows, n_out, n_in, swiglu))       // a decode token: stream the weights once, no tiles
     return launch_gemv(x, weight, residual, y, (int)n_rows, n_out, n_in, swiglu, static_cast<cudaStream_t>(stream_));
-  if (n_rows <= kSkinnyMaxRows) {   // the query's tokens, a decoded batch
+  // The query's tokens, a decoded batch.  Not gate/up matrices of more than two tiles per SM with 97 rows and more, where the few-row
+  // kernel's two blocks per SM have three stages each and start over for every tile (128 rows: 57344 x 8192 200 us in the
+  // kernel below against 211 to 218, 128256 x 4096 220 to 226 against 245; 96 rows equal, 34816 x 5120, 272 tiles, 89 / 72).
+  const int sms_here = sm_count_of_current_device();
+  if (n_rows <= kSkinnyMaxRows && !(swiglu && n_rows > 96 && (n_out + 127) / 128 > 2 * sms_here)) {
     SkinnyOut outs = {};
     outs.y[0] = static_cast<uint16_t*>(y);
     outs.residual[0] = static_cast<const uint16_t*>(residual);

@@ -444,9 +444,9 @@ def test_linear_swiglu_fused(M, I, K):
     assert float((out.float() - two.float()).abs().max()) <= 2.0 ** -6 * float(two.float().abs().max()) + 1e-2
 
 
-@pytest.mark.parametrize("M,I,K", [(2, 1024, 4096), (2, 3584, 4096), (2, 3712, 4096), (3, 1024, 4096), (4, 1024, 4104), (4, 1152, 4096), (3, 1024, 2048), (4, 2560, 5120)])
-def test_gate_up_of_two_to_four_rows(M, I, K):
-    """Both sides of the lines between the streaming kernel and the tiles for gate/up matrices: against the oracle."""
+@pytest.mark.parametrize("M,I,K", [(96, 19072, 136), (97, 19072, 136), (128, 19072, 136), (128, 18944, 136), (2, 1024, 4096), (2, 3584, 4096), (2, 3712, 4096), (3, 1024, 4096), (4, 1024, 4104), (4, 1152, 4096), (3, 1024, 2048), (4, 2560, 5120)])
+def test_gate_up_routes(M, I, K):
+    """Both sides of the lines between the streaming kernel, the few-row tiles and the large kernel for gate/up matrices: against the oracle."""
     x, w = rnd(M, K, seed=57), rnd(2 * I, K, scale=K ** -0.5, seed=58)
     buf = torch.full((M + 2, I), 7.0, dtype=torch.bfloat16, device="cuda")
     B().relaxkv_linear_swiglu(x, B().tile_gate_up(w), buf[1:M + 1])
