@@ -68,7 +68,7 @@ decode_attention_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
   using L = DecSmem<D>;
   const int G = H / Hkv;
   // rt.tile_cu: prefix of the splits per request.  KV heads fastest: the blocks of a long request start one behind the other in
-  // request order (heads slowest, its last head waited for all other requests' blocks: 64 requests, one of 128 K, 699 us, 678 so)
+  // request order (heads slowest, its last head waited for all other requests' blocks: 64 requests, one of 128 K in one block, 699 us, 678 so)
   const int hd = (int)blockIdx.x % Hkv, at = (int)blockIdx.x / Hkv;
   int b = 0;                               // by halves: a walk over the requests costs a block of the 64th a microsecond before it starts
   for (int hi = rt.n_req; hi - b > 1;) { const int mid = (b + hi) >> 1; if (rt.tile_cu[mid] <= at) b = mid; else hi = mid; }
