@@ -41,6 +41,7 @@ constexpr int kSkWBytes = kSkFeat * kSkBK * 2;                             // we
 constexpr int kSkRing2 = 108 * 1024, kSkRing1 = 192 * 1024;                // two blocks, one block per SM
 constexpr int kSkCols2 = 64;                                               // widest MMA that always takes the two-block form
 constexpr int kSkPitch = kSkFeat + 4;                                      // floats per staged row: 16-byte reads of 8 rows hit all banks
+constexpr int kSkDeepK = 8192;                                             // few rows: K from which eight blocks share a tile
 constexpr int kSkParts = 8, kSkPartCols = 16;                               // few rows: parts of K, MMA columns of each
 constexpr int kSkBars = 2 * kSkStagesMax + 1;                              // full, empty per stage; accumulator full
 constexpr int kSkTail = 8 * kSkBars + 16 + 1024;                           // barriers, slots, alignment
@@ -198,7 +199,7 @@ gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_
     uint16_t* y = outs.y[sg] + (col0 - outs.col0[sg]);
     const uint16_t* res = outs.residual[sg] ? outs.residual[sg] + (col0 - outs.col0[sg]) : nullptr;
     if (m0 < rows && col0 < n_feat && status != RELAXKV_ERR_TIMEOUT) {
-      constexpr int R = 4;                                       // rounds whose loads are in flight together
+      constexpr int R = PL > 1 ? 1 : 4;                          // rounds whose loads are in flight together (up to four rows: one in all)
       for (int mb = m0; mb < M; mb += R * rows) {
         uint2 r[R];
         float4 f[R], u[R];
@@ -328,8 +329,10 @@ relaxkv_status launch_gemm_skinny(const void* x, const void* weight, const Skinn
   relaxkv_status rc = RELAXKV_OK;
   // The largest cluster that fits.  A projection of up to four rows is always summed over K in kSkParts parts, however many blocks
   // share them, so that it has the same bits stacked with others and by itself.
+  // Eight blocks where K is long, or where each gets an SM: else they fill the SMs that the next kernel's blocks would start on.
   if (n_rows <= kGemvMaxRows && !swiglu && (n_in + kSkBK - 1) / kSkBK >= kSkParts) {
-    if (try_launch<8, 1>(p, tm_w, tm_x, outs, &rc) || try_launch<4, 2>(p, tm_w, tm_x, outs, &rc) || try_launch<2, 4>(p, tm_w, tm_x, outs, &rc))
+    const bool eight = n_in >= kSkDeepK || p.tiles * 8 <= p.sms;
+    if ((eight && try_launch<8, 1>(p, tm_w, tm_x, outs, &rc)) || try_launch<4, 2>(p, tm_w, tm_x, outs, &rc) || try_launch<2, 4>(p, tm_w, tm_x, outs, &rc))
       return rc;
     try_launch<1, 8>(p, tm_w, tm_x, outs, &rc);
     return rc;
