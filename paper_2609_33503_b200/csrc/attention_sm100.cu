@@ -38,6 +38,7 @@ constexpr int kBM = 128;                      // query rows per tile (TMEM lanes
 constexpr int kBN = 128;                      // keys per context tile
 constexpr int kHalfBytes = 128 * 128;         // 128 rows x 64 bf16: one 128B-swizzled half tile
 constexpr int kRing = 5;                      // K/V tile buffers, used in the order K0 V0 K1 V1 ...
+constexpr int kNoLimit = 0x7fffffff;          // causal limit of a row that nobody reads: no tile is masked for it
 constexpr int kPersistMaxTiles = 128;          // contexts up to this many key tiles take the persistent form
 constexpr int kAttnThreads = 384;             // 2 x 4 softmax warps + a control warpgroup (TMA warp, MMA warp, 2 idle)
 
@@ -399,7 +400,10 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     const int t_local = row / G, j_head = row - t_local * G;
     const bool row_valid = (row < tile_targets * G) && (t_local < n_valid[x]);
     const int rho_t = rho0 + x * tile_targets + t_local;
-    int limit = 0;
+    // Rows without a target (125 of 128 rows are used with five heads per KV head) and rows of an empty context see every key: what
+    // they hold is not used, and a limit below the tile sends their whole warp through the masking of every tile, 1.0 k clk of
+    // a 3.5 k step (12 layers of 40 / 8 heads at 32 K, repaired: 40.8 -> 37.4 ms; every row used, 32 / 8 heads: 8.48 -> 8.43).
+    int limit = kNoLimit;
     bool row_empty = false;                                     // explicit lists: a target that sees no context entry
     if (row_valid) {
       const int c = r_cu ? r_rank[row_b + rho_t] : first_pos + rho_t;
@@ -407,6 +411,7 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         row_empty = true;
       } else if (c < 0 || c >= nu) {
         report(st, RELAXKV_ERR_BAD_INDEX, KID_ATTN_SM100, c, nu);
+        limit = 0;
       } else {
         limit = (mode == RELAXKV_CTX_UNION) ? c : u_pos[u_cu[b] + c];
         if (limit < 0 || limit >= ctx_len_b) { report(st, RELAXKV_ERR_BAD_INDEX, KID_ATTN_SM100, limit, ctx_len_b); limit = 0; }
@@ -902,7 +907,7 @@ attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
     int c = ok ? row_rank(0, row_valid) : 0;
     while (ok) {
       const uint32_t k = ph >> 2;
-      int limit = 0, my_n;
+      int limit = kNoLimit, my_n;
       bool row_empty = false;
       {
         const int4 a = rec_ld(k, 0);
@@ -915,6 +920,7 @@ attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
             row_empty = true;
           } else if (c < 0 || c >= nu) {
             report(st, RELAXKV_ERR_BAD_INDEX, KID_ATTN_SM100, c, nu);
+            limit = 0;
           } else {
             limit = (mode == RELAXKV_CTX_UNION) ? c : u_pos[d.x + c];
             if (limit < 0 || limit >= ctx_len_b) { report(st, RELAXKV_ERR_BAD_INDEX, KID_ATTN_SM100, limit, ctx_len_b); limit = 0; }
