@@ -37,6 +37,7 @@ constexpr float kRescaleThreshold = 8.0f;     // log2 units: rescale O only when
 constexpr int kBM = 128;                      // query rows per tile (TMEM lanes)
 constexpr int kBN = 128;                      // keys per context tile
 constexpr int kHalfBytes = 128 * 128;         // 128 rows x 64 bf16: one 128B-swizzled half tile
+constexpr int kPLo = 3;                        // P is handed over in two groups of 32 keys each: the first kPLo, the rest
 constexpr int kRing = 5;                      // K/V tile buffers, used in the order K0 V0 K1 V1 ...
 constexpr int kNoLimit = 0x7fffffff;          // causal limit of a row that nobody reads: no tile is masked for it
 constexpr int kPersistMaxTiles = 128;          // contexts up to this many key tiles take the persistent form
@@ -56,11 +57,52 @@ struct AttnSmem {
   static constexpr int kDynamic = kTotal + 1024;                // slack to align the base to 1024 B
 };
 
+// P of keys [32 C0, 32 C1) of a row's tile: p = 2^(s * scale - m), row sums, bf16 into TMEM over S.  The scaling and the sums use packed
+// fp32 pairs.  MAX: mx8 collects the maxima of the whole tile meanwhile (the maximum is an ALU instruction: it costs nothing
+// beside the exponentials, which leave seven of eight issue slots free).
+template <int C0, int C1, bool MAX>
+__device__ __forceinline__ void softmax_keys(uint32_t t_s, const uint32_t* s, float scale_log2, float neg_m, float* mx8, float& zs0,
+                                             float& zs1, float& zs2, float& zs3) {
+  constexpr int kGroups = 4 * (C1 - C0);                      // groups of eight exponentials
+  constexpr int kMaxPerGroup = (kBN + 2 * kGroups - 1) / (2 * kGroups) * 2;      // values each of them adds to the maxima
+#pragma unroll
+  for (int c = C0; c < C1; ++c) {
+    uint32_t pk[16];
+#pragma unroll
+    for (int i = 0; i < 32; i += 8) {
+      float x[8], p[8];
+#pragma unroll
+      for (int e = 0; e < 8; e += 2)
+        fma2(x[e], x[e + 1], __uint_as_float(s[c * 32 + i + e]), __uint_as_float(s[c * 32 + i + e + 1]), scale_log2, scale_log2, neg_m, neg_m);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) p[e] = fast_exp2(x[e]);
+      add2(zs0, zs1, p[0], p[1]); add2(zs2, zs3, p[2], p[3]);
+      add2(zs0, zs1, p[4], p[5]); add2(zs2, zs3, p[6], p[7]);
+#pragma unroll
+      for (int e = 0; e < 8; e += 2) {
+        __nv_bfloat162 h = __floats2bfloat162_rn(p[e], p[e + 1]);
+        pk[(i + e) >> 1] = *reinterpret_cast<uint32_t*>(&h);
+      }
+      if (MAX) {
+        const int g0 = ((c - C0) * 4 + i / 8) * kMaxPerGroup;
+#pragma unroll
+        for (int e = 0; e < kMaxPerGroup && g0 + e < kBN; e += 2)
+          mx8[(e >> 1) & 7] = fmax3(mx8[(e >> 1) & 7], __uint_as_float(s[g0 + e]), __uint_as_float(s[g0 + e + 1]));
+      }
+    }
+    tmem_st16(t_s + c * 16, pk);
+  }
+}
+
 // One step of a query row's online softmax (thread = query row = TMEM lane): S_x(j) is read from TMEM, the keys
 // past the row's limit are masked on the tiles that straddle the staircase (col0 = index of the tile's first key),
 // the running maximum m and sum z are updated (O_x is rescaled only when the maximum grew by more than the
-// threshold), and P is written over S as bf16 in two column halves, each handed to the MMA warp (bar_p_lo,
+// threshold), and P is written over S as bf16 in two column groups, each handed to the MMA warp (bar_p_lo,
 // bar_p_hi) as soon as it is stored.
+// The step is a link of the chain S -> P -> P V -> next S that bounds the kernel (a step of both tiles took 3.08 k clk, of which
+// 2.93 k are one tile's chain, 1.70 k of them here), so the exponentials do not wait for the maximum: they are begun with the
+// reference of the tile before, and only if the maximum turns out to have grown by more than the threshold are they
+// done again.  Same decisions and bits as with the maximum first.
 template <int D>
 __device__ __forceinline__ void softmax_step(uint32_t t_s, uint32_t t_o, int col0, int limit, bool first, float scale_log2,
                                              float& m, float& z, uint32_t bar_p_lo, uint32_t bar_p_hi) {
@@ -73,29 +115,28 @@ __device__ __forceinline__ void softmax_step(uint32_t t_s, uint32_t t_o, int col
     for (int i = 0; i < kBN; ++i)
       if (col0 + i > limit) s[i] = 0xff800000u;              // -inf
   }
-  // row maximum: eight independent chains instead of one 128-deep dependency chain
-  float mx8[8];
+  float zs0 = 0.f, zs1 = 0.f, zs2 = 0.f, zs3 = 0.f;
+  float mx8[8];                         // eight independent chains instead of one 128-deep dependency chain
 #pragma unroll
-  for (int e = 0; e < 8; ++e) mx8[e] = __uint_as_float(s[e]);
-#pragma unroll
-  for (int i = 8; i + 16 <= kBN; i += 16) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) mx8[e] = fmax3(mx8[e], __uint_as_float(s[i + e]), __uint_as_float(s[i + 8 + e]));
-  }
-#pragma unroll
-  for (int e = 0; e < 8; ++e) mx8[e] = fmaxf(mx8[e], __uint_as_float(s[kBN - 8 + e]));
-  const float mx = fmaxf(fmaxf(fmaxf(mx8[0], mx8[1]), fmaxf(mx8[2], mx8[3])),
-                         fmaxf(fmaxf(mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7])));
-  const float m_new = mx * scale_log2;
+  for (int e = 0; e < 8; ++e) mx8[e] = -INFINITY;
+  auto row_max = [&]() {
+    return fmaxf(fmaxf(fmaxf(mx8[0], mx8[1]), fmaxf(mx8[2], mx8[3])), fmaxf(fmaxf(mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7]))) * scale_log2;
+  };
   if (first) {
-    m = fmaxf(m_new, -1.0e30f);           // a row whose first tile of this split is fully masked keeps a finite reference
+#pragma unroll
+    for (int i = 0; i < kBN; i += 2) mx8[(i >> 1) & 7] = fmax3(mx8[(i >> 1) & 7], __uint_as_float(s[i]), __uint_as_float(s[i + 1]));
+    m = fmaxf(row_max(), -1.0e30f);       // a row whose first tile of this split is fully masked keeps a finite reference
+    softmax_keys<0, kPLo, false>(t_s, s, scale_log2, -m, mx8, zs0, zs1, zs2, zs3);
   } else {
+    softmax_keys<0, kPLo, true>(t_s, s, scale_log2, -m, mx8, zs0, zs1, zs2, zs3);
+    const float m_new = row_max();
     // S_x(j) is complete, hence so is O_x += P_x V_{j-1}: O_x may be rescaled here
     const bool need = m_new > m + kRescaleThreshold;
     if (__any_sync(0xffffffffu, need)) {
       float alpha = 1.f;
       if (need) { alpha = fast_exp2(m - m_new); z *= alpha; m = m_new; }
-#pragma unroll
+      tmem_wait_st();
+#pragma unroll 1
       for (int c = 0; c < D / 32; ++c) {
         uint32_t o[32];
         tmem_ld32(t_o + c * 32, o);
@@ -104,39 +145,14 @@ __device__ __forceinline__ void softmax_step(uint32_t t_s, uint32_t t_o, int col
         for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
         tmem_st32(t_o + c * 32, o);
       }
-      tmem_wait_st();
+      zs0 = zs1 = zs2 = zs3 = 0.f;
+      softmax_keys<0, kPLo, false>(t_s, s, scale_log2, -m, mx8, zs0, zs1, zs2, zs3);
     }
   }
-  float zs0 = 0.f, zs1 = 0.f, zs2 = 0.f, zs3 = 0.f;
-  const float neg_m = -m;
-#pragma unroll
-  for (int c = 0; c < kBN / 32; ++c) {
-    uint32_t pk[16];
-#pragma unroll
-    for (int i = 0; i < 32; i += 8) {
-      // p = 2^(s * scale - m) for eight keys; the scaling and the row sums use packed fp32 pairs
-      float x[8], p[8];
-#pragma unroll
-      for (int e = 0; e < 8; e += 2)
-        fma2(x[e], x[e + 1], __uint_as_float(s[c * 32 + i + e]), __uint_as_float(s[c * 32 + i + e + 1]), scale_log2,
-             scale_log2, neg_m, neg_m);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) p[e] = fast_exp2(x[e]);
-      add2(zs0, zs1, p[0], p[1]); add2(zs2, zs3, p[2], p[3]);
-      add2(zs0, zs1, p[4], p[5]); add2(zs2, zs3, p[6], p[7]);
-#pragma unroll
-      for (int e = 0; e < 8; e += 2) {
-        __nv_bfloat162 h = __floats2bfloat162_rn(p[e], p[e + 1]);
-        pk[(i + e) >> 1] = *reinterpret_cast<uint32_t*>(&h);
-      }
-    }
-    tmem_st16(t_s + c * 16, pk);
-    if (c == kBN / 64 - 1) {          // first 64 keys done: hand them to the MMA warp early
-      tmem_wait_st();
-      tc_fence_before();
-      mbar_arrive(bar_p_lo);
-    }
-  }
+  tmem_wait_st();
+  tc_fence_before();
+  mbar_arrive(bar_p_lo);                  // the first keys are done: hand them to the MMA warp early
+  softmax_keys<kPLo, kBN / 32, false>(t_s, s, scale_log2, -m, mx8, zs0, zs1, zs2, zs3);
   z += (zs0 + zs1) + (zs2 + zs3);
   tmem_wait_st();
   tc_fence_before();
@@ -340,11 +356,12 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         const uint32_t v_lo = desc_lo(kv_smem + sv * L::kTileBytes, kHalfBytes);
         if (!mbar_wait(bar_pfull + 8 * x, par, abort_flag)) return false;
         tc_fence_after();
-        mma_ts_4steps(tmem_base + 256 + x * 128, tmem_base + x * 128, v_lo, desc_hi_sw128(1024), idesc_pv, acc);
+        mma_ts_steps<2 * kPLo>(tmem_base + 256 + x * 128, tmem_base + x * 128, v_lo, desc_hi_sw128(1024), idesc_pv, acc);
         // the second half of P arrives while the first half is being multiplied
         if (!mbar_wait(bar_pfull_hi + 8 * x, par, abort_flag)) return false;
         tc_fence_after();
-        mma_ts_4steps(tmem_base + 256 + x * 128, tmem_base + x * 128 + 32, v_lo + 512, desc_hi_sw128(1024), idesc_pv, 1u);
+        mma_ts_steps<8 - 2 * kPLo>(tmem_base + 256 + x * 128, tmem_base + x * 128 + 16 * kPLo, v_lo + 256 * kPLo, desc_hi_sw128(1024),
+                                   idesc_pv, 1u);
         return true;
       };
       // pair 0 = K_0 alone
@@ -773,10 +790,11 @@ attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
         const uint32_t v_lo = desc_lo(kv_smem + sv * L::kTileBytes, kHalfBytes);
         if (!mbar_wait(bar_pfull + 8 * x, par, abort_flag)) return false;
         tc_fence_after();
-        mma_ts_4steps(tmem_base + 256 + x * 128, tmem_base + x * 128, v_lo, desc_hi_sw128(1024), idesc_pv, acc);
+        mma_ts_steps<2 * kPLo>(tmem_base + 256 + x * 128, tmem_base + x * 128, v_lo, desc_hi_sw128(1024), idesc_pv, acc);
         if (!mbar_wait(bar_pfull_hi + 8 * x, par, abort_flag)) return false;
         tc_fence_after();
-        mma_ts_4steps(tmem_base + 256 + x * 128, tmem_base + x * 128 + 32, v_lo + 512, desc_hi_sw128(1024), idesc_pv, 1u);
+        mma_ts_steps<8 - 2 * kPLo>(tmem_base + 256 + x * 128, tmem_base + x * 128 + 16 * kPLo, v_lo + 256 * kPLo, desc_hi_sw128(1024),
+                                   idesc_pv, 1u);
         return true;
       };
       auto advance = [&]() {

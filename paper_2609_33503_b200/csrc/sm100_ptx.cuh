@@ -241,15 +241,24 @@ __device__ __forceinline__ void mma_ss_4steps(uint32_t d_tmem, uint32_t a_lo, ui
   "mov.b64 db, {tb, %3};\n\t"                                                                  \
   "tcgen05.mma.cta_group::1.kind::f16 [%0], [ta], db, %4, " #PRED ";\n\t"
 
-// D[tmem] (+)= A[tmem] * B[smem] for four K steps of 16: A advances 8 columns, B (MN-major, 128B swizzle)
+// D[tmem] (+)= A[tmem] * B[smem] for N = 2, 4 or 6 K steps of 16: A advances 8 columns, B (MN-major, 128B swizzle)
 // 2048 bytes per step.  acc_first = 0 makes the first MMA overwrite D.
-__device__ __forceinline__ void mma_ts_4steps(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi, uint32_t idesc,
-                                              uint32_t acc_first) {
-  asm volatile(
-      "{\n\t.reg .pred p0, p1;\n\t.reg .b32 ta, tb;\n\t.reg .b64 db;\n\t"
-      "setp.ne.b32 p0, %5, 0;\n\tsetp.eq.b32 p1, 0, 0;\n\t"
-      RELAXKV_MMA_TS_STEP(0, 0, p0) RELAXKV_MMA_TS_STEP(8, 128, p1) RELAXKV_MMA_TS_STEP(16, 256, p1) RELAXKV_MMA_TS_STEP(24, 384, p1)
-      "}" ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"(acc_first) : "memory");
+template <int N>
+__device__ __forceinline__ void mma_ts_steps(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi, uint32_t idesc,
+                                             uint32_t acc_first) {
+  static_assert(N == 2 || N == 4 || N == 6, "K steps");
+#define RELAXKV_MMA_TS_HEAD                                                  \
+  "{\n\t.reg .pred p0, p1;\n\t.reg .b32 ta, tb;\n\t.reg .b64 db;\n\t"    \
+  "setp.ne.b32 p0, %5, 0;\n\tsetp.eq.b32 p1, 0, 0;\n\t"                    \
+  RELAXKV_MMA_TS_STEP(0, 0, p0) RELAXKV_MMA_TS_STEP(8, 128, p1)
+#define RELAXKV_MMA_TS_ARGS "}" ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"(acc_first) : "memory"
+  if (N == 2) asm volatile(RELAXKV_MMA_TS_HEAD RELAXKV_MMA_TS_ARGS);
+  if (N == 4) asm volatile(RELAXKV_MMA_TS_HEAD RELAXKV_MMA_TS_STEP(16, 256, p1) RELAXKV_MMA_TS_STEP(24, 384, p1) RELAXKV_MMA_TS_ARGS);
+  if (N == 6)
+    asm volatile(RELAXKV_MMA_TS_HEAD RELAXKV_MMA_TS_STEP(16, 256, p1) RELAXKV_MMA_TS_STEP(24, 384, p1)
+                 RELAXKV_MMA_TS_STEP(32, 512, p1) RELAXKV_MMA_TS_STEP(40, 640, p1) RELAXKV_MMA_TS_ARGS);
+#undef RELAXKV_MMA_TS_HEAD
+#undef RELAXKV_MMA_TS_ARGS
 }
 
 // ---- CTA pairs (cta_group::2): one MMA instruction drives the tensor cores of two SMs ----------------------
