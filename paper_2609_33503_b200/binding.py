@@ -109,18 +109,38 @@ def _check(status: int, where: str) -> None:
         raise RelaxKVError(status, where)
 
 
+_i32_types = {}                    # array types by length: making one is most of what a short array costs
+
+
 def _i32(xs: Optional[Sequence[int]]):
     if xs is None:
         return None
-    return (ctypes.c_int32 * len(xs))(*map(int, xs))
+    n = len(xs)
+    kind = _i32_types.get(n)
+    if kind is None:
+        kind = ctypes.c_int32 * n
+        if n <= 64:                # (the most requests of a call; longer lists are refused by the library)
+            _i32_types[n] = kind
+    return kind(*map(int, xs))
 
 
-def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
-    return None if t is None else t.data_ptr()
+def _ptr(t) -> Optional[int]:
+    """Address of a tensor; an address (int) stands for itself."""
+    return t if t is None or type(t) is int else t.data_ptr()
 
 
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)     # the handle without a Stream object around it
 _current_device = getattr(torch._C, "_cuda_getDevice", None)
+_raw_synchronize = getattr(torch._C, "_cuda_synchronize", None)
+
+
+def synchronize(device: torch.device) -> None:
+    """torch.cuda.synchronize; without its change of device where the device is the current one."""
+    if (_raw_synchronize is not None and _current_device is not None and torch.cuda.is_initialized()
+            and (device.index is None or device.index == _current_device())):
+        _raw_synchronize()
+    else:
+        torch.cuda.synchronize(device)
 
 
 def _stream(stream) -> int:

@@ -60,7 +60,7 @@ class RepairSession:
     def counts(self):
         """(|U_b| per request, |R_{l,b}| as [n_layers][n_req]) - synchronises the device."""
         if self._counts is None:
-            torch.cuda.synchronize(self.device)
+            B.synchronize(self.device)
             nb = self.shape.n_req
             c = self.counts_pinned.tolist()
             self._counts = (c[:nb], [c[nb + l * nb: nb + (l + 1) * nb] for l in range(self.n_layers)])
@@ -70,18 +70,23 @@ class RepairSession:
         nb = self.shape.n_req
         return self.r_cu[layer * nb: layer * nb + nb + 1]
 
+    def _r_cu_ptr(self, layer: int) -> int:
+        """Address of r_cu_layer(layer): a tensor slice costs the host 1 to 3 us, as much as marshalling the rest of a call."""
+        assert 0 <= layer < self.n_layers
+        return self.r_cu.data_ptr() + 4 * layer * self.shape.n_req
+
     # -- (b) repair -----------------------------------------------------------------------------
     def attention(self, layer: int, cache: B.CacheView, q_new, k_new, v_new, out, max_targets, max_ctx,
                   mode: int = B.CTX_UNION, lse_out=None, stream=None, simt: bool = False) -> None:
         fn = B.relaxkv_sparse_ctx_attention_simt if simt else B.relaxkv_sparse_ctx_attention
         fn(self.shape, mode, cache, q_new, k_new, v_new, self.u_pos, self.u_cu, self.r_rank,
-           self.r_cu_layer(layer), max_targets, max_ctx, out, self.workspace, lse_out=lse_out, stream=stream)
+           self._r_cu_ptr(layer), max_targets, max_ctx, out, self.workspace, lse_out=lse_out, stream=stream)
 
     def scatter(self, layer: int, cache: B.CacheView, k_new, v_new, max_targets, stream=None) -> None:
         B.relaxkv_scatter_kv(self.shape, cache, k_new, v_new, self.u_pos, self.u_cu, self.r_rank,
-                             self.r_cu_layer(layer), max_targets, stream=stream)
+                             self._r_cu_ptr(layer), max_targets, stream=stream)
 
     def gather(self, layer: int, cache: B.CacheView, k_new, v_new, max_ctx, k_ctx_out, v_ctx_out,
                mode: int = B.CTX_UNION, stream=None) -> None:
         B.relaxkv_gather_kv(self.shape, mode, cache, k_new, v_new, self.u_pos, self.u_cu, self.r_rank,
-                            self.r_cu_layer(layer), max_ctx, k_ctx_out, v_ctx_out, stream=stream)
+                            self._r_cu_ptr(layer), max_ctx, k_ctx_out, v_ctx_out, stream=stream)
