@@ -258,8 +258,8 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const uint32_t bar0 = base + L::kBar;
   const uint32_t bar_q = bar0;
   const uint32_t bar_sfull = bar0 + 8;          // [2]
-  const uint32_t bar_pfull = bar0 + 24;         // [2] first 64 keys of P ready
-  const uint32_t bar_pfull_hi = bar0 + 40;      // [2] last 64 keys of P ready
+  const uint32_t bar_pfull = bar0 + 24;         // [2] first 32 kPLo keys of P ready
+  const uint32_t bar_pfull_hi = bar0 + 40;      // [2] the other keys of P ready
   const uint32_t bar_ofinal = bar0 + 56;        // [2]
   const uint32_t bar_full = bar0 + 72;          // [kPairBars] pair p = (V_{p-1}, K_p) has landed
   const uint32_t bar_empty = bar_full + 8 * L::kPairBars;   // [kPairBars] pair p has been consumed by both tiles

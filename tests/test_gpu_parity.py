@@ -401,6 +401,30 @@ def test_attention_call_replays_from_a_cuda_graph(persistent):
         s.shape.set_tuning()
 
 
+@pytest.mark.parametrize("shape", ["five_heads", "four_heads", "head_dim_64"])
+@pytest.mark.parametrize("growth", [3.0, 30.0])
+def test_row_maxima_that_grow_along_the_context(shape, growth):
+    """Keys that grow along the context: the row maxima outgrow the reference the exponentials of a tile were begun with, once
+    or several times per row, so that P is computed again and O rescaled (at 3 a few rows of a warp, at 30 all of them).  One
+    block per tile pair, the persistent form and a context split.  Values at a quarter: a row that one key dominates takes its value, of up
+    to 4.5, rounded twice (P and O, 2^-9 each) = 0.018, which is the tolerance itself."""
+    w = {"five_heads": inputs.scaled_down(inputs.qwen14b_32k("literal"), (1500,), (5,), n_layers=1, chunk=64),
+         "four_heads": small_llama(n_layers=1, ctx=(1300, 700), q=(8, 8)), "head_dim_64": inputs.tiny()}[shape].replace(ratio=0.5)
+    case = Case(w)
+    f = case.fresh[0]
+    n = f.k_new.shape[0]
+    ramp = torch.linspace(1.0, growth, n, device=f.k_new.device)[:, None, None]
+    f.k_new = (f.k_new.float() * ramp).to(torch.bfloat16)
+    f.v_new = (f.v_new.float() * 0.25).to(torch.bfloat16)
+    s = case.make_session()
+    s.build_active_sets(case.anchors_tensor())
+    for tuning in (dict(attention_ctx_splits=1, attention_persistent=2), dict(attention_ctx_splits=1, attention_persistent=1, attention_grid_blocks=3),
+                   dict(attention_ctx_splits=2)):
+        s.shape.set_tuning(**tuning)
+        out, lse = run_attention(case, s, 0, B().CTX_UNION, simt=False)
+        check_attention(case, 0, out, lse, False)
+
+
 def test_attention_orders_agree_and_is_deterministic(case):
     """Update-then-attend from the cache equals mix-then-attend (Algorithm 1's order), bit for bit;
     two runs give identical bits."""
