@@ -72,6 +72,7 @@ class RepairSession:
 
     def _r_cu_ptr(self, layer: int) -> int:
         """Address of r_cu_layer(layer): a tensor slice costs the host 1 to 3 us, as much as marshalling the rest of a call."""
+        layer = int(layer)                      # (numpy and torch integers index a tensor, too)
         assert 0 <= layer < self.n_layers
         return self.r_cu.data_ptr() + 4 * layer * self.shape.n_req
 

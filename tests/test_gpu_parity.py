@@ -425,6 +425,22 @@ def test_row_maxima_that_grow_along_the_context(shape, growth):
         check_attention(case, 0, out, lse, False)
 
 
+@pytest.mark.parametrize("kind", [np.int64, np.int32, torch.tensor], ids=["int64", "int32", "tensor"])
+def test_a_layer_is_any_integer(kind):
+    """The layer of a session's calls may be a numpy or torch integer, as an index of a tensor may."""
+    case = Case(small_llama())
+    s = case.make_session()
+    s.build_active_sets(case.anchors_tensor())
+    l = case.w.n_layers - 1
+    ref, _ = run_attention(case, s, l, B().CTX_UNION, simt=False)
+    f = case.fresh[l]
+    out = torch.zeros_like(ref)
+    s.attention(kind(l), case.cache_views()[l], f.q_new, f.k_new, f.v_new, out, case.max_targets(l), case.max_ctx())
+    s.scatter(kind(l), case.cache_views()[l], f.k_new, f.v_new, case.max_targets(l))
+    assert_status_ok()
+    assert torch.equal(out, ref)
+
+
 def test_attention_orders_agree_and_is_deterministic(case):
     """Update-then-attend from the cache equals mix-then-attend (Algorithm 1's order), bit for bit;
     two runs give identical bits."""
