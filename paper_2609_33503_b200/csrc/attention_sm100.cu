@@ -417,9 +417,10 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     const int t_local = row / G, j_head = row - t_local * G;
     const bool row_valid = (row < tile_targets * G) && (t_local < n_valid[x]);
     const int rho_t = rho0 + x * tile_targets + t_local;
-    // Rows without a target (125 of 128 rows are used with five heads per KV head) and rows of an empty context see every key: what
-    // they hold is not used, and a limit below the tile sends their whole warp through the masking of every tile, 1.0 k clk of
-    // a 3.5 k step (12 layers of 40 / 8 heads at 32 K, repaired: 40.8 -> 37.4 ms; every row used, 32 / 8 heads: 8.48 -> 8.43).
+    // Rows without a target (125 of 128 rows are used with five heads per KV head) and rows of an empty context see every key: what they
+    // hold is not stored (an empty context's row is written as zeros), and a limit below the tile sends their whole warp through the
+    // masking of every tile, 1.0 k clk of a 3.5 k step (12 layers of 40 / 8 heads at 32 K, repaired: 40.7 -> 37.3 ms; every row used,
+    // 32 / 8 heads at 8 K: 8.42 -> 8.37).
     int limit = kNoLimit;
     bool row_empty = false;                                     // explicit lists: a target that sees no context entry
     if (row_valid) {
@@ -474,7 +475,8 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                                                           __uint_as_float(o[i + 2 * e + 1]) * inv);
                 w[e] = *reinterpret_cast<uint32_t*>(&h2);
               }
-              *reinterpret_cast<uint4*>(optr + c * 32 + i) = make_uint4(w[0], w[1], w[2], w[3]);
+              // a row of an empty context is zero whatever the keys gave it (0 x NaN is not)
+              *reinterpret_cast<uint4*>(optr + c * 32 + i) = row_empty ? make_uint4(0, 0, 0, 0) : make_uint4(w[0], w[1], w[2], w[3]);
             }
           }
         }
@@ -986,7 +988,7 @@ attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
                 __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(o[i + 2 * e]) * inv, __uint_as_float(o[i + 2 * e + 1]) * inv);
                 w[e] = *reinterpret_cast<uint32_t*>(&h2);
               }
-              *reinterpret_cast<uint4*>(optr + cc * 32 + i) = make_uint4(w[0], w[1], w[2], w[3]);
+              *reinterpret_cast<uint4*>(optr + cc * 32 + i) = row_empty ? make_uint4(0, 0, 0, 0) : make_uint4(w[0], w[1], w[2], w[3]);
             }
           }
         }

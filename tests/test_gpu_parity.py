@@ -677,6 +677,31 @@ def test_controlled_configurations_match_oracle(case, variant, persistent):
         np.testing.assert_array_equal(v2_b[case.ctx_cu[b]:case.ctx_cu[b + 1]], rv)
 
 
+@pytest.mark.parametrize("bad", ["later", "next", "first"])
+@pytest.mark.parametrize("tuning", [dict(attention_ctx_splits=1, attention_persistent=2), dict(attention_ctx_splits=1, attention_persistent=1),
+                                    dict(attention_ctx_splits=2)], ids=["one_shot", "persistent", "split"])
+def test_targets_before_their_context_are_zero_whatever_the_keys(tuning, bad):
+    """A target that sees no context entry is a zero row with lse = -inf, also where the key tiles its query tile walks hold NaN or
+    infinities: in entries past every target of the request, in the next request's rows behind them, or in the very first entry."""
+    case = Case(small_llama(n_layers=1, ctx=(700, 400), q=(8, 8)))
+    s = case.make_session()
+    s.shape.set_tuning(**tuning)
+    ctx_lists = [np.arange(100, 700, 3, dtype=np.int32), np.arange(5, 400, 2, dtype=np.int32)]       # 200 = 1.6 tiles, 198 entries
+    early = [0, 17, 60, 99]
+    tgt_lists = [np.array(early if bad == "first" else early + [250, 401, 652], dtype=np.int32), np.array([0, 6, 300], dtype=np.int32)]
+    rows = {"later": [655, 658, 697], "next": [700 + 5, 700 + 7], "first": [100]}[bad]
+    for i, r in enumerate(rows):
+        case.k_cache[0][r] = float("nan") if i % 2 == 0 else float("inf")
+    out, lse, fresh, tcu = _run_lists(case, s, 0, ctx_lists, tgt_lists)
+    assert torch.all(out[:len(early)] == 0) and torch.all(torch.isneginf(lse[:, :len(early)]))
+    if bad != "first":                  # the rows that see something: entries past their position do not count
+        n = int(tcu[1])
+        qn, kn, vn = (inputs.bf16_bits(t[:n]) for t in fresh)
+        ref, _ = orc.list_attention(case.req_k(0, 0), case.req_v(0, 0), qn, kn, vn, ctx_lists[0], tgt_lists[0], case.scale)
+        mx, mean = attention_errors(out[:n], ref)
+        assert mx <= MAX_ABS and mean <= MEAN_ABS, (mx, mean)
+
+
 def test_mean_scores_and_global_topk(case):
     """g = mean over layers of the normalised scores (fixed summation order), then top-m of g."""
     w = case.w
