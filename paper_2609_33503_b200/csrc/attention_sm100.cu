@@ -37,7 +37,10 @@ constexpr float kRescaleThreshold = 8.0f;     // log2 units: rescale O only when
 constexpr int kBM = 128;                      // query rows per tile (TMEM lanes)
 constexpr int kBN = 128;                      // keys per context tile
 constexpr int kHalfBytes = 128 * 128;         // 128 rows x 64 bf16: one 128B-swizzled half tile
-constexpr int kPLo = 3;                        // P is handed over in two groups of 32 keys each: the first kPLo, the rest
+// P of a tile is handed to the MMA warp in two groups: its first 32 * kPLo keys, then the rest.  96 + 32 against 64 + 64 keys, us per call
+// of one layer with every entry repaired: 24 K entries, 40 / 8 heads 5350 / 5440, 32 / 8 heads of dim 64 3155 / 3150; 6 K entries, 32 / 8
+// heads of dim 64 212 / 214: one value for both head dims.
+constexpr int kPLo = 3;
 constexpr int kRing = 5;                      // K/V tile buffers, used in the order K0 V0 K1 V1 ...
 constexpr int kNoLimit = 0x7fffffff;          // causal limit of a row that nobody reads: no tile is masked for it
 constexpr int kPersistMaxTiles = 128;          // contexts up to this many key tiles take the persistent form
@@ -58,13 +61,10 @@ struct AttnSmem {
 };
 
 // P of keys [32 C0, 32 C1) of a row's tile: p = 2^(s * scale - m), row sums, bf16 into TMEM over S.  The scaling and the sums use packed
-// fp32 pairs.  MAX: mx8 collects the maxima of the whole tile meanwhile (the maximum is an ALU instruction: it costs nothing
-// beside the exponentials, which leave seven of eight issue slots free).
-template <int C0, int C1, bool MAX>
-__device__ __forceinline__ void softmax_keys(uint32_t t_s, const uint32_t* s, float scale_log2, float neg_m, float* mx8, float& zs0,
-                                             float& zs1, float& zs2, float& zs3) {
-  constexpr int kGroups = 4 * (C1 - C0);                      // groups of eight exponentials
-  constexpr int kMaxPerGroup = (kBN + 2 * kGroups - 1) / (2 * kGroups) * 2;      // values each of them adds to the maxima
+// fp32 pairs.
+template <int C0, int C1>
+__device__ __forceinline__ void softmax_keys(uint32_t t_s, const uint32_t* s, float scale_log2, float neg_m, float& zs0, float& zs1,
+                                             float& zs2, float& zs3) {
 #pragma unroll
   for (int c = C0; c < C1; ++c) {
     uint32_t pk[16];
@@ -83,76 +83,63 @@ __device__ __forceinline__ void softmax_keys(uint32_t t_s, const uint32_t* s, fl
         __nv_bfloat162 h = __floats2bfloat162_rn(p[e], p[e + 1]);
         pk[(i + e) >> 1] = *reinterpret_cast<uint32_t*>(&h);
       }
-      if (MAX) {
-        const int g0 = ((c - C0) * 4 + i / 8) * kMaxPerGroup;
-#pragma unroll
-        for (int e = 0; e < kMaxPerGroup && g0 + e < kBN; e += 2)
-          mx8[(e >> 1) & 7] = fmax3(mx8[(e >> 1) & 7], __uint_as_float(s[g0 + e]), __uint_as_float(s[g0 + e + 1]));
-      }
     }
     tmem_st16(t_s + c * 16, pk);
   }
 }
 
 // One step of a query row's online softmax (thread = query row = TMEM lane): S_x(j) is read from TMEM, the keys
-// past the row's limit are masked on the tiles that straddle the staircase (col0 = index of the tile's first key),
+// past the row's limit (counted from the tile's first key) are masked on the tiles that straddle the staircase,
 // the running maximum m and sum z are updated (O_x is rescaled only when the maximum grew by more than the
 // threshold), and P is written over S as bf16 in two column groups, each handed to the MMA warp (bar_p_lo,
-// bar_p_hi) as soon as it is stored.
-// The step is a link of the chain S -> P -> P V -> next S that bounds the kernel (a step of both tiles took 3.08 k clk, of which
-// 2.93 k are one tile's chain, 1.70 k of them here), so the exponentials do not wait for the maximum: they are begun with the
-// reference of the tile before, and only if the maximum turns out to have grown by more than the threshold are they
-// done again.  Same decisions and bits as with the maximum first.
+// bar_p_hi) as soon as it is stored.  m starts at -1e30, so that a row whose first tile is fully masked keeps a finite reference.
+// The step is a link of the chain S -> P -> P V -> next S that bounds the kernel.  The maximum comes first.  Exponentials begun with the
+// tile before's reference are no faster where both tiles of a pair keep the SM busy (8 K stack 8.12 ms either way, 12 layers of 40 / 8
+// heads at 32 K 35.8; ragged query passes of one to 25 rows per tile 1 to 3 % faster), and where maxima grow along the context they have
+// to be done again, four warps waiting for the slowest of them (6 K entries, 32 / 8 heads, keys that grow thirtyfold: 400 us against 325
+// with the maximum first; of dim 64 333 against 230).
 template <int D>
-__device__ __forceinline__ void softmax_step(uint32_t t_s, uint32_t t_o, int col0, int limit, bool first, float scale_log2,
+__device__ __forceinline__ void softmax_step(uint32_t t_s, uint32_t t_o, int limit, bool first, float scale_log2,
                                              float& m, float& z, uint32_t bar_p_lo, uint32_t bar_p_hi) {
   uint32_t s[kBN];
 #pragma unroll
   for (int c = 0; c < kBN / 32; ++c) tmem_ld32(t_s + c * 32, &s[c * 32]);
   tmem_wait_ld();
-  if (col0 + kBN - 1 > limit) {
+  if (limit < kBN - 1) {
 #pragma unroll
     for (int i = 0; i < kBN; ++i)
-      if (col0 + i > limit) s[i] = 0xff800000u;              // -inf
+      if (i > limit) s[i] = 0xff800000u;                      // -inf
   }
-  float zs0 = 0.f, zs1 = 0.f, zs2 = 0.f, zs3 = 0.f;
   float mx8[8];                         // eight independent chains instead of one 128-deep dependency chain
 #pragma unroll
-  for (int e = 0; e < 8; ++e) mx8[e] = -INFINITY;
-  auto row_max = [&]() {
-    return fmaxf(fmaxf(fmaxf(mx8[0], mx8[1]), fmaxf(mx8[2], mx8[3])), fmaxf(fmaxf(mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7]))) * scale_log2;
-  };
-  if (first) {
+  for (int e = 0; e < 8; ++e) mx8[e] = fmaxf(__uint_as_float(s[2 * e]), __uint_as_float(s[2 * e + 1]));
 #pragma unroll
-    for (int i = 0; i < kBN; i += 2) mx8[(i >> 1) & 7] = fmax3(mx8[(i >> 1) & 7], __uint_as_float(s[i]), __uint_as_float(s[i + 1]));
-    m = fmaxf(row_max(), -1.0e30f);       // a row whose first tile of this split is fully masked keeps a finite reference
-    softmax_keys<0, kPLo, false>(t_s, s, scale_log2, -m, mx8, zs0, zs1, zs2, zs3);
-  } else {
-    softmax_keys<0, kPLo, true>(t_s, s, scale_log2, -m, mx8, zs0, zs1, zs2, zs3);
-    const float m_new = row_max();
-    // S_x(j) is complete, hence so is O_x += P_x V_{j-1}: O_x may be rescaled here
-    const bool need = m_new > m + kRescaleThreshold;
-    if (__any_sync(0xffffffffu, need)) {
-      float alpha = 1.f;
-      if (need) { alpha = fast_exp2(m - m_new); z *= alpha; m = m_new; }
-      tmem_wait_st();
+  for (int i = 16; i < kBN; i += 2) mx8[(i >> 1) & 7] = fmax3(mx8[(i >> 1) & 7], __uint_as_float(s[i]), __uint_as_float(s[i + 1]));
+  const float m_new =
+      fmax3(fmax3(mx8[0], mx8[1], mx8[2]), fmax3(mx8[3], mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7])) * scale_log2;
+  const float m_old = m;
+  const bool need = m_new > m + kRescaleThreshold;
+  if (need) m = m_new;
+  // S_x(j) is complete, hence so is O_x += P_x V_{j-1}: O_x may be rescaled here (nothing lies in it before the first tile)
+  if (__any_sync(0xffffffffu, need) && !first) {
+    const float alpha = fast_exp2(m_old - m);
+    z *= alpha;
 #pragma unroll 1
-      for (int c = 0; c < D / 32; ++c) {
-        uint32_t o[32];
-        tmem_ld32(t_o + c * 32, o);
-        tmem_wait_ld();
+    for (int c = 0; c < D / 32; ++c) {
+      uint32_t o[32];
+      tmem_ld32(t_o + c * 32, o);
+      tmem_wait_ld();
 #pragma unroll
-        for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-        tmem_st32(t_o + c * 32, o);
-      }
-      zs0 = zs1 = zs2 = zs3 = 0.f;
-      softmax_keys<0, kPLo, false>(t_s, s, scale_log2, -m, mx8, zs0, zs1, zs2, zs3);
+      for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+      tmem_st32(t_o + c * 32, o);
     }
   }
+  float zs0 = 0.f, zs1 = 0.f, zs2 = 0.f, zs3 = 0.f;
+  softmax_keys<0, kPLo>(t_s, s, scale_log2, -m, zs0, zs1, zs2, zs3);
   tmem_wait_st();
   tc_fence_before();
   mbar_arrive(bar_p_lo);                  // the first keys are done: hand them to the MMA warp early
-  softmax_keys<kPLo, kBN / 32, false>(t_s, s, scale_log2, -m, mx8, zs0, zs1, zs2, zs3);
+  softmax_keys<kPLo, kBN / 32>(t_s, s, scale_log2, -m, zs0, zs1, zs2, zs3);
   z += (zs0 + zs1) + (zs2 + zs3);
   tmem_wait_st();
   tc_fence_before();
@@ -357,7 +344,7 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         if (!mbar_wait(bar_pfull + 8 * x, par, abort_flag)) return false;
         tc_fence_after();
         mma_ts_steps<2 * kPLo>(tmem_base + 256 + x * 128, tmem_base + x * 128, v_lo, desc_hi_sw128(1024), idesc_pv, acc);
-        // the second half of P arrives while the first half is being multiplied
+        // the last keys of P arrive while the first 32 * kPLo are being multiplied
         if (!mbar_wait(bar_pfull_hi + 8 * x, par, abort_flag)) return false;
         tc_fence_after();
         mma_ts_steps<8 - 2 * kPLo>(tmem_base + 256 + x * 128, tmem_base + x * 128 + 16 * kPLo, v_lo + 256 * kPLo, desc_hi_sw128(1024),
@@ -439,14 +426,15 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     const uint32_t t_s = lane_base + x * 128, t_o = lane_base + 256 + x * 128;
     const uint32_t my_sfull = bar_sfull + 8 * x, my_pfull = bar_pfull + 8 * x;
     const int my_n = n_my[x];
-    float m = -INFINITY, z = 0.f;
+    limit -= j0 * kBN;                                          // counted from the split's first tile
+    float m = -1.0e30f, z = 0.f;
     bool ok = true;
     for (int j = 0; j < my_n; ++j) {
       ok = mbar_wait(my_sfull, j & 1, abort_flag);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
-      softmax_step<D>(t_s, t_o, (j0 + j) * kBN, limit, j == 0, scale_log2, m, z, my_pfull, bar_pfull_hi + 8 * x);
+      softmax_step<D>(t_s, t_o, limit - j * kBN, j == 0, scale_log2, m, z, my_pfull, bar_pfull_hi + 8 * x);
     }
     if (ok && my_n > 0) {
       ok = mbar_wait(bar_ofinal + 8 * x, 0, abort_flag);
@@ -947,13 +935,13 @@ attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
           }
         }
       }
-      float m = -INFINITY, z = 0.f;
+      float m = -1.0e30f, z = 0.f;
       for (int j = 0; j < my_n; ++j) {
         ok = mbar_wait(my_sfull, (ph + (uint32_t)j) & 1u, abort_flag);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         tc_fence_after();
-        softmax_step<D>(t_s, t_o, j * kBN, limit, j == 0, scale_log2, m, z, my_pfull, bar_pfull_hi + 8 * x);
+        softmax_step<D>(t_s, t_o, limit - j * kBN, j == 0, scale_log2, m, z, my_pfull, bar_pfull_hi + 8 * x);
       }
       if (!ok) break;
       // the next item's record (shown long ago) and this thread's row of it: the load travels under the epilogue

@@ -404,9 +404,8 @@ def test_attention_call_replays_from_a_cuda_graph(persistent):
 @pytest.mark.parametrize("shape", ["five_heads", "four_heads", "head_dim_64"])
 @pytest.mark.parametrize("growth", [3.0, 30.0])
 def test_row_maxima_that_grow_along_the_context(shape, growth):
-    """Keys that grow along the context: the row maxima outgrow the reference the exponentials of a tile were begun with, once
-    or several times per row, so that P is computed again and O rescaled (at 3 a few rows of a warp, at 30 all of them).  One
-    block per tile pair, the persistent form and a context split.  Values at a quarter: a row that one key dominates takes its value, of up
+    """Keys that grow along the context: the row maxima outgrow the reference of the tiles before, once or several times per row, so that
+    O is rescaled (at 3 a few rows of a warp, at 30 all of them).  One block per tile pair, the persistent form and a context split.  Values at a quarter: a row that one key dominates takes its value, of up
     to 4.5, rounded twice (P and O, 2^-9 each) = 0.018, which is the tolerance itself."""
     w = {"five_heads": inputs.scaled_down(inputs.qwen14b_32k("literal"), (1500,), (5,), n_layers=1, chunk=64),
          "four_heads": small_llama(n_layers=1, ctx=(1300, 700), q=(8, 8)), "head_dim_64": inputs.tiny()}[shape].replace(ratio=0.5)
@@ -423,6 +422,37 @@ def test_row_maxima_that_grow_along_the_context(shape, growth):
         s.shape.set_tuning(**tuning)
         out, lse = run_attention(case, s, 0, B().CTX_UNION, simt=False)
         check_attention(case, 0, out, lse, False)
+
+
+def test_row_maxima_that_grow_do_not_cost_the_exponentials_twice():
+    """One layer of 8 K tokens (dim 64, where the exponential unit bounds the step) with keys that grow thirtyfold along the context
+    against keys that do not.  Rescaling O in most steps costs 9 %; exponentials done again besides cost 56 %: the bound lies between."""
+    g = torch.Generator(device="cuda").manual_seed(1)
+    rnd = lambda n, h: torch.randn(n, h, 64, device="cuda", generator=g).to(torch.bfloat16)
+    from paper_2609_33503_b200.pipeline import RepairSession
+    n = 6144
+    s = RepairSession(32, 8, 64, [8192], [8], 1, [n])
+    s.build_active_sets(torch.randperm(8192, device="cuda", generator=g)[:n].sort().values.to(torch.int32).view(1, n).contiguous())
+    view = B().CacheView(rnd(8192, 8), rnd(8192, 8), [0])
+    q, k, v = rnd(n, 32), rnd(n, 8), rnd(n, 8)
+    grown = (k.float() * torch.linspace(1.0, 30.0, n, device="cuda")[:, None, None]).to(torch.bfloat16)
+    out = torch.empty_like(q)
+
+    def us(keys, reps=20):
+        t = []
+        for _ in range(2):
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            e[0].record()
+            for _ in range(reps):
+                s.attention(0, view, q, keys, v, out, [n], [n])
+            e[1].record()
+            torch.cuda.synchronize()
+            t.append(e[0].elapsed_time(e[1]) / reps * 1e3)
+        return t[-1]
+
+    ratio = sorted(us(grown) / us(k) for _ in range(7))[3]
+    assert_status_ok()
+    assert ratio < 1.3, ratio
 
 
 @pytest.mark.parametrize("kind", [np.int64, np.int32, torch.tensor], ids=["int64", "int32", "tensor"])
