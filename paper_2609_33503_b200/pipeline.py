@@ -4,6 +4,7 @@ step runs in the kernels behind `binding`.
 """
 from __future__ import annotations
 
+import operator
 from typing import List, Optional, Sequence
 
 import torch
@@ -72,8 +73,9 @@ class RepairSession:
 
     def _r_cu_ptr(self, layer: int) -> int:
         """Address of r_cu_layer(layer): a tensor slice costs the host 1 to 3 us, as much as marshalling the rest of a call."""
-        layer = int(layer)                      # (numpy and torch integers index a tensor, too)
-        assert 0 <= layer < self.n_layers
+        layer = operator.index(layer)           # numpy and torch integers, as an index of a tensor; nothing else
+        if not 0 <= layer < self.n_layers:
+            raise B.RelaxKVError(B.ERR_INVALID_ARG, f"layer {layer} of {self.n_layers}")
         return self.r_cu.data_ptr() + 4 * layer * self.shape.n_req
 
     # -- (b) repair -----------------------------------------------------------------------------

@@ -5,9 +5,12 @@ import os
 import random
 import re
 
+import numpy as np
 import pytest
+import torch
 
 from paper_2609_33503_b200 import binding as B
+from paper_2609_33503_b200.pipeline import RepairSession
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 GOLDEN = os.path.join(os.path.dirname(__file__), "golden")
@@ -164,6 +167,54 @@ def test_chained_launch_switch_is_host_state_only():
     assert B.relaxkv_set_chained_launch(False) is False
     assert B.relaxkv_set_chained_launch(True) is False
     assert B.relaxkv_set_chained_launch(True) is True
+
+
+class _AnyCall:
+    """In the place of the library: every entry point notes its arguments and reports success."""
+
+    def __init__(self):
+        self.calls = []
+
+    def __getattr__(self, name):
+        return lambda *args: self.calls.append((name, args)) or 0
+
+
+def _host_session(monkeypatch, n_layers=3, n_req=2):
+    """A session's bookkeeping without its device buffers, over a library that launches nothing."""
+    lib = _AnyCall()
+    monkeypatch.setattr(B, "_lib", lib)
+    monkeypatch.setattr(B, "_stream", lambda stream: 0)
+    monkeypatch.setattr(B, "status_string", lambda status: "refused")
+    t = lambda n: torch.zeros(n, dtype=torch.int32)
+    s = object.__new__(RepairSession)
+    s.shape, s.n_layers = B.Shape(8, 2, 128, [64] * n_req, [4] * n_req), n_layers
+    s.u_pos, s.u_cu, s.r_rank, s.workspace = t(64), t(n_req + 1), t(64), t(64)
+    s.r_cu = torch.arange(n_layers * n_req + 1, dtype=torch.int32)
+    rows = torch.zeros(4, 8, 128, dtype=torch.bfloat16)
+    cache = B.CacheView(torch.zeros(128, 2, 128, dtype=torch.bfloat16), torch.zeros(128, 2, 128, dtype=torch.bfloat16), [0, 64])
+    calls = {"relaxkv_sparse_ctx_attention": lambda l: s.attention(l, cache, rows, rows, rows, rows, [2, 2], [4, 4]),
+             "relaxkv_scatter_kv": lambda l: s.scatter(l, cache, rows, rows, [2, 2]),
+             "relaxkv_gather_kv": lambda l: s.gather(l, cache, rows, rows, [4, 4], rows, rows)}
+    return s, lib, calls
+
+
+@pytest.mark.parametrize("name", ["relaxkv_sparse_ctx_attention", "relaxkv_scatter_kv", "relaxkv_gather_kv"])
+def test_a_sessions_layer_is_an_index_in_range(monkeypatch, name):
+    """The layer of a session's calls: any integer type in range; other types and other layers end on the host."""
+    s, lib, calls = _host_session(monkeypatch)
+    for layer in (0, 2, np.int32(1), np.int64(2), torch.tensor(1), True):
+        lib.calls.clear()
+        calls[name](layer)
+        assert [n for n, _ in lib.calls] == [name]
+        assert s.r_cu_layer(int(layer)).data_ptr() in lib.calls[0][1]
+    lib.calls.clear()
+    for layer in (1.7, 1.0, "1", torch.tensor(1.0), np.float32(2.0), None):
+        with pytest.raises(TypeError):
+            calls[name](layer)
+    for layer in (-1, 3, 4, 100):
+        with pytest.raises(B.RelaxKVError, match="layer"):
+            calls[name](layer)
+    assert not lib.calls
 
 
 def test_missing_library_fails_loudly(monkeypatch):
