@@ -71,25 +71,25 @@ class RepairSession:
         nb = self.shape.n_req
         return self.r_cu[layer * nb: layer * nb + nb + 1]
 
-    def _r_cu_ptr(self, layer: int) -> int:
-        """Address of r_cu_layer(layer): a tensor slice costs the host 1 to 3 us, as much as marshalling the rest of a call."""
+    def _r_cu_at(self, layer: int) -> B.Offsets:
+        """r_cu_layer(layer) without its slice."""
         layer = operator.index(layer)           # numpy and torch integers, as an index of a tensor; nothing else
         if not 0 <= layer < self.n_layers:
             raise B.RelaxKVError(B.ERR_INVALID_ARG, f"layer {layer} of {self.n_layers}")
-        return self.r_cu.data_ptr() + 4 * layer * self.shape.n_req
+        return B.Offsets(self.r_cu, layer * self.shape.n_req)
 
     # -- (b) repair -----------------------------------------------------------------------------
     def attention(self, layer: int, cache: B.CacheView, q_new, k_new, v_new, out, max_targets, max_ctx,
                   mode: int = B.CTX_UNION, lse_out=None, stream=None, simt: bool = False) -> None:
         fn = B.relaxkv_sparse_ctx_attention_simt if simt else B.relaxkv_sparse_ctx_attention
         fn(self.shape, mode, cache, q_new, k_new, v_new, self.u_pos, self.u_cu, self.r_rank,
-           self._r_cu_ptr(layer), max_targets, max_ctx, out, self.workspace, lse_out=lse_out, stream=stream)
+           self._r_cu_at(layer), max_targets, max_ctx, out, self.workspace, lse_out=lse_out, stream=stream)
 
     def scatter(self, layer: int, cache: B.CacheView, k_new, v_new, max_targets, stream=None) -> None:
         B.relaxkv_scatter_kv(self.shape, cache, k_new, v_new, self.u_pos, self.u_cu, self.r_rank,
-                             self._r_cu_ptr(layer), max_targets, stream=stream)
+                             self._r_cu_at(layer), max_targets, stream=stream)
 
     def gather(self, layer: int, cache: B.CacheView, k_new, v_new, max_ctx, k_ctx_out, v_ctx_out,
                mode: int = B.CTX_UNION, stream=None) -> None:
         B.relaxkv_gather_kv(self.shape, mode, cache, k_new, v_new, self.u_pos, self.u_cu, self.r_rank,
-                            self._r_cu_ptr(layer), max_ctx, k_ctx_out, v_ctx_out, stream=stream)
+                            self._r_cu_at(layer), max_ctx, k_ctx_out, v_ctx_out, stream=stream)

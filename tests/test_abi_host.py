@@ -217,6 +217,25 @@ def test_a_sessions_layer_is_an_index_in_range(monkeypatch, name):
     assert not lib.calls
 
 
+def test_a_number_is_not_a_device_address(monkeypatch):
+    """A number where a tensor belongs ends on the host, whatever the argument."""
+    s, lib, _ = _host_session(monkeypatch)
+    t = torch.zeros(4, 1024, dtype=torch.bfloat16)
+    rows, cache = t.view(4, 8, 128), B.CacheView(t.view(8, 4, 128), t.view(8, 4, 128), [0, 4])
+    att = [s.shape, B.CTX_UNION, cache, rows, rows, rows, s.u_pos, s.u_cu, s.r_rank, s.r_cu, [1, 1], [1, 1], rows, s.workspace]
+    scatter = [s.shape, cache, rows, rows, s.u_pos, s.u_cu, s.r_rank, s.r_cu, [1, 1]]
+    for fn, args, where in ((B.relaxkv_sparse_ctx_attention, att, (3, 4, 5, 6, 7, 8, 9, 12, 13)), (B.relaxkv_scatter_kv, scatter, range(2, 8)),
+                            (B.relaxkv_rmsnorm, [t, t, t, 1e-6], (0, 1, 2)), (B.relaxkv_linear, [t, t, t], (0, 1, 2)),
+                            (B.relaxkv_target_positions, [s.shape, s.u_pos, s.u_cu, s.r_rank, s.r_cu, [1, 1], s.u_pos], (1, 2, 3, 4, 6))):
+        fn(*args)
+        assert lib.calls.pop()[0] == fn.__name__
+        for i in where:
+            for number in (0x10000, 0, 3.5):
+                with pytest.raises(AttributeError):
+                    fn(*args[:i], number, *args[i + 1:])
+                assert not lib.calls, (fn.__name__, i)
+
+
 def test_missing_library_fails_loudly(monkeypatch):
     monkeypatch.setattr(B, "_lib", None)
     monkeypatch.setattr(B, "LIB_PATH", "/nonexistent/librelaxkv.so")
