@@ -148,7 +148,7 @@ _raw_synchronize = getattr(torch._C, "_cuda_synchronize", None)
 
 def synchronize(device: torch.device) -> None:
     """torch.cuda.synchronize; without its change of device where the device is the current one."""
-    if (_raw_synchronize is not None and _current_device is not None and torch.cuda.is_initialized()
+    if (_raw_synchronize is not None and _current_device is not None and device.type == "cuda" and torch.cuda.is_initialized()
             and (device.index is None or device.index == _current_device())):
         _raw_synchronize()
     else:

@@ -236,6 +236,22 @@ def test_a_number_is_not_a_device_address(monkeypatch):
                 assert not lib.calls, (fn.__name__, i)
 
 
+def test_synchronize_leaves_other_devices_to_torch(monkeypatch):
+    """Only the current CUDA device is waited for directly; everything else, refusals included, is torch.cuda.synchronize's."""
+    direct, by_torch = [], []
+    monkeypatch.setattr(B, "_raw_synchronize", lambda: direct.append(1))
+    monkeypatch.setattr(B, "_current_device", lambda: 0)
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(torch.cuda, "synchronize", lambda device=None: by_torch.append(device))
+    B.synchronize(torch.device("cuda"))
+    B.synchronize(torch.device("cuda:0"))
+    assert len(direct) == 2 and not by_torch
+    others = [torch.device("cpu"), torch.device("cpu:0"), torch.device("cuda:1")]
+    for device in others:
+        B.synchronize(device)
+    assert len(direct) == 2 and by_torch == others
+
+
 def test_missing_library_fails_loudly(monkeypatch):
     monkeypatch.setattr(B, "_lib", None)
     monkeypatch.setattr(B, "LIB_PATH", "/nonexistent/librelaxkv.so")
