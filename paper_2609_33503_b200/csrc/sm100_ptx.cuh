@@ -169,20 +169,6 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
 }
 
 // ---- tcgen05.mma (issued by one thread) -----------------------------------------------------------
-// D[tmem] (+)= A[smem desc] * B[smem desc]
-__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-}
-// D[tmem] (+)= A[tmem] * B[smem desc]
-__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-}
 // The mbarrier receives one arrival once every tcgen05.mma issued so far by this thread has completed.
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -192,6 +178,10 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
 // The issuing thread is a single lane, so every instruction it spends on descriptor arithmetic delays
 // the next MMA.  A descriptor's low word holds the (address >> 4); stepping along K only adds a small
 // constant to it, so a whole K-loop is emitted as add / mov.b64 / mma triples with immediates.
+// Shared-memory matrix descriptor, 128-byte swizzle, tiles whose 8-row groups are 1024 bytes apart.
+//   K-major operand  (rows of 64 bf16 = 128 B):       lbo ignored (1),  sbo = 1024
+//   MN-major operand (64 contiguous MN elements per K row): lbo = bytes between 64-element MN blocks,
+//                                                           sbo = 1024 (between groups of 8 K rows)
 //   lo word: (smem address >> 4) | (leading byte offset >> 4) << 16      hi word: see desc_hi_sw128()
 __host__ __device__ constexpr uint32_t desc_hi_sw128(uint32_t sbo_bytes) {
   return ((sbo_bytes >> 4) & 0x3FFFu) | (1u << 14) | (2u << 29);        // stride offset | version | 128B swizzle
@@ -241,19 +231,18 @@ __device__ __forceinline__ void mma_ss_4steps(uint32_t d_tmem, uint32_t a_lo, ui
   "mov.b64 db, {tb, %3};\n\t"                                                                  \
   "tcgen05.mma.cta_group::1.kind::f16 [%0], [ta], db, %4, " #PRED ";\n\t"
 
-// D[tmem] (+)= A[tmem] * B[smem] for N = 2, 4 or 6 K steps of 16: A advances 8 columns, B (MN-major, 128B swizzle)
+// D[tmem] (+)= A[tmem] * B[smem] for N = 2 or 6 K steps of 16: A advances 8 columns, B (MN-major, 128B swizzle)
 // 2048 bytes per step.  acc_first = 0 makes the first MMA overwrite D.
 template <int N>
 __device__ __forceinline__ void mma_ts_steps(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi, uint32_t idesc,
                                              uint32_t acc_first) {
-  static_assert(N == 2 || N == 4 || N == 6, "K steps");
+  static_assert(N == 2 || N == 6, "K steps");
 #define RELAXKV_MMA_TS_HEAD                                                  \
   "{\n\t.reg .pred p0, p1;\n\t.reg .b32 ta, tb;\n\t.reg .b64 db;\n\t"    \
   "setp.ne.b32 p0, %5, 0;\n\tsetp.eq.b32 p1, 0, 0;\n\t"                    \
   RELAXKV_MMA_TS_STEP(0, 0, p0) RELAXKV_MMA_TS_STEP(8, 128, p1)
 #define RELAXKV_MMA_TS_ARGS "}" ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"(acc_first) : "memory"
   if (N == 2) asm volatile(RELAXKV_MMA_TS_HEAD RELAXKV_MMA_TS_ARGS);
-  if (N == 4) asm volatile(RELAXKV_MMA_TS_HEAD RELAXKV_MMA_TS_STEP(16, 256, p1) RELAXKV_MMA_TS_STEP(24, 384, p1) RELAXKV_MMA_TS_ARGS);
   if (N == 6)
     asm volatile(RELAXKV_MMA_TS_HEAD RELAXKV_MMA_TS_STEP(16, 256, p1) RELAXKV_MMA_TS_STEP(24, 384, p1)
                  RELAXKV_MMA_TS_STEP(32, 512, p1) RELAXKV_MMA_TS_STEP(40, 640, p1) RELAXKV_MMA_TS_ARGS);
@@ -329,17 +318,6 @@ __device__ __forceinline__ void mma_commit2_mc(uint32_t bar, uint16_t mask) {
   "add.u32 ta, %1, " #AOFF ";\n\tadd.u32 tb, %2, " #BOFF ";\n\t"                                  \
   "mov.b64 da, {ta, %3};\n\tmov.b64 db, {tb, %3};\n\t"                                           \
   "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, " #PRED ";\n\t"
-// D[tmem] = A[smem] * B[smem] over K = 128 (two 64-element halves; A's halves 16 KB apart, B's 8 KB: this CTA's
-// 64 of the tile's 128 N rows): the first MMA overwrites D.
-__device__ __forceinline__ void mma2_ss_kloop(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc) {
-  asm volatile(
-      "{\n\t.reg .pred p0, p1;\n\t.reg .b32 ta, tb;\n\t.reg .b64 da, db;\n\t"
-      "setp.ne.b32 p0, 0, 0;\n\tsetp.eq.b32 p1, 0, 0;\n\t"
-      RELAXKV_MMA2_SS_STEP(0, 0, p0) RELAXKV_MMA2_SS_STEP(2, 2, p1) RELAXKV_MMA2_SS_STEP(4, 4, p1) RELAXKV_MMA2_SS_STEP(6, 6, p1)
-      RELAXKV_MMA2_SS_STEP(1024, 512, p1) RELAXKV_MMA2_SS_STEP(1026, 514, p1) RELAXKV_MMA2_SS_STEP(1028, 516, p1)
-      RELAXKV_MMA2_SS_STEP(1030, 518, p1)
-      "}" ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc) : "memory");
-}
 // D[tmem] (+)= A[smem] * B[smem] for four K steps of 16 inside one 64-element swizzled K block (both K-major).
 __device__ __forceinline__ void mma2_ss_4steps(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc,
                                                uint32_t acc_first) {
@@ -349,35 +327,8 @@ __device__ __forceinline__ void mma2_ss_4steps(uint32_t d_tmem, uint32_t a_lo, u
       RELAXKV_MMA2_SS_STEP(0, 0, p0) RELAXKV_MMA2_SS_STEP(2, 2, p1) RELAXKV_MMA2_SS_STEP(4, 4, p1) RELAXKV_MMA2_SS_STEP(6, 6, p1)
       "}" ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(acc_first) : "memory");
 }
-#define RELAXKV_MMA2_TS_STEP(AOFF, BOFF, PRED)                                               \
-  "add.u32 ta, %1, " #AOFF ";\n\tadd.u32 tb, %2, " #BOFF ";\n\t"                                  \
-  "mov.b64 db, {tb, %3};\n\t"                                                                  \
-  "tcgen05.mma.cta_group::2.kind::f16 [%0], [ta], db, %4, " #PRED ";\n\t"
-// D[tmem] (+)= A[tmem] * B[smem] for four K steps of 16: A advances 8 columns, B (MN-major) 2048 bytes per step.
-__device__ __forceinline__ void mma2_ts_4steps(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi, uint32_t idesc,
-                                               uint32_t acc_first) {
-  asm volatile(
-      "{\n\t.reg .pred p0, p1;\n\t.reg .b32 ta, tb;\n\t.reg .b64 db;\n\t"
-      "setp.ne.b32 p0, %5, 0;\n\tsetp.eq.b32 p1, 0, 0;\n\t"
-      RELAXKV_MMA2_TS_STEP(0, 0, p0) RELAXKV_MMA2_TS_STEP(8, 128, p1) RELAXKV_MMA2_TS_STEP(16, 256, p1) RELAXKV_MMA2_TS_STEP(24, 384, p1)
-      "}" ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"(acc_first) : "memory");
-}
 
-// ---- descriptors ------------------------------------------------------------------------------------
-// Shared-memory matrix descriptor, 128-byte swizzle, tiles whose 8-row groups are 1024 bytes apart.
-//   K-major operand  (rows of 64 bf16 = 128 B):       lbo ignored (1),  sbo = 1024
-//   MN-major operand (64 contiguous MN elements per K row): lbo = bytes between 64-element MN blocks,
-//                                                           sbo = 1024 (between groups of 8 K rows)
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t smem_addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-  uint64_t d = 0;
-  d |= static_cast<uint64_t>((smem_addr >> 4) & 0x3FFFu);
-  d |= static_cast<uint64_t>((lbo_bytes >> 4) & 0x3FFFu) << 16;
-  d |= static_cast<uint64_t>((sbo_bytes >> 4) & 0x3FFFu) << 32;
-  d |= 1ull << 46;      // descriptor version of this architecture
-  d |= 2ull << 61;      // 128-byte swizzle
-  return d;
-}
-
+// ---- instruction descriptor ------------------------------------------------------------------------------------
 // Instruction descriptor: bf16 x bf16 -> fp32, A K-major, dense.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int m, int n, int b_mn_major) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(b_mn_major) << 16) |
