@@ -610,6 +610,33 @@ def test_expired_wait_is_reported_and_the_context_stays_usable():
     check_attention(case, 0, out, lse, False)
 
 
+@pytest.mark.parametrize("given_lse", [False, True], ids=["both_passes", "given_lse"])
+@pytest.mark.parametrize("head_dim", [128, 64])
+def test_scoring_after_an_expired_wait_adds_nothing_up(head_dim, given_lse):
+    """While the status word says RELAXKV_ERR_TIMEOUT the scoring passes leave their partial sums alone (the workspace is zero, so the
+    scores are sums of zeros) and give their tensor memory back: the same call works once the word has been read."""
+    w = small_llama(n_layers=2, ctx=(1500, 300), q=(40, 8)) if head_dim == 128 else inputs.tiny()
+    case = Case(w)
+    s = case.make_session()
+    lses = None
+    if given_lse:               # (their values only have to be finite: what they scale is not looked at)
+        lses = [torch.zeros(w.n_q_heads, int(case.q_cu[-1]), dtype=torch.float32, device=case.device) for _ in range(w.n_layers)]
+    s.workspace.zero_()
+    s.raw.fill_(3.0)
+    B().relaxkv_debug_wait_timeout()
+    s.score_select(case.q_layers, case.cache_views(), row_lse_layers=lses)
+    st, _ = B().relaxkv_read_device_status()
+    assert st == B().ERR_TIMEOUT
+    assert torch.all(s.raw == 0)
+    s.score_select(case.q_layers, case.cache_views())
+    assert_status_ok()
+    raw = s.raw.cpu().numpy().astype(np.float64)
+    for l in range(w.n_layers):
+        for b in range(w.n_req):
+            ref = case.raw[(l, b)]
+            assert np.all(np.abs(raw[l, case.ctx_cu[b]:case.ctx_cu[b + 1]] - ref) <= 1e-3 * ref + 1e-6 / w.ctx_lens[b])
+
+
 # ------------------------------------------------ controlled configurations (explicit lists) ----
 
 def _pack(lists, device):
