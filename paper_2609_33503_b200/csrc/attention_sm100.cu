@@ -96,8 +96,8 @@ __device__ __forceinline__ void softmax_keys(uint32_t t_s, const uint32_t* s, fl
 // The step is a link of the chain S -> P -> P V -> next S that bounds the kernel.  The maximum comes first.  Exponentials begun with the
 // tile before's reference are no faster where both tiles of a pair keep the SM busy (8 K stack 8.12 ms either way, 12 layers of 40 / 8
 // heads at 32 K 35.8; ragged query passes of one to 25 rows per tile 1 to 3 % faster), and where maxima grow along the context they have
-// to be done again, four warps waiting for the slowest of them (6 K entries, 32 / 8 heads, keys that grow thirtyfold: 400 us against 325
-// with the maximum first; of dim 64 333 against 230).
+// to be done again, four warps waiting for the slowest of them (6 K entries, 32 / 8 heads, keys that grow thirtyfold: 397 us against 321
+// with the maximum first; of dim 64 333 against 229).
 template <int D>
 __device__ __forceinline__ void softmax_step(uint32_t t_s, uint32_t t_o, int limit, bool first, float scale_log2,
                                              float& m, float& z, uint32_t bar_p_lo, uint32_t bar_p_hi) {
