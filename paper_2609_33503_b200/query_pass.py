@@ -20,6 +20,12 @@ from . import binding as B
 from .inputs import BlockShape
 
 
+# Layers whose context scores are computed by one launch behind the last of them, and the query rows kept for that (10 MB of Q at 40
+# heads of 128).  By itself a layer of few rows is mostly its launch's start and end: 57 rows over 8K of context 15 + 4 us of which 4 are
+# work; 8 layers of such a pass took 1321 us, 1278 so, 12 layers of 128 rows over 32K 4264 / 4221.  With more rows a launch is full by itself.
+_SCORE_LAYERS, _SCORE_ROWS = 8, 1024
+
+
 class QueryPass:
     """Buffers for the block work of the query rows of a batch (`q_lens` tokens per request after `ctx_lens` context
     tokens).  The caches handed to `prefill` / `decode` must have room for ctx + query (+ decoded) tokens per request."""
@@ -49,6 +55,12 @@ class QueryPass:
         self.q, self.k, self.v, self.o = e(n, H, D), e(n, Hkv, D), e(n, Hkv, D), e(n, H, D)
         self.gu, self.m = e(n, 2 * I), e(n, I)
         self.lse = torch.empty(H, n, dtype=torch.float32, device=self.device)
+        # rotated queries and row normalisers of the layers that are scored together, as far as the workspace reaches
+        g = max(1, min(_SCORE_LAYERS, _SCORE_ROWS // max(1, n)))
+        while g > 1 and B.relaxkv_workspace_bytes(self.shape_prefill, g) > nbytes:
+            g -= 1
+        self.q_kept = torch.empty(g, n, H, D, **bf) if g > 1 else None
+        self.lse_kept = torch.empty(g, H, n, dtype=torch.float32, device=self.device) if g > 1 else None
         # positions of the query tokens (request-local) and their offsets: plain index data, built once
         pos, cu = [], [0]
         for c, q in zip(self.ctx_lens, self.q_lens):
@@ -105,18 +117,28 @@ class QueryPass:
                 taps: Optional[list] = None) -> torch.Tensor:
         """h0: input representations of the query tokens [sum Q_b, hidden].  caches[l]: layer l's cache with the context
         rows in place and room behind them; the query's K/V are written there.  scores_out: fp32 [n_layers, sum T_c]
-        or None; when given, row l receives the context scores of layer l from this very pass.  Returns the hidden rows
-        after the last layer."""
+        or None; when given, row l receives the context scores of layer l from this very pass (computed for several layers
+        at once where its rows lie one behind the other).  Returns the hidden rows after the last layer."""
         rec = self._rec(events)
         h = h0
+        # scored in groups where the rows of scores_out lie one behind the other, as a call over several layers writes them
+        together = (self.q_kept is not None and isinstance(scores_out, torch.Tensor) and scores_out.dim() == 2
+                    and scores_out.shape[1] == sum(self.ctx_lens) and scores_out.is_contiguous())
+        group = self.q_kept.shape[0] if together else 1
         for l, w in enumerate(weights):
             h_out = self.h[l % 2]
             raw = scores_out[l] if scores_out is not None else None
+            q, lse = (self.q_kept[l % group], self.lse_kept[l % group]) if together else (self.q, self.lse)
 
             def attend():
-                B.relaxkv_query_prefill_attention(self.shape_prefill, caches[l], self.q, self.o, self.lse, raw, self.workspace)
-            self._block(l, w, caches[l], h, self.x, self.a, self.q, self.k, self.v, self.o, self.gu, self.m, h_out,
+                B.relaxkv_query_prefill_attention(self.shape_prefill, caches[l], q, self.o, lse, None if together else raw, self.workspace)
+            self._block(l, w, caches[l], h, self.x, self.a, q, self.k, self.v, self.o, self.gu, self.m, h_out,
                         self.q_pos, self.q_cu, self.q_lens, self.shape_ext, attend, rec)
+            if together and (l % group == group - 1 or l == len(weights) - 1):
+                l0, n = l - l % group, l % group + 1
+                rec("scores", lambda: B.relaxkv_score_select(
+                    self.shape_prefill, [self.q_kept[i] for i in range(n)], [caches[i] for i in range(l0, l + 1)], [1] * len(self.ctx_lens),
+                    scores_out[l0:l + 1], None, self.workspace, row_lse_layers=[self.lse_kept[i] for i in range(n)]))
             if taps is not None:
                 taps.append((h.clone(), h_out.clone()))
             h = h_out

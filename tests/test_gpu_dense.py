@@ -648,3 +648,31 @@ def test_decode_step_with_chained_launches_equals_plain_launches(graph):
     for b in range(nb):
         for s in range(steps):
             assert plain[1][0][0][offs[b] + ctx[b] + qn[b] + s].float().abs().max() > 0
+
+
+@pytest.mark.parametrize("layers", [7, 8, 9])
+def test_scores_of_several_layers_in_one_launch_equal_the_layers_own(layers):
+    """A query pass scores groups of eight layers behind the last of each where the rows of scores_out are one matrix, and each layer in
+    its own launch where they are not: the same hidden rows, and scores that differ by the order of their fp32 sums alone (a
+    column sum adds H * Q_b = 112 positive terms in at most 2 H_kv runs: 112 * 2^-24 < 1e-5 relative)."""
+    from paper_2609_33503_b200.query_pass import QueryPass
+    H, Hkv, D = 8, 2, 64
+    ctx, qn = (700, 129), (9, 5)
+    blkshape = inputs.BlockShape(hidden=256, inter=512, rope_theta=1.0e4, eps=1.0e-5, qk_norm=True)
+    w = inputs.Workload("grouped", layers, H, Hkv, D, 64, ctx, qn, 0.15, base_seed=13)
+    room = [c + q for c, q in zip(ctx, qn)]
+    weights = [inputs.block_weights(w, blkshape, l, "cuda") for l in range(layers)]
+    h0 = rnd(sum(qn), blkshape.hidden, seed=3)
+    qp = QueryPass(H, Hkv, D, ctx, qn, blkshape)
+    assert qp.q_kept.shape[0] == 8
+    got = []
+    for width in (sum(ctx), sum(ctx) + 4):                  # one matrix; rows with a gap between them
+        views = [B().CacheView(rnd(sum(room), Hkv, D, seed=100 + l), rnd(sum(room), Hkv, D, seed=200 + l), [0, room[0]]) for l in range(layers)]
+        scores = torch.full((layers, width), -1.0, dtype=torch.float32, device="cuda")[:, :sum(ctx)]
+        h = qp.prefill(h0, weights, views, scores_out=scores)
+        st, detail = B().relaxkv_read_device_status()
+        assert st == 0, (st, detail)
+        got.append((h.clone(), scores.contiguous()))
+    assert torch.equal(got[0][0], got[1][0])
+    assert (got[1][1] > 0).all()
+    assert ((got[0][1] - got[1][1]).abs() <= 1e-5 * got[1][1]).all()
