@@ -122,7 +122,7 @@ class QueryPass:
         rec = self._rec(events)
         h = h0
         # scored in groups where the rows of scores_out lie one behind the other, as a call over several layers writes them
-        together = (self.q_kept is not None and isinstance(scores_out, torch.Tensor) and scores_out.dim() == 2
+        together = (self.q_kept is not None and isinstance(scores_out, torch.Tensor) and scores_out.dtype == torch.float32 and scores_out.dim() == 2
                     and scores_out.shape[1] == sum(self.ctx_lens) and scores_out.is_contiguous())
         group = self.q_kept.shape[0] if together else 1
         for l, w in enumerate(weights):
