@@ -1,13 +1,13 @@
 // Sparse-context repair attention on the Blackwell tensor cores (Section 3.3; Algorithm 1, steps 16-19).
 //
-// One CTA owns a tile of 128 query rows = (floor(128/G) consecutive active targets) x (the G query
+// One CTA owns a pair of tiles of 128 query rows = (floor(256/G) consecutive active targets) x (the G query
 // heads of one KV head), so every K/V tile it stages is shared by the whole GQA group.  It walks the
-// context prefix the tile can see in 128-key tiles of the materialised mixed context:
+// context prefix a tile can see in 128-key tiles of the materialised mixed context:
 //   TMA (128B swizzle)  ->  S = Q K^T  (tcgen05.mma, fp32 accumulator in TMEM)
 //   softmax warps: tcgen05.ld S, position-based causal mask on the staircase edge, online max/sum with
 //                  lazy rescaling, P -> bf16 back into TMEM (over S)
 //   O += P V            (tcgen05.mma, A operand = P from TMEM, B = V tile MN-major from shared memory)
-// A CTA runs TWO such query tiles (A, B) in ping-pong: while the softmax warps of one tile work, the
+// A CTA runs the TWO tiles (A, B) in ping-pong: while the softmax warps of one tile work, the
 // tensor pipe runs the other tile's MMAs; both tiles share every K/V tile staged in shared memory.
 // Warp roles: warps 0-3 softmax/epilogue of tile A, warps 4-7 of tile B (thread = query row = TMEM
 // lane), warp 8 TMA producer, warp 9 MMA issuer and TMEM owner, warp 10 a helper for cache-only calls.  K/V tiles
@@ -150,7 +150,7 @@ template <int D>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                        const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ ReqTable rt,
-                       int mode, int allow_empty, int head_inner, int dense_ctx, int H, int Hkv, int tile_targets, float scale_log2,
+                       int mode, int allow_empty, int head_inner, int dense_ctx, int H, int Hkv, int pair_targets, float scale_log2,
                        const int* u_pos, const int* u_cu, const int* r_rank, const int* r_cu,
                        long long n_target_rows, uint16_t* __restrict__ out, float* __restrict__ lse_out,
                        float* __restrict__ part_o, float* __restrict__ part_lse, DeviceStatus* st) {
@@ -180,7 +180,6 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const int first_pos = rt.ctx_len[b] - nr;
   // dense_ctx: the context is the cache itself (every position of the request), a target's limit is its position
   const int nu = dense_ctx ? rt.ctx_len[b] : (u_cu[b + 1] - u_cu[b]);
-  const int pair_targets = 2 * tile_targets;
   const int n_pairs_true = (nr + pair_targets - 1) / pair_targets;
   if (p_rev >= n_pairs_true) return;
   // a true count above its host bound, or more target rows than q_new / out hold: report, touch nothing
@@ -194,15 +193,15 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const int rho0 = pair * pair_targets;                       // first target of tile A
   const int ctx_len_b = (mode == RELAXKV_CTX_UNION) ? nu : rt.ctx_len[b];
   const long long ctx_base = dense_ctx ? rt.tok_off[b] : ((mode == RELAXKV_CTX_UNION) ? (long long)u_cu[b] : rt.ctx_cu[b]);
-  const long long q_row_base = row0 + rho0;
-  // valid targets and context tiles of each query tile
-  int n_valid[2], n_kv[2];
+  const int q_row_base = (int)row0 + rho0;                    // (offsets of the lists are 32-bit)
+  // targets of the pair, context tiles of each query tile
+  const int n_tgt = min(pair_targets, nr - rho0);
+  int n_kv[2];
 #pragma unroll
   for (int x = 0; x < 2; ++x) {
-    n_valid[x] = max(0, min(tile_targets, nr - rho0 - x * tile_targets));
     n_kv[x] = 0;
-    if (n_valid[x] > 0) {
-      const int rho_last = rho0 + x * tile_targets + n_valid[x] - 1;
+    if (n_tgt * G > x * kBM) {
+      const int rho_last = rho0 + (min(n_tgt * G, (x + 1) * kBM) - 1) / G;
       const int c = r_cu ? r_rank[row_b + rho_last] : first_pos + rho_last;
       const int cc = min(max(c, 0), max(nu - 1, 0));
       int lim_last = (mode == RELAXKV_CTX_UNION) ? cc : u_pos[u_cu[b] + cc];
@@ -222,9 +221,9 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const int n_my_max = max(n_my[0], n_my[1]);
   if (n_my_max == 0) {                        // nothing of this pair's context falls into this split
     if (n_splits > 1 && threadIdx.x < 2 * kBM) {
-      const int x = threadIdx.x >> 7, row = threadIdx.x & 127, t_local = row / G;
-      if (row < tile_targets * G && t_local < n_valid[x]) {
-        const long long orow = q_row_base + x * tile_targets + t_local;
+      const int row = threadIdx.x, t_local = row / G;
+      if (t_local < n_tgt) {
+        const int orow = q_row_base + t_local;
         part_lse[((long long)split * n_target_rows + orow) * H + hd * G + (row - t_local * G)] = -INFINITY;
       }
     }
@@ -273,11 +272,11 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   }
   // rows of the Q tiles that no (target, head) pair fills: zero them (they feed unused MMA rows)
   {
-    const int used = tile_targets * G;
-    const int n_pad = kBM - used;
-    for (int i = threadIdx.x; i < n_pad * 8 * kHalves * 2; i += kAttnThreads) {
-      const int piece = i & 7, r = (i >> 3) % n_pad, blk = (i >> 3) / n_pad;    // blk = tile * kHalves + half
-      *reinterpret_cast<uint4*>(base_ptr + L::kQ + blk * kHalfBytes + (used + r) * 128 + piece * 16) = make_uint4(0, 0, 0, 0);
+    const int used = pair_targets * G;
+    const int n_pad = 2 * kBM - used;
+    for (int i = threadIdx.x; i < n_pad * 8 * kHalves; i += kAttnThreads) {
+      const int piece = i & 7, r = (i >> 3) % n_pad, hf = (i >> 3) / n_pad;
+      *reinterpret_cast<uint4*>(base_ptr + L::kQ + hf * 2 * kHalfBytes + (used + r) * 128 + piece * 16) = make_uint4(0, 0, 0, 0);
     }
     fence_proxy_async_smem();
   }
@@ -293,11 +292,9 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   if (warp == 8) {
     // ================= TMA producer =================
     if (lane == 0) {
-      mbar_expect_tx(bar_q, (uint32_t)(2 * kHalves * tile_targets * G * 128));
-      for (int x = 0; x < 2; ++x)
-        for (int hf = 0; hf < kHalves; ++hf)
-          tma_load_3d(q_smem + (x * kHalves + hf) * kHalfBytes, &tm_q, bar_q, hf * 64, hd * G,
-                      (int)(q_row_base + x * tile_targets));
+      mbar_expect_tx(bar_q, (uint32_t)(kHalves * pair_targets * G * 128));
+      for (int hf = 0; hf < kHalves; ++hf)
+        tma_load_3d(q_smem + hf * 2 * kHalfBytes, &tm_q, bar_q, hf * 64, hd * G, q_row_base);
       // The tiles travel in the order K_0 V_0 K_1 V_1 ... through the ring slots u % kRing (u = 2j for K_j, 2j + 1
       // for V_j; j counted from j0).  They are signalled in PAIRS p = (V_{p-1}, K_p): step j of the MMA warp needs
       // exactly pair j + 1 (V_j for P V, K_{j+1} for the next Q K^T), so it waits once and frees once per step.
@@ -334,7 +331,7 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       uint32_t sv = 1, sk = 2, pk = 8, pph = 0;
       const int n0 = n_my[0], n1 = n_my[1];
       auto issue_qk = [&](int x, uint32_t slot) {                   // S_x = Q_x K^T with the K tile in `slot` -> bar_sfull[x]
-        mma_ss_kloop<kHalves>(tmem_base + x * 128, desc_lo(q_smem + x * L::kTileBytes, 16),
+        mma_ss_kloop<kHalves>(tmem_base + x * 128, desc_lo(q_smem + x * kHalfBytes, 16),
                               desc_lo(kv_smem + slot * L::kTileBytes, 16), desc_hi_sw128(1024), idesc_qk);
         mma_commit(bar_sfull + 8 * x);
       };
@@ -400,11 +397,10 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     reg_alloc<224>();
     // ================= softmax + epilogue: thread = query row = TMEM lane =================
     const int x = warp >> 2;                                    // 0: tile A, 1: tile B
-    const int row = threadIdx.x & 127;
-    const int t_local = row / G, j_head = row - t_local * G;
-    const bool row_valid = (row < tile_targets * G) && (t_local < n_valid[x]);
-    const int rho_t = rho0 + x * tile_targets + t_local;
-    // Rows without a target (125 of 128 rows are used with five heads per KV head) and rows of an empty context see every key: what they
+    const int t_local = (int)threadIdx.x / G, j_head = (int)threadIdx.x - t_local * G;      // flat rows of the pair: tile A, then B
+    const bool row_valid = t_local < n_tgt;
+    const int rho_t = rho0 + t_local;
+    // Rows without a target (one of 256 with five heads per KV head; three of 128 when a target's heads had to share a tile) and rows of an empty context see every key: what they
     // hold is not stored (an empty context's row is written as zeros), and a limit below the tile sends their whole warp through the
     // masking of every tile, 1.0 k clk of a 3.5 k step (12 layers of 40 / 8 heads at 32 K, repaired: 40.7 -> 37.3 ms; every row used,
     // 32 / 8 heads at 8 K: 8.42 -> 8.37).
@@ -445,9 +441,9 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       const bool none = row_empty || !(z > 0.f);                // an empty context is defined as a zero output row
       const float inv = none ? 0.f : 1.f / z;
       const float lse = none ? -INFINITY : (m + log2f(z)) * kLn2A;
-      const long long orow = q_row_base + x * tile_targets + t_local;
+      const int orow = q_row_base + t_local;
       if (n_splits == 1) {
-        uint16_t* optr = out + (orow * H + hd * G + j_head) * D;
+        uint16_t* optr = out + ((long long)orow * H + hd * G + j_head) * D;
 #pragma unroll
         for (int c = 0; c < D / 32; ++c) {
           uint32_t o[32];
@@ -490,7 +486,7 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       }
     } else if (ok && my_n == 0 && n_splits > 1 && row_valid) {
       // this tile's context ends before the split begins (the pair's other tile still has work here)
-      const long long orow = q_row_base + x * tile_targets + t_local;
+      const int orow = q_row_base + t_local;
       part_lse[((long long)split * n_target_rows + orow) * H + hd * G + j_head] = -INFINITY;
     }
   }
@@ -541,15 +537,14 @@ struct PersistSmem {
 struct WorkItem {
   int work;            // 1: work, -1: the list is exhausted
   int n_max, n_my0, n_my1;
-  int n_valid0, n_valid1, hd, q_row_base;
+  int n_tgt, pad0, hd, q_row_base;
   int nu, ctx_len_b, r_base, rho0;      // r_base = r_cu[b]
   int u_base, ctx_base, b, pad;         // u_base = u_cu[b]
-  __device__ __forceinline__ int n_valid(int x) const { return x ? n_valid1 : n_valid0; }
   __device__ __forceinline__ int n_my(int x) const { return x ? n_my1 : n_my0; }
 };
 __device__ __forceinline__ void item_store(int4* rec, const WorkItem& it) {
   rec[0] = make_int4(it.work, it.n_max, it.n_my0, it.n_my1);
-  rec[1] = make_int4(it.n_valid0, it.n_valid1, it.hd, it.q_row_base);
+  rec[1] = make_int4(it.n_tgt, 0, it.hd, it.q_row_base);
   rec[2] = make_int4(it.nu, it.ctx_len_b, it.r_base, it.rho0);
   rec[3] = make_int4(it.u_base, it.ctx_base, it.b, 0);
 }
@@ -560,16 +555,16 @@ __device__ __forceinline__ void item_load_head(const int4* rec, WorkItem& it) { 
 __device__ __forceinline__ void item_load(const int4* rec, WorkItem& it) {
   item_load_head(rec, it);
   const int4 b = rec[1], c = rec[2], d = rec[3];
-  it.n_valid0 = b.x; it.n_valid1 = b.y; it.hd = b.z; it.q_row_base = b.w;
+  it.n_tgt = b.x; it.pad0 = 0; it.hd = b.z; it.q_row_base = b.w;
   it.nu = c.x; it.ctx_len_b = c.y; it.r_base = c.z; it.rho0 = c.w;
   it.u_base = d.x; it.ctx_base = d.y; it.b = d.z; it.pad = 0;
 }
 
-__device__ __forceinline__ WorkItem decode_item(int id, const ReqTable& rt, int head_inner, int Hkv, int mode, int tile_targets,
+__device__ __forceinline__ WorkItem decode_item(int id, const ReqTable& rt, int head_inner, int G, int Hkv, int mode, int pair_targets,
                                                 const int* u_pos, const int* u_cu, const int* r_rank, const int* r_cu,
                                                 long long n_target_rows, DeviceStatus* st) {
   WorkItem it;
-  it.work = 0; it.pad = 0;
+  it.work = 0; it.pad = it.pad0 = 0;
   const int B = rt.n_req;
   const int n_pairs_total = rt.tile_cu[B];
   it.hd = head_inner ? (id % Hkv) : (id / n_pairs_total);
@@ -581,9 +576,8 @@ __device__ __forceinline__ WorkItem decode_item(int id, const ReqTable& rt, int 
   const int nr = r_cu[b + 1] - it.r_base;
   const int nu = u_cu[b + 1] - it.u_base;
   it.nu = nu;
-  const int pair_targets = 2 * tile_targets;
   const int n_pairs_true = (nr + pair_targets - 1) / pair_targets;
-  it.n_max = 0; it.n_my0 = it.n_my1 = 0; it.n_valid0 = it.n_valid1 = 0;
+  it.n_max = 0; it.n_my0 = it.n_my1 = 0; it.n_tgt = 0;
   it.rho0 = 0; it.ctx_len_b = 0; it.ctx_base = 0; it.q_row_base = 0;
   if (p_rev >= n_pairs_true) return it;
   if (nr > rt.bound_a[b] || (mode == RELAXKV_CTX_UNION && nu > rt.bound_b[b]) || (long long)(r_cu[b + 1] - r_cu[0]) > n_target_rows) {
@@ -595,19 +589,19 @@ __device__ __forceinline__ WorkItem decode_item(int id, const ReqTable& rt, int 
   it.ctx_len_b = (mode == RELAXKV_CTX_UNION) ? nu : rt.ctx_len[b];
   it.ctx_base = (int)((mode == RELAXKV_CTX_UNION) ? (long long)it.u_base : rt.ctx_cu[b]);
   it.q_row_base = (it.r_base - r_cu[0]) + it.rho0;
-  int nm[2] = {0, 0}, nv[2] = {0, 0};
+  it.n_tgt = min(pair_targets, nr - it.rho0);
+  int nm[2] = {0, 0};
 #pragma unroll
   for (int x = 0; x < 2; ++x) {
-    nv[x] = max(0, min(tile_targets, nr - it.rho0 - x * tile_targets));
-    if (nv[x] > 0) {
-      const int c = r_rank[it.r_base + it.rho0 + x * tile_targets + nv[x] - 1];
+    if (it.n_tgt * G > x * kBM) {
+      const int c = r_rank[it.r_base + it.rho0 + (min(it.n_tgt * G, (x + 1) * kBM) - 1) / G];
       const int cc = min(max(c, 0), max(nu - 1, 0));
       int lim_last = (mode == RELAXKV_CTX_UNION) ? cc : u_pos[it.u_base + cc];
       lim_last = min(max(lim_last, 0), it.ctx_len_b - 1);
       nm[x] = lim_last / kBN + 1;
     }
   }
-  it.n_valid0 = nv[0]; it.n_valid1 = nv[1]; it.n_my0 = nm[0]; it.n_my1 = nm[1];
+  it.n_my0 = nm[0]; it.n_my1 = nm[1];
   it.n_max = max(nm[0], nm[1]);
   it.work = it.n_max > 0;
   return it;
@@ -617,7 +611,7 @@ template <int D>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                          const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ ReqTable rt,
-                         int mode, int allow_empty, int head_inner, int H, int Hkv, int tile_targets, float scale_log2,
+                         int mode, int allow_empty, int head_inner, int H, int Hkv, int pair_targets, float scale_log2,
                          const int* u_pos, const int* u_cu, const int* r_rank, const int* r_cu,
                          long long n_target_rows, uint16_t* __restrict__ out, float* __restrict__ lse_out,
                          int total_items, int* __restrict__ work_counter, DeviceStatus* st) {
@@ -658,11 +652,11 @@ attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
   }
   if (warp == 9) { tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols); tmem_relinquish(); }
   {
-    const int used = tile_targets * G;
-    const int n_pad = kBM - used;
-    for (int i = threadIdx.x; i < n_pad * 8 * kHalves * 2; i += kAttnThreads) {
-      const int piece = i & 7, r = (i >> 3) % n_pad, blk = (i >> 3) / n_pad;
-      *reinterpret_cast<uint4*>(base_ptr + L::kQ + blk * kHalfBytes + (used + r) * 128 + piece * 16) = make_uint4(0, 0, 0, 0);
+    const int used = pair_targets * G;
+    const int n_pad = 2 * kBM - used;
+    for (int i = threadIdx.x; i < n_pad * 8 * kHalves; i += kAttnThreads) {
+      const int piece = i & 7, r = (i >> 3) % n_pad, hf = (i >> 3) / n_pad;
+      *reinterpret_cast<uint4*>(base_ptr + L::kQ + hf * 2 * kHalfBytes + (used + r) * 128 + piece * 16) = make_uint4(0, 0, 0, 0);
     }
     fence_proxy_async_smem();
   }
@@ -692,7 +686,7 @@ attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
           const int id = (n_fetched == 0) ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(work_counter, 1);
           ++n_fetched;
           if (id >= total_items) { it.work = -1; return false; }
-          it = decode_item(id, rt, head_inner, Hkv, mode, tile_targets, u_pos, u_cu, r_rank, r_cu, n_target_rows, st);
+          it = decode_item(id, rt, head_inner, G, Hkv, mode, pair_targets, u_pos, u_cu, r_rank, r_cu, n_target_rows, st);
           if (it.work) return true;
         }
       };
@@ -705,10 +699,8 @@ attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
         return true;
       };
       auto load_q = [&](const WorkItem& it) {
-        mbar_expect_tx(bar_q, (uint32_t)(2 * kHalves * tile_targets * G * 128));
-        for (int x = 0; x < 2; ++x)
-          for (int hf = 0; hf < kHalves; ++hf)
-            tma_load_3d(q_smem + (x * kHalves + hf) * kHalfBytes, &tm_q, bar_q, hf * 64, it.hd * G, it.q_row_base + x * tile_targets);
+        mbar_expect_tx(bar_q, (uint32_t)(kHalves * pair_targets * G * 128));
+        for (int hf = 0; hf < kHalves; ++hf) tma_load_3d(q_smem + hf * 2 * kHalfBytes, &tm_q, bar_q, hf * 64, it.hd * G, it.q_row_base);
       };
       auto load_tile = [&](int u, const WorkItem& it, int j, uint32_t bar) {      // u = 2 g for K of global tile g, 2 g + 1 for V
         const int s = u % kRing;
@@ -772,7 +764,7 @@ attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       uint32_t sv = 1, sk = 2, pk = 8;
       uint32_t pph = 0;
       auto issue_qk = [&](int x, uint32_t slot) {                   // S_x = Q_x K^T with the K tile in `slot`
-        mma_ss_kloop<kHalves>(tmem_base + x * 128, desc_lo(q_smem + x * L::kTileBytes, 16), desc_lo(kv_smem + slot * L::kTileBytes, 16),
+        mma_ss_kloop<kHalves>(tmem_base + x * 128, desc_lo(q_smem + x * kHalfBytes, 16), desc_lo(kv_smem + slot * L::kTileBytes, 16),
                               desc_hi_sw128(1024), idesc_qk);
         mma_commit(bar_sfull + 8 * x);
       };
@@ -888,8 +880,7 @@ attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
     reg_alloc<224>();
     // ================= softmax + epilogue =================
     const int x = warp >> 2;
-    const int row = threadIdx.x & 127;
-    const int t_local = row / G, j_head = row - t_local * G;
+    const int t_local = (int)threadIdx.x / G, j_head = (int)threadIdx.x - t_local * G;      // flat rows of the pair: tile A, then B
     const uint32_t lane_base = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
     const uint32_t t_s = lane_base + x * 128, t_o = lane_base + 256 + x * 128;
     const uint32_t my_sfull = bar_sfull + 8 * x, my_pfull = bar_pfull + 8 * x;
@@ -907,8 +898,8 @@ attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
     // this thread's row of item k: validity and the load of its context rank
     auto row_rank = [&](uint32_t k, bool& valid) -> int {
       const int4 a = rec_ld(k, 0), b = rec_ld(k, 1), cc = rec_ld(k, 2);
-      valid = a.x > 0 && (row < tile_targets * G) && (t_local < (x ? b.y : b.x));
-      return valid ? r_rank[cc.z + cc.w + x * tile_targets + t_local] : 0;
+      valid = a.x > 0 && t_local < b.x;
+      return valid ? r_rank[cc.z + cc.w + t_local] : 0;
     };
     bool ok = wait_rec(0);
     bool row_valid = false;
@@ -960,8 +951,8 @@ attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
         const float lse = none ? -INFINITY : (m + log2f(z)) * kLn2A;
         const int4 b = rec_ld(k, 1);
         const int hd = b.z;
-        const long long orow = (long long)b.w + x * tile_targets + t_local;
-        uint16_t* optr = out + (orow * H + hd * G + j_head) * D;
+        const long long orow = (long long)b.w + t_local;
+        uint16_t* optr = out + ((long long)orow * H + hd * G + j_head) * D;
 #pragma unroll
         for (int cc = 0; cc < D / 32; ++cc) {
           uint32_t o[32];
@@ -1183,16 +1174,19 @@ static relaxkv_status launch_attention(const relaxkv_shape* shape, int mode, Att
                                        const int32_t* r_cu_layer, long long n_target_rows, void* out, float* lse_out,
                                        cudaStream_t stream, int allow_empty = 0) {
   const int H = shape->n_q_heads, Hkv = shape->n_kv_heads, G = H / Hkv;
-  const int tile_targets = kBM / G;
+  // A pair of query tiles is 256 rows: whole targets with the G heads of a KV head each, the one in the middle with heads in both tiles
+  // where 128 is no multiple of G.  Five heads: 51 targets; with 25 in each tile, 2 % more pairs, 12 repaired layers of 40 / 8 heads at
+  // 32 K took 36.09 ms, now 35.71, four of eight requests of 8 to 64 K 49.65 / 49.04.
+  const int pair_targets = 2 * kBM / G;
   const int B = shape->n_req;
   for (int b = 0; b < B; ++b)     // tile_cu counts the launch units per request: PAIRS of query tiles
-    plan.rt.tile_cu[b + 1] = plan.rt.tile_cu[b] + (plan.rt.bound_a[b] + 2 * tile_targets - 1) / (2 * tile_targets);
+    plan.rt.tile_cu[b + 1] = plan.rt.tile_cu[b] + (plan.rt.bound_a[b] + pair_targets - 1) / pair_targets;
   const long long grid = (long long)plan.rt.tile_cu[B] * Hkv;
   if (grid == 0) return RELAXKV_OK;
   if (grid > 0x7fffffffLL) return RELAXKV_ERR_UNSUPPORTED_SHAPE;
   CUtensorMap tm_q, tm_k, tm_v;
   const uint64_t row_q = (uint64_t)H * D * 2, row_kv = (uint64_t)Hkv * D * 2;
-  if (!make_map_3d(&tm_q, q_new, D, H, (uint64_t)n_target_rows, (uint64_t)D * 2, row_q, (uint32_t)G, (uint32_t)tile_targets) ||
+  if (!make_map_3d(&tm_q, q_new, D, H, (uint64_t)n_target_rows, (uint64_t)D * 2, row_q, (uint32_t)G, (uint32_t)pair_targets) ||
       !make_map_3d(&tm_k, plan.k_base, D, Hkv, (uint64_t)plan.ctx_rows, plan.kv_head_stride_bytes, plan.kv_token_stride_bytes, 1u,
                    (uint32_t)kBN) ||
       !make_map_3d(&tm_v, plan.v_base, D, Hkv, (uint64_t)plan.ctx_rows, plan.kv_head_stride_bytes, plan.kv_token_stride_bytes, 1u,
@@ -1247,12 +1241,12 @@ static relaxkv_status launch_attention(const relaxkv_shape* shape, int mode, Att
     if (tun && tun->attention_grid_blocks > 0) pgrid = std::min<long long>(grid, tun->attention_grid_blocks);
     RELAXKV_RANGE("attention_persist_kernel");
     return cuda_ok(launch_chained(pk, (unsigned)pgrid, kAttnThreads, PersistSmem<D>::kDynamic, stream,
-        tm_q, tm_k, tm_v, plan.rt, mode, allow_empty, head_inner, H, Hkv, tile_targets, shape->softmax_scale * kLog2eA,
+        tm_q, tm_k, tm_v, plan.rt, mode, allow_empty, head_inner, H, Hkv, pair_targets, shape->softmax_scale * kLog2eA,
         u_pos, u_cu, r_rank, r_cu_layer, n_target_rows, static_cast<uint16_t*>(out), lse_out, (int)grid, counter, st));
   }
   RELAXKV_RANGE("attention_sm100_kernel");
   relaxkv_status rc = cuda_ok(launch_chained(kern, dim3((unsigned)grid, (unsigned)n_splits), kAttnThreads, AttnSmem<D>::kDynamic, stream,
-      tm_q, tm_k, tm_v, plan.rt, mode, allow_empty, head_inner, plan.dense_ctx, H, Hkv, tile_targets, shape->softmax_scale * kLog2eA,
+      tm_q, tm_k, tm_v, plan.rt, mode, allow_empty, head_inner, plan.dense_ctx, H, Hkv, pair_targets, shape->softmax_scale * kLog2eA,
       u_pos, u_cu, r_rank, r_cu_layer, n_target_rows, static_cast<uint16_t*>(out), lse_out, plan.split_o, plan.split_lse, st));
   if (rc != RELAXKV_OK || n_splits == 1) return rc;
   return launch_combine_splits(plan.split_o, plan.split_lse, (int)n_splits, n_target_rows, H, D, r_cu_layer, B, plan.sum_targets,

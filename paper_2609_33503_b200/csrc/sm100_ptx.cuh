@@ -195,8 +195,13 @@ __device__ __forceinline__ uint32_t desc_lo(uint32_t smem_addr, uint32_t lbo_byt
   "mov.b64 da, {ta, %3};\n\tmov.b64 db, {tb, %3};\n\t"                                           \
   "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, " #PRED ";\n\t"
 
-// D[tmem] = A[smem] * B[smem] over K = 64 * HALVES (both operands K-major, 128B swizzle, halves 16 KB apart
-// for A when a_half_step16 = 1024 and for B when the same): the first MMA overwrites D.
+#define RELAXKV_MMA_SS_STEP2(AOFF, BOFF, PRED)                                                 \
+  "add.u32 ta, %1, " #AOFF ";\n\tadd.u32 tb, %2, " #BOFF ";\n\t"                                  \
+  "mov.b64 da, {ta, %3};\n\tmov.b64 db, {tb, %3};\n\t"                                           \
+  "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, " #PRED ";\n\t"
+
+// D[tmem] = A[smem] * B[smem] over K = 64 * HALVES (both operands K-major, 128B swizzle, halves 32 KB apart for A, two tiles of
+// 128 rows behind each other, and 16 KB for B): the first MMA overwrites D.
 template <int HALVES>
 __device__ __forceinline__ void mma_ss_kloop(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc) {
   if (HALVES == 2) {
@@ -204,7 +209,8 @@ __device__ __forceinline__ void mma_ss_kloop(uint32_t d_tmem, uint32_t a_lo, uin
         "{\n\t.reg .pred p0, p1;\n\t.reg .b32 ta, tb;\n\t.reg .b64 da, db;\n\t"
         "setp.ne.b32 p0, 0, 0;\n\tsetp.eq.b32 p1, 0, 0;\n\t"
         RELAXKV_MMA_SS_STEP(0, p0) RELAXKV_MMA_SS_STEP(2, p1) RELAXKV_MMA_SS_STEP(4, p1) RELAXKV_MMA_SS_STEP(6, p1)
-        RELAXKV_MMA_SS_STEP(1024, p1) RELAXKV_MMA_SS_STEP(1026, p1) RELAXKV_MMA_SS_STEP(1028, p1) RELAXKV_MMA_SS_STEP(1030, p1)
+        RELAXKV_MMA_SS_STEP2(2048, 1024, p1) RELAXKV_MMA_SS_STEP2(2050, 1026, p1) RELAXKV_MMA_SS_STEP2(2052, 1028, p1)
+        RELAXKV_MMA_SS_STEP2(2054, 1030, p1)
         "}" ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc) : "memory");
   } else {
     asm volatile(

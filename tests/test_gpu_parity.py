@@ -1213,3 +1213,26 @@ def test_other_geometries_and_head_major_cache(H, Hkv, D, head_major):
         for full_prefix in (False, True):
             out, lse = run_attention(case, s, l, B().CTX_FULL_PREFIX if full_prefix else B().CTX_UNION, simt=False)
             check_attention(case, l, out, lse, full_prefix)
+
+
+@pytest.mark.parametrize("G,D", [(1, 64), (3, 128), (5, 128), (7, 64), (11, 128), (16, 64)])
+def test_targets_at_the_edges_of_a_pair_of_query_tiles(G, D):
+    """A pair of query tiles is 256 rows of floor(256 / G) whole targets; where 128 is no multiple of G one target has heads in both
+    tiles.  Target counts around one tile, one pair and two, all three forms of the launch."""
+    pair = 256 // G
+    for n in sorted({1, 128 // G, 128 // G + 1, pair - 1, pair, pair + 1, 2 * pair, 2 * pair + 1}):
+        w = inputs.Workload("pairs", 1, 2 * G, 2, D, 64, (600,), (4,), 0.1, base_seed=n)
+        pos = np.sort(np.random.default_rng(n).choice(600, n, replace=False)).astype(np.int32)
+        case = Case(w, anchors_override=[[pos]])
+        case.k = [n]
+        s = case.make_session()
+        s.build_active_sets(case.anchors_tensor())
+        outs = []
+        for tuning in (dict(attention_ctx_splits=1, attention_persistent=2), dict(attention_ctx_splits=1, attention_persistent=1),
+                       dict(attention_ctx_splits=3)):
+            s.shape.set_tuning(**tuning)
+            for full_prefix in (False, True):
+                out, lse = run_attention(case, s, 0, B().CTX_FULL_PREFIX if full_prefix else B().CTX_UNION, simt=False)
+                check_attention(case, 0, out, lse, full_prefix)
+                outs.append(out)
+        assert torch.equal(outs[0], outs[2]) and torch.equal(outs[1], outs[3])
