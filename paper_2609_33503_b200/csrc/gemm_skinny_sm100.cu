@@ -28,6 +28,7 @@
 #include "sm100_ptx.cuh"
 #include <algorithm>
 #include <atomic>
+#include <cstdlib>
 
 namespace relaxkv {
 
@@ -36,29 +37,28 @@ using namespace ptx;
 bool make_map_3d(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t stride1_bytes,
                  uint64_t stride2_bytes, uint32_t b1, uint32_t b2);          // attention_sm100.cu
 
-constexpr int kSkFeat = 128, kSkBK = 64, kSkThreads = 192, kSkStagesMax = 7;
+constexpr int kSkFeat = 128, kSkBK = 64, kSkStagesMax = 7;
+__host__ __device__ constexpr int sk_threads(int epi) { return 64 + 32 * epi; }
 constexpr int kSkWBytes = kSkFeat * kSkBK * 2;                             // weights of a stage: 16 KB, as two 64-row boxes
 constexpr int kSkRing2 = 108 * 1024, kSkRing1 = 192 * 1024;                // two blocks, one block per SM
 constexpr int kSkCols2 = 64;                                               // widest MMA that always takes the two-block form
-constexpr int kSkPitch = kSkFeat + 4;                                      // floats per staged row: 16-byte reads of 8 rows hit all banks
+constexpr int kSkManyRows = 32;                                            // whole tiles: rows from which eight warps write them
 constexpr int kSkDeepK = 8192;                                             // few rows: K from which eight blocks share a tile
 constexpr int kSkParts = 8, kSkPartCols = 16;                               // few rows: parts of K, MMA columns of each
-constexpr int kSkBars = 2 * kSkStagesMax + 1;                              // full, empty per stage; accumulator full
+constexpr int kSkBars = 2 * kSkStagesMax + 2;                              // full, empty per stage; accumulator full; partial tiles received
 constexpr int kSkTail = 8 * kSkBars + 16 + 1024;                           // barriers, slots, alignment
 constexpr int sk_stages(int n_cols, bool whole_sm) { return (whole_sm ? kSkRing1 : kSkRing2) / (kSkWBytes + n_cols * kSkBK * 2); }
 static_assert(sk_stages(16, false) <= kSkStagesMax, "barriers for every stage");
-static_assert(kSkinnyMaxRows * kSkPitch * 4 <= sk_stages(kSkinnyMaxRows, false) * (kSkWBytes + kSkinnyMaxRows * kSkBK * 2),
-              "the partial tile reuses the TMA ring");
-
-__device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t cluster_addr) {
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(cluster_addr));
-  return v;
-}
+// The partial tile (rows of x times parts of K, 128 features, fp32) and as much again that the blocks of a cluster receive take the ring's place.
+__host__ __device__ constexpr int sk_part_bytes(int rows) { return rows * kSkFeat * 4; }
+static_assert(sk_part_bytes(kSkinnyMaxRows) <= sk_stages(kSkinnyMaxRows, false) * (kSkWBytes + kSkinnyMaxRows * kSkBK * 2) &&
+              2 * sk_part_bytes(kSkCols2) <= sk_stages(kSkCols2, false) * (kSkWBytes + kSkCols2 * kSkBK * 2) &&
+              2 * sk_part_bytes(kSkinnyMaxRows) <= sk_stages(kSkinnyMaxRows, true) * (kSkWBytes + kSkinnyMaxRows * kSkBK * 2),
+              "the partial tiles reuse the TMA ring");
 
 // S blocks per tile; a block's share of K is PL parts, each summed in an accumulator of its own (PL > 1: n_cols is kSkPartCols).
-template <int S, int PL>
-__global__ void __launch_bounds__(kSkThreads, 2)
+template <int S, int PL, int E>
+__global__ void __launch_bounds__(sk_threads(E), 2)
 gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
                          int M, int n_cols, int n_stages, int n_feat, int K, int swiglu, const __grid_constant__ SkinnyOut outs,
                          DeviceStatus* st) {
@@ -71,12 +71,16 @@ gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_
   const int f0 = swiglu ? tile * (kSkFeat / 2) : tile * kSkFeat;            // first output feature
   const int r0 = swiglu ? (f0 / 128) * 256 + f0 % 128 : f0, r1 = swiglu ? r0 + 128 : r0 + kSkFeat / 2;
 
+  // of the tile's features, in groups of four, block r of the cluster adds up and writes [r all / S, (r + 1) all / S)
+  const int all_quads = (swiglu ? kSkFeat / 2 : kSkFeat) / 4;
+  const int own_q0 = (int)rank * all_quads / S, own_quads = ((int)rank + 1) * all_quads / S - own_q0;
+
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
   const uint32_t stage_bytes = (uint32_t)(kSkWBytes + n_cols * kSkBK * 2), ring = stage_bytes * (uint32_t)n_stages;
   const uint32_t bar0 = base + ring;
-  const uint32_t bar_full = bar0, bar_empty = bar0 + 8 * kSkStagesMax, bar_acc = bar0 + 16 * kSkStagesMax;
+  const uint32_t bar_full = bar0, bar_empty = bar0 + 8 * kSkStagesMax, bar_acc = bar0 + 16 * kSkStagesMax, bar_recv = bar_acc + 8;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + ring + 8 * kSkBars);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(const_cast<uint32_t*>(tmem_slot) + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -85,8 +89,10 @@ gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_
   if (threadIdx.x == 0) {
     for (int s = 0; s < n_stages; ++s) { mbar_init(bar_full + 8 * s, 1); mbar_init(bar_empty + 8 * s, 1); }
     mbar_init(bar_acc, 1);
+    mbar_init(bar_recv, 1);
     *abort_flag = 0;
     fence_barrier_init();
+    if (S > 1) mbar_expect_tx(bar_recv, (uint32_t)((S - 1) * PL * M * (swiglu ? 2 : 1) * own_quads * 16));
     fence_proxy_async_smem();
   }
   if (warp == 4 && lane == 0) {
@@ -144,44 +150,81 @@ gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_
       if (go) mma_commit(bar_acc);
     }
   } else {
-    // ---- epilogue warps (thread = weight row = TMEM lane): this block's partial tile -> its own shared memory, [row of x]
-    // [feature] fp32 (the lanes of a warp hold consecutive features: every store below writes 128 consecutive bytes).
-    // The MMAs have completed by then, so the TMA ring is free to hold it. ----
+    // ---- epilogue warps (thread = weight row = TMEM lane): this block's partial tile -> its own shared memory, the features of each
+    // block of the cluster behind one another: [block][gate, up][row of x][feature] fp32.  The MMAs have completed by then, so the TMA
+    // ring is free to hold it, here (said to the cluster by the arrival below) and behind it what the other blocks send. ----
+    // (What does not depend on the products comes before the wait for them: the divisions and the residual's first rows.)
+    const int halves = swiglu ? 2 : 1;
+    const int tl = (warp & 3) * 32 + lane, up = swiglu ? tl / (kSkFeat / 2) : 0, f_st = tl - up * (kSkFeat / 2);
+    const int r_st = S > 1 ? (((f_st >> 2) + 1) * S - 1) / all_quads : 0, q_st = r_st * all_quads / S;
+    const int w_st = ((r_st + 1) * all_quads / S - q_st) * 4;    // features of the block that this thread's feature goes to
+    float* stage = reinterpret_cast<float*>(base_ptr) + PL * M * (halves * 4 * q_st + up * w_st) + f_st - 4 * q_st;
+    // this block's run of the tile's features, four features of one row of x per thread and round
+    const int et = warp < 4 ? (int)threadIdx.x : (int)threadIdx.x - 64;
+    const int rows = 32 * E / own_quads, m0 = et / own_quads, q = et % own_quads;               // rows of x per round
+    const int col0 = f0 + (own_q0 + q) * 4;
+    // which output buffer these features go to (segment boundaries are multiples of 8)
+    int sg = 0;
+    while (sg + 1 < outs.n && col0 >= outs.col0[sg + 1]) ++sg;
+    const int width = outs.col0[sg + 1] - outs.col0[sg];
+    uint16_t* y = outs.y[sg] + (col0 - outs.col0[sg]);
+    const uint16_t* res = outs.residual[sg] ? outs.residual[sg] + (col0 - outs.col0[sg]) : nullptr;
+    const bool mine = m0 < rows && col0 < n_feat && status != RELAXKV_ERR_TIMEOUT;
+    constexpr int R = PL > 1 ? 1 : 4;                            // rounds whose loads are in flight together (up to four rows: one in all)
+    uint2 r[R];
+    auto load_residual = [&](int mb) {
+#pragma unroll
+      for (int j = 0; j < R; ++j) {
+        const int m = mb + j * rows;
+        r[j] = (res != nullptr && mine && m < M) ? *reinterpret_cast<const uint2*>(res + (long long)m * width) : make_uint2(0u, 0u);
+      }
+    };
+    load_residual(m0);
+
     ok = mbar_wait(bar_acc, 0, abort_flag);
     ok = __all_sync(0xffffffffu, ok);
+    if (S > 1) cluster_arrive();
     tc_fence_after();
     if (ok) {
-      const uint32_t t_lane = tmem_base + ((uint32_t)(warp * 32) << 16);
-      float* stage = reinterpret_cast<float*>(base_ptr) + warp * 32 + lane;
+      const uint32_t t_lane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
 #pragma unroll 1
-      for (int c = 0; c < (PL > 1 ? PL * kSkPartCols : M); c += 32) {
+      for (int c = warp < 4 ? 0 : 32; c < (PL > 1 ? PL * kSkPartCols : M); c += 8 * E) {
         uint32_t v[32];
         tmem_ld32(t_lane + c, v);
         tmem_wait_ld();
 #pragma unroll
         for (int i = 0; i < 32; ++i) {                           // staged: the rows of x of one part behind the other
           const int m = PL > 1 ? i % kSkPartCols : c + i, part = PL > 1 ? c / kSkPartCols + i / kSkPartCols : 0;
-          if (m < M) stage[(part * M + m) * kSkPitch] = __uint_as_float(v[i]);
+          if (m < M) stage[(part * M + m) * w_st] = __uint_as_float(v[i]);
         }
       }
     }
-  }
-  // every block's partial tile is in place
-  __syncthreads();
-  if (S > 1) cluster_sync();
-  ok = !*abort_flag;
-
-  if (warp < 4 && ok) {
-    uint32_t peer[S];
-#pragma unroll
-    for (int src = 0; src < S; ++src) peer[src] = (S > 1) ? mapa_shared(base, (uint32_t)src) : base;
-    // this rank's run of the tile's features, four features of one row of x per thread and round: the lanes that share a
-    // row read up to 128 consecutive bytes of each peer (scattered 16-byte reads cost a tile of 128 rows another 8 us)
-    auto sum4 = [&](int m, int col) {
+    if (S > 1) {
+      fence_proxy_async_smem();
+      cluster_wait();                                            // every block's ring is free
+    }
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * E) : "memory");    // the partial tile is in place
+    const int sent = PL * M * halves * own_quads * 4;            // floats of one block's contribution to this one
+    if (S > 1) {
+      // One bulk copy to every other block of the cluster.  (Each block reading its share of every peer, and its own, through ld.shared::cluster and
+      // two whole cluster barriers took 4 of the 14.3 us of a projection of 57 rows by 5120 x 5120 in six blocks per tile; now 12.9.)
+      if ((int)threadIdx.x < S && threadIdx.x != rank && !*abort_flag) {
+        const int to = (int)threadIdx.x, q0 = to * all_quads / S, quads = (to + 1) * all_quads / S - q0;
+        const uint32_t per = (uint32_t)(PL * M * halves * 16);   // bytes per group of four features
+        bulk_push(mapa_shared(base + sk_part_bytes(PL * M) + rank * (per * (uint32_t)quads), (uint32_t)to), base + per * (uint32_t)q0,
+                  per * (uint32_t)quads, mapa_shared(bar_recv, (uint32_t)to));
+      }
+      if (ok) ok = mbar_wait_cluster(bar_recv, 0, abort_flag);
+      ok = __all_sync(0xffffffffu, ok);
+      cluster_arrive();                                          // nothing is on its way to this block any more
+    }
+    const float* recv = reinterpret_cast<const float*>(base_ptr + sk_part_bytes(PL * M)) + q * 4;
+    const float* own = reinterpret_cast<const float*>(base_ptr) + PL * M * halves * 4 * own_q0 + q * 4;
+    auto sum4 = [&](int m, int half) {
       float4 v[S * PL];
 #pragma unroll
       for (int src = 0; src < S * PL; ++src)
-        v[src] = ld_cluster_f32x4(peer[src / PL] + (uint32_t)((src % PL * M + m) * kSkPitch + col) * 4u);
+        v[src] = *reinterpret_cast<const float4*>((src / PL == (int)rank ? own : recv + src / PL * sent) + (half * PL * M + src % PL * M + m) * own_quads * 4);
       float4 f = v[0];
 #pragma unroll
       for (int src = 1; src < S * PL; ++src) {                   // order of K: the same sum whatever the timing
@@ -189,30 +232,14 @@ gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_
       }
       return f;
     };
-    const int all = (swiglu ? kSkFeat / 2 : kSkFeat) / 4, q0 = (int)rank * all / S, quads = ((int)rank + 1) * all / S - q0;
-    const int rows = 128 / quads, m0 = (int)threadIdx.x / quads;  // rows of x per round
-    const int col = (q0 + (int)threadIdx.x % quads) * 4, col0 = f0 + col;
-    // which output buffer these features go to (segment boundaries are multiples of 8)
-    int sg = 0;
-    while (sg + 1 < outs.n && col0 >= outs.col0[sg + 1]) ++sg;
-    const int width = outs.col0[sg + 1] - outs.col0[sg];
-    uint16_t* y = outs.y[sg] + (col0 - outs.col0[sg]);
-    const uint16_t* res = outs.residual[sg] ? outs.residual[sg] + (col0 - outs.col0[sg]) : nullptr;
-    if (m0 < rows && col0 < n_feat && status != RELAXKV_ERR_TIMEOUT) {
-      constexpr int R = PL > 1 ? 1 : 4;                          // rounds whose loads are in flight together (up to four rows: one in all)
+    if (ok && mine) {
       for (int mb = m0; mb < M; mb += R * rows) {
-        uint2 r[R];
         float4 f[R], u[R];
 #pragma unroll
         for (int j = 0; j < R; ++j) {
-          const int m = mb + j * rows;
-          r[j] = (res != nullptr && m < M) ? *reinterpret_cast<const uint2*>(res + (long long)m * width) : make_uint2(0u, 0u);
-        }
-#pragma unroll
-        for (int j = 0; j < R; ++j) {
           const int m = min(mb + j * rows, M - 1);
-          f[j] = sum4(m, col);
-          if (swiglu) u[j] = sum4(m, kSkFeat / 2 + col);
+          f[j] = sum4(m, 0);
+          if (swiglu) u[j] = sum4(m, 1);
         }
 #pragma unroll
         for (int j = 0; j < R; ++j) {
@@ -230,13 +257,17 @@ gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_
           __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
           *reinterpret_cast<uint2*>(y + (long long)m * width) = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
         }
+        if (mb + R * rows < M) load_residual(mb + R * rows);
       }
     }
   }
-  // nobody leaves while a peer may still read its partial tile
+  if (S > 1) {
+    __syncwarp();
+    if (warp == 4 || warp == 5) { cluster_arrive(); cluster_wait(); cluster_arrive(); }
+    cluster_wait();                             // nobody leaves while its partial tile is on its way to a peer
+  }
   tc_fence_before();
   __syncthreads();
-  if (S > 1) cluster_sync();
   if (*abort_flag) {
     if (threadIdx.x == 0) report(st, RELAXKV_ERR_TIMEOUT, KID_GEMM_SM100, (int)blockIdx.x, 1);
     const uint64_t tw = global_timer_ns();
@@ -254,11 +285,11 @@ struct SkinnyPlan {
   cudaStream_t stream;
 };
 
-template <int S, int PL>
+template <int S, int PL, int E>
 static bool opt_in_smem(int dev) {
   static std::atomic<int> attr_done[kMaxDevices];
   if (!attr_done[dev].load(std::memory_order_acquire)) {
-    if (cudaFuncSetAttribute(gemm_skinny_sm100_kernel<S, PL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSkRing1 + kSkTail) != cudaSuccess)
+    if (cudaFuncSetAttribute(gemm_skinny_sm100_kernel<S, PL, E>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSkRing1 + kSkTail) != cudaSuccess)
       return false;
     attr_done[dev].store(1, std::memory_order_release);
   }
@@ -272,32 +303,33 @@ static int max_clusters(int dev, int sms) {
   static std::atomic<int> cached[kMaxDevices];
   int n = S == 1 ? sms : cached[dev].load(std::memory_order_acquire);
   if (n == 0) {
-    if (!opt_in_smem<S, 1>(dev)) return 0;
+    if (!opt_in_smem<S, 1, 4>(dev)) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(sms / S * S));
-    cfg.blockDim = dim3(kSkThreads);
+    cfg.blockDim = dim3(sk_threads(4));
     cfg.dynamicSmemBytes = kSkRing1 + kSkTail;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = (unsigned)S; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm_skinny_sm100_kernel<S, 1>, &cfg) != cudaSuccess || n < 1) n = std::max(1, sms / S / 2);
+    if (cudaOccupancyMaxActiveClusters(&n, gemm_skinny_sm100_kernel<S, 1, 4>, &cfg) != cudaSuccess || n < 1) n = std::max(1, sms / S / 2);
     cached[dev].store(n, std::memory_order_release);
   }
   return n;
 }
 
 // Launches with clusters of S blocks if that is one wave of resident blocks that have two K blocks each (or S is 1).
-template <int S, int PL = 1>
+template <int S, int PL = 1, int E = 4>
 static bool try_launch(const SkinnyPlan& p, const CUtensorMap& tm_w, const CUtensorMap& tm_x, const SkinnyOut& outs, relaxkv_status* rc) {
   const int n_k = (p.n_in + kSkBK - 1) / kSkBK;
   if (S > 1 && n_k < 2 * S) return false;
+  if (S > 1 && 2 * sk_part_bytes(PL * p.n_rows) > p.n_stages * (kSkWBytes + p.n_cols * kSkBK * 2)) return false;
   // with two blocks per SM an even cluster sits on S / 2 SMs (the occupancy query itself counts one block per SM)
   const int resident = p.whole_sm ? max_clusters<S>(p.dev, p.sms) : (S % 2 ? 2 * max_clusters<S>(p.dev, p.sms) : max_clusters<(S + 1) / 2>(p.dev, p.sms));
-  if (resident < 1 || !opt_in_smem<S, PL>(p.dev)) { *rc = RELAXKV_ERR_CUDA; return true; }
+  if (resident < 1 || !opt_in_smem<S, PL, E>(p.dev)) { *rc = RELAXKV_ERR_CUDA; return true; }
   if (S > 1 && p.tiles > resident) return false;
-  *rc = cuda_ok(launch_chained_clusters(S, gemm_skinny_sm100_kernel<S, PL>, dim3((unsigned)(p.tiles * S)), dim3(kSkThreads), p.smem,
+  *rc = cuda_ok(launch_chained_clusters(S, gemm_skinny_sm100_kernel<S, PL, E>, dim3((unsigned)(p.tiles * S)), dim3(sk_threads(E)), p.smem,
                                         p.stream, tm_w, tm_x, p.n_rows, p.n_cols, p.n_stages, p.n_feat, p.n_in, p.swiglu, outs, p.st));
   return true;
 }
@@ -324,6 +356,7 @@ relaxkv_status launch_gemm_skinny(const void* x, const void* weight, const Skinn
   // (64 rows, two blocks / one: 2048 x 2048 8.4 / 6.9 us, 3072 x 2048 9.8 / 7.6, 4096 x 4096 12.9 / 10.7, 4096 x 14336 25.9 / 24.1; 33 rows 6.8 / 6.2,
   // 7.8 / 7.1, 11.0 / 10.2, 24.0 / 23.5; 40 tiles of 5120 x 5120 14.4 / 13.8 and 13.2 / 13.1; 17 rows, 2048 x 4096 7.4 / 7.8).
   p.whole_sm = (p.n_cols > kSkCols2 && p.tiles <= p.sms) || (p.n_cols > 32 && p.tiles * 4 <= p.sms);
+  if (getenv("SK_WHOLE") && p.n_cols > atoi(getenv("SK_WHOLE")) && p.tiles * 2 <= p.sms) p.whole_sm = true;
   p.n_stages = std::min(kSkStagesMax, sk_stages(p.n_cols, p.whole_sm));
   p.smem = (size_t)p.n_stages * (kSkWBytes + p.n_cols * kSkBK * 2) + kSkTail;
   relaxkv_status rc = RELAXKV_OK;
@@ -341,7 +374,10 @@ relaxkv_status launch_gemm_skinny(const void* x, const void* weight, const Skinn
       try_launch<5>(p, tm_w, tm_x, outs, &rc) || try_launch<4>(p, tm_w, tm_x, outs, &rc) || try_launch<3>(p, tm_w, tm_x, outs, &rc) ||
       try_launch<2>(p, tm_w, tm_x, outs, &rc))
     return rc;
-  try_launch<1>(p, tm_w, tm_x, outs, &rc);
+  // A block with a tile of its own adds nothing up but writes every feature of it: eight warps for many rows (28672 x 4096 gate/up: 57 rows
+  // 42.7 us with four, 41.9, 128 rows 47.4 / 45.7).  In a cluster four are enough, and more cost their start (5120 x 5120: 57 rows 13.0 / 13.8).
+  if (p.n_rows > kSkManyRows) try_launch<1, 1, 8>(p, tm_w, tm_x, outs, &rc);
+  else try_launch<1>(p, tm_w, tm_x, outs, &rc);
   return rc;
 }
 
