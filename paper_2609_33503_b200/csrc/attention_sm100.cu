@@ -88,6 +88,16 @@ __device__ __forceinline__ void softmax_keys(uint32_t t_s, const uint32_t* s, fl
   }
 }
 
+// 16 bf16 values of an output row; as one sector where the output is 32-byte aligned (the call asks for 16).
+__device__ __forceinline__ void store_16(uint16_t* p, const uint32_t* w, bool sectors) {
+  if (sectors) {
+    st_global_32b(p, w);
+  } else {
+    reinterpret_cast<uint4*>(p)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    reinterpret_cast<uint4*>(p)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+  }
+}
+
 // One step of a query row's online softmax (thread = query row = TMEM lane): S_x(j) is read from TMEM, the keys
 // past the row's limit (counted from the tile's first key) are masked on the tiles that straddle the staircase,
 // the running maximum m and sum z are updated (O_x is rescaled only when the maximum grew by more than the
@@ -444,6 +454,7 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       const int orow = q_row_base + t_local;
       if (n_splits == 1) {
         uint16_t* optr = out + ((long long)orow * H + hd * G + j_head) * D;
+        const bool sectors = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;
 #pragma unroll
         for (int c = 0; c < D / 32; ++c) {
           uint32_t o[32];
@@ -451,16 +462,15 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           tmem_wait_ld();
           if (row_valid) {
 #pragma unroll
-            for (int i = 0; i < 32; i += 8) {
-              uint32_t w[4];
+            for (int i = 0; i < 32; i += 16) {
+              uint32_t w[8];
 #pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(o[i + 2 * e]) * inv,
-                                                          __uint_as_float(o[i + 2 * e + 1]) * inv);
-                w[e] = *reinterpret_cast<uint32_t*>(&h2);
+              for (int e = 0; e < 8; ++e) {
+                __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(o[i + 2 * e]) * inv, __uint_as_float(o[i + 2 * e + 1]) * inv);
+                // a row of an empty context is zero whatever the keys gave it (0 x NaN is not)
+                w[e] = row_empty ? 0u : *reinterpret_cast<uint32_t*>(&h2);
               }
-              // a row of an empty context is zero whatever the keys gave it (0 x NaN is not)
-              *reinterpret_cast<uint4*>(optr + c * 32 + i) = row_empty ? make_uint4(0, 0, 0, 0) : make_uint4(w[0], w[1], w[2], w[3]);
+              store_16(optr + c * 32 + i, w, sectors);
             }
           }
         }
@@ -476,10 +486,9 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           tmem_wait_ld();
           if (row_valid) {
 #pragma unroll
-            for (int i = 0; i < 32; i += 4)
-              *reinterpret_cast<float4*>(optr + c * 32 + i) =
-                  make_float4(__uint_as_float(o[i]) * inv, __uint_as_float(o[i + 1]) * inv, __uint_as_float(o[i + 2]) * inv,
-                              __uint_as_float(o[i + 3]) * inv);
+            for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * inv);
+#pragma unroll
+            for (int i = 0; i < 32; i += 8) st_global_32b(optr + c * 32 + i, o + i);      // (the workspace is 256-byte aligned)
           }
         }
         if (row_valid) part_lse[slot] = lse;
@@ -953,6 +962,7 @@ attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
         const int hd = b.z;
         const long long orow = (long long)b.w + t_local;
         uint16_t* optr = out + ((long long)orow * H + hd * G + j_head) * D;
+        const bool sectors = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;
 #pragma unroll
         for (int cc = 0; cc < D / 32; ++cc) {
           uint32_t o[32];
@@ -960,14 +970,15 @@ attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
           tmem_wait_ld();
           if (row_valid) {
 #pragma unroll
-            for (int i = 0; i < 32; i += 8) {
-              uint32_t w[4];
+            for (int i = 0; i < 32; i += 16) {
+              uint32_t w[8];
 #pragma unroll
-              for (int e = 0; e < 4; ++e) {
+              for (int e = 0; e < 8; ++e) {
                 __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(o[i + 2 * e]) * inv, __uint_as_float(o[i + 2 * e + 1]) * inv);
-                w[e] = *reinterpret_cast<uint32_t*>(&h2);
+                // a row of an empty context is zero whatever the keys gave it (0 x NaN is not)
+                w[e] = row_empty ? 0u : *reinterpret_cast<uint32_t*>(&h2);
               }
-              *reinterpret_cast<uint4*>(optr + cc * 32 + i) = row_empty ? make_uint4(0, 0, 0, 0) : make_uint4(w[0], w[1], w[2], w[3]);
+              store_16(optr + cc * 32 + i, w, sectors);
             }
           }
         }
