@@ -43,6 +43,7 @@ constexpr int kHalfBytes = 128 * 128;         // 128 rows x 64 bf16: one 128B-sw
 constexpr int kPLo = 3;
 constexpr int kRing = 5;                      // K/V tile buffers, used in the order K0 V0 K1 V1 ...
 constexpr int kNoLimit = 0x7fffffff;          // causal limit of a row that nobody reads: no tile is masked for it
+constexpr int kL2Tiles = 5;                     // query calls: key tiles of a block requested into L2 before its wait
 constexpr int kPersistMaxTiles = 128;          // contexts up to this many key tiles take the persistent form
 constexpr int kAttnThreads = 384;             // 2 x 4 softmax warps + a control warpgroup (TMA warp, MMA warp, 2 idle)
 
@@ -174,15 +175,83 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const int B = rt.n_req;
   const int G = H / Hkv;
   const int n_pairs_total = rt.tile_cu[B];
+  // ---- shared memory -----------------------------------------------------------------------------
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
+  const uint32_t q_smem = base + L::kQ, kv_smem = base + L::kKV;
+  const uint32_t bar0 = base + L::kBar;
+  const uint32_t bar_q = bar0;
+  const uint32_t bar_sfull = bar0 + 8;          // [2]
+  const uint32_t bar_pfull = bar0 + 24;         // [2] first 32 kPLo keys of P ready
+  const uint32_t bar_pfull_hi = bar0 + 40;      // [2] the other keys of P ready
+  const uint32_t bar_ofinal = bar0 + 56;        // [2]
+  const uint32_t bar_full = bar0 + 72;          // [kPairBars] pair p = (V_{p-1}, K_p) has landed
+  const uint32_t bar_empty = bar_full + 8 * L::kPairBars;   // [kPairBars] pair p has been consumed by both tiles
+  const uint32_t bar_vreq = bar_empty + 8 * L::kPairBars;   // the request's last V tile has landed (MMA warp -> helper warp)
+  const uint32_t bar_vfix = bar_vreq + 8;                   // its rows past the request's end are zeroed (helper -> MMA warp)
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + L::kMisc);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + L::kMisc + 4);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+  // Barriers, tensor memory, zeroed padding: this block's own.  A call without lists, whose every block has work, sets them up while the
+  // kernels in front finish; with lists a block may turn out to have none (loose host bounds), so it looks first.
+  auto set_up = [&]() {
+    if (threadIdx.x == 0) {
+      mbar_init(bar_q, 1);
+      for (int x = 0; x < 2; ++x) { mbar_init(bar_sfull + 8 * x, 1); mbar_init(bar_pfull + 8 * x, 128); mbar_init(bar_pfull_hi + 8 * x, 128); mbar_init(bar_ofinal + 8 * x, 1); }
+      for (int s = 0; s < L::kPairBars; ++s) { mbar_init(bar_full + 8 * s, 1); mbar_init(bar_empty + 8 * s, 1); }
+      mbar_init(bar_vreq, 1);
+      mbar_init(bar_vfix, 32);
+      *abort_flag = 0;
+      fence_barrier_init();
+      fence_proxy_async_smem();
+    }
+    if (warp == 9) {
+      tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
+      tmem_relinquish();
+    }
+    // rows of the Q tiles that no (target, head) pair fills: zero them (they feed unused MMA rows)
+    {
+      const int used = pair_targets * G;
+      const int n_pad = 2 * kBM - used;
+      for (int i = threadIdx.x; i < n_pad * 8 * kHalves; i += kAttnThreads) {
+        const int piece = i & 7, r = (i >> 3) % n_pad, hf = (i >> 3) / n_pad;
+        *reinterpret_cast<uint4*>(base_ptr + L::kQ + hf * 2 * kHalfBytes + (used + r) * 128 + piece * 16) = make_uint4(0, 0, 0, 0);
+      }
+      fence_proxy_async_smem();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+  };
+  const bool early = r_cu == nullptr;
+  auto give_back = [&]() {                                          // of a block that leaves with what it has set up
+    if (!early) return;
+    __syncthreads();
+    if (warp == 9) { tc_fence_after(); tmem_dealloc(*tmem_slot, kTmemCols); }
+  };
   if (threadIdx.x == 256) { prefetch_tensormap(&tm_q); prefetch_tensormap(&tm_k); prefetch_tensormap(&tm_v); }
-  griddep_wait();
-  const int status = *reinterpret_cast<volatile int*>(&st->status);       // (fetched beside the lists)
   // Block order.  Large contexts: KV head outermost, so one head's K/V stays in L2 while its tiles run.
   // Contexts that fit L2 whole (head_inner): tile pair outermost, so the longest tiles of every head start first.
   const int hd = head_inner ? (int)(blockIdx.x % Hkv) : (int)(blockIdx.x / n_pairs_total);
   const int tt = head_inner ? (int)(blockIdx.x / Hkv) : (int)(blockIdx.x - hd * n_pairs_total);
   const int b = find_segment(rt.tile_cu, B, tt);
   const int p_rev = tt - rt.tile_cu[b];
+  if (early) set_up();
+  if (early && threadIdx.x == 256) {
+    // the first K/V tiles into L2 (a prefetch only: they are read after the wait)
+    const int nr = rt.q_len[b], last = min(nr, ((nr + pair_targets - 1) / pair_targets - p_rev) * pair_targets) - 1;
+    const int n = (rt.ctx_len[b] - nr + last) / kBN + 1, chunk = (n + (int)gridDim.y - 1) / (int)gridDim.y, t0 = (int)blockIdx.y * chunk;
+    for (int t = t0; t < min(n, t0 + min(chunk, kL2Tiles)); ++t)
+      for (int hf = 0; hf < kHalves; ++hf) {
+        tma_prefetch_3d(&tm_k, hf * 64, hd, (int)rt.tok_off[b] + t * kBN);
+        tma_prefetch_3d(&tm_v, hf * 64, hd, (int)rt.tok_off[b] + t * kBN);
+      }
+  }
+  griddep_wait();
+  const int status = *reinterpret_cast<volatile int*>(&st->status);       // (fetched beside the lists)
   // no lists (r_cu == NULL): the targets are the last q_len tokens of every request
   const int row_b = r_cu ? r_cu[b] : rt.q_cu[b];
   const int nr = r_cu ? r_cu[b + 1] - row_b : rt.q_len[b];
@@ -191,14 +260,16 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   // dense_ctx: the context is the cache itself (every position of the request), a target's limit is its position
   const int nu = dense_ctx ? rt.ctx_len[b] : (u_cu[b + 1] - u_cu[b]);
   const int n_pairs_true = (nr + pair_targets - 1) / pair_targets;
-  if (p_rev >= n_pairs_true) return;
+  if (p_rev >= n_pairs_true) { give_back(); return; }
   // a true count above its host bound, or more target rows than q_new / out hold: report, touch nothing
   if (nr > rt.bound_a[b] || (mode == RELAXKV_CTX_UNION && nu > rt.bound_b[b]) ||
       row0 + nr > n_target_rows) {
     if (threadIdx.x == 0) report(st, RELAXKV_ERR_BAD_INDEX, KID_ATTN_SM100, nr, nu);
+    give_back();
     return;
   }
-  if (status == RELAXKV_ERR_TIMEOUT) return;                  // drain after a timeout
+  // After a timeout nothing is written.  (Without lists to wait for, the word is looked at where the outputs are written.)
+  if (!early && status == RELAXKV_ERR_TIMEOUT) return;
   const int pair = n_pairs_true - 1 - p_rev;
   const int rho0 = pair * pair_targets;                       // first target of tile A
   const int ctx_len_b = (mode == RELAXKV_CTX_UNION) ? nu : rt.ctx_len[b];
@@ -237,6 +308,7 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         part_lse[((long long)split * n_target_rows + orow) * H + hd * G + (row - t_local * G)] = -INFINITY;
       }
     }
+    give_back();
     return;
   }
 
@@ -246,53 +318,7 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const int v_fix_tile = (dense_ctx && (ctx_len_b % kBN) != 0) ? (ctx_len_b / kBN - j0) : -1;
   const bool need_v_fix = v_fix_tile >= 0 && v_fix_tile < n_my_max;
 
-  // ---- shared memory -----------------------------------------------------------------------------
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
-  const uint32_t q_smem = base + L::kQ, kv_smem = base + L::kKV;
-  const uint32_t bar0 = base + L::kBar;
-  const uint32_t bar_q = bar0;
-  const uint32_t bar_sfull = bar0 + 8;          // [2]
-  const uint32_t bar_pfull = bar0 + 24;         // [2] first 32 kPLo keys of P ready
-  const uint32_t bar_pfull_hi = bar0 + 40;      // [2] the other keys of P ready
-  const uint32_t bar_ofinal = bar0 + 56;        // [2]
-  const uint32_t bar_full = bar0 + 72;          // [kPairBars] pair p = (V_{p-1}, K_p) has landed
-  const uint32_t bar_empty = bar_full + 8 * L::kPairBars;   // [kPairBars] pair p has been consumed by both tiles
-  const uint32_t bar_vreq = bar_empty + 8 * L::kPairBars;   // the request's last V tile has landed (MMA warp -> helper warp)
-  const uint32_t bar_vfix = bar_vreq + 8;                   // its rows past the request's end are zeroed (helper -> MMA warp)
-  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + L::kMisc);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + L::kMisc + 4);
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-
-  if (threadIdx.x == 0) {
-    mbar_init(bar_q, 1);
-    for (int x = 0; x < 2; ++x) { mbar_init(bar_sfull + 8 * x, 1); mbar_init(bar_pfull + 8 * x, 128); mbar_init(bar_pfull_hi + 8 * x, 128); mbar_init(bar_ofinal + 8 * x, 1); }
-    for (int s = 0; s < L::kPairBars; ++s) { mbar_init(bar_full + 8 * s, 1); mbar_init(bar_empty + 8 * s, 1); }
-    mbar_init(bar_vreq, 1);
-    mbar_init(bar_vfix, 32);
-    *abort_flag = 0;
-    fence_barrier_init();
-    fence_proxy_async_smem();
-  }
-  if (warp == 9) {
-    tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
-    tmem_relinquish();
-  }
-  // rows of the Q tiles that no (target, head) pair fills: zero them (they feed unused MMA rows)
-  {
-    const int used = pair_targets * G;
-    const int n_pad = 2 * kBM - used;
-    for (int i = threadIdx.x; i < n_pad * 8 * kHalves; i += kAttnThreads) {
-      const int piece = i & 7, r = (i >> 3) % n_pad, hf = (i >> 3) / n_pad;
-      *reinterpret_cast<uint4*>(base_ptr + L::kQ + hf * 2 * kHalfBytes + (used + r) * 128 + piece * 16) = make_uint4(0, 0, 0, 0);
-    }
-    fence_proxy_async_smem();
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
+  if (!early) set_up();
   const uint32_t tmem_base = *tmem_slot;
 
   // Register budget: the control warpgroup gives registers to the two softmax warpgroups
@@ -408,7 +434,7 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     // ================= softmax + epilogue: thread = query row = TMEM lane =================
     const int x = warp >> 2;                                    // 0: tile A, 1: tile B
     const int t_local = (int)threadIdx.x / G, j_head = (int)threadIdx.x - t_local * G;      // flat rows of the pair: tile A, then B
-    const bool row_valid = t_local < n_tgt;
+    bool row_valid = t_local < n_tgt;
     const int rho_t = rho0 + t_local;
     // Rows without a target (one of 256 with five heads per KV head; three of 128 when a target's heads had to share a tile) and rows of an empty context see every key: what they
     // hold is not stored (an empty context's row is written as zeros), and a limit below the tile sends their whole warp through the
@@ -446,6 +472,7 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       ok = mbar_wait(bar_ofinal + 8 * x, 0, abort_flag);
       ok = __all_sync(0xffffffffu, ok);
     }
+    row_valid = row_valid && status != RELAXKV_ERR_TIMEOUT;
     if (ok && my_n > 0) {
       tc_fence_after();
       const bool none = row_empty || !(z > 0.f);                // an empty context is defined as a zero output row
@@ -1213,7 +1240,11 @@ static relaxkv_status launch_attention(const relaxkv_shape* shape, int mode, Att
   if (sms <= 0) return RELAXKV_ERR_CUDA;
   // Context split.  A block's work is its pair's context length; with fewer blocks than a few waves of SMs (a query
   // prefill, a decode step, a layer with few targets, a short context) the longest pairs would run alone at the end,
-  // so every pair's context is cut into pieces of at least four tiles until the launch has about four blocks per SM.
+  // so every pair's context is cut: with fewer pairs than SMs into as many pieces as there are SMs, of a tile each if need be (the merge behind
+  // them takes as long as about three tiles, so up to four are left whole), with more until the launch has about four blocks per SM, in pieces of at least
+  // four tiles.  Pieces of four tiles at least with few pairs too, as against one, us per query attention: 64 rows over 2 K 18.0 / 16.2, 30 rows over 2 K with 8 / 2
+  // heads 13.9 / 10.2, 100 rows over 5 K 17.9 / 15.6, 32 rows over 1 K with 4 / 1 heads of dim 64 10.5 / 8.5, requests of 512 and 900 17.4 / 12.3; 57 rows over 8 K
+  // (five tiles in 13 pieces because 15 had been asked for, four in 16) 22.7 / 21.4.
   long long max_tiles = 1;
   for (int b = 0; b < B; ++b) max_tiles = std::max<long long>(max_tiles, (plan.rt.bound_b[b] + kBN - 1) / kBN);
   long long n_splits = 1;
@@ -1221,7 +1252,8 @@ static relaxkv_status launch_attention(const relaxkv_shape* shape, int mode, Att
   if (forced > 0) {
     n_splits = forced;
   } else if (grid < 4ll * sms) {
-    n_splits = std::min<long long>(std::max<long long>(1, (grid < sms ? sms : 4ll * sms) / grid), std::max<long long>(1, max_tiles / 4));
+    n_splits = grid < sms ? std::min<long long>(sms / grid, max_tiles > 4 ? max_tiles : 1)
+                          : std::min<long long>(std::max<long long>(1, 4ll * sms / grid), std::max<long long>(1, max_tiles / 4));
   }
   n_splits = std::min<long long>(n_splits, kMaxCtxSplits);
   n_splits = std::min<long long>(n_splits, kSplitRowsCap / n_target_rows);   // partial slots: [split][row of the call]
