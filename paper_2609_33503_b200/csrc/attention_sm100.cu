@@ -1240,11 +1240,12 @@ static relaxkv_status launch_attention(const relaxkv_shape* shape, int mode, Att
   if (sms <= 0) return RELAXKV_ERR_CUDA;
   // Context split.  A block's work is its pair's context length; with fewer blocks than a few waves of SMs (a query
   // prefill, a decode step, a layer with few targets, a short context) the longest pairs would run alone at the end,
-  // so every pair's context is cut: with fewer pairs than SMs into as many pieces as there are SMs, of a tile each if need be (the merge behind
-  // them takes as long as about three tiles, so up to four are left whole), with more until the launch has about four blocks per SM, in pieces of at least
-  // four tiles.  Pieces of four tiles at least with few pairs too, as against one, us per query attention: 64 rows over 2 K 18.0 / 16.2, 30 rows over 2 K with 8 / 2
-  // heads 13.9 / 10.2, 100 rows over 5 K 17.9 / 15.6, 32 rows over 1 K with 4 / 1 heads of dim 64 10.5 / 8.5, requests of 512 and 900 17.4 / 12.3; 57 rows over 8 K
-  // (five tiles in 13 pieces because 15 had been asked for, four in 16) 22.7 / 21.4.
+  // so every pair's context is cut into pieces of at least four tiles until the launch has about four blocks per SM, one with fewer pairs than SMs.
+  // A query's own rows (no lists) see their whole context and are few: as many pieces as there are SMs, of one tile if need be; the merge
+  // takes as long as about three tiles, so up to four are left whole.  Pieces of four tiles at least as against one, us: 64 rows over 2 K 18.0 / 16.2,
+  // 30 rows over 2 K with 8 / 2 heads 13.9 / 10.3, 100 rows over 5 K 17.9 / 15.7, 32 rows over 1 K with 4 / 1 heads of dim 64 10.5 / 8.6, requests of 512 and
+  // 900 17.4 / 12.3; 57 rows over 8 K (of the 15 pieces asked for, 13 of five tiles; now 16 of four) 22.7 / 21.4.  Targets along the context
+  // have shorter pairs and more rows to merge: 16 layers over 836 tokens, repaired, 503 / 511.
   long long max_tiles = 1;
   for (int b = 0; b < B; ++b) max_tiles = std::max<long long>(max_tiles, (plan.rt.bound_b[b] + kBN - 1) / kBN);
   long long n_splits = 1;
@@ -1252,8 +1253,9 @@ static relaxkv_status launch_attention(const relaxkv_shape* shape, int mode, Att
   if (forced > 0) {
     n_splits = forced;
   } else if (grid < 4ll * sms) {
-    n_splits = grid < sms ? std::min<long long>(sms / grid, max_tiles > 4 ? max_tiles : 1)
-                          : std::min<long long>(std::max<long long>(1, 4ll * sms / grid), std::max<long long>(1, max_tiles / 4));
+    n_splits = grid < sms && !r_cu_layer
+                   ? std::min<long long>(sms / grid, max_tiles > 4 ? max_tiles : 1)
+                   : std::min<long long>(std::max<long long>(1, (grid < sms ? sms : 4ll * sms) / grid), std::max<long long>(1, max_tiles / 4));
   }
   n_splits = std::min<long long>(n_splits, kMaxCtxSplits);
   n_splits = std::min<long long>(n_splits, kSplitRowsCap / n_target_rows);   // partial slots: [split][row of the call]
