@@ -58,7 +58,7 @@ static_assert(sk_part_bytes(kSkinnyMaxRows) <= sk_stages(kSkinnyMaxRows, false) 
 
 // S blocks per tile; a block's share of K is PL parts, each summed in an accumulator of its own (PL > 1: n_cols is kSkPartCols).
 template <int S, int PL, int E>
-__global__ void __launch_bounds__(sk_threads(E), 2)
+__global__ void __launch_bounds__(64 + 32 * E, 2)
 gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
                          int M, int n_cols, int n_stages, int n_feat, int K, int swiglu, const __grid_constant__ SkinnyOut outs,
                          DeviceStatus* st) {
