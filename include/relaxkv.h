@@ -392,6 +392,14 @@ relaxkv_status relaxkv_qk_norm_rope(void* q, void* k, int64_t n_rows, int32_t n_
                                     int32_t head_dim, const void* w_q_norm, const void* w_k_norm, float eps,
                                     const int32_t* positions, float theta, relaxkv_stream stream);
 
+/* relaxkv_qk_norm_rope of q and k [n_rows, ..] at positions tgt_pos, then relaxkv_scatter_kv_lists of k and v to the same positions: the
+ * rows of a decode step or a query pass, packed in list order (tgt_cu[0] = 0), rotated and appended to the cache in one launch (more
+ * than 512 rows: in two).  Errors as for the two calls. */
+relaxkv_status relaxkv_qk_norm_rope_append(
+    const relaxkv_shape* shape, const relaxkv_cache_view* cache, void* q, void* k, const void* v, int64_t n_rows, const void* w_q_norm,
+    const void* w_k_norm, float eps, const int32_t* tgt_pos, const int32_t* tgt_cu, const int32_t* h_max_targets, float theta,
+    relaxkv_stream stream);
+
 /* out[r, i] = silu(gate_up[r, i]) * gate_up[r, n_inter + i]      gate_up [n_rows, 2*n_inter], out [n_rows, n_inter] */
 relaxkv_status relaxkv_swiglu(const void* gate_up, void* out, int64_t n_rows, int32_t n_inter, relaxkv_stream stream);
 

@@ -25,7 +25,7 @@ ENTRY_POINTS = (
     "relaxkv_sparse_ctx_attention_simt", "relaxkv_read_device_status", "relaxkv_select_topk",
     "relaxkv_build_active_sets_static", "relaxkv_debug_wait_timeout",
     "relaxkv_list_attention", "relaxkv_cache_attention",
-    "relaxkv_scatter_kv_lists", "relaxkv_mean_scores", "relaxkv_scale_scores", "relaxkv_query_prefill_attention", "relaxkv_rmsnorm", "relaxkv_linear", "relaxkv_linear_qkv", "relaxkv_linear_swiglu", "relaxkv_rope", "relaxkv_qk_norm_rope",
+    "relaxkv_scatter_kv_lists", "relaxkv_mean_scores", "relaxkv_scale_scores", "relaxkv_query_prefill_attention", "relaxkv_rmsnorm", "relaxkv_linear", "relaxkv_linear_qkv", "relaxkv_linear_swiglu", "relaxkv_rope", "relaxkv_qk_norm_rope", "relaxkv_qk_norm_rope_append",
     "relaxkv_swiglu", "relaxkv_target_positions", "relaxkv_carry_rows", "relaxkv_set_chained_launch",
 )
 
@@ -71,7 +71,8 @@ _SIGNATURES = {
     "relaxkv_scale_scores": (_ST, "pi pf p"), "relaxkv_query_prefill_attention": (_ST, "pp ppp p pzp"),
     "relaxkv_rmsnorm": (_ST, "ppp li f p"), "relaxkv_linear": (_ST, "pppp lii p"), "relaxkv_linear_qkv": (_ST, "pp ppp liii p"),
     "relaxkv_linear_swiglu": (_ST, "ppp lii p"), "relaxkv_rope": (_ST, "p lii p f p"),
-    "relaxkv_qk_norm_rope": (_ST, "pp liii pp f p f p"), "relaxkv_swiglu": (_ST, "pp li p"),
+    "relaxkv_qk_norm_rope": (_ST, "pp liii pp f p f p"),
+    "relaxkv_qk_norm_rope_append": (_ST, "pp ppp l pp f ppp f p"), "relaxkv_swiglu": (_ST, "pp li p"),
     "relaxkv_target_positions": (_ST, "p pppp p p p"), "relaxkv_carry_rows": (_ST, "p pp i ppp p p"),
     "relaxkv_debug_wait_timeout": (_ST, "p"), "relaxkv_read_device_status": (_ST, "pp p"),
 }
@@ -429,6 +430,15 @@ def relaxkv_qk_norm_rope(q: torch.Tensor, k: torch.Tensor, positions: torch.Tens
     _check(lib().relaxkv_qk_norm_rope(_ptr(q), _ptr(k), q.shape[0], int(q.shape[1]), int(k.shape[1]),
                                       int(q.shape[2]), _ptr(w_q_norm), _ptr(w_k_norm), float(eps), _ptr(positions),
                                       float(theta), _stream(stream)), "relaxkv_qk_norm_rope")
+
+
+def relaxkv_qk_norm_rope_append(shape: Shape, cache: CacheView, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, tgt_pos: torch.Tensor,
+                                tgt_cu: torch.Tensor, max_targets: Sequence[int], theta: float, w_q_norm: Optional[torch.Tensor] = None,
+                                w_k_norm: Optional[torch.Tensor] = None, eps: float = 1e-6, stream=None) -> None:
+    """relaxkv_qk_norm_rope of q [n, H, D] and k [n, H_kv, D], then relaxkv_scatter_kv_lists of k and v, both at tgt_pos."""
+    _check(lib().relaxkv_qk_norm_rope_append(shape.ref(), cache.ref(), _ptr(q), _ptr(k), _ptr(v), q.shape[0], _ptr(w_q_norm), _ptr(w_k_norm),
+                                             float(eps), _ptr(tgt_pos), _ptr(tgt_cu), _i32(max_targets), float(theta), _stream(stream)),
+           "relaxkv_qk_norm_rope_append")
 
 
 def relaxkv_swiglu(gate_up: torch.Tensor, out: torch.Tensor, stream=None) -> None:

@@ -5,7 +5,7 @@ region).  Call sequencing over torch buffers only; every operation runs in the C
 `binding`.
 
 Per layer the query's rows run the decoder block: RMSNorm, the stacked Q/K/V projection, per-head Q/K norm where the
-model has one and rotary embedding at positions T_c, T_c + 1, ... (one launch), their K/V are appended to the cache behind the context rows,
+model has one, rotary embedding at positions T_c, T_c + 1, ... and the append of their K/V to the cache behind the context rows (one launch),
 then causal attention over [context, query] (`relaxkv_query_prefill_attention`, which can emit the context scores of
 that very pass), output projection + residual, MLP + residual.  The decode step is the same block for one new token
 (the projections take the streaming one-row kernel), followed by the final norm and the output head.
@@ -90,8 +90,8 @@ class QueryPass:
         if "w_qkv" not in w:                            # weight-loading step, once per layer: [Wq; Wk; Wv] stacked
             w["w_qkv"] = B.stack_qkv(w["wq"], w["wk"], w["wv"])
         rec("qkv_proj", lambda: B.relaxkv_linear_qkv(x, w["w_qkv"], q, k, v))
-        rec("rope", lambda: B.relaxkv_qk_norm_rope(q, k, pos, blk.rope_theta, w.get("w_q_norm"), w.get("w_k_norm"), blk.eps))
-        rec("append_kv", lambda: B.relaxkv_scatter_kv_lists(shape, cache, k, v, pos, cu, counts))
+        rec("rope_append", lambda: B.relaxkv_qk_norm_rope_append(shape, cache, q, k, v, pos, cu, counts, blk.rope_theta,
+                                                                 w.get("w_q_norm"), w.get("w_k_norm"), blk.eps))
         rec("attention", attend)
         rec("o_proj", lambda: B.relaxkv_linear(o, w["wo"], a, residual=h))
         rec("norm", lambda: B.relaxkv_rmsnorm(a, w["w_post_norm"], x, blk.eps))

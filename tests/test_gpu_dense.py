@@ -676,3 +676,40 @@ def test_scores_of_several_layers_in_one_launch_equal_the_layers_own(layers):
     assert torch.equal(got[0][0], got[1][0])
     assert (got[1][1] > 0).all()
     assert ((got[0][1] - got[1][1]).abs() <= 1e-5 * got[1][1]).all()
+
+
+@pytest.mark.parametrize("head_major", [False, True], ids=["token_major", "head_major"])
+@pytest.mark.parametrize("H,Hkv,D,with_norm,counts", [(4, 1, 64, False, (1,)), (6, 2, 128, True, (1, 0, 7)), (40, 8, 128, True, (130,)), (8, 8, 64, True, (256, 257))],
+                         ids=["one_row", "ragged", "query", "two_launches"])
+def test_rotating_and_appending_in_one_launch(H, Hkv, D, with_norm, counts, head_major):
+    """relaxkv_qk_norm_rope_append: the bits of relaxkv_qk_norm_rope followed by relaxkv_scatter_kv_lists, in q, k and the cache (513 rows:
+    more than one launch takes); rows past a request's host bound or at a position outside it are reported and appended nowhere."""
+    n, nb = sum(counts), len(counts)
+    ctx = [300 + 11 * b for b in range(nb)]
+    offs = [sum(ctx[:b]) + 5 * b for b in range(nb)]
+    rows = offs[-1] + ctx[-1]
+    rng = np.random.default_rng(n)
+    pos = torch.from_numpy(np.concatenate([np.sort(rng.choice(c, m, replace=False)) for c, m in zip(ctx, counts)]).astype(np.int32)).cuda()
+    cu = torch.tensor([sum(counts[:b]) for b in range(nb + 1)], dtype=torch.int32, device="cuda")
+    wq, wk = (rnd(D, seed=3), rnd(D, seed=4)) if with_norm else (None, None)
+    shape = B().Shape(H, Hkv, D, ctx)
+
+    def run(fn, pos, bounds):
+        q, k, v = rnd(n, H, D, seed=5), rnd(n, Hkv, D, seed=6), rnd(n, Hkv, D, seed=7)
+        kv = [rnd(Hkv, rows, D, seed=8 + i).transpose(0, 1) if head_major else rnd(rows, Hkv, D, seed=8 + i) for i in range(2)]
+        fn(B().CacheView(kv[0], kv[1], offs), q, k, v, pos, bounds)
+        return [t.clone() for t in (q, k, *kv)], B().relaxkv_read_device_status()[0]
+
+    def two(cache, q, k, v, pos, bounds):
+        B().relaxkv_qk_norm_rope(q, k, pos, 1e6, wq, wk, 1e-6)
+        B().relaxkv_scatter_kv_lists(shape, cache, k, v, pos, cu, bounds)
+
+    def one(cache, q, k, v, pos, bounds):
+        B().relaxkv_qk_norm_rope_append(shape, cache, q, k, v, pos, cu, bounds, 1e6, wq, wk, 1e-6)
+
+    outside = pos.clone()
+    outside[-1] = ctx[-1]
+    for p, bounds in ((pos, counts), (outside, counts), (pos, [max(0, c - 1) for c in counts])):
+        (want, st2), (got, st1) = run(two, p, bounds), run(one, p, bounds)
+        assert all(torch.equal(a, b) for a, b in zip(want, got))
+        assert st1 == st2 and (st1 != 0) == (p is outside or (bounds is not counts and any(bounds)))
