@@ -91,7 +91,8 @@ decode_attention_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
   uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
   const uint32_t bar_full = base + L::kBar, bar_empty = bar_full + 8 * kDecStages;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + L::kMisc);
-  __shared__ __align__(16) float q_s[GMAX][D];                      // the query heads of this KV head
+  constexpr bool kQDirect = GMAX > 4;
+  __shared__ __align__(16) float q_s[kQDirect ? 1 : GMAX][D];       // the query heads of this KV head
   __shared__ float m_s[kDecConsumers][GMAX], z_s[kDecConsumers][GMAX];
   // the warps' partial outputs for the merge take the ring's place once every tile has been consumed
   float (*o_s)[GMAX][D] = reinterpret_cast<float (*)[GMAX][D]>(base_ptr);
@@ -148,25 +149,36 @@ decode_attention_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
     }
   } else {
     // ================= consumers =================
-    // the query heads (the producer is on its way already: the consumers' own barrier)
-    for (int i = threadIdx.x; i < GMAX * D; i += kDecConsumers * 32) {
-      const int g = i / D, d = i - g * D;
-      q_s[g][d] = (g < G) ? bf16_bits_to_float(q[(row * H + hd * G + g) * D + d]) : 0.f;     // exact; the scale goes on S
-    }
-    asm volatile("bar.sync 1, %0;" ::"n"(kDecConsumers * 32) : "memory");
     const int gid = lane >> 2, tig = lane & 3;                        // fragment coordinates: row gid (and gid + 8), column pair tig
-    // Q as A fragments, one per 16 dims: rows = the G query heads (zero beyond)
+    // Q as A fragments, one per 16 dims: rows = the G query heads of this KV head (zero beyond), the bf16 pairs as stored (the scale goes on S).
+    // With more than four heads every warp fetches its pairs itself, a latency and a barrier less than through shared memory (12 layers
+    // of a decode step of 40 / 8 heads at 32 K 1985 us, 1968 so; with four the lanes are half idle: 16 layers of four requests of 32 / 8 heads 1969 / 1977).
     uint32_t qa[D / 16][4];
+    if constexpr (kQDirect) {
+      const uint16_t* q_head = q + (row * H + hd * G) * D + tig * 2;
 #pragma unroll
-    for (int ks = 0; ks < D / 16; ++ks) {
+      for (int ks = 0; ks < D / 16; ++ks) {
 #pragma unroll
-      for (int h2 = 0; h2 < 2; ++h2) {                                // columns ks*16 + tig*2 (+8 for h2 = 1)
-        const int col = ks * 16 + h2 * 8 + tig * 2;
-        const __nv_bfloat162 lo = __floats2bfloat162_rn(q_s[gid % GMAX][col] * (gid < GMAX ? 1.f : 0.f), q_s[gid % GMAX][col + 1] * (gid < GMAX ? 1.f : 0.f));
-        const __nv_bfloat162 hi = (GMAX > 8) ? __floats2bfloat162_rn(q_s[(gid + 8) % GMAX][col], q_s[(gid + 8) % GMAX][col + 1])
-                                             : __floats2bfloat162_rn(0.f, 0.f);
-        qa[ks][h2 * 2] = *reinterpret_cast<const uint32_t*>(&lo);
-        qa[ks][h2 * 2 + 1] = *reinterpret_cast<const uint32_t*>(&hi);
+        for (int h2 = 0; h2 < 2; ++h2) {                              // columns ks*16 + tig*2 (+8 for h2 = 1)
+          qa[ks][h2 * 2] = gid < G ? *reinterpret_cast<const uint32_t*>(q_head + gid * D + ks * 16 + h2 * 8) : 0u;
+          qa[ks][h2 * 2 + 1] = (GMAX > 8 && gid + 8 < G) ? *reinterpret_cast<const uint32_t*>(q_head + (gid + 8) * D + ks * 16 + h2 * 8) : 0u;
+        }
+      }
+    } else {
+      for (int i = threadIdx.x; i < GMAX * D; i += kDecConsumers * 32) {
+        const int g = i / D, d = i - g * D;
+        q_s[g][d] = (g < G) ? bf16_bits_to_float(q[(row * H + hd * G + g) * D + d]) : 0.f;     // exact
+      }
+      asm volatile("bar.sync 1, %0;" ::"n"(kDecConsumers * 32) : "memory");      // (the producer is on its way already)
+#pragma unroll
+      for (int ks = 0; ks < D / 16; ++ks) {
+#pragma unroll
+        for (int h2 = 0; h2 < 2; ++h2) {
+          const int col = ks * 16 + h2 * 8 + tig * 2;
+          const __nv_bfloat162 lo = __floats2bfloat162_rn(q_s[gid % GMAX][col] * (gid < GMAX ? 1.f : 0.f), q_s[gid % GMAX][col + 1] * (gid < GMAX ? 1.f : 0.f));
+          qa[ks][h2 * 2] = *reinterpret_cast<const uint32_t*>(&lo);
+          qa[ks][h2 * 2 + 1] = 0u;
+        }
       }
     }
     float m_r[2] = {-INFINITY, -INFINITY}, z_r[2] = {0.f, 0.f};       // rows gid and gid + 8
