@@ -71,17 +71,23 @@ __global__ void finalize_raw_kernel(ReqTable rt, int n_layers, int H, int Hkv, i
   const long long sum_t = rt.ctx_cu[rt.n_req];
   const long long gi = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (gi >= sum_t * n_layers) return;
-  const long long layer = gi / sum_t, i = gi - layer * sum_t;
+  const long long layer = n_layers == 1 ? 0 : gi / sum_t, i = gi - layer * sum_t;
   int b = 0;
   while (b + 1 < rt.n_req && i >= rt.ctx_cu[b + 1]) ++b;
   const int n_super = rt.tile_cu[b + 1] - rt.tile_cu[b];
   const float* cp = colpart + layer * (2 * Hkv * max_super) * sum_t;
   float s = 0.f;
   const int per_head = 2 * n_super, n_part = Hkv * per_head;
+  if (n_super == max_super) {                      // one behind the other, sixteen in flight (a call over one 16 K layer 39.5 us, 38.4 so)
+    cp += i;
+#pragma unroll 16
+    for (int m = 0; m < n_part; ++m) s += cp[(long long)m * sum_t];
+  } else {
 #pragma unroll 8
-  for (int m = 0; m < n_part; ++m) {               // one loop, so that eight loads are in flight
-    const int g = m / per_head;
-    s += cp[(long long)(g * 2 * max_super + (m - g * per_head)) * sum_t + i];
+    for (int m = 0; m < n_part; ++m) {             // one loop, so that eight loads are in flight
+      const int g = m / per_head;
+      s += cp[(long long)(g * 2 * max_super + (m - g * per_head)) * sum_t + i];
+    }
   }
   raw[gi] = s / ((float)H * (float)rt.q_len[b]);
 }
