@@ -73,7 +73,8 @@ typedef struct {
   int32_t attention_ctx_splits;  /* > 0: the attention calls split every query tile's context over this many thread   */
                                  /* blocks (up to 32, and as far as the workspace's 2048 row-splits allow) and merge   */
                                  /* the partial results by their log-sum-exp; automatic = only when the call has too   */
-                                 /* few query tiles to fill the GPU (a query prefill, a decode step, few targets)      */
+                                 /* few query tiles to fill the GPU (a query prefill, a decode step, few targets), and */
+                                 /* then, for targets along the context, the longest of them alone                     */
   int32_t attention_persistent;  /* the repair / list attention calls have a persistent form (one thread block per SM  */
                                  /* walks the call's query tiles, longest context first).  0: the library takes it     */
                                  /* for one-split calls over gathered contexts of at most 128 key tiles; 1: for every  */

@@ -11,7 +11,7 @@ struct AttnPlan {
   uint16_t* vctx;
   long long ctx_rows;     // rows the two buffers hold (tensor-map extent)
   long long sum_targets;  // sum of the host bounds on |R_{l,b}|
-  float* split_o;         // workspace for a context split across blocks: [kSplitRowsCap, H, D] and [kSplitRowsCap, H]
+  float* split_o;         // workspace for a context split across blocks: [split_rows_cap, H, D] and [split_rows_cap, H]
   float* split_lse;       // (its first word, zeroed by the gather, is the work counter of the persistent form)
   // what the attention kernel's K/V tensor maps cover: the materialised context, or the cache itself
   const void* k_base; const void* v_base;

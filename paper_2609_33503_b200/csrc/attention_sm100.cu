@@ -21,6 +21,7 @@
 // Every wait is bounded; an expired wait raises the block's abort flag, records RELAXKV_ERR_TIMEOUT in the
 // device status word and the block tears down normally.
 #include "attention_common.cuh"
+#include "attention_pieces.cuh"
 #include "decode_attention.cuh"
 #include "sm100_ptx.cuh"
 #include <algorithm>
@@ -161,7 +162,7 @@ template <int D>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                        const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ ReqTable rt,
-                       int mode, int allow_empty, int head_inner, int dense_ctx, int H, int Hkv, int pair_targets, float scale_log2,
+                       const __grid_constant__ PieceTable pt, int mode, int allow_empty, int head_inner, int dense_ctx, int H, int Hkv, int pair_targets, float scale_log2,
                        const int* u_pos, const int* u_cu, const int* r_rank, const int* r_cu,
                        long long n_target_rows, uint16_t* __restrict__ out, float* __restrict__ lse_out,
                        float* __restrict__ part_o, float* __restrict__ part_lse, DeviceStatus* st) {
@@ -238,7 +239,15 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const int hd = head_inner ? (int)(blockIdx.x % Hkv) : (int)(blockIdx.x / n_pairs_total);
   const int tt = head_inner ? (int)(blockIdx.x / Hkv) : (int)(blockIdx.x - hd * n_pairs_total);
   const int b = find_segment(rt.tile_cu, B, tt);
-  const int p_rev = tt - rt.tile_cu[b];
+  // Context split: this block walks the context tiles [j0, j0 + chunk) of its pair and leaves a normalised partial result + its log-sum-exp.
+  // Either all pairs alike (gridDim.y, used when there are too few query tiles to fill the GPU) or the longest pairs of a request in pieces (pt).
+  int p_rev = tt - rt.tile_cu[b], n_splits = (int)gridDim.y, split = (int)blockIdx.y, slot0 = 0;
+  if (pt.most > 0) {
+    split = unit_piece(p_rev, rt.tile_cu[b + 1] - rt.tile_cu[b], pt.pieces[b], pt.long_pairs[b], &p_rev);
+    n_splits = split < 0 ? 1 : pt.pieces[b];
+    split = max(split, 0);
+    slot0 = pt.slot_cu[b] + p_rev * pair_targets;
+  }
   if (early) set_up();
   if (early && threadIdx.x == 256) {
     // the first K/V tiles into L2 (a prefetch only: they are read after the wait)
@@ -291,9 +300,8 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     }
   }
   const int n_kv_max = max(n_kv[0], n_kv[1]);
-  // Context split (gridDim.y > 1, used when there are too few query tiles to fill the GPU): this block walks the
-  // context tiles [j0, j0 + chunk) of its pair and leaves a normalised partial result + its log-sum-exp.
-  const int n_splits = (int)gridDim.y, split = (int)blockIdx.y;
+  // slot of the pair's first row in the workspace (which holds some ten thousand); -1: the only piece, written to the output
+  const int slot_base = n_splits == 1 ? -1 : (pt.most > 0 ? split * pt.slot_cu[B] + slot0 : split * (int)n_target_rows + q_row_base);
   const int chunk = (n_kv_max + n_splits - 1) / n_splits;
   const int j0 = split * chunk;
   int n_my[2];
@@ -301,11 +309,10 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   for (int x = 0; x < 2; ++x) n_my[x] = max(0, min(n_kv[x], j0 + chunk) - j0);
   const int n_my_max = max(n_my[0], n_my[1]);
   if (n_my_max == 0) {                        // nothing of this pair's context falls into this split
-    if (n_splits > 1 && threadIdx.x < 2 * kBM) {
+    if (slot_base >= 0 && threadIdx.x < 2 * kBM) {
       const int row = threadIdx.x, t_local = row / G;
       if (t_local < n_tgt) {
-        const int orow = q_row_base + t_local;
-        part_lse[((long long)split * n_target_rows + orow) * H + hd * G + (row - t_local * G)] = -INFINITY;
+        part_lse[(long long)(slot_base + t_local) * H + hd * G + (row - t_local * G)] = -INFINITY;
       }
     }
     give_back();
@@ -479,7 +486,7 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       const float inv = none ? 0.f : 1.f / z;
       const float lse = none ? -INFINITY : (m + log2f(z)) * kLn2A;
       const int orow = q_row_base + t_local;
-      if (n_splits == 1) {
+      if (slot_base < 0) {
         uint16_t* optr = out + ((long long)orow * H + hd * G + j_head) * D;
         const bool sectors = (reinterpret_cast<uintptr_t>(out) & 31u) == 0;
 #pragma unroll
@@ -504,7 +511,7 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         if (row_valid && lse_out) lse_out[(long long)(hd * G + j_head) * n_target_rows + orow] = lse;
       } else {
         // partial result of this split: fp32, normalised by this split's own sum
-        const long long slot = ((long long)split * n_target_rows + orow) * H + hd * G + j_head;
+        const long long slot = (long long)(slot_base + t_local) * H + hd * G + j_head;
         float* optr = part_o + slot * D;
 #pragma unroll
         for (int c = 0; c < D / 32; ++c) {
@@ -520,10 +527,9 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         }
         if (row_valid) part_lse[slot] = lse;
       }
-    } else if (ok && my_n == 0 && n_splits > 1 && row_valid) {
+    } else if (ok && my_n == 0 && slot_base >= 0 && row_valid) {
       // this tile's context ends before the split begins (the pair's other tile still has work here)
-      const int orow = q_row_base + t_local;
-      part_lse[((long long)split * n_target_rows + orow) * H + hd * G + j_head] = -INFINITY;
+      part_lse[(long long)(slot_base + t_local) * H + hd * G + j_head] = -INFINITY;
     }
   }
 
@@ -1090,22 +1096,28 @@ constexpr int kMaxCombineSplits = 1024;       // four warps x 4 KB of weights
 
 // Merges the partial results of a context split: out = sum_s w_s O_s / sum_s w_s with w_s = exp(lse_s - max lse).
 // One warp per (target row, query head), U partial results of it in flight; rows past the true target count are left alone.
-template <int U>
+// PIECES: the rows are the slots of the pairs that were cut (pt).
+template <int U, bool PIECES>
 __global__ void __launch_bounds__(kCombineThreads)
 combine_splits_kernel(const float* part_o, const float* part_lse, int n_splits,
                       long long n_target_rows, int H, int D, const int* r_cu, int n_req,
-                      uint16_t* __restrict__ out, float* __restrict__ lse_out) {
+                      uint16_t* __restrict__ out, float* __restrict__ lse_out, const __grid_constant__ PieceTable pt, int pair_targets) {
   // the splits' weights of this warp's (row, head): the lanes fetch the log-sum-exps side by side (a serial walk over
   // the splits would pay one memory latency per split), the sums below still run in split order
   __shared__ float wgt_s[kCombineThreads / 32][kMaxCombineSplits];
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long w = (long long)blockIdx.x * (kCombineThreads / 32) + wib;
-  const long long row = w / H;
-  const int h = (int)(w - row * H);
-  const bool mine = row < n_target_rows;
+  const long long slot = w / H, slot_rows = PIECES ? pt.slot_cu[n_req] : n_target_rows;
+  const int h = (int)(w - slot * H);
+  const bool mine = slot < slot_rows;
+  int b = 0;
+  if (PIECES) {
+    while (b + 1 < n_req && slot >= pt.slot_cu[b + 1]) ++b;
+    n_splits = pt.pieces[b];
+  }
   const int per = D / 32;                       // 2 or 4 consecutive floats per lane
-  const float* o = part_o + (row * H + h) * D + lane * per;
-  const long long sp_stride = n_target_rows * H * D;
+  const float* o = part_o + (slot * H + h) * D + lane * per;
+  const long long sp_stride = slot_rows * H * D;
   auto load = [&](int sp) -> float4 {
     if (per == 4) return *reinterpret_cast<const float4*>(o + sp * sp_stride);
     const float2 v = *reinterpret_cast<const float2*>(o + sp * sp_stride);
@@ -1120,14 +1132,23 @@ combine_splits_kernel(const float* part_o, const float* part_lse, int n_splits,
   float4 v[U];
 #pragma unroll
   for (int u = 0; u < U; ++u) v[u] = u < n_splits ? load(u) : make_float4(0.f, 0.f, 0.f, 0.f);
-  const long long rows_true = r_cu ? min((long long)(r_cu[n_req] - r_cu[0]), n_target_rows) : n_target_rows;
+  long long row = slot;
+  bool here = true;                             // rows past the true counts (and requests that were refused) hold nothing
+  if (PIECES) {
+    const int c0 = r_cu[0], cb = r_cu[b], nr = r_cu[b + 1] - cb, rel = (int)slot - pt.slot_cu[b], p_rev = rel / pair_targets;
+    const int rho = ((nr + pair_targets - 1) / pair_targets - 1 - p_rev) * pair_targets + rel - p_rev * pair_targets;
+    row = (long long)(cb - c0) + rho;
+    here = rho >= 0 && rho < nr && nr <= pt.bound[b] && (long long)(cb - c0) + nr <= n_target_rows;
+  } else {
+    here = slot < (r_cu ? min((long long)(r_cu[n_req] - r_cu[0]), n_target_rows) : n_target_rows);
+  }
   float mx = -INFINITY;
   for (int sp = lane; sp < n_splits; sp += 32) {
-    const float l = part_lse[((long long)sp * n_target_rows + row) * H + h];
+    const float l = part_lse[((long long)sp * slot_rows + slot) * H + h];
     wgt_s[wib][sp] = l;
     mx = fmaxf(mx, l);
   }
-  if (row >= rows_true) return;
+  if (!here) return;
   mx = warp_reduce_max(mx);
   __syncwarp();
   for (int sp = lane; sp < n_splits; sp += 32) {
@@ -1172,9 +1193,9 @@ relaxkv_status launch_combine_splits(const float* part_o, const float* part_lse,
   // A decoded row whose context one wave of blocks shares (18 splits with eight KV heads): all of them in one go, one memory latency less (12 layers of a
   // decode step at 32 K 1985 us, 1970 so).  Up to eight splits the small form: with the registers of the large one beside it the next projection's
   // blocks come later (16 layers of four requests 1969 / 2017).
-  auto kern = n_splits > 8 && warps <= kCombineFewWarps ? combine_splits_kernel<20> : combine_splits_kernel<8>;
+  auto kern = n_splits > 8 && warps <= kCombineFewWarps ? combine_splits_kernel<20, false> : combine_splits_kernel<8, false>;
   return cuda_ok(launch_chained(kern, (unsigned)((warps + wpb - 1) / wpb), kCombineThreads, 0, stream, part_o,
-                                part_lse, n_splits, (long long)n_target_rows, H, D, r_cu, n_req, static_cast<uint16_t*>(out), lse_out));
+                                part_lse, n_splits, (long long)n_target_rows, H, D, r_cu, n_req, static_cast<uint16_t*>(out), lse_out, PieceTable{}, 0));
 }
 
 // ---- host side ---------------------------------------------------------------------------------------
@@ -1265,6 +1286,31 @@ static relaxkv_status launch_attention(const relaxkv_shape* shape, int mode, Att
   n_splits = std::min<long long>(n_splits, kMaxCtxSplits);
   n_splits = std::min<long long>(n_splits, kSplitRowsCap / n_target_rows);   // partial slots: [split][row of the call]
   if (n_splits < 1) n_splits = 1;
+  // Or only the longest pairs of the call, in pieces.
+  PieceTable pt{};
+  const bool automatic = forced == 0 && (!shape->h_tuning || shape->h_tuning->attention_persistent == 0);
+  if (automatic && r_cu_layer && !plan.dense_ctx && grid <= 4ll * sms) {
+    int tiles[kMaxReqInline], pairs[kMaxReqInline];
+    double steps = 0.0;
+    for (int b = 0; b < B; ++b) {
+      tiles[b] = (plan.rt.bound_b[b] + kBN - 1) / kBN;
+      pairs[b] = tiles[b] > 0 ? plan.rt.tile_cu[b + 1] - plan.rt.tile_cu[b] : 0;
+      steps += 0.5 * tiles[b] * (pairs[b] + 1) * (pairs[b] > 0);
+    }
+    const double per_sm = steps * Hkv / sms;
+    const double bytes = 2.0 * n_splits * plan.sum_targets * H * D * 4;
+    const double uncut = std::max((double)max_tiles / (double)n_splits, 1.05 * per_sm) + (n_splits > 1 ? kPieceMergeSteps + bytes / kPieceBytesPerStep : 0.0);
+    pt = plan_pieces(tiles, pairs, plan.rt.bound_a, B, pair_targets, Hkv, (long long)H * D * 4, split_rows_cap(shape), sms, uncut);
+  }
+  if (pt.most > 0) {
+    n_splits = 1;
+    int cu = 0;
+    for (int b = 0; b < B; ++b) {
+      cu += (plan.rt.bound_a[b] + pair_targets - 1) / pair_targets + pt.long_pairs[b] * (pt.pieces[b] - 1);
+      plan.rt.tile_cu[b + 1] = cu;
+    }
+  }
+  const long long units = (long long)plan.rt.tile_cu[B] * Hkv;
   auto kern = attention_sm100_kernel<D>;
   static std::atomic<int> attr_done[kMaxDevices];          // per device: the opt-in to > 48 KB of dynamic shared memory
   int dev = 0;
@@ -1278,7 +1324,7 @@ static relaxkv_status launch_attention(const relaxkv_shape* shape, int mode, Att
   // 3 % at an 8K context; nothing at 32K, where the chip runs at its power cap either way).
   const relaxkv_tuning* tun = shape->h_tuning;
   const int want_persist = tun ? tun->attention_persistent : 0;
-  if (n_splits == 1 && !plan.dense_ctx && (want_persist == 1 || (want_persist == 0 && max_tiles <= kPersistMaxTiles && grid > sms))) {
+  if (n_splits == 1 && pt.most == 0 && !plan.dense_ctx && (want_persist == 1 || (want_persist == 0 && max_tiles <= kPersistMaxTiles && grid > sms))) {
     auto pk = attention_persist_kernel<D>;
     static std::atomic<int> pattr_done[kMaxDevices];
     if (!pattr_done[dev].load(std::memory_order_acquire)) {
@@ -1295,9 +1341,15 @@ static relaxkv_status launch_attention(const relaxkv_shape* shape, int mode, Att
         u_pos, u_cu, r_rank, r_cu_layer, n_target_rows, static_cast<uint16_t*>(out), lse_out, (int)grid, counter, st));
   }
   RELAXKV_RANGE("attention_sm100_kernel");
-  relaxkv_status rc = cuda_ok(launch_chained(kern, dim3((unsigned)grid, (unsigned)n_splits), kAttnThreads, AttnSmem<D>::kDynamic, stream,
-      tm_q, tm_k, tm_v, plan.rt, mode, allow_empty, head_inner, plan.dense_ctx, H, Hkv, pair_targets, shape->softmax_scale * kLog2eA,
+  relaxkv_status rc = cuda_ok(launch_chained(kern, dim3((unsigned)units, (unsigned)n_splits), kAttnThreads, AttnSmem<D>::kDynamic, stream,
+      tm_q, tm_k, tm_v, plan.rt, pt, mode, allow_empty, head_inner, plan.dense_ctx, H, Hkv, pair_targets, shape->softmax_scale * kLog2eA,
       u_pos, u_cu, r_rank, r_cu_layer, n_target_rows, static_cast<uint16_t*>(out), lse_out, plan.split_o, plan.split_lse, st));
+  if (rc == RELAXKV_OK && pt.most > 0) {
+    const long long warps = (long long)pt.slot_cu[B] * H;
+    constexpr int wpb = kCombineThreads / 32;
+    return cuda_ok(launch_chained(combine_splits_kernel<8, true>, (unsigned)((warps + wpb - 1) / wpb), kCombineThreads, 0, stream,
+                                  plan.split_o, plan.split_lse, pt.most, n_target_rows, H, D, r_cu_layer, B, static_cast<uint16_t*>(out), lse_out, pt, pair_targets));
+  }
   if (rc != RELAXKV_OK || n_splits == 1) return rc;
   return launch_combine_splits(plan.split_o, plan.split_lse, (int)n_splits, n_target_rows, H, D, r_cu_layer, B, plan.sum_targets,
                                out, lse_out, stream);

@@ -1236,3 +1236,43 @@ def test_targets_at_the_edges_of_a_pair_of_query_tiles(G, D):
                 check_attention(case, 0, out, lse, full_prefix)
                 outs.append(out)
         assert torch.equal(outs[0], outs[2]) and torch.equal(outs[1], outs[3])
+
+
+@pytest.mark.parametrize("H,Hkv,D,ctx,targets", [(4, 1, 64, (4000,), 4000), (4, 1, 64, (2600, 130, 3100), 3100), (5, 1, 128, (4500,), 4500),
+                                                 (8, 2, 128, (6000,), 1229), (6, 2, 64, (5000, 3000), 400)],
+                         ids=["one", "ragged", "five_heads", "few_targets", "few_targets_ragged"])
+def test_longest_pairs_in_pieces(H, Hkv, D, ctx, targets):
+    """A call of few tile pairs cuts its longest ones into pieces and merges them: against the oracle, with exact and with loose host
+    bounds, beside the whole form (other bits: pieces were taken), and refused where a count is above its bound."""
+    w = inputs.Workload("pieces", 1, H, Hkv, D, 64, ctx, (4,) * len(ctx), 0.1, base_seed=H)
+    case = Case(w, anchors_override=[[np.arange(1, dtype=np.int32) for _ in ctx]])
+    rng = np.random.default_rng(len(ctx))
+    tgt = [np.sort(rng.choice(t, min(t, targets), replace=False)).astype(np.int32) for t in ctx]
+    ctx_lists = [np.unique(np.concatenate([x, rng.choice(t, (5 * t) // 6, replace=False)])).astype(np.int32) for x, t in zip(tgt, ctx)]
+    ctx_pos, ctx_cu, _ = _pack(ctx_lists, case.device)
+    tgt_pos, tgt_cu, tcu = _pack(tgt, case.device)
+    fresh = [torch.cat(x).contiguous() for x in zip(*[inputs.fresh_qkv(w, 0, b, case.k_cache[0][case.ctx_cu[b]:case.ctx_cu[b + 1]],
+                                                                      case.v_cache[0][case.ctx_cu[b]:case.ctx_cu[b + 1]],
+                                                                      torch.from_numpy(tgt[b].astype(np.int64))) for b in range(len(ctx))])]
+    refs = [orc.list_attention(case.req_k(0, b), case.req_v(0, b), *(inputs.bf16_bits(t[tcu[b]:tcu[b + 1]]) for t in fresh), ctx_lists[b], tgt[b],
+                               case.scale) for b in range(len(ctx))]
+    n_t, n_c = [len(x) for x in tgt], [len(x) for x in ctx_lists]
+    outs = []
+    for tuning, max_t, max_c in ((dict(), n_t, n_c), (dict(), ctx, ctx), (dict(attention_ctx_splits=1), n_t, n_c), (dict(), [max(1, n - 1) for n in n_t], n_c)):
+        shape = B().Shape(H, Hkv, D, ctx, None, case.scale, **tuning)
+        ws = torch.empty(B().relaxkv_workspace_bytes(shape, 1), dtype=torch.uint8, device="cuda")
+        out, lse = torch.full_like(fresh[0], 3.0), torch.zeros(H, fresh[0].shape[0], dtype=torch.float32, device="cuda")
+        B().relaxkv_list_attention(shape, case.cache_views()[0], *fresh, ctx_pos, ctx_cu, tgt_pos, tgt_cu, max_t, max_c, out, ws, lse_out=lse)
+        outs.append(out)
+        if len(outs) == 4:
+            break
+        assert_status_ok()
+        for b, (ref, ref_lse) in enumerate(refs):
+            lo, hi = int(tcu[b]), int(tcu[b + 1])
+            mx, mean = attention_errors(out[lo:hi], ref)
+            assert mx <= MAX_ABS and mean <= MEAN_ABS, (b, mx, mean)
+            np.testing.assert_allclose(lse[:, lo:hi].cpu().numpy().astype(np.float64).T, ref_lse, atol=2e-3, rtol=1e-4)
+    assert not torch.equal(outs[0], outs[2])
+    assert B().relaxkv_read_device_status()[0] == B().ERR_BAD_INDEX
+    refused = torch.cat([torch.full((n,), n > 1) for n in n_t]).cuda()
+    assert torch.all(outs[3][refused] == 3.0)
