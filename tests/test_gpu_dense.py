@@ -713,3 +713,20 @@ def test_rotating_and_appending_in_one_launch(H, Hkv, D, with_norm, counts, head
         (want, st2), (got, st1) = run(two, p, bounds), run(one, p, bounds)
         assert all(torch.equal(a, b) for a, b in zip(want, got))
         assert st1 == st2 and (st1 != 0) == (p is outside or (bounds is not counts and any(bounds)))
+
+
+@pytest.mark.parametrize("M", [129, 300, 1000])
+@pytest.mark.parametrize("N,off_y,off_r", [(512, 0, 0), (512, 8, 0), (512, 0, 8), (264, 0, 0), (272, 8, 8), (8, 0, 0)])
+def test_rows_of_any_alignment_leave_a_gemm_alike(M, N, off_y, off_r):
+    """Both GEMM kernels store (and add) whole 32-byte sectors where every row is 32-byte aligned and 16-byte pieces elsewhere: the same bits
+    as an aligned output of a width of 512, neighbours untouched."""
+    K = 192
+    x, w, r = rnd(M, K, seed=1), rnd(512, K, scale=K ** -0.5, seed=2), rnd(M, 512, seed=3)
+    ref = torch.empty(M, 512, dtype=torch.bfloat16, device="cuda")
+    B().relaxkv_linear(x, w, ref, residual=r)
+    res = torch.zeros(M * N + 16, dtype=torch.bfloat16, device="cuda")
+    res[off_r:off_r + M * N] = r[:, :N].reshape(-1)
+    out = torch.full((M * N + 16,), 3.0, dtype=torch.bfloat16, device="cuda")
+    B().relaxkv_linear(x, w[:N].contiguous(), out[off_y:off_y + M * N].view(M, N), residual=res[off_r:off_r + M * N].view(M, N))
+    assert torch.equal(out[off_y:off_y + M * N].view(M, N), ref[:, :N])
+    assert torch.all(out[:off_y] == 3.0) and torch.all(out[off_y + M * N:] == 3.0)
