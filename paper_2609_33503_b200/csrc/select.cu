@@ -51,7 +51,7 @@ __device__ __forceinline__ int block_prefix(int v, int* warp_tot) {
 // of 16 K / 32 K / 64 K scores (each pass a block-wide walk through L2).  Here a slice's keys are read once and stay in
 // shared memory (slices above kSelKeysMax keys are read again from L2 in each pass), the histograms of a
 // cluster's blocks are added through distributed shared memory by every block for itself, and the bin is found by a
-// block-wide prefix: 5.5 us, and 12.5 / 32 (40 segments) / 38 us.
+// block-wide prefix: 4.5 us, and 10.1 / 12.3 (15.7 for 40 segments) / 15.6 us.
 template <int NS>                                          // slices = blocks of a cluster
 __global__ void __launch_bounds__(kSelThreads)
 select_topk_kernel(ReqTable rt, int n_layers, int keys_cap, const float* raw, float* norm, int* anchors, DeviceStatus* st) {
@@ -210,12 +210,25 @@ __global__ void scale_scores_kernel(long long n, float factor, float* __restrict
   if (i < n) scores[i] *= factor;
 }
 
-// Blocks per segment: slices of at least 4 K keys (below that the kernel is its fixed chain of barriers: 5.5 us at 1 K keys),
-// fewer when the launch would not fit the GPU at once (two blocks of 1024 threads per SM).
+// Blocks per segment, by the longest segment of the call and by what the GPU holds at once: a block of 1024 threads has an SM
+// to itself, 32 clusters of four run together (36 take two waves: 11 -> 21 us at 16 K keys) and eight or nine of eight do (ten
+// take two: 17 -> 22 us at 64 K).  Measured in us, by slices:
+//   segments x keys     1      2      4      8        segments x keys     1      2      4      8
+//    1 x  6 K          7.4    8.2    8.8   11.6        12 x 32 K         25.1   15.6   12.6   22.7
+//    1 x  8 K          8.1    8.6    9.3   11.8        28 x 32 K         25.0   15.6   13.2   26.8
+//    1 x 12 K         10.4   10.1   10.0   12.1        40 x 32 K           -    15.7   25.4   40.4
+//    1 x 16 K         12.6   10.7   10.1   12.6         1 x 48 K         40.9   19.8   14.7   15.0
+//    8 x 16 K         12.8   11.0   10.3   14.1         1 x 64 K         65.1   39.3   17.1   15.6
+//    1 x 32 K         24.7   15.4   12.3   13.5        64 x 64 K         78.5   40.4   35.8   58.5
+// So one block up to 8 K keys (the chain of cluster barriers costs what the shorter walk gives), four up to 48 K, eight above,
+// fewer where they would not all run at once; and more again, two waves of them, rather than slices too long for shared memory.
 static int select_slices(const ReqTable& rt, long long n_seg, int sms) {
   int t_max = 1, s = 1;
   for (int b = 0; b < rt.n_req; ++b) t_max = std::max(t_max, rt.ctx_len[b]);
-  while (s < 8 && t_max > 4096 * s && n_seg * (2 * s) <= 2ll * sms) s *= 2;
+  const int want = t_max <= 8192 ? 1 : (t_max <= 49152 ? 4 : 8);
+  auto together = [&](int n) { return n == 8 ? n_seg * 16 <= sms : n_seg * n * 8 <= 7ll * sms; };
+  while (s < want && together(2 * s)) s *= 2;
+  while (s < 8 && t_max > kSelKeysMax * s && n_seg * (2 * s) <= 2ll * sms) s *= 2;
   return s;
 }
 

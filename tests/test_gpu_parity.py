@@ -193,6 +193,25 @@ def test_selection_and_schedule_at_slice_edges(ctx):
                 np.testing.assert_array_equal(got, ref.ranks(l))
 
 
+@pytest.mark.parametrize("ctx,L", [((8192, 100), 70), ((8193,), 32), ((8193, 5), 32), ((30000,), 33), ((49153,), 9), ((49153, 1), 5), ((24577,), 70),
+                                   ((98305,), 12)])
+def test_selection_by_segments_of_a_call(ctx, L):
+    """The slices of a segment follow from the longest one and from how many segments run at once (32 of four slices, 64 of two): on
+    both sides of each limit the anchors are the oracle's, with ties, bit for bit."""
+    rng = np.random.default_rng(L + sum(ctx))
+    cu = np.concatenate([[0], np.cumsum(ctx)])
+    k = [max(1, round(0.15 * t)) for t in ctx]
+    k_cu = np.concatenate([[0], np.cumsum(k)])
+    raw = (np.round(rng.standard_normal((L, cu[-1])) * 200) / 200).astype(np.float32)
+    anchors = torch.full((L, k_cu[-1]), -1, dtype=torch.int32, device="cuda")
+    B().relaxkv_select_topk(B().Shape(8, 2, 128, list(ctx)), L, k, torch.from_numpy(raw).cuda(), anchors)
+    assert_status_ok()
+    got = anchors.cpu().numpy()
+    for l in range(L):
+        for b in range(len(ctx)):
+            np.testing.assert_array_equal(got[l, k_cu[b]:k_cu[b + 1]], orc.topk(raw[l, cu[b]:cu[b + 1]].astype(np.float64), k[b]))
+
+
 @pytest.mark.parametrize("ctx,L", [((1,) + tuple(range(33, 96)), 6), ((1024,) * 64, 40), ((4097,) * 3 + (31, 32, 1), 40), ((65536, 640), 60),
                                    ((32768,), 40), ((32769, 5), 12), ((100001,), 6), ((70000, 4096, 1, 16385), 3)])
 def test_schedule_by_the_blocks_per_list(ctx, L):
