@@ -28,7 +28,6 @@
 #include "sm100_ptx.cuh"
 #include <algorithm>
 #include <atomic>
-#include <cstdlib>
 
 namespace relaxkv {
 
@@ -356,7 +355,6 @@ relaxkv_status launch_gemm_skinny(const void* x, const void* weight, const Skinn
   // (64 rows, two blocks / one: 2048 x 2048 8.4 / 6.9 us, 3072 x 2048 9.8 / 7.6, 4096 x 4096 12.9 / 10.7, 4096 x 14336 25.9 / 24.1; 33 rows 6.8 / 6.2,
   // 7.8 / 7.1, 11.0 / 10.2, 24.0 / 23.5; 40 tiles of 5120 x 5120 14.4 / 13.8 and 13.2 / 13.1; 17 rows, 2048 x 4096 7.4 / 7.8).
   p.whole_sm = (p.n_cols > kSkCols2 && p.tiles <= p.sms) || (p.n_cols > 32 && p.tiles * 4 <= p.sms);
-  if (getenv("SK_WHOLE") && p.n_cols > atoi(getenv("SK_WHOLE")) && p.tiles * 2 <= p.sms) p.whole_sm = true;
   p.n_stages = std::min(kSkStagesMax, sk_stages(p.n_cols, p.whole_sm));
   p.smem = (size_t)p.n_stages * (kSkWBytes + p.n_cols * kSkBK * 2) + kSkTail;
   relaxkv_status rc = RELAXKV_OK;
