@@ -2,8 +2,8 @@
 
 `binding` mirrors the C ABI of include/relaxkv.h one to one; `pipeline.RepairSession` keeps the
 device buffers of a request batch and issues the calls in the order of the paper's Algorithm 1;
-`inputs` holds the seeded synthetic workloads.  All computation is in librelaxkv.so (CUDA); build
-it with `python -m paper_2609_33503_b200.build`.
+`inputs` holds the seeded synthetic workloads.  All computation is in librelaxkv.so (CUDA), called
+through _calls.so (csrc/py_calls.cpp); `python -m paper_2609_33503_b200.build` builds both.
 """
 from . import inputs  # noqa: F401
 

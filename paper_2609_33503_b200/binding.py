@@ -80,6 +80,16 @@ _SIGNATURES = {
 _lib = None
 
 
+def _native():
+    """The module of csrc/py_calls.cpp: arguments and calls in native code."""
+    try:
+        from . import _calls
+    except ImportError as e:
+        raise RuntimeError(f"{os.path.join(_HERE, '_calls.so')} is missing or cannot be loaded ({e}): build it with "
+                           "`python -m paper_2609_33503_b200.build`") from e
+    return _calls
+
+
 def lib() -> ctypes.CDLL:
     """The loaded C-ABI library.  Raises if it has not been built (no fallback exists)."""
     global _lib
@@ -91,6 +101,7 @@ def lib() -> ctypes.CDLL:
         for name, (restype, args) in _SIGNATURES.items():
             fn = getattr(l, name)
             fn.restype, fn.argtypes = restype, [_CTYPE[c] for c in args.replace(" ", "")]
+            setattr(l, name, _native().bind(name, ctypes.cast(fn, ctypes.c_void_p).value, fn))
         _lib = l
     return _lib
 
@@ -127,6 +138,14 @@ def _i32(xs: Optional[Sequence[int]]):
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     return None if t is None else t.data_ptr()
+
+
+def _args(codes: str, *args):
+    """The arguments of an entry point as its bound form takes them, one code each: p a tensor (or None), h host integers (or None), s a
+    ctypes structure, . a plain value.  The first call puts the native function in this one's place."""
+    global _args
+    _args = _native().marshal
+    return _args(codes, *args)
 
 
 class Offsets:
@@ -247,8 +266,8 @@ def relaxkv_score_select(shape: Shape, q_layers: List[torch.Tensor], cache_layer
 def relaxkv_select_topk(shape: Shape, n_layers: int, k: Sequence[int], raw_scores: torch.Tensor,
                         anchors_out: torch.Tensor, norm_scores_out: Optional[torch.Tensor] = None,
                         stream=None) -> None:
-    _check(lib().relaxkv_select_topk(shape.ref(), int(n_layers), _i32(k), _ptr(raw_scores), _ptr(norm_scores_out),
-                                     _ptr(anchors_out), _stream(stream)), "relaxkv_select_topk")
+    _check(lib().relaxkv_select_topk(*_args("s.hppp.", shape.c, int(n_layers), k, raw_scores, norm_scores_out, anchors_out,
+                                            _stream(stream))), "relaxkv_select_topk")
 
 
 def relaxkv_build_active_sets(shape: Shape, n_layers: int, k: Sequence[int], anchors: torch.Tensor,
@@ -256,12 +275,9 @@ def relaxkv_build_active_sets(shape: Shape, n_layers: int, k: Sequence[int], anc
                               u_rank_out: torch.Tensor, r_rank_out: torch.Tensor, r_cu_out: torch.Tensor,
                               workspace: torch.Tensor, counts_pinned: Optional[torch.Tensor] = None,
                               stream=None) -> None:
-    _check(lib().relaxkv_build_active_sets(shape.ref(), int(n_layers), _i32(k), _ptr(anchors),
-                                           _ptr(highest_layer_out), _ptr(u_pos_out), _ptr(u_cu_out),
-                                           _ptr(u_rank_out), _ptr(r_rank_out), _ptr(r_cu_out), _ptr(counts_pinned),
-                                           _ptr(workspace),
-                                           workspace.nbytes,
-                                           _stream(stream)),
+    _check(lib().relaxkv_build_active_sets(*_args("s.hppppppppp..", shape.c, int(n_layers), k, anchors, highest_layer_out, u_pos_out,
+                                                  u_cu_out, u_rank_out, r_rank_out, r_cu_out, counts_pinned, workspace, workspace.nbytes,
+                                                  _stream(stream))),
            "relaxkv_build_active_sets")
 
 
@@ -272,20 +288,16 @@ def relaxkv_build_active_sets_static(shape: Shape, n_layers: int, k: Sequence[in
                                      stream=None) -> None:
     """Same outputs as relaxkv_build_active_sets, for callers that cannot supply a workspace: the
     scratch is a fixed array inside the library (at most 8192 counts: n_req * (1 + n_layers))."""
-    _check(lib().relaxkv_build_active_sets_static(shape.ref(), int(n_layers), _i32(k), _ptr(anchors),
-                                                  _ptr(highest_layer_out), _ptr(u_pos_out), _ptr(u_cu_out),
-                                                  _ptr(u_rank_out), _ptr(r_rank_out), _ptr(r_cu_out),
-                                                  _ptr(counts_pinned), _stream(stream)),
+    _check(lib().relaxkv_build_active_sets_static(*_args("s.hpppppppp.", shape.c, int(n_layers), k, anchors, highest_layer_out, u_pos_out,
+                                                         u_cu_out, u_rank_out, r_rank_out, r_cu_out, counts_pinned, _stream(stream))),
            "relaxkv_build_active_sets_static")
 
 
 def _attention(fn_name, shape, mode, cache, q_new, k_new, v_new, u_pos, u_cu, r_rank, r_cu_layer, max_targets,
                max_ctx, out, lse_out, workspace, stream):
     fn = getattr(lib(), fn_name)
-    _check(fn(shape.ref(), int(mode), cache.ref(), _ptr(q_new), _ptr(k_new), _ptr(v_new), _ptr(u_pos), _ptr(u_cu),
-              _ptr(r_rank), _ptr(r_cu_layer), q_new.shape[0], _i32(max_targets), _i32(max_ctx),
-              _ptr(out), _ptr(lse_out), _ptr(workspace),
-              workspace.nbytes, _stream(stream)), fn_name)
+    _check(fn(*_args("s.sppppppp.hhppp..", shape.c, int(mode), cache.c, q_new, k_new, v_new, u_pos, u_cu, r_rank, r_cu_layer,
+                     q_new.shape[0], max_targets, max_ctx, out, lse_out, workspace, workspace.nbytes, _stream(stream))), fn_name)
 
 
 def relaxkv_sparse_ctx_attention(shape: Shape, mode: int, cache: CacheView, q_new: torch.Tensor,
@@ -308,19 +320,16 @@ def relaxkv_sparse_ctx_attention_simt(shape, mode, cache, q_new, k_new, v_new, u
 def relaxkv_scatter_kv(shape: Shape, cache: CacheView, k_new: torch.Tensor, v_new: torch.Tensor,
                        u_pos: torch.Tensor, u_cu: torch.Tensor, r_rank: torch.Tensor, r_cu_layer: torch.Tensor,
                        max_targets: Sequence[int], stream=None) -> None:
-    _check(lib().relaxkv_scatter_kv(shape.ref(), cache.ref(), _ptr(k_new), _ptr(v_new), _ptr(u_pos), _ptr(u_cu),
-                                    _ptr(r_rank), _ptr(r_cu_layer), _i32(max_targets), _stream(stream)),
-           "relaxkv_scatter_kv")
+    _check(lib().relaxkv_scatter_kv(*_args("sspppppph.", shape.c, cache.c, k_new, v_new, u_pos, u_cu, r_rank, r_cu_layer, max_targets,
+                                           _stream(stream))), "relaxkv_scatter_kv")
 
 
 def relaxkv_gather_kv(shape: Shape, mode: int, cache: CacheView, k_new: Optional[torch.Tensor],
                       v_new: Optional[torch.Tensor], u_pos: torch.Tensor, u_cu: torch.Tensor, r_rank: torch.Tensor,
                       r_cu_layer: torch.Tensor, max_ctx: Sequence[int], k_ctx_out: torch.Tensor,
                       v_ctx_out: torch.Tensor, stream=None) -> None:
-    _check(lib().relaxkv_gather_kv(shape.ref(), int(mode), cache.ref(), _ptr(k_new), _ptr(v_new), _ptr(u_pos),
-                                   _ptr(u_cu), _ptr(r_rank), _ptr(r_cu_layer), _i32(max_ctx), _ptr(k_ctx_out),
-                                   _ptr(v_ctx_out), k_ctx_out.shape[0], _stream(stream)),
-           "relaxkv_gather_kv")
+    _check(lib().relaxkv_gather_kv(*_args("s.spppppphpp..", shape.c, int(mode), cache.c, k_new, v_new, u_pos, u_cu, r_rank, r_cu_layer,
+                                          max_ctx, k_ctx_out, v_ctx_out, k_ctx_out.shape[0], _stream(stream))), "relaxkv_gather_kv")
 
 
 def relaxkv_list_attention(shape: Shape, cache: CacheView, q_new: torch.Tensor, k_new: Optional[torch.Tensor],
@@ -328,21 +337,16 @@ def relaxkv_list_attention(shape: Shape, cache: CacheView, q_new: torch.Tensor, 
                            tgt_pos: torch.Tensor, tgt_cu: torch.Tensor, max_targets: Sequence[int],
                            max_ctx: Sequence[int], out: torch.Tensor, workspace: torch.Tensor,
                            lse_out: Optional[torch.Tensor] = None, stream=None) -> None:
-    _check(lib().relaxkv_list_attention(shape.ref(), cache.ref(), _ptr(q_new), _ptr(k_new), _ptr(v_new), _ptr(ctx_pos),
-                                        _ptr(ctx_cu), _ptr(tgt_pos), _ptr(tgt_cu), q_new.shape[0],
-                                        _i32(max_targets), _i32(max_ctx), _ptr(out), _ptr(lse_out), _ptr(workspace),
-                                        workspace.nbytes, _stream(stream)),
-           "relaxkv_list_attention")
+    _check(lib().relaxkv_list_attention(*_args("ssppppppp.hhppp..", shape.c, cache.c, q_new, k_new, v_new, ctx_pos, ctx_cu, tgt_pos, tgt_cu,
+                                               q_new.shape[0], max_targets, max_ctx, out, lse_out, workspace, workspace.nbytes,
+                                               _stream(stream))), "relaxkv_list_attention")
 
 
 def relaxkv_cache_attention(shape: Shape, cache: CacheView, q_new: torch.Tensor, tgt_pos: torch.Tensor, tgt_cu: torch.Tensor,
                             max_targets: Sequence[int], out: torch.Tensor, workspace: torch.Tensor,
                             lse_out: Optional[torch.Tensor] = None, stream=None) -> None:
-    _check(lib().relaxkv_cache_attention(shape.ref(), cache.ref(), _ptr(q_new), _ptr(tgt_pos), _ptr(tgt_cu),
-                                         q_new.shape[0], _i32(max_targets), _ptr(out), _ptr(lse_out),
-                                         _ptr(workspace), workspace.nbytes,
-                                         _stream(stream)),
-           "relaxkv_cache_attention")
+    _check(lib().relaxkv_cache_attention(*_args("ssppp.hppp..", shape.c, cache.c, q_new, tgt_pos, tgt_cu, q_new.shape[0], max_targets, out,
+                                                lse_out, workspace, workspace.nbytes, _stream(stream))), "relaxkv_cache_attention")
 
 
 def relaxkv_query_prefill_attention(shape: Shape, cache: CacheView, q: torch.Tensor, out: torch.Tensor, lse_out: torch.Tensor,
@@ -357,8 +361,8 @@ def relaxkv_query_prefill_attention(shape: Shape, cache: CacheView, q: torch.Ten
 
 def relaxkv_scatter_kv_lists(shape: Shape, cache: CacheView, k_new: torch.Tensor, v_new: torch.Tensor,
                              tgt_pos: torch.Tensor, tgt_cu: torch.Tensor, max_targets: Sequence[int], stream=None) -> None:
-    _check(lib().relaxkv_scatter_kv_lists(shape.ref(), cache.ref(), _ptr(k_new), _ptr(v_new), _ptr(tgt_pos), _ptr(tgt_cu),
-                                          _i32(max_targets), _stream(stream)), "relaxkv_scatter_kv_lists")
+    _check(lib().relaxkv_scatter_kv_lists(*_args("sspppph.", shape.c, cache.c, k_new, v_new, tgt_pos, tgt_cu, max_targets,
+                                                 _stream(stream))), "relaxkv_scatter_kv_lists")
 
 
 def relaxkv_mean_scores(shape: Shape, n_layers: int, scores: torch.Tensor, mean_out: torch.Tensor, stream=None) -> None:
@@ -436,8 +440,8 @@ def relaxkv_qk_norm_rope_append(shape: Shape, cache: CacheView, q: torch.Tensor,
                                 tgt_cu: torch.Tensor, max_targets: Sequence[int], theta: float, w_q_norm: Optional[torch.Tensor] = None,
                                 w_k_norm: Optional[torch.Tensor] = None, eps: float = 1e-6, stream=None) -> None:
     """relaxkv_qk_norm_rope of q [n, H, D] and k [n, H_kv, D], then relaxkv_scatter_kv_lists of k and v, both at tgt_pos."""
-    _check(lib().relaxkv_qk_norm_rope_append(shape.ref(), cache.ref(), _ptr(q), _ptr(k), _ptr(v), q.shape[0], _ptr(w_q_norm), _ptr(w_k_norm),
-                                             float(eps), _ptr(tgt_pos), _ptr(tgt_cu), _i32(max_targets), float(theta), _stream(stream)),
+    _check(lib().relaxkv_qk_norm_rope_append(*_args("ssppp.pp.pph..", shape.c, cache.c, q, k, v, q.shape[0], w_q_norm, w_k_norm, float(eps),
+                                                    tgt_pos, tgt_cu, max_targets, float(theta), _stream(stream))),
            "relaxkv_qk_norm_rope_append")
 
 
@@ -448,16 +452,14 @@ def relaxkv_swiglu(gate_up: torch.Tensor, out: torch.Tensor, stream=None) -> Non
 
 def relaxkv_target_positions(shape: Shape, u_pos, u_cu, r_rank, r_cu_layer, max_targets: Sequence[int],
                              positions_out: torch.Tensor, stream=None) -> None:
-    _check(lib().relaxkv_target_positions(shape.ref(), _ptr(u_pos), _ptr(u_cu), _ptr(r_rank), _ptr(r_cu_layer),
-                                          _i32(max_targets), _ptr(positions_out), _stream(stream)),
-           "relaxkv_target_positions")
+    _check(lib().relaxkv_target_positions(*_args("spppphp.", shape.c, u_pos, u_cu, r_rank, r_cu_layer, max_targets, positions_out,
+                                                 _stream(stream))), "relaxkv_target_positions")
 
 
 def relaxkv_carry_rows(shape: Shape, h_in: torch.Tensor, h_out: torch.Tensor, r_rank, r_cu_layer, r_cu_next,
                        max_next: Sequence[int], stream=None) -> None:
-    _check(lib().relaxkv_carry_rows(shape.ref(), _ptr(h_in), _ptr(h_out), int(h_in.shape[1]), _ptr(r_rank),
-                                    _ptr(r_cu_layer), _ptr(r_cu_next), _i32(max_next), _stream(stream)),
-           "relaxkv_carry_rows")
+    _check(lib().relaxkv_carry_rows(*_args("spp.ppph.", shape.c, h_in, h_out, int(h_in.shape[1]), r_rank, r_cu_layer, r_cu_next, max_next,
+                                           _stream(stream))), "relaxkv_carry_rows")
 
 
 def relaxkv_debug_wait_timeout(stream=None) -> None:

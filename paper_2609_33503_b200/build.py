@@ -1,4 +1,5 @@
-"""Builds the CUDA library (sm_100a only) in-tree: paper_2609_33503_b200/librelaxkv.so.
+"""Builds the CUDA library (sm_100a only) in-tree, paper_2609_33503_b200/librelaxkv.so, and the Python module through which the
+binding calls it, paper_2609_33503_b200/_calls.so.
 
 nvcc cross-compiles without a GPU.  Each .cu file is one translation unit, compiled in parallel.
 """
@@ -8,12 +9,14 @@ import concurrent.futures as cf
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 OBJ = os.path.join(HERE, "build")
 LIB = os.path.join(HERE, "librelaxkv.so")
+CALLS = os.path.join(HERE, "_calls.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
          "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
@@ -61,7 +64,18 @@ def build(force: bool = False, verbose: bool = False, ptxas_v: bool = False) -> 
         tmp = LIB + f".tmp{os.getpid()}"
         subprocess.check_call([NVCC, "-shared", "-o", tmp, *objs, *(["-ldl"] if NVTX else [])])
         os.replace(tmp, LIB)
+    build_calls(force)
     return LIB
+
+
+def build_calls(force: bool = False) -> str:
+    src, header = os.path.join(CSRC, "py_calls.cpp"), os.path.join(INCLUDE, "relaxkv.h")
+    if force or not os.path.exists(CALLS) or os.path.getmtime(CALLS) < max(os.path.getmtime(src), os.path.getmtime(header)):
+        tmp = CALLS + f".tmp{os.getpid()}"
+        subprocess.check_call([os.environ.get("CXX", "g++"), "-shared", "-fPIC", "-O2", "-std=c++17", "-Wall", "-I", INCLUDE,
+                               "-I", sysconfig.get_paths()["include"], src, "-o", tmp])
+        os.replace(tmp, CALLS)
+    return CALLS
 
 
 if __name__ == "__main__":
