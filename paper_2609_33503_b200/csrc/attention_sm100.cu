@@ -14,7 +14,8 @@
 // move through a 5-slot ring in the order K_0 V_0 K_1 V_1 ... and are signalled in pairs (V_j, K_{j+1}) - what
 // step j of the MMA warp consumes.
 // When a call has too few query tiles to fill the GPU, grid.y splits every pair's context; the blocks leave
-// normalised partial results that combine_splits_kernel merges by their log-sum-exp.  The K/V tensor maps
+// normalised partial results that combine_splits_kernel merges by their log-sum-exp.  Of a call over lists that
+// has pairs enough but none to follow its longest ones, only those are cut (attention_pieces.cuh).  The K/V tensor maps
 // cover either the materialised mixed context (the repair calls) or the cache itself (relaxkv_cache_attention).
 // Calls over short gathered contexts (at most 128 key tiles, one split) take attention_persist_kernel below: one
 // block per SM walks the same list of (tile pair, KV head) items and overlaps each turn-over with its neighbours.

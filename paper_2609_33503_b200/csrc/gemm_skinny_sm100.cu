@@ -6,18 +6,19 @@
 // whole SM's above 64 rows, where x takes as much of a stage as the weights, and from 33 rows on for few tiles).  128 to 192 KB of weights per SM are in
 // flight, and x rows that do not exist are neither multiplied nor, past the 16
 // granularity, staged.  A thread-block CLUSTER of S blocks shares a tile and splits K: block r multiplies K blocks
-// [r n_k / S, (r + 1) n_k / S) into its own TMEM accumulator, writes the partial tile into its own shared memory, and
-// after a cluster barrier every block sums, for the 128 / S features it owns, the S
-// partials in rank order - through distributed shared memory - adds the residual and writes bf16.  A fixed order: results
+// [r n_k / S, (r + 1) n_k / S) into its own TMEM accumulator, writes the partial tile into its own shared memory and
+// pushes to every other block, in one bulk copy each, the features that one owns (128 / S); every block then sums the S
+// partials of its own features in rank order, adds the residual and writes bf16.  A fixed order: results
 // do not depend on timing.  No scratch in global memory.  Up to four rows (a decoded batch) K is always summed in eight parts, each
 // in TMEM columns of its own where a block has several: the bits then depend on K alone, not on how many blocks share a tile, so a
 // projection gives the same bits stacked with others and by itself.
 // Up to three output segments (feature ranges going to different buffers) serve the fused Q/K/V projection; the fused
 // gate/up projection takes 64 gate rows and their 64 up rows as one tile and applies the activation in the epilogue.
 // Bound by HBM (N K 2 bytes); with 128 rows of x as the M side, one block per SM and plain launches, four rows of a decode
-// step went through the FMA pipe (gate/up 34816 x 5120 77 us, 5120 x 17408 40 us, 6144 x 4096 13.6 us; now 56, 32 and 12.2:
-// 6.2, 5.6 and 4.1 TB/s), 57 rows took 65 / 36 / 16.2 us (now 59 / 34 / 13.8) and 128 rows 65 / 37.7 / 17.2 us (64 / 37.8 /
-// 17.4, and 2 to 3 us less behind a short kernel, where the start is hidden).
+// step went through the FMA pipe (gate/up 34816 x 5120 77 us, 5120 x 17408 40 us, 6144 x 4096 13.6 us; now 55, 32 and 12.3:
+// 6.5, 5.6 and 4.1 TB/s), 57 rows took 65 / 36 / 16.2 us (now 56 / 32.5 / 12.3) and 128 rows 65 / 37.7 / 17.2 us (60.5 / 35.9 /
+// 15.5, and 2 to 3 us less behind a short kernel, where the start is hidden).  What is left above the bytes is about 4 us of a launch: the first
+// products 3 us behind the wait, the exchange of the partial tiles and the hand-over to the next kernel behind the last.
 // Launched chained: barriers, tensor memory and an L2 prefetch of the ring's first weight tiles come before the wait for
 // the kernels in front (a prefetch only: the weights are read after the wait, whoever wrote them).
 // The cluster barriers have no time limit, so every thread executes all of them whatever its (bounded) waits on the
