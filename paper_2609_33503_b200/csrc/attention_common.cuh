@@ -16,6 +16,8 @@ struct AttnPlan {
   // what the attention kernel's K/V tensor maps cover: the materialised context, or the cache itself
   const void* k_base; const void* v_base;
   unsigned long long kv_token_stride_bytes, kv_head_stride_bytes;
+  const void* k_new = nullptr; const void* v_new = nullptr;
+  int all_fresh = 0;      // > 0: if both lists hold that many entries the context is k_new / v_new themselves (all_rows_fresh)
   int dense_ctx;          // 1: context = the cache's own rows (request b starts at rt.tok_off[b]), limits are positions
 };
 
@@ -32,7 +34,7 @@ inline relaxkv_status prepare_attention(
     const int32_t* u_pos, const int32_t* u_cu, const int32_t* r_rank, const int32_t* r_cu_layer,
     int64_t n_target_rows, const int32_t* h_max_targets, const int32_t* h_max_ctx,
     void* out, void* workspace, size_t workspace_bytes, cudaStream_t stream, AttnPlan& plan,
-    const int32_t* fresh_row = nullptr) {
+    const int32_t* fresh_row = nullptr, bool fresh_in_place = false) {
   relaxkv_status rc = check_shape(shape);
   if (rc != RELAXKV_OK) return rc;
   if ((rc = check_cache(shape, cache, true)) != RELAXKV_OK) return rc;
@@ -71,9 +73,15 @@ inline relaxkv_status prepare_attention(
   plan.kv_head_stride_bytes = (unsigned long long)shape->head_dim * 2;
   plan.kv_token_stride_bytes = (unsigned long long)shape->n_kv_heads * shape->head_dim * 2;
   plan.dense_ctx = 0;
+  // The first layer of a repair renews its whole context (R_0 = U).  Whether a layer does is in the device's lists; the host's bounds say
+  // where it can be.
+  plan.k_new = k_new;
+  plan.v_new = v_new;
+  plan.all_fresh = fresh_in_place && shape->n_req == 1 && mode == RELAXKV_CTX_UNION && k_new && !fresh_row &&
+                           h_max_targets[0] == h_max_ctx[0] && n_target_rows == h_max_ctx[0] ? (int)n_target_rows : 0;
   return launch_gather(shape, mode, cache, k_new, v_new, u_pos, u_cu, r_rank, r_cu_layer, fresh_row,
                        fresh_row ? need_ctx : 0, n_target_rows, need_ctx + kCtxPadRows, plan.kctx, plan.vctx, plan.ctx_rows,
-                       reinterpret_cast<int*>(plan.split_lse), stream);
+                       reinterpret_cast<int*>(plan.split_lse), plan.all_fresh, stream);
 }
 
 }  // namespace relaxkv

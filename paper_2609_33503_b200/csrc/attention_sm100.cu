@@ -162,7 +162,8 @@ __device__ __forceinline__ void softmax_step(uint32_t t_s, uint32_t t_o, int lim
 template <int D>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                       const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ ReqTable rt,
+                       const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_k_new,
+                       const __grid_constant__ CUtensorMap tm_v_new, int all_fresh, const __grid_constant__ ReqTable rt,
                        const __grid_constant__ PieceTable pt, int mode, int allow_empty, int head_inner, int dense_ctx, int H, int Hkv, int pair_targets, float scale_log2,
                        const int* u_pos, const int* u_cu, const int* r_rank, const int* r_cu,
                        long long n_target_rows, uint16_t* __restrict__ out, float* __restrict__ lse_out,
@@ -342,10 +343,12 @@ attention_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       // The tiles travel in the order K_0 V_0 K_1 V_1 ... through the ring slots u % kRing (u = 2j for K_j, 2j + 1
       // for V_j; j counted from j0).  They are signalled in PAIRS p = (V_{p-1}, K_p): step j of the MMA warp needs
       // exactly pair j + 1 (V_j for P V, K_{j+1} for the next Q K^T), so it waits once and frees once per step.
+      const bool fresh = all_rows_fresh(all_fresh, u_cu, r_cu);
+      const CUtensorMap *map_k = fresh ? &tm_k_new : &tm_k, *map_v = fresh ? &tm_v_new : &tm_v;
       auto load_tile = [&](int u, uint32_t bar) {
         const int s = u % kRing;
         const int row = (int)(ctx_base + (long long)(j0 + (u >> 1)) * kBN);
-        const CUtensorMap* tm = (u & 1) ? &tm_v : &tm_k;
+        const CUtensorMap* tm = (u & 1) ? map_v : map_k;
         for (int hf = 0; hf < kHalves; ++hf)
           tma_load_3d(kv_smem + s * L::kTileBytes + hf * kHalfBytes, tm, bar, hf * 64, hd, row);
       };
@@ -653,7 +656,8 @@ __device__ __forceinline__ WorkItem decode_item(int id, const ReqTable& rt, int 
 template <int D>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                         const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ ReqTable rt,
+                         const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_k_new,
+                         const __grid_constant__ CUtensorMap tm_v_new, int all_fresh, const __grid_constant__ ReqTable rt,
                          int mode, int allow_empty, int head_inner, int H, int Hkv, int pair_targets, float scale_log2,
                          const int* u_pos, const int* u_cu, const int* r_rank, const int* r_cu,
                          long long n_target_rows, uint16_t* __restrict__ out, float* __restrict__ lse_out,
@@ -745,10 +749,12 @@ attention_persist_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
         mbar_expect_tx(bar_q, (uint32_t)(kHalves * pair_targets * G * 128));
         for (int hf = 0; hf < kHalves; ++hf) tma_load_3d(q_smem + hf * 2 * kHalfBytes, &tm_q, bar_q, hf * 64, it.hd * G, it.q_row_base);
       };
+      const bool fresh = all_rows_fresh(all_fresh, u_cu, r_cu);
+      const CUtensorMap *map_k = fresh ? &tm_k_new : &tm_k, *map_v = fresh ? &tm_v_new : &tm_v;
       auto load_tile = [&](int u, const WorkItem& it, int j, uint32_t bar) {      // u = 2 g for K of global tile g, 2 g + 1 for V
         const int s = u % kRing;
         const int row = it.ctx_base + j * kBN;
-        const CUtensorMap* tm = (u & 1) ? &tm_v : &tm_k;
+        const CUtensorMap* tm = (u & 1) ? map_v : map_k;
         for (int hf = 0; hf < kHalves; ++hf) tma_load_3d(kv_smem + s * L::kTileBytes + hf * kHalfBytes, tm, bar, hf * 64, it.hd, row);
       };
       WorkItem cur, nxt;
@@ -1257,6 +1263,12 @@ static relaxkv_status launch_attention(const relaxkv_shape* shape, int mode, Att
       !make_map_3d(&tm_v, plan.v_base, D, Hkv, (uint64_t)plan.ctx_rows, plan.kv_head_stride_bytes, plan.kv_token_stride_bytes, 1u,
                    (uint32_t)kBN))
     return RELAXKV_ERR_CUDA;
+  // The fresh rows as a context (rows past the last read as zeros, as the materialised context's do).
+  CUtensorMap tm_k_new = tm_k, tm_v_new = tm_v;
+  if (plan.all_fresh > 0 &&
+      (!make_map_3d(&tm_k_new, plan.k_new, D, Hkv, (uint64_t)plan.all_fresh, (uint64_t)D * 2, row_kv, 1u, (uint32_t)kBN) ||
+       !make_map_3d(&tm_v_new, plan.v_new, D, Hkv, (uint64_t)plan.all_fresh, (uint64_t)D * 2, row_kv, 1u, (uint32_t)kBN)))
+    return RELAXKV_ERR_CUDA;
   DeviceStatus* st = status_word();
   if (!st) return RELAXKV_ERR_CUDA;
   // the materialised context (K and V, all heads) against the 126 MB L2
@@ -1338,12 +1350,12 @@ static relaxkv_status launch_attention(const relaxkv_shape* shape, int mode, Att
     if (tun && tun->attention_grid_blocks > 0) pgrid = std::min<long long>(grid, tun->attention_grid_blocks);
     RELAXKV_RANGE("attention_persist_kernel");
     return cuda_ok(launch_chained(pk, (unsigned)pgrid, kAttnThreads, PersistSmem<D>::kDynamic, stream,
-        tm_q, tm_k, tm_v, plan.rt, mode, allow_empty, head_inner, H, Hkv, pair_targets, shape->softmax_scale * kLog2eA,
+        tm_q, tm_k, tm_v, tm_k_new, tm_v_new, plan.all_fresh, plan.rt, mode, allow_empty, head_inner, H, Hkv, pair_targets, shape->softmax_scale * kLog2eA,
         u_pos, u_cu, r_rank, r_cu_layer, n_target_rows, static_cast<uint16_t*>(out), lse_out, (int)grid, counter, st));
   }
   RELAXKV_RANGE("attention_sm100_kernel");
   relaxkv_status rc = cuda_ok(launch_chained(kern, dim3((unsigned)units, (unsigned)n_splits), kAttnThreads, AttnSmem<D>::kDynamic, stream,
-      tm_q, tm_k, tm_v, plan.rt, pt, mode, allow_empty, head_inner, plan.dense_ctx, H, Hkv, pair_targets, shape->softmax_scale * kLog2eA,
+      tm_q, tm_k, tm_v, tm_k_new, tm_v_new, plan.all_fresh, plan.rt, pt, mode, allow_empty, head_inner, plan.dense_ctx, H, Hkv, pair_targets, shape->softmax_scale * kLog2eA,
       u_pos, u_cu, r_rank, r_cu_layer, n_target_rows, static_cast<uint16_t*>(out), lse_out, plan.split_o, plan.split_lse, st));
   if (rc == RELAXKV_OK && pt.most > 0) {
     const long long warps = (long long)pt.slot_cu[B] * H;
@@ -1368,10 +1380,21 @@ extern "C" relaxkv_status relaxkv_sparse_ctx_attention(
     void* out, float* lse_out, void* workspace, size_t workspace_bytes, relaxkv_stream stream_) {
   RELAXKV_RANGE("relaxkv_sparse_ctx_attention");
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
+  // The fresh rows may be read while outputs are written, unless a caller has the outputs take their place.
+  bool fresh_in_place = false;
+  if (shape && n_target_rows > 0) {
+    auto apart = [&](const void* x, const void* y, long long y_bytes) {
+      const uintptr_t x0 = reinterpret_cast<uintptr_t>(x), y0 = reinterpret_cast<uintptr_t>(y);
+      const uintptr_t x_bytes = (uintptr_t)n_target_rows * shape->n_kv_heads * shape->head_dim * 2;
+      return y == nullptr || x0 + x_bytes <= y0 || y0 + (uintptr_t)y_bytes <= x0;
+    };
+    const long long o_bytes = (long long)n_target_rows * shape->n_q_heads * shape->head_dim * 2, l_bytes = (long long)n_target_rows * shape->n_q_heads * 4;
+    fresh_in_place = apart(k_new, out, o_bytes) && apart(v_new, out, o_bytes) && apart(k_new, lse_out, l_bytes) && apart(v_new, lse_out, l_bytes);
+  }
   AttnPlan plan;
   relaxkv_status rc = prepare_attention(shape, mode, cache, q_new, k_new, v_new, u_pos, u_cu, r_rank, r_cu_layer,
                                         n_target_rows, h_max_targets, h_max_ctx, out, workspace, workspace_bytes,
-                                        stream, plan);
+                                        stream, plan, nullptr, fresh_in_place);
   if (rc != RELAXKV_OK) return rc;
   if (shape->head_dim == 128)
     return launch_attention<128>(shape, mode, plan, q_new, u_pos, u_cu, r_rank, r_cu_layer, n_target_rows, out, lse_out, stream);

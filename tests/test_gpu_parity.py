@@ -1295,3 +1295,56 @@ def test_longest_pairs_in_pieces(H, Hkv, D, ctx, targets):
     assert B().relaxkv_read_device_status()[0] == B().ERR_BAD_INDEX
     refused = torch.cat([torch.full((n,), n > 1) for n in n_t]).cuda()
     assert torch.all(outs[3][refused] == 3.0)
+
+
+@pytest.mark.parametrize("n,H,Hkv,D", [(1, 8, 2, 128), (51, 40, 8, 128), (127, 8, 2, 128), (128, 32, 8, 128), (129, 8, 2, 64), (300, 40, 8, 128),
+                                       (2458, 32, 8, 128), (2500, 8, 8, 64)])
+def test_a_context_of_fresh_rows_alone_is_read_in_place(n, H, Hkv, D):
+    """One request whose layer renews its whole context (exact bounds): the fresh rows are the context.  The same bits as by the general way
+    (a bound that is one too large), whatever lies behind the rows and in the workspace, and nothing but the lists decides: equal bounds
+    over a layer that renews less take the general way."""
+    from paper_2609_33503_b200.pipeline import RepairSession
+    b, T = B(), n + 1700
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    normal = lambda *s: torch.randn(*s, device="cuda", generator=gen).to(torch.bfloat16)
+    few = max(1, n - 3)
+    s = RepairSession(H, Hkv, D, [T], [4], 2, [n])
+    pos = torch.randperm(T, device="cuda", generator=gen)[:n].sort().values.to(torch.int32)
+    # layer 0 renews all n, layer 1 the first `few` of them
+    s.u_pos[:n] = pos
+    s.u_cu.copy_(torch.tensor([0, n], dtype=torch.int32))
+    ranks = torch.cat([torch.arange(n), torch.arange(n - few, n)]).to(torch.int32).cuda()
+    s.r_rank[:n + few] = ranks
+    s.r_cu.copy_(torch.tensor([0, n, n + few], dtype=torch.int32))
+    cache = b.CacheView(normal(T, Hkv, D), normal(T, Hkv, D), [0])
+
+    def rows(m, heads):                                      # with NaN behind them
+        t = torch.full((m + 200, heads, D), float("nan"), dtype=torch.bfloat16, device="cuda")
+        t[:m] = normal(m, heads, D)
+        return t[:m]
+    q, k, v = rows(n, H), rows(n, Hkv), rows(n, Hkv)
+
+    def run(layer, n_r, bound_r, bound_u):
+        s.workspace.fill_(0xFF)
+        out, lse = torch.zeros(n_r, H, D, dtype=torch.bfloat16, device="cuda"), torch.zeros(H, n_r, device="cuda")
+        s.attention(layer, cache, q[:n_r], k[:n_r], v[:n_r], out, [bound_r], [bound_u], lse_out=lse)
+        assert_status_ok()
+        return out, lse
+    got, want = run(0, n, n, n), run(0, n, n, n + 1)
+    assert torch.isfinite(got[0]).all() and torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    if H == Hkv:                                             # an output in the place of the fresh values
+        v_kept = v.clone()
+        s.attention(0, cache, q, k, v, v, [n], [n])
+        assert_status_ok()
+        assert torch.equal(v, want[0])
+        v.copy_(v_kept)
+    if few < n:
+        want = run(1, few, few, n)
+        got = run(1, n, n, n)                                # rows past the layer's own stay as they were
+        assert torch.isfinite(got[0]).all() and torch.equal(got[0][:few], want[0]) and not got[0][few:].any()
+        lists = s.r_rank.clone()
+        s.r_rank[1] = 0                                      # a rank twice: no list of the schedule
+        s.attention(0, cache, q, k, v, torch.empty(n, H, D, dtype=torch.bfloat16, device="cuda"), [n], [n])
+        status, detail = b.relaxkv_read_device_status()
+        assert status == b.ERR_BAD_INDEX
+        s.r_rank.copy_(lists)
