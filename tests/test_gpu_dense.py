@@ -142,6 +142,27 @@ def test_stacked_projections_give_the_bits_of_single_ones(M, n_q, n_kv, K):
     assert st == 0, (st, detail)
 
 
+@pytest.mark.parametrize("n_q,n_kv,K", [(264, 8, 3576), (2368, 8, 3584), (264, 136, 4088), (4096, 512, 4096), (264, 8, 4104), (264, 8, 8184), (1024, 264, 8192),
+                                        (2400, 264, 16376), (1024, 264, 16384)])
+def test_one_row_by_the_features_of_a_warp(n_q, n_kv, K):
+    """One row: whether a warp has one feature or two follows from K alone.  A stacked matrix and its pieces on both sides of each line: equal
+    bits, rows around the output untouched, and against the oracle."""
+    x = rnd(1, K, seed=71)
+    ws = [rnd(n, K, scale=K ** -0.5, seed=72 + i) for i, n in enumerate((n_q, n_kv, n_kv))]
+    outs = [torch.full((1, n), 7.0, dtype=torch.bfloat16, device="cuda") for n in (n_q, n_kv, n_kv)]
+    B().relaxkv_linear_qkv(x, B().stack_qkv(*ws), *outs)
+    for w, out in zip(ws, outs):
+        one, res = torch.full((3, w.shape[0]), 7.0, dtype=torch.bfloat16, device="cuda"), rnd(1, w.shape[0], seed=75)
+        B().relaxkv_linear(x, w, one[1:2])
+        assert torch.equal(one[1:2], out) and (one[0] == 7.0).all() and (one[2] == 7.0).all()
+        ref = blk.linear(blk.f64(bits(x)), blk.f64(bits(w)), None)
+        close(out, ref, abs_floor=2e-3)
+        B().relaxkv_linear(x, w, one[1:2], residual=res)
+        close(one[1:2], ref + blk.f64(bits(res)), abs_floor=2e-3)
+    st, detail = B().relaxkv_read_device_status()
+    assert st == 0, (st, detail)
+
+
 @pytest.mark.parametrize("M,N,K", [(32, 4736, 520), (33, 4736, 520), (33, 4744, 520), (49, 4096, 4104), (64, 4736, 1032), (64, 128, 8), (48, 2048, 1000)])
 def test_one_block_per_sm_from_33_rows(M, N, K):
     """Both sides of the line where few tiles (37 of 128 weight rows) take a whole SM's shared memory per block: against the oracle,
