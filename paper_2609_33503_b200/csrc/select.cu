@@ -220,12 +220,13 @@ __global__ void scale_scores_kernel(long long n, float factor, float* __restrict
 //    1 x 16 K         12.6   10.7   10.1   12.6         1 x 48 K         40.9   19.8   14.7   15.0
 //    8 x 16 K         12.8   11.0   10.3   14.1         1 x 64 K         65.1   39.3   17.1   15.6
 //    1 x 32 K         24.7   15.4   12.3   13.5        64 x 64 K         78.5   40.4   35.8   58.5
-// So one block up to 8 K keys (the chain of cluster barriers costs what the shorter walk gives), four up to 48 K, eight above,
-// fewer where they would not all run at once; and more again, two waves of them, rather than slices too long for shared memory.
+// (scores spread over many bins).  Equal leading bits make the histogram's additions queue up, the longer the more keys a block has: scores of 16 query
+// rows over 6719 keys took 4.6 us more in one block than in two.  So slices of at most 4 K keys, up to eight, but fewer where they would not
+// all run at once; and more again, two waves of them, rather than slices too long for shared memory.
 static int select_slices(const ReqTable& rt, long long n_seg, int sms) {
   int t_max = 1, s = 1;
   for (int b = 0; b < rt.n_req; ++b) t_max = std::max(t_max, rt.ctx_len[b]);
-  const int want = t_max <= 8192 ? 1 : (t_max <= 49152 ? 4 : 8);
+  const int want = t_max <= 4096 ? 1 : (t_max <= 8192 ? 2 : (t_max <= 16384 ? 4 : 8));
   auto together = [&](int n) { return n == 8 ? n_seg * 16 <= sms : n_seg * n * 8 <= 7ll * sms; };
   while (s < want && together(2 * s)) s *= 2;
   while (s < 8 && t_max > kSelKeysMax * s && n_seg * (2 * s) <= 2ll * sms) s *= 2;
