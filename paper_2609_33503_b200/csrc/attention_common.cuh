@@ -12,7 +12,8 @@ struct AttnPlan {
   long long ctx_rows;     // rows the two buffers hold (tensor-map extent)
   long long sum_targets;  // sum of the host bounds on |R_{l,b}|
   float* split_o;         // workspace for a context split across blocks: [split_rows_cap, H, D] and [split_rows_cap, H]
-  float* split_lse;       // (its first word, zeroed by the gather, is the work counter of the persistent form)
+  float* split_lse;       // (the first word of split_o, zeroed by the gather, is the work counter of the persistent form)
+  int* refused = nullptr; // workspace: per request, whether its blocks refuse it (written by the gather)
   // what the attention kernel's K/V tensor maps cover: the materialised context, or the cache itself
   const void* k_base; const void* v_base;
   unsigned long long kv_token_stride_bytes, kv_head_stride_bytes;
@@ -68,6 +69,7 @@ inline relaxkv_status prepare_attention(
   plan.ctx_rows = ws.ctx_rows_cap;
   plan.split_o = reinterpret_cast<float*>(base + ws.split_o);
   plan.split_lse = reinterpret_cast<float*>(base + ws.split_lse);
+  plan.refused = reinterpret_cast<int*>(base + ws.refused);
   plan.k_base = plan.kctx;
   plan.v_base = plan.vctx;
   plan.kv_head_stride_bytes = (unsigned long long)shape->head_dim * 2;
@@ -81,7 +83,8 @@ inline relaxkv_status prepare_attention(
                            h_max_targets[0] == h_max_ctx[0] && n_target_rows == h_max_ctx[0] ? (int)n_target_rows : 0;
   return launch_gather(shape, mode, cache, k_new, v_new, u_pos, u_cu, r_rank, r_cu_layer, fresh_row,
                        fresh_row ? need_ctx : 0, n_target_rows, need_ctx + kCtxPadRows, plan.kctx, plan.vctx, plan.ctx_rows,
-                       reinterpret_cast<int*>(plan.split_lse), plan.all_fresh, stream);
+                       reinterpret_cast<int*>(plan.split_o),
+                       {plan.refused, plan.split_lse, split_rows_cap(shape), shape->n_q_heads, plan.rt.bound_a, plan.rt.bound_b}, plan.all_fresh, stream);
 }
 
 }  // namespace relaxkv

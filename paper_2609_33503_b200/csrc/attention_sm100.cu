@@ -1102,23 +1102,29 @@ constexpr long long kCombineFewWarps = 64;
 constexpr int kMaxCombineSplits = 1024;       // four warps x 4 KB of weights
 
 // Merges the partial results of a context split: out = sum_s w_s O_s / sum_s w_s with w_s = exp(lse_s - max lse).
-// One warp per (target row, query head), U partial results of it in flight; rows past the true target count are left alone.
-// PIECES: the rows are the slots of the pairs that were cut (pt).
-template <int U, bool PIECES>
+// One warp per (target row, query head), U partial results of it in flight.  Rows past the true target count, the rows of requests that the
+// blocks in front refused (marked, kRefusedLse) and, after an expired wait, all rows are left alone: there are no partial results of them.
+// ROWS: the rows of the call.  PIECES: the slots of the pairs that were cut (pt); what was refused is said per request.  LISTS: the rows of a call that
+// no gather went before, whose counts are held against the bounds here.
+// The loads are asked for side by side and whether a row is written is looked at last: a return before the sums lets the compiler move the
+// loads behind it (attention of four requests of 700 to 1300 tokens, in pieces, 30.9 us a call / 27.8).
+enum MergeForm { ROWS, PIECES, LISTS };
+template <int U, MergeForm FORM>
 __global__ void __launch_bounds__(kCombineThreads)
 combine_splits_kernel(const float* part_o, const float* part_lse, int n_splits,
-                      long long n_target_rows, int H, int D, const int* r_cu, int n_req,
-                      uint16_t* __restrict__ out, float* __restrict__ lse_out, const __grid_constant__ PieceTable pt, int pair_targets) {
+                      long long n_target_rows, int H, int D, const int* r_cu, const int* refused, int n_req,
+                      uint16_t* __restrict__ out, float* __restrict__ lse_out, const __grid_constant__ PieceTable pt, int pair_targets,
+                      DeviceStatus* st) {
   // the splits' weights of this warp's (row, head): the lanes fetch the log-sum-exps side by side (a serial walk over
   // the splits would pay one memory latency per split), the sums below still run in split order
   __shared__ float wgt_s[kCombineThreads / 32][kMaxCombineSplits];
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long w = (long long)blockIdx.x * (kCombineThreads / 32) + wib;
-  const long long slot = w / H, slot_rows = PIECES ? pt.slot_cu[n_req] : n_target_rows;
+  const long long slot = w / H, slot_rows = FORM == PIECES ? pt.slot_cu[n_req] : n_target_rows;
   const int h = (int)(w - slot * H);
   const bool mine = slot < slot_rows;
   int b = 0;
-  if (PIECES) {
+  if (FORM == PIECES) {
     while (b + 1 < n_req && slot >= pt.slot_cu[b + 1]) ++b;
     n_splits = pt.pieces[b];
   }
@@ -1136,16 +1142,17 @@ combine_splits_kernel(const float* part_o, const float* part_lse, int n_splits,
   // A launch of a few rows is a chain of memory latencies, so the first partial results, the log-sum-exps and the row
   // count are fetched side by side (what rows past the true count or empty splits hold is not used), and each further
   // group of partial results while the one before is added up.
+  const int status = *reinterpret_cast<volatile int*>(&st->status);
   float4 v[U];
 #pragma unroll
   for (int u = 0; u < U; ++u) v[u] = u < n_splits ? load(u) : make_float4(0.f, 0.f, 0.f, 0.f);
   long long row = slot;
   bool here = true;                             // rows past the true counts (and requests that were refused) hold nothing
-  if (PIECES) {
+  if (FORM == PIECES) {
     const int c0 = r_cu[0], cb = r_cu[b], nr = r_cu[b + 1] - cb, rel = (int)slot - pt.slot_cu[b], p_rev = rel / pair_targets;
     const int rho = ((nr + pair_targets - 1) / pair_targets - 1 - p_rev) * pair_targets + rel - p_rev * pair_targets;
     row = (long long)(cb - c0) + rho;
-    here = rho >= 0 && rho < nr && nr <= pt.bound[b] && (long long)(cb - c0) + nr <= n_target_rows;
+    here = rho >= 0 && rho < nr && nr <= pt.bound[b] && (long long)(cb - c0) + nr <= n_target_rows && refused[b] == 0;
   } else {
     here = slot < (r_cu ? min((long long)(r_cu[n_req] - r_cu[0]), n_target_rows) : n_target_rows);
   }
@@ -1155,7 +1162,6 @@ combine_splits_kernel(const float* part_o, const float* part_lse, int n_splits,
     wgt_s[wib][sp] = l;
     mx = fmaxf(mx, l);
   }
-  if (!here) return;
   mx = warp_reduce_max(mx);
   __syncwarp();
   for (int sp = lane; sp < n_splits; sp += 32) {
@@ -1179,6 +1185,11 @@ combine_splits_kernel(const float* part_o, const float* part_lse, int n_splits,
       v[u] = nx[u];
     }
   }
+  if (FORM == LISTS) {
+    while (b + 1 < n_req && slot >= r_cu[b + 1] - r_cu[0]) ++b;
+    here = here && r_cu[b + 1] - r_cu[b] <= pt.bound[b] && r_cu[b + 1] - r_cu[0] <= n_target_rows;
+  }
+  if (!here || mx == __uint_as_float(kRefusedLse) || status == RELAXKV_ERR_TIMEOUT) return;
   const float inv = den > 0.f ? 1.f / den : 0.f;
   uint16_t* optr = out + (row * H + h) * D + lane * per;
   __nv_bfloat162 h01 = __floats2bfloat162_rn(acc[0] * inv, acc[1] * inv);
@@ -1192,7 +1203,7 @@ combine_splits_kernel(const float* part_o, const float* part_lse, int n_splits,
 
 relaxkv_status launch_combine_splits(const float* part_o, const float* part_lse, int n_splits, long long n_target_rows, int H,
                                      int D, const int32_t* r_cu, int n_req, long long rows_bound, void* out, float* lse_out,
-                                     cudaStream_t stream) {
+                                     DeviceStatus* st, cudaStream_t stream) {
   const long long warps = rows_bound * H;
   if (warps <= 0) return RELAXKV_OK;
   if (n_splits > kMaxCombineSplits) return RELAXKV_ERR_UNSUPPORTED_SHAPE;
@@ -1200,9 +1211,9 @@ relaxkv_status launch_combine_splits(const float* part_o, const float* part_lse,
   // A decoded row whose context one wave of blocks shares (18 splits with eight KV heads): all of them in one go, one memory latency less (12 layers of a
   // decode step at 32 K 1985 us, 1970 so).  Up to eight splits the small form: with the registers of the large one beside it the next projection's
   // blocks come later (16 layers of four requests 1969 / 2017).
-  auto kern = n_splits > 8 && warps <= kCombineFewWarps ? combine_splits_kernel<20, false> : combine_splits_kernel<8, false>;
+  auto kern = n_splits > 8 && warps <= kCombineFewWarps ? combine_splits_kernel<20, ROWS> : combine_splits_kernel<8, ROWS>;
   return cuda_ok(launch_chained(kern, (unsigned)((warps + wpb - 1) / wpb), kCombineThreads, 0, stream, part_o,
-                                part_lse, n_splits, (long long)n_target_rows, H, D, r_cu, n_req, static_cast<uint16_t*>(out), lse_out, PieceTable{}, 0));
+                                part_lse, n_splits, (long long)n_target_rows, H, D, r_cu, nullptr, n_req, static_cast<uint16_t*>(out), lse_out, PieceTable{}, 0, st));
 }
 
 // ---- host side ---------------------------------------------------------------------------------------
@@ -1345,7 +1356,7 @@ static relaxkv_status launch_attention(const relaxkv_shape* shape, int mode, Att
         return RELAXKV_ERR_CUDA;
       pattr_done[dev].store(1, std::memory_order_release);
     }
-    int* counter = reinterpret_cast<int*>(plan.split_lse);          // unused by a one-split call; zeroed by the gather
+    int* counter = reinterpret_cast<int*>(plan.split_o);            // unused by a one-split call; zeroed by the gather
     long long pgrid = std::min<long long>(grid, sms);
     if (tun && tun->attention_grid_blocks > 0) pgrid = std::min<long long>(grid, tun->attention_grid_blocks);
     RELAXKV_RANGE("attention_persist_kernel");
@@ -1357,15 +1368,16 @@ static relaxkv_status launch_attention(const relaxkv_shape* shape, int mode, Att
   relaxkv_status rc = cuda_ok(launch_chained(kern, dim3((unsigned)units, (unsigned)n_splits), kAttnThreads, AttnSmem<D>::kDynamic, stream,
       tm_q, tm_k, tm_v, tm_k_new, tm_v_new, plan.all_fresh, plan.rt, pt, mode, allow_empty, head_inner, plan.dense_ctx, H, Hkv, pair_targets, shape->softmax_scale * kLog2eA,
       u_pos, u_cu, r_rank, r_cu_layer, n_target_rows, static_cast<uint16_t*>(out), lse_out, plan.split_o, plan.split_lse, st));
-  if (rc == RELAXKV_OK && pt.most > 0) {
-    const long long warps = (long long)pt.slot_cu[B] * H;
-    constexpr int wpb = kCombineThreads / 32;
-    return cuda_ok(launch_chained(combine_splits_kernel<8, true>, (unsigned)((warps + wpb - 1) / wpb), kCombineThreads, 0, stream,
-                                  plan.split_o, plan.split_lse, pt.most, n_target_rows, H, D, r_cu_layer, B, static_cast<uint16_t*>(out), lse_out, pt, pair_targets));
-  }
-  if (rc != RELAXKV_OK || n_splits == 1) return rc;
-  return launch_combine_splits(plan.split_o, plan.split_lse, (int)n_splits, n_target_rows, H, D, r_cu_layer, B, plan.sum_targets,
-                               out, lse_out, stream);
+  if (rc != RELAXKV_OK || (n_splits == 1 && pt.most == 0)) return rc;
+  const bool own_counts = plan.dense_ctx && r_cu_layer;      // (no gather has marked what is refused)
+  if (pt.most == 0 && !own_counts)
+    return launch_combine_splits(plan.split_o, plan.split_lse, (int)n_splits, n_target_rows, H, D, r_cu_layer, B, plan.sum_targets, out, lse_out, st, stream);
+  if (own_counts) std::copy_n(plan.rt.bound_a, B, pt.bound);
+  const long long warps = (own_counts ? plan.sum_targets : pt.slot_cu[B]) * H;
+  constexpr int wpb = kCombineThreads / 32;
+  return cuda_ok(launch_chained(own_counts ? combine_splits_kernel<8, LISTS> : combine_splits_kernel<8, PIECES>, (unsigned)((warps + wpb - 1) / wpb), kCombineThreads,
+                                0, stream, plan.split_o, plan.split_lse, own_counts ? (int)n_splits : pt.most, n_target_rows, H, D, r_cu_layer, plan.refused, B,
+                                static_cast<uint16_t*>(out), lse_out, pt, pair_targets, st));
 }
 
 }  // namespace relaxkv

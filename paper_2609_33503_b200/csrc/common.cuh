@@ -257,6 +257,7 @@ struct WsLayout {
   size_t list_limit, list_fresh;
   // context split across blocks (few targets): partial O [split_rows_cap, H, D] f32 | partial lse [split_rows_cap, H] f32
   size_t split_o, split_lse;
+  size_t refused;           // [kMaxReqInline] i32: requests that the attention kernel refuses
   // scoring (per launch of Lc <= kScoreLayersPerLaunch layers): lse [Lc, H, sumQ] f32 |
   // part [Lc, 2*n_splits, H, sumQ] float2 | colpart [Lc, 2*H_kv*max_blocks, sumT] f32
   size_t lse, part, colpart;
@@ -278,6 +279,7 @@ inline WsLayout ws_layout(const relaxkv_shape* s, int n_layers) {
   w.list_fresh = a; a = align_up(a + (size_t)sum_t * 4, 256);
   w.split_o = a; a = align_up(a + (size_t)split_rows_cap(s) * s->n_q_heads * s->head_dim * 4, 256);
   w.split_lse = a; a = align_up(a + (size_t)split_rows_cap(s) * s->n_q_heads * 4, 256);
+  w.refused = a; a = align_up(a + kMaxReqInline * 4, 256);
   size_t attn_total = a;
   a = 0;
   const int lc_max = n_layers < kScoreLayersPerLaunch ? n_layers : kScoreLayersPerLaunch;

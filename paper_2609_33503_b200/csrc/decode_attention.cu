@@ -110,13 +110,12 @@ decode_attention_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
   const int c0 = tgt_cu ? tgt_cu[0] : 0, cb = tgt_cu ? tgt_cu[b] : rt.q_cu[b], nr = tgt_cu ? tgt_cu[b + 1] - cb : rt.q_len[b];
   if (nr <= 0) return;
   const long long row = (long long)cb - c0;
-  if (nr > rt.bound_a[b] || nr > 1 || row >= n_target_rows) {      // more targets than the host bound (one): touch nothing
-    if (threadIdx.x == 0) report(st, RELAXKV_ERR_BAD_INDEX, KID_ATTN_SIMT, nr, (int)row);
-    return;
-  }
-  const int pos = tgt_cu ? tgt_pos[cb] : rt.ctx_len[b] - 1;
+  const bool many = nr > rt.bound_a[b] || nr > 1 || row >= n_target_rows;      // more targets than the host bound (one): touch nothing
+  const int pos = many ? -1 : (tgt_cu ? tgt_pos[cb] : rt.ctx_len[b] - 1);
   if (pos < 0 || pos >= rt.ctx_len[b]) {
-    if (threadIdx.x == 0) report(st, RELAXKV_ERR_BAD_INDEX, KID_ATTN_SIMT, pos, rt.ctx_len[b]);
+    if (threadIdx.x == 0) report(st, RELAXKV_ERR_BAD_INDEX, KID_ATTN_SIMT, many ? nr : pos, many ? (int)row : rt.ctx_len[b]);
+    if (max_splits > 1 && split == 0 && threadIdx.x < G)             // nor does the merge
+      for (long long r = row; r < min(row + nr, n_target_rows); ++r) part_lse[r * H + hd * G + threadIdx.x] = __uint_as_float(kRefusedLse);
     return;
   }
   if (status == RELAXKV_ERR_TIMEOUT) return;                         // drain after a timeout
@@ -391,7 +390,7 @@ static relaxkv_status launch_d(const relaxkv_shape* shape, AttnPlan plan, const 
   else rc = launch_g<D, 16>(tm_k, tm_v, plan, max_splits, q, tgt_pos, tgt_cu, n_target_rows, H, Hkv, scale_log2, out, lse_out, st, stream);
   if (rc != RELAXKV_OK || max_splits == 1) return rc;
   return launch_combine_splits(plan.split_o, plan.split_lse, max_splits, n_target_rows, H, shape->head_dim, tgt_cu, B,
-                               plan.sum_targets, out, lse_out, stream);
+                               plan.sum_targets, out, lse_out, st, stream);
 }
 
 relaxkv_status launch_decode_attention(const relaxkv_shape* shape, const AttnPlan& plan, const void* q, const int32_t* tgt_pos,

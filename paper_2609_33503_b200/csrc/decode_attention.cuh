@@ -11,9 +11,9 @@ relaxkv_status launch_decode_attention(const relaxkv_shape* shape, const AttnPla
                                        cudaStream_t stream);
 
 // Merges the normalised partial results [n_splits][n_target_rows][H][D] and their log-sum-exp by a fixed-order sum
-// (attention_sm100.cu).  rows_bound: sum of the host bounds on the targets.
+// (attention_sm100.cu).  rows_bound: sum of the host bounds on the targets.  Marked rows (kRefusedLse) are not written.
 relaxkv_status launch_combine_splits(const float* part_o, const float* part_lse, int n_splits, long long n_target_rows, int H,
                                      int D, const int32_t* r_cu, int n_req, long long rows_bound, void* out, float* lse_out,
-                                     cudaStream_t stream);
+                                     DeviceStatus* st, cudaStream_t stream);
 
 }  // namespace relaxkv

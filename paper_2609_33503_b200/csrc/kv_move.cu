@@ -108,7 +108,8 @@ gather_ctx_kernel(ReqTable rt, int mode, int n_kv_heads, int head_dim,
                   const uint16_t* k_new, const uint16_t* v_new,
                   const int* u_pos, const int* u_cu, const int* r_rank, const int* r_cu, const int* fresh_row,
                   uint16_t* __restrict__ k_out, uint16_t* __restrict__ v_out, long long ctx_rows,
-                  long long fresh_map_rows, long long n_new_rows, int rows_per_warp, int* work_counter, int all_fresh, DeviceStatus* st) {
+                  long long fresh_map_rows, long long n_new_rows, int rows_per_warp, int* work_counter,
+                  int* refused, float* part_lse, long long part_rows, int H, int all_fresh, DeviceStatus* st) {
   // fresh_map_rows: entries of fresh_row that were written (the host bound on the context rows of an explicit-list
   // call); n_new_rows: rows k_new / v_new hold.  An index past either is reported and the row zero-filled.
   extern __shared__ __align__(128) uint8_t stage[];          // [warp][row of the warp][K row | V row]
@@ -121,6 +122,15 @@ gather_ctx_kernel(ReqTable rt, int mode, int n_kv_heads, int head_dim,
   if (lane == 0) { gave_up[warp] = 0; mbar_init(bar, 1); fence_barrier_init(); }
   griddep_wait();                              // the rows and the index lists come from earlier kernels
   if (work_counter != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *work_counter = 0;
+  // (the last block, which has padding to write at most: the counts are a memory latency of their own)
+  if (refused != nullptr && blockIdx.x == gridDim.x - 1 && threadIdx.x < B) {
+    const int b = threadIdx.x, row = r_cu[b] - r_cu[0], nr = r_cu[b + 1] - r_cu[b], nu = u_cu[b + 1] - u_cu[b];
+    const bool no = nr > rt.bound_a[b] || (mode == RELAXKV_CTX_UNION && nu > rt.bound_b[b]) || (long long)row + nr > n_new_rows;
+    refused[b] = no;
+    if (no)
+      for (long long i = max(row, 0) * (long long)H; i < min((long long)row + nr, min(n_new_rows, part_rows)) * H; ++i)
+        part_lse[i] = __uint_as_float(kRefusedLse);
+  }
   if (x0 >= ctx_rows) return;
   if (all_rows_fresh(all_fresh, u_cu, r_cu)) {
     // Nothing to bring together: the lists are only looked over.  One layer of 16 K tokens, 2458 rows of 4 KB, from selection to cache update
@@ -316,9 +326,10 @@ relaxkv_status launch_gather(const relaxkv_shape* shape, int mode, const relaxkv
                              const int32_t* r_rank, const int32_t* r_cu_layer, const int32_t* fresh_row,
                              long long fresh_map_rows, long long n_new_rows,
                              long long rows_to_cover, void* k_out, void* v_out, long long ctx_rows, int* work_counter,
-                             int all_fresh, cudaStream_t stream) {
+                             const RefusedRows& refused, int all_fresh, cudaStream_t stream) {
   ReqTable rt;
   fill_req_table(rt, shape, cache, nullptr);
+  for (int b = 0; refused.flag && b < shape->n_req; ++b) { rt.bound_a[b] = refused.bound_targets[b]; rt.bound_b[b] = refused.bound_ctx[b]; }
   DeviceStatus* st = status_word();
   if (!st) return RELAXKV_ERR_CUDA;
   if (rows_to_cover > ctx_rows) rows_to_cover = ctx_rows;
@@ -339,7 +350,7 @@ relaxkv_status launch_gather(const relaxkv_shape* shape, int mode, const relaxkv
       (long long)cache->token_stride, (long long)cache->head_stride,
       static_cast<const uint16_t*>(k_new), static_cast<const uint16_t*>(v_new),
       u_pos, u_cu, r_rank, r_cu_layer, fresh_row, static_cast<uint16_t*>(k_out), static_cast<uint16_t*>(v_out), ctx_rows,
-      fresh_map_rows, n_new_rows, rows_per_warp, work_counter, all_fresh, st));
+      fresh_map_rows, n_new_rows, rows_per_warp, work_counter, refused.flag, refused.part_lse, refused.part_rows, refused.H, all_fresh, st));
 }
 
 // Launches the cache update for `total` target rows (host bound); direct: see scatter_kv_kernel.
@@ -399,7 +410,7 @@ extern "C" relaxkv_status relaxkv_gather_kv(
   if (ctx_rows < need) return RELAXKV_ERR_INVALID_ARG;
   // this entry point is not told how many rows k_new / v_new hold: the fresh-row index is bounded by the R list only
   return launch_gather(shape, mode, cache, k_new, v_new, u_pos, u_cu, r_rank, r_cu_layer, nullptr, 0, 0x7fffffffffffffffLL,
-                       need + kCtxPadRows, k_ctx_out, v_ctx_out, ctx_rows, nullptr, 0, static_cast<cudaStream_t>(stream));
+                       need + kCtxPadRows, k_ctx_out, v_ctx_out, ctx_rows, nullptr, {}, 0, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" relaxkv_status relaxkv_scatter_kv(

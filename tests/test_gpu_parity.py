@@ -1348,3 +1348,98 @@ def test_a_context_of_fresh_rows_alone_is_read_in_place(n, H, Hkv, D):
         status, detail = b.relaxkv_read_device_status()
         assert status == b.ERR_BAD_INDEX
         s.r_rank.copy_(lists)
+
+
+def _merged_calls(form):
+    """A call whose context is split over blocks and merged: H, the rows per request, run(out, lse, bounds) and the call's own bounds.  form:
+    "pieces" (the longest pairs alone), "splits" (every pair, in three), each "_lists" or "_sets"; "query" (a query's rows over six key
+    tiles, no lists); "decode" (a token per request); "cache" (rows at given positions of the cache)."""
+    b, g = B(), torch.Generator(device="cuda").manual_seed(len(form))
+    normal = lambda *s: torch.randn(*s, device="cuda", generator=g).to(torch.bfloat16)
+    i32 = lambda x: torch.tensor(np.asarray(x, dtype=np.int32)).cuda()
+    if form in ("query", "decode", "cache"):
+        H, Hkv, D, ctx, n = {"query": (8, 2, 128, (700, 640), (30, 9)), "decode": (8, 2, 64, (900, 2000, 700), (1, 1, 1)),
+                             "cache": (8, 4, 128, (500, 130, 900), (40, 1, 70))}[form]
+        room = [c + m for c, m in zip(ctx, n)]
+        shape = b.Shape(H, Hkv, D, list(ctx) if form == "query" else room, list(n), attention_ctx_splits=0 if form == "query" else 4)
+        ext = b.Shape(H, Hkv, D, room, list(n))
+        view = b.CacheView(normal(sum(room), Hkv, D), normal(sum(room), Hkv, D), [sum(room[:i]) for i in range(len(n))])
+        q = normal(sum(n), H, D)
+        ws = torch.zeros(max(b.relaxkv_workspace_bytes(s, 1) for s in (shape, ext)), dtype=torch.uint8, device="cuda")
+        tgt_cu = i32(np.concatenate([[0], np.cumsum(n)]))
+
+        def run(out, lse, pos, counts=n):
+            ws.zero_()
+            rows = out.shape[0]
+            if form == "query":
+                b.relaxkv_query_prefill_attention(shape, view, q, out, lse, None, ws)
+            else:
+                b.relaxkv_cache_attention(shape, view, q[:rows], i32(pos), tgt_cu, counts, out, ws, lse_out=lse)
+        if form == "cache":
+            return H, D, n, lambda out, lse, counts: run(out, lse, np.concatenate([c + np.arange(m) for c, m in zip(ctx, n)]), counts), (list(n),)
+        return H, D, n, run, (list(ctx),)
+    H, Hkv, D, ctx = 4, 1, 64, (2600, 130, 3100) if form.startswith("pieces") else (300, 130, 250)
+    cu = i32(np.concatenate([[0], np.cumsum(ctx)]))
+    pos = i32(np.concatenate([np.arange(t) for t in ctx]))                   # every position is an entry and a target
+    shape = b.Shape(H, Hkv, D, list(ctx), None, attention_ctx_splits=3 if form.startswith("splits") else 0)
+    view = b.CacheView(normal(sum(ctx), Hkv, D), normal(sum(ctx), Hkv, D), [sum(ctx[:i]) for i in range(3)])
+    q, k, v = normal(sum(ctx), H, D), normal(sum(ctx), Hkv, D), normal(sum(ctx), Hkv, D)
+    ws = torch.zeros(b.relaxkv_workspace_bytes(shape, 1), dtype=torch.uint8, device="cuda")
+
+    def run(out, lse, max_t, max_c):
+        ws.zero_()
+        rows = out.shape[0]
+        if form.endswith("lists"):
+            b.relaxkv_list_attention(shape, view, q[:rows], k, v, pos, cu, pos, cu, max_t, max_c, out, ws, lse_out=lse)
+        else:
+            b.relaxkv_sparse_ctx_attention(shape, b.CTX_UNION, view, q[:rows], k, v, pos, cu, pos, cu, max_t, max_c, out, ws, lse_out=lse)
+    return H, D, ctx, run, (list(ctx), list(ctx))
+
+
+_MERGED = ["pieces_lists", "pieces_sets", "splits_lists", "splits_sets", "cache", "decode"]
+
+
+def _filled(n, H, D):
+    return torch.full((n, H, D), 3.0, dtype=torch.bfloat16, device="cuda"), torch.full((H, n), 3.0, dtype=torch.float32, device="cuda")
+
+
+@pytest.mark.parametrize("form,what", [(f, w) for f in _MERGED[:4] for w in ("targets", "context", "rows")] +
+                         [("cache", "targets"), ("cache", "rows"), ("decode", "rows"), ("decode", "position")])
+def test_a_refused_request_of_a_merged_call_keeps_its_rows(form, what):
+    """The last request's targets or context entries are above their host bound, its rows past the output's end, or its token's position
+    past the cache: reported, its rows of out and lse untouched (the workspace holds zeros, whose merge would be a zero row), the
+    other requests' rows as in the call without the fault."""
+    H, D, n, run, bounds = _merged_calls(form)
+    want = _filled(sum(n), H, D)
+    run(*want, *bounds)
+    assert_status_ok()
+    rows = sum(n) - ((5 if n[-1] > 5 else 1) if what == "rows" else 0)
+    got = _filled(rows, H, D)
+    wrong = [list(x) for x in bounds]
+    if what != "rows":
+        wrong[1 if what == "context" else 0][-1] += {"position": 1}.get(what, -1)
+    run(*got, *wrong)
+    st, _ = B().relaxkv_read_device_status()
+    assert st == B().ERR_BAD_INDEX
+    lo = sum(n[:-1])
+    assert torch.equal(got[0][:lo], want[0][:lo]) and torch.equal(got[1][:, :lo], want[1][:, :lo])
+    assert torch.all(got[0][lo:] == 3.0) and torch.all(got[1][:, lo:] == 3.0)
+
+
+@pytest.mark.parametrize("form", _MERGED + ["query"])
+def test_a_merged_call_after_an_expired_wait_writes_nothing(form):
+    """While the status word says RELAXKV_ERR_TIMEOUT the blocks leave no partial results, and nothing is merged; once the word has
+    been read the same call has its results."""
+    H, D, n, run, bounds = _merged_calls(form)
+    want, got = _filled(sum(n), H, D), _filled(sum(n), H, D)
+    run(*want, *bounds)
+    assert_status_ok()
+    assert not torch.any(want[1] == 3.0)
+    B().relaxkv_debug_wait_timeout()
+    run(*got, *bounds)
+    st, _ = B().relaxkv_read_device_status()
+    assert st == B().ERR_TIMEOUT
+    assert torch.all(got[0] == 3.0) and torch.all(got[1] == 3.0)
+    run(*got, *bounds)
+    assert_status_ok()
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
