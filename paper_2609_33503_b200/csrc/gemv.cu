@@ -1,9 +1,10 @@
 // Projections of a handful of rows (a decode token, the last query row going through the output head): y = x W^T with
 // one row of x, or two to four where K is short (more rows or a longer K take the tensor-core tiles of
 // gemm_skinny_sm100.cu: a weight byte then meets more multiply-adds than the FMA pipe does in its HBM time).  The work is
-// reading W once (HBM-bound), so this is a plain streaming kernel without tiles: each warp owns one or two output
-// features, its lanes stride over K in 16-byte pieces with four or eight independent weight loads in flight per lane, x stays in
-// L1, and a shuffle tree sums the lanes' partial dot products in a fixed order.  (Algorithm 1 runs the model's
+// reading W once (HBM-bound), so this is a plain streaming kernel without tiles: each warp owns two output
+// features (16 per block: a 5120-wide projection is 320 blocks, all resident at once), its lanes stride over K in
+// 16-byte pieces with eight independent weight loads in flight per lane, x stays in L1, and a shuffle tree sums the
+// lanes' partial dot products in a fixed order.  (Algorithm 1 runs the model's
 // own block unchanged; after the repair loop the same block serves the decode step of the TTFT region.)
 #include "common.cuh"
 #include "gemv.cuh"
@@ -11,6 +12,8 @@
 namespace relaxkv {
 
 constexpr int kGemvThreads = 256;
+constexpr int kGemvFeatPerWarp = 2;        // few features per warp: many blocks, so that enough bytes are in flight
+constexpr int kGemvFeatPerBlock = (kGemvThreads / 32) * kGemvFeatPerWarp;
 constexpr int kGemvPrefetchElems = 1024;   // weights per row and warp requested into L2 before the dependency wait
 
 __device__ __forceinline__ void unpack8_gemv(const uint4& v, float* f) {
@@ -27,21 +30,20 @@ __device__ __forceinline__ void unpack8_gemv(const uint4& v, float* f) {
 // KS > 1: KS warps share a warp's features and split K among them (partial sums added through shared memory in a
 //         fixed order): a matrix of a few tens of MB then has four times as many, four times shorter dependent load
 //         chains, which is what bounds such a launch (not bandwidth).
-// F: features per warp.
-template <int M, int SWIGLU, int SEG, int KS, int F>
+template <int M, int SWIGLU, int SEG, int KS>
 __global__ void __launch_bounds__(kGemvThreads)
 gemv_kernel(const uint16_t* x, const uint16_t* w, const uint16_t* residual,
             uint16_t* __restrict__ y, int n_out, int K, const GemvOut outs) {
   constexpr int kWarps = kGemvThreads / 32, kGroups = kWarps / KS;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int grp = warp / KS, kp = warp % KS;
-  const int f0 = (blockIdx.x * kGroups + grp) * F;
-  constexpr int R = SWIGLU ? 2 * F : F;      // weight rows this warp streams
+  const int f0 = (blockIdx.x * kGroups + grp) * kGemvFeatPerWarp;
+  constexpr int R = SWIGLU ? 2 * kGemvFeatPerWarp : kGemvFeatPerWarp;      // weight rows this warp streams
   const uint16_t* wr[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    const int f = min(f0 + (r % F), n_out - 1);              // the tail warp re-reads the last feature
-    const long long row = SWIGLU ? ((long long)(f / 128) * 256 + (f % 128) + (r >= F ? 128 : 0)) : f;
+    const int f = min(f0 + (r % kGemvFeatPerWarp), n_out - 1);              // the tail warp re-reads the last feature
+    const long long row = SWIGLU ? ((long long)(f / 128) * 256 + (f % 128) + (r >= kGemvFeatPerWarp ? 128 : 0)) : f;
     wr[r] = w + row * K;
   }
   float acc[R][M];
@@ -107,17 +109,17 @@ gemv_kernel(const uint16_t* x, const uint16_t* w, const uint16_t* residual,
         acc[r][m] = v;
       }
   }
-  if (lane < F) {
+  if (lane < kGemvFeatPerWarp) {
     const int f = f0 + lane;
     if (f < n_out) {
 #pragma unroll
       for (int m = 0; m < M; ++m) {
         float v = 0.f;
 #pragma unroll
-        for (int r = 0; r < F; ++r) {          // static indexing keeps the accumulators in registers
+        for (int r = 0; r < kGemvFeatPerWarp; ++r) {          // static indexing keeps the accumulators in registers
           if (r == lane) {
             if (SWIGLU) {                                     // one rounding, after the activation
-              const float g = acc[r][m], u = acc[r + (SWIGLU ? F : 0)][m];
+              const float g = acc[r][m], u = acc[r + (SWIGLU ? kGemvFeatPerWarp : 0)][m];
               v = g / (1.f + __expf(-g)) * u;
             } else {
               v = acc[r][m];
@@ -138,51 +140,30 @@ gemv_kernel(const uint16_t* x, const uint16_t* w, const uint16_t* residual,
 }
 
 constexpr long long kGemvSplitKBelowBytes = 256ll << 20;     // matrices below this size split K over four warps
-// One row of a plain projection takes one feature per warp (32 registers, eight blocks per SM, twice as many of them; with two, four or five blocks
-// share an SM, and a projection is a wave of them and a part of another) where that gained in a whole decode step too: by K alone, and
-// with the parts of K that two features have, so that stacked matrices and their pieces have the same bits.  us, two features / one: 512 x
-// 3584 2.8 / 2.3, 3584 x 3584 6.8 / 6.0, 1024 x 4096 3.7 / 2.9, 4096 x 4096 8.2 / 7.3, 6144 x 4096 10.5 / 9.5, 128256 x 4096 153.6 / 143.3, 8192 x 8192 24.1 /
-// 22.0, 4096 x 11008 18.7 / 15.9, 4096 x 14336 24.0 / 20.1; twelve layers of a decoded token over 8 K, 32 / 8 heads, 1354 / 1326.  Shorter K has too few steps
-// per warp (5120 x 3072 7.3 / 7.2, 3072 x 2048 3.8 / 4.1, 8192 x 2048 7.4 / 7.9).  5120 x 5120 alone is 10.4 / 9.9 and 5120 x 17408 in
-// eight parts 30.4 / 28.8, but the step of 40 / 8 heads that holds them 2005 / 2048 and 2004 / 2012; two rows lose (4096 x 4096 8.2 / 11.6).
-static bool one_feature(int K) { return (K >= 3584 && K <= 4096) || (K >= 8192 && K < 16384); }
 
-template <int M, int SWIGLU, int SEG, int KS, int F>
-static relaxkv_status launch_one(const uint16_t* x, const uint16_t* w, const uint16_t* residual, uint16_t* y, int n_out, int K,
-                                 const GemvOut& outs, cudaStream_t stream) {
-  constexpr int feat_per_block = kGemvThreads / 32 / KS * F;
-  return cuda_ok(launch_chained(gemv_kernel<M, SWIGLU, SEG, KS, F>, (unsigned)((n_out + feat_per_block - 1) / feat_per_block), kGemvThreads, 0,
-                                stream, x, w, residual, y, n_out, K, outs));
+template <int SWIGLU, int SEG, int KS>
+static relaxkv_status launch_mk(const uint16_t* x, const uint16_t* w, const uint16_t* residual, uint16_t* y, int n_rows,
+                                int n_out, int K, const GemvOut& outs, cudaStream_t stream) {
+  constexpr int feat_per_block = kGemvFeatPerBlock / KS;
+  const unsigned blocks = (unsigned)((n_out + feat_per_block - 1) / feat_per_block);
+  cudaError_t e = cudaSuccess;
+  switch (n_rows) {
+    case 1: e = launch_chained(gemv_kernel<1, SWIGLU, SEG, KS>, blocks, kGemvThreads, 0, stream, x, w, residual, y, n_out, K, outs); break;
+    case 2: e = launch_chained(gemv_kernel<2, SWIGLU, SEG, KS>, blocks, kGemvThreads, 0, stream, x, w, residual, y, n_out, K, outs); break;
+    case 3: e = launch_chained(gemv_kernel<3, SWIGLU, SEG, KS>, blocks, kGemvThreads, 0, stream, x, w, residual, y, n_out, K, outs); break;
+    case 4: e = launch_chained(gemv_kernel<4, SWIGLU, SEG, KS>, blocks, kGemvThreads, 0, stream, x, w, residual, y, n_out, K, outs); break;
+    default: return RELAXKV_ERR_INVALID_ARG;
+  }
+  return cuda_ok(e);
 }
 
-// Two features per warp, four warps along K where the matrix is small (a block of 256 threads for 4 or 16 features).
-template <int M, int SWIGLU, int SEG>
-static relaxkv_status launch_two_features(const uint16_t* x, const uint16_t* w, const uint16_t* residual, uint16_t* y, int n_out, int K,
-                                          const GemvOut& outs, cudaStream_t stream) {
-  const long long bytes = (long long)(SWIGLU ? 2 : 1) * n_out * K * 2;
-  return bytes < kGemvSplitKBelowBytes && K >= 4 * 256 ? launch_one<M, SWIGLU, SEG, 4, 2>(x, w, residual, y, n_out, K, outs, stream)
-                                                       : launch_one<M, SWIGLU, SEG, 1, 2>(x, w, residual, y, n_out, K, outs, stream);
-}
-
-// One row with a K that is not short takes more and shorter blocks: with two features per warp four or five of them shared an SM, and a
-// projection was a wave of them and a part of another.  A plain projection has one feature per warp (32 registers, eight blocks per SM) and
-// four warps along K, eight for a long K; gate/up four warps, then eight with two features.  By K alone, so that stacked matrices and
-// their pieces have the same bits.  us, two features / now: 512 x 3584 2.8 / 2.3, 1024 x 5120 4.1 / 3.4, 4096 x 4096 8.2 / 7.3, 6144 x 4096 10.5 / 9.5,
-// 5120 x 5120 10.4 / 9.9, 7168 x 5120 13.6 / 13.2, 4096 x 14336 24.0 / 20.0, 3584 x 18944 30.5 / 24.0, 5120 x 17408 30.4 / 28.8, 128256 x 4096
-// 153.6 / 143.3; gate/up 16384 x 2048 12.8 / 12.3, 28672 x 4096 39.2 / 36.6, 34816 x 5120 54.5 / 52.4, 57344 x 8192 147 / 143.  Shorter: 5120 x 3072 7.3 / 7.2, 3072 x
-// 2048 3.8 / 4.1, 8192 x 2048 7.4 / 7.9, 4096 x 1024 3.2 / 3.8; gate/up 8192 x 1024 4.8 / 5.0.  Two to four rows have more work per weight
-// and lose by it (two rows, 4096 x 4096 8.2 / 11.6).
 template <int SWIGLU, int SEG>
 static relaxkv_status launch_m(const uint16_t* x, const uint16_t* w, const uint16_t* residual, uint16_t* y, int n_rows,
                                int n_out, int K, const GemvOut& outs, cudaStream_t stream) {
-  if (!SWIGLU && n_rows == 1 && one_feature(K)) return launch_one<1, 0, SEG, 4, 1>(x, w, residual, y, n_out, K, outs, stream);
-  switch (n_rows) {
-    case 1: return launch_two_features<1, SWIGLU, SEG>(x, w, residual, y, n_out, K, outs, stream);
-    case 2: return launch_two_features<2, SWIGLU, SEG>(x, w, residual, y, n_out, K, outs, stream);
-    case 3: return launch_two_features<3, SWIGLU, SEG>(x, w, residual, y, n_out, K, outs, stream);
-    case 4: return launch_two_features<4, SWIGLU, SEG>(x, w, residual, y, n_out, K, outs, stream);
-    default: return RELAXKV_ERR_INVALID_ARG;
-  }
+  const long long bytes = (long long)(SWIGLU ? 2 : 1) * n_out * K * 2;
+  if (bytes < kGemvSplitKBelowBytes && K >= 4 * 256)
+    return launch_mk<SWIGLU, SEG, 4>(x, w, residual, y, n_rows, n_out, K, outs, stream);
+  return launch_mk<SWIGLU, SEG, 1>(x, w, residual, y, n_rows, n_out, K, outs, stream);
 }
 
 relaxkv_status launch_gemv(const void* x, const void* weight, const void* residual, void* y, int n_rows, int n_out,

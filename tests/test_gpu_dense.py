@@ -145,8 +145,8 @@ def test_stacked_projections_give_the_bits_of_single_ones(M, n_q, n_kv, K):
 @pytest.mark.parametrize("n_q,n_kv,K", [(264, 8, 3576), (2368, 8, 3584), (264, 136, 4088), (4096, 512, 4096), (264, 8, 4104), (264, 8, 8184), (1024, 264, 8192),
                                         (2400, 264, 16376), (1024, 264, 16384)])
 def test_one_row_by_the_features_of_a_warp(n_q, n_kv, K):
-    """One row: whether a warp has one feature or two follows from K alone.  A stacked matrix and its pieces on both sides of each line: equal
-    bits, rows around the output untouched, and against the oracle."""
+    """One row: a stacked matrix and its pieces, on both sides of K = 3584, 4096, 8192 and 16384: equal bits, rows around the output
+    untouched, and against the oracle."""
     x = rnd(1, K, seed=71)
     ws = [rnd(n, K, scale=K ** -0.5, seed=72 + i) for i, n in enumerate((n_q, n_kv, n_kv))]
     outs = [torch.full((1, n), 7.0, dtype=torch.bfloat16, device="cuda") for n in (n_q, n_kv, n_kv)]
