@@ -79,7 +79,8 @@ typedef struct {
                                  /* walks the call's query tiles, longest context first).  0: the library takes it     */
                                  /* for one-split calls over gathered contexts of at most 128 key tiles; 1: for every  */
                                  /* one-split call over a gathered context; 2: never.  Same results bit for bit.       */
-  int32_t attention_grid_blocks; /* > 0: number of thread blocks of the persistent form (default: one per SM)          */
+  int32_t attention_grid_blocks; /* > 0: number of thread blocks of the persistent form (default: one per SM); the     */
+                                 /* automatic choice then cuts no call at its longest targets                          */
 } relaxkv_tuning;
 
 /* Shapes shared by all calls. */

@@ -1310,9 +1310,10 @@ static relaxkv_status launch_attention(const relaxkv_shape* shape, int mode, Att
   n_splits = std::min<long long>(n_splits, kMaxCtxSplits);
   n_splits = std::min<long long>(n_splits, kSplitRowsCap / n_target_rows);   // partial slots: [split][row of the call]
   if (n_splits < 1) n_splits = 1;
-  // Or only the longest pairs of the call, in pieces.
+  // Or only the longest pairs of the call, in pieces.  Decided without a look at attention_persistent, whose settings have the same bits; a number of
+  // blocks asked for is one of the persistent form, which has no pieces.
   PieceTable pt{};
-  const bool automatic = forced == 0 && (!shape->h_tuning || shape->h_tuning->attention_persistent == 0);
+  const bool automatic = forced == 0 && (!shape->h_tuning || shape->h_tuning->attention_grid_blocks <= 0);
   if (automatic && r_cu_layer && !plan.dense_ctx && grid <= 4ll * sms) {
     int tiles[kMaxReqInline], pairs[kMaxReqInline];
     double steps = 0.0;

@@ -1443,3 +1443,29 @@ def test_a_merged_call_after_an_expired_wait_writes_nothing(form):
     run(*got, *bounds)
     assert_status_ok()
     assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+
+
+def test_the_forms_of_a_call_that_is_cut_have_the_same_bits():
+    """A call of more tile pairs than SMs whose longest are cut: attention_persistent = 0, 1 and 2 give the same bits, which are not the whole
+    form's; a number of blocks of the persistent form is one of a call that is not cut, and gives the bits of the whole form."""
+    b, T = B(), 12000
+    g = torch.Generator(device="cuda").manual_seed(3)
+    normal = lambda: torch.randn(T, 4, 64, device="cuda", generator=g).to(torch.bfloat16)
+    view, q, k, v = b.CacheView(normal(), normal(), [0]), normal(), normal(), normal()
+    pos, cu = torch.arange(T, dtype=torch.int32, device="cuda"), torch.tensor([0, T], dtype=torch.int32, device="cuda")
+
+    def run(**tuning):
+        shape = b.Shape(4, 4, 64, [T], None, **tuning)
+        ws = torch.empty(b.relaxkv_workspace_bytes(shape, 1), dtype=torch.uint8, device="cuda")
+        out, lse = torch.empty_like(q), torch.empty(4, T, device="cuda")
+        b.relaxkv_list_attention(shape, view, q, k, v, pos, cu, pos, cu, [T], [T], out, ws, lse_out=lse)
+        assert_status_ok()
+        return out, lse
+    same = lambda x, y: torch.equal(x[0], y[0]) and torch.equal(x[1], y[1])
+    cut, whole = run(), run(attention_ctx_splits=1)
+    assert not same(cut, whole) and (cut[0].float() - whole[0].float()).abs().max() <= MAX_ABS
+    for persistent in (1, 2):
+        assert same(run(attention_persistent=persistent), cut)
+        assert same(run(attention_persistent=persistent, attention_ctx_splits=1), whole)
+    for blocks in (3, 100):
+        assert same(run(attention_grid_blocks=blocks), whole)
