@@ -117,32 +117,54 @@ class QueryPass:
                 taps: Optional[list] = None) -> torch.Tensor:
         """h0: input representations of the query tokens [sum Q_b, hidden].  caches[l]: layer l's cache with the context
         rows in place and room behind them; the query's K/V are written there.  scores_out: fp32 [n_layers, sum T_c]
-        or None; when given, row l receives the context scores of layer l from this very pass (computed for several layers
-        at once where its rows lie one behind the other).  Returns the hidden rows after the last layer."""
+        or None; when given, row l receives the context scores of layer l from this very pass.  Where scores_out is one matrix and
+        weights and caches are lists (or tuples) whose layers have memory of their own, they are computed for up to eight layers at once,
+        behind the last of them: the context rows stay as they are until the call's work is done.  A cache that
+        several layers share, or that another kind of sequence hands out, is scored before the next layer is asked for.
+        Returns the hidden rows after the last layer."""
         rec = self._rec(events)
         h = h0
-        # scored in groups where the rows of scores_out lie one behind the other, as a call over several layers writes them
-        together = (self.q_kept is not None and isinstance(scores_out, torch.Tensor) and scores_out.dtype == torch.float32 and scores_out.dim() == 2
-                    and scores_out.shape[1] == sum(self.ctx_lens) and scores_out.is_contiguous())
-        group = self.q_kept.shape[0] if together else 1
+        group, keep = 1, self.q_kept is not None and scores_out is not None
         for l, w in enumerate(weights):
             h_out = self.h[l % 2]
+            cache = caches[l]
             raw = scores_out[l] if scores_out is not None else None
-            q, lse = (self.q_kept[l % group], self.lse_kept[l % group]) if together else (self.q, self.lse)
+            q, lse = (self.q_kept[l % group], self.lse_kept[l % group]) if keep else (self.q, self.lse)
 
             def attend():
-                B.relaxkv_query_prefill_attention(self.shape_prefill, caches[l], q, self.o, lse, None if together else raw, self.workspace)
-            self._block(l, w, caches[l], h, self.x, self.a, q, self.k, self.v, self.o, self.gu, self.m, h_out,
+                nonlocal group
+                if l == 0 and keep:                     # (10 us of a host that has three launches ahead of it by now)
+                    group = self._score_group(weights, caches, scores_out, events, taps)
+                B.relaxkv_query_prefill_attention(self.shape_prefill, cache, q, self.o, lse, None if group > 1 else raw, self.workspace)
+            self._block(l, w, cache, h, self.x, self.a, q, self.k, self.v, self.o, self.gu, self.m, h_out,
                         self.q_pos, self.q_cu, self.q_lens, self.shape_ext, attend, rec)
-            if together and (l % group == group - 1 or l == len(weights) - 1):
+            if group > 1 and (l % group == group - 1 or l == len(weights) - 1):
                 l0, n = l - l % group, l % group + 1
                 rec("scores", lambda: B.relaxkv_score_select(
-                    self.shape_prefill, [self.q_kept[i] for i in range(n)], [caches[i] for i in range(l0, l + 1)], [1] * len(self.ctx_lens),
+                    self.shape_prefill, [self.q_kept[i] for i in range(n)], caches[l0:l + 1], [1] * len(self.ctx_lens),
                     scores_out[l0:l + 1], None, self.workspace, row_lse_layers=[self.lse_kept[i] for i in range(n)]))
             if taps is not None:
                 taps.append((h.clone(), h_out.clone()))
             h = h_out
         return h
+
+    def _score_group(self, weights, caches, scores_out, events, taps) -> int:
+        """Layers that are scored by one launch (1: each in its own).  More than one need rows of scores_out one behind the other, as a call over
+        several layers writes them, and keys that are still there when the last of them has run: nothing of the caller's runs between two
+        layers (a generator, a sequence or a list of its own making may fill the next layer's cache then), and no two layers share a byte."""
+        if (not isinstance(scores_out, torch.Tensor) or scores_out.dtype != torch.float32 or scores_out.dim() != 2
+                or scores_out.shape[1] != sum(self.ctx_lens) or not scores_out.is_contiguous()):
+            return 1
+        if (any(type(x) not in (list, tuple) for x in (weights, caches)) or any(type(x) not in (list, type(None)) for x in (events, taps))
+                or len(caches) < len(weights)):
+            return 1
+        spans = []
+        for c in caches[:len(weights)]:
+            v = c.c                                     # (v.v is None for a view without values: refused by the layer's own calls)
+            n = 2 * ((c.k.shape[0] - 1) * v.token_stride + (self.Hkv - 1) * v.head_stride + self.D)
+            spans += {(v.k, v.k + n), (v.v or 0, (v.v or 0) + n)}          # (one, where K and V are one tensor)
+        spans.sort()
+        return self.q_kept.shape[0] if all(a[1] <= b[0] for a, b in zip(spans, spans[1:])) else 1
 
     def decode(self, h_tok: torch.Tensor, weights: List[Dict[str, torch.Tensor]], caches: List[B.CacheView], step: int = 0,
                events: Optional[list] = None) -> torch.Tensor:

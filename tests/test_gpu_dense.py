@@ -751,3 +751,80 @@ def test_rows_of_any_alignment_leave_a_gemm_alike(M, N, off_y, off_r):
     B().relaxkv_linear(x, w[:N].contiguous(), out[off_y:off_y + M * N].view(M, N), residual=res[off_r:off_r + M * N].view(M, N))
     assert torch.equal(out[off_y:off_y + M * N].view(M, N), ref[:, :N])
     assert torch.all(out[:off_y] == 3.0) and torch.all(out[off_y + M * N:] == 3.0)
+
+
+def _grouped_pass(layers=3):
+    """A small query pass with scores: the pass, weights, query rows, per-layer K/V, a view of a layer's tensors, its scores by single layers."""
+    from paper_2609_33503_b200.query_pass import QueryPass
+    H, Hkv, D, ctx, qn = 8, 2, 64, (700,), (9,)
+    blkshape = inputs.BlockShape(hidden=256, inter=512, rope_theta=1.0e4, eps=1.0e-5, qk_norm=True)
+    w = inputs.Workload("staged", layers, H, Hkv, D, 64, ctx, qn, 0.15, base_seed=13)
+    rows = ctx[0] + qn[0]
+    weights = [inputs.block_weights(w, blkshape, l, "cuda") for l in range(layers)]
+    kv = [(rnd(rows, Hkv, D, seed=100 + l), rnd(rows, Hkv, D, seed=200 + l)) for l in range(layers)]
+    view = lambda k, v: B().CacheView(k, v, [0])
+    qp, h0 = QueryPass(H, Hkv, D, ctx, qn, blkshape), rnd(qn[0], blkshape.hidden, seed=3)
+    apart = torch.full((layers, ctx[0] + 4), -1.0, device="cuda")[:, :ctx[0]]            # rows with a gap: a launch per layer
+    h = qp.prefill(h0, weights, [view(k.clone(), v.clone()) for k, v in kv], scores_out=apart).clone()
+    return qp, weights, h0, kv, view, h, apart
+
+
+class _Staged:
+    """Caches that a program streams: asked for a layer, it copies that layer into the one staging buffer there is, and hands it out once."""
+
+    def __init__(self, kv, view, n_buffers):
+        self.kv, self.next = kv, 0
+        self.views = [view(torch.empty_like(kv[0][0]), torch.empty_like(kv[0][1])) for _ in range(n_buffers)]
+
+    def __len__(self):
+        return len(self.kv)
+
+    def __getitem__(self, l):
+        assert l == self.next, "a layer that was handed out, or is not due yet"
+        self.next += 1
+        c = self.views[l % len(self.views)]
+        c.k.copy_(self.kv[l][0])
+        c.v.copy_(self.kv[l][1])
+        return c
+
+
+@pytest.mark.parametrize("n_buffers", [1, 2])
+@pytest.mark.parametrize("by", ["sequence", "weights"])
+def test_scores_of_a_pass_whose_caches_are_staged(by, n_buffers):
+    """One or two staging buffers for the caches of all layers, filled when a layer is asked for, or by the generator of the layers' weights
+    (which has no length): every layer's scores are its own, to the order of fp32 sums (112 positive terms at most: 1e-5)."""
+    qp, weights, h0, kv, view, h_ref, ref = _grouped_pass()
+    staged, scores = _Staged(kv, view, n_buffers), torch.full(ref.shape, -1.0, device="cuda")
+    if by == "sequence":
+        h = qp.prefill(h0, weights, staged, scores_out=scores)
+    else:
+        def stream():
+            for l, w in enumerate(weights):
+                staged[l]
+                yield w
+        h = qp.prefill(h0, stream(), [staged.views[l % n_buffers] for l in range(len(weights))], scores_out=scores)
+    assert B().relaxkv_read_device_status()[0] == 0
+    assert torch.equal(h, h_ref)
+    assert ((scores - ref).abs() <= 1e-5 * ref).all()
+
+
+@pytest.mark.parametrize("layout", ["one_tensor", "interleaved", "same"])
+def test_scores_of_a_pass_by_the_memory_of_its_layers(layout):
+    """Layers whose caches are slices of one tensor, lie between one another's rows, or are one cache (each layer then sees the query rows
+    of the layers before in the rows behind the context, which no score reads)."""
+    qp, weights, h0, kv, view, h_ref, ref = _grouped_pass()
+    L = len(kv)
+    if layout == "same":
+        kv = [kv[0]] * L
+        views = [view(*kv[0])] * L
+        ref = torch.cat([ref[:1]] * L)                   # (of layer 0 alone: the others' queries differ from the reference pass)
+    else:
+        stacked = [torch.stack([x[i] for x in kv], dim=0 if layout == "one_tensor" else 1) for i in range(2)]
+        views = [view(*(t[l] if layout == "one_tensor" else t[:, l] for t in stacked)) for l in range(L)]
+    scores = torch.full(ref.shape, -1.0, device="cuda")
+    h = qp.prefill(h0, weights, views, scores_out=scores)
+    assert B().relaxkv_read_device_status()[0] == 0
+    n = 1 if layout == "same" else L
+    assert ((scores[:n] - ref[:n]).abs() <= 1e-5 * ref[:n]).all() and (scores > 0).all()
+    if layout != "same":
+        assert torch.equal(h, h_ref)
