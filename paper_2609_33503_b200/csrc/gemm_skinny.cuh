@@ -2,10 +2,9 @@
 // cluster, K split over the cluster's blocks, partial tiles summed through distributed shared memory.
 #pragma once
 #include "common.cuh"
+#include "gemm_skinny_layout.cuh"
 
 namespace relaxkv {
-
-constexpr int kSkinnyMaxRows = 128;
 
 // Where the features of y = x W^T go: segment i takes features [col0[i], col0[i + 1]) and is a row-major matrix of that
 // width of its own (+ an optional residual of the same shape).  Segment widths are multiples of 8.

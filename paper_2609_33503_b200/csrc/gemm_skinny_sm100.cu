@@ -37,24 +37,13 @@ using namespace ptx;
 bool make_map_3d(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t stride1_bytes,
                  uint64_t stride2_bytes, uint32_t b1, uint32_t b2);          // attention_sm100.cu
 
-constexpr int kSkFeat = 128, kSkBK = 64, kSkStagesMax = 7;
 __host__ __device__ constexpr int sk_threads(int epi) { return 64 + 32 * epi; }
-constexpr int kSkWBytes = kSkFeat * kSkBK * 2;                             // weights of a stage: 16 KB, as two 64-row boxes
-constexpr int kSkRing2 = 108 * 1024, kSkRing1 = 192 * 1024;                // two blocks, one block per SM
-constexpr int kSkCols2 = 64;                                               // widest MMA that always takes the two-block form
 constexpr int kSkManyRows = 32;                                            // whole tiles: rows from which eight warps write them
 constexpr int kSkDeepK = 8192;                                             // few rows: K from which eight blocks share a tile
 constexpr int kSkParts = 8, kSkPartCols = 16;                               // few rows: parts of K, MMA columns of each
 constexpr int kSkBars = 2 * kSkStagesMax + 2;                              // full, empty per stage; accumulator full; partial tiles received
 constexpr int kSkTail = 8 * kSkBars + 16 + 1024;                           // barriers, slots, alignment
-constexpr int sk_stages(int n_cols, bool whole_sm) { return (whole_sm ? kSkRing1 : kSkRing2) / (kSkWBytes + n_cols * kSkBK * 2); }
-static_assert(sk_stages(16, false) <= kSkStagesMax, "barriers for every stage");
-// The partial tile (rows of x times parts of K, 128 features, fp32) and as much again that the blocks of a cluster receive take the ring's place.
-__host__ __device__ constexpr int sk_part_bytes(int rows) { return rows * kSkFeat * 4; }
-static_assert(sk_part_bytes(kSkinnyMaxRows) <= sk_stages(kSkinnyMaxRows, false) * (kSkWBytes + kSkinnyMaxRows * kSkBK * 2) &&
-              2 * sk_part_bytes(kSkCols2) <= sk_stages(kSkCols2, false) * (kSkWBytes + kSkCols2 * kSkBK * 2) &&
-              2 * sk_part_bytes(kSkinnyMaxRows) <= sk_stages(kSkinnyMaxRows, true) * (kSkWBytes + kSkinnyMaxRows * kSkBK * 2),
-              "the partial tiles reuse the TMA ring");
+static_assert(sk_exchange_fits(1, 1, kSkinnyMaxRows, false, kSkinnyMaxRows, sk_stages(kSkinnyMaxRows, false)), "a tile of its own reuses the TMA ring");
 
 // S blocks per tile; a block's share of K is PL parts, each summed in an accumulator of its own (PL > 1: n_cols is kSkPartCols).
 template <int S, int PL, int E>
@@ -72,8 +61,8 @@ gemm_skinny_sm100_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_
   const int r0 = swiglu ? (f0 / 128) * 256 + f0 % 128 : f0, r1 = swiglu ? r0 + 128 : r0 + kSkFeat / 2;
 
   // of the tile's features, in groups of four, block r of the cluster adds up and writes [r all / S, (r + 1) all / S)
-  const int all_quads = (swiglu ? kSkFeat / 2 : kSkFeat) / 4;
-  const int own_q0 = (int)rank * all_quads / S, own_quads = ((int)rank + 1) * all_quads / S - own_q0;
+  const int all_quads = sk_quads(swiglu != 0);
+  const int own_q0 = sk_quad((int)rank, S, swiglu != 0), own_quads = sk_quad((int)rank + 1, S, swiglu != 0) - own_q0;
 
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -324,7 +313,7 @@ template <int S, int PL = 1, int E = 4>
 static bool try_launch(const SkinnyPlan& p, const CUtensorMap& tm_w, const CUtensorMap& tm_x, const SkinnyOut& outs, relaxkv_status* rc) {
   const int n_k = (p.n_in + kSkBK - 1) / kSkBK;
   if (S > 1 && n_k < 2 * S) return false;
-  if (S > 1 && 2 * sk_part_bytes(PL * p.n_rows) > p.n_stages * (kSkWBytes + p.n_cols * kSkBK * 2)) return false;
+  if (S > 1 && !sk_exchange_fits(S, PL, p.n_rows, p.swiglu != 0, p.n_cols, p.n_stages)) return false;
   // with two blocks per SM an even cluster sits on S / 2 SMs (the occupancy query itself counts one block per SM)
   const int resident = p.whole_sm ? max_clusters<S>(p.dev, p.sms) : (S % 2 ? 2 * max_clusters<S>(p.dev, p.sms) : max_clusters<(S + 1) / 2>(p.dev, p.sms));
   if (resident < 1 || !opt_in_smem<S, PL, E>(p.dev)) { *rc = RELAXKV_ERR_CUDA; return true; }
@@ -356,8 +345,8 @@ relaxkv_status launch_gemm_skinny(const void* x, const void* weight, const Skinn
   // (64 rows, two blocks / one: 2048 x 2048 8.4 / 6.9 us, 3072 x 2048 9.8 / 7.6, 4096 x 4096 12.9 / 10.7, 4096 x 14336 25.9 / 24.1; 33 rows 6.8 / 6.2,
   // 7.8 / 7.1, 11.0 / 10.2, 24.0 / 23.5; 40 tiles of 5120 x 5120 14.4 / 13.8 and 13.2 / 13.1; 17 rows, 2048 x 4096 7.4 / 7.8).
   p.whole_sm = (p.n_cols > kSkCols2 && p.tiles <= p.sms) || (p.n_cols > 32 && p.tiles * 4 <= p.sms);
-  p.n_stages = std::min(kSkStagesMax, sk_stages(p.n_cols, p.whole_sm));
-  p.smem = (size_t)p.n_stages * (kSkWBytes + p.n_cols * kSkBK * 2) + kSkTail;
+  p.n_stages = sk_stages(p.n_cols, p.whole_sm);
+  p.smem = (size_t)p.n_stages * sk_stage_bytes(p.n_cols) + kSkTail;
   relaxkv_status rc = RELAXKV_OK;
   // The largest cluster that fits.  A projection of up to four rows is always summed over K in kSkParts parts, however many blocks
   // share them, so that it has the same bits stacked with others and by itself.
