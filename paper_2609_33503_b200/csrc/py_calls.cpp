@@ -8,9 +8,10 @@
 //                                '.' anything, as it is.
 //   bind(name, address, other)   the entry point at `address` as a callable over integers, floats, bytes and None.  A call with
 //                                anything else among its arguments (a ctypes reference, a wrong count) is `other`'s.
-// The interpreter's lock is released during the call, as ctypes does it.
+// The interpreter's lock is released during the call, as ctypes does it.  Python 3.10 or newer.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
+#include <structmember.h>                                  // T_PYSSIZET, READONLY: the names that Python 3.10 and 3.11 have, too
 #include <cstddef>
 #include <cstdint>
 #include <cstring>
@@ -143,7 +144,7 @@ void entry_dealloc(PyObject* self) {
 }
 
 PyMemberDef entry_members[] = {
-    {"__vectorcalloffset__", Py_T_PYSSIZET, offsetof(Entry, vectorcall), Py_READONLY, nullptr}, {nullptr, 0, 0, 0, nullptr}};
+    {"__vectorcalloffset__", T_PYSSIZET, offsetof(Entry, vectorcall), READONLY, nullptr}, {nullptr, 0, 0, 0, nullptr}};
 PyType_Slot entry_slots[] = {{Py_tp_dealloc, (void*)entry_dealloc}, {Py_tp_call, (void*)PyVectorcall_Call},
                              {Py_tp_members, entry_members}, {0, nullptr}};
 PyType_Spec entry_spec = {"paper_2609_33503_b200._calls.Entry", sizeof(Entry), 0,

@@ -115,3 +115,18 @@ def test_references_and_threads():
     entry_refs = sys.getrefcount(plain)
     del bound
     assert sys.getrefcount(plain) == entry_refs - 1
+
+
+def test_the_calls_name_nothing_newer_than_python_3_10():
+    """The member descriptors go by the names of structmember.h (their Py_ forms came with 3.12), and nothing else of the C API that came with
+    3.11 to 3.14 is named."""
+    import os
+    import re
+    from paper_2609_33503_b200 import build
+    with open(os.path.join(build.CSRC, "py_calls.cpp")) as f:
+        words = set(re.findall(r"\w+", re.sub(r"//.*", "", f.read())))
+    newer = {w for w in words if re.fullmatch(r"Py_(T_\w+|READONLY|RELATIVE_OFFSET|AUDIT_READ|mod_gil|MOD_GIL_\w+|tp_vectorcall)", w)}
+    newer |= words & {"PyType_GetName", "PyType_GetQualName", "PyType_FromMetaclass", "PyErr_GetRaisedException", "PyErr_SetRaisedException", "PyObject_GetOptionalAttr",
+                      "PyLong_AsInt", "PyLong_AsNativeBytes", "PyList_GetItemRef", "PyDict_GetItemRef", "PyUnicode_EqualToUTF8", "PyBuffer_ReleaseBuffer",
+                      "Py_HashPointer", "PyWeakref_GetRef", "PyUnstable_Long_IsCompact", "PyImport_AddModuleRef"}
+    assert not newer and "structmember" in words
