@@ -51,7 +51,7 @@ __device__ __forceinline__ int block_prefix(int v, int* warp_tot) {
 // of 16 K / 32 K / 64 K scores (each pass a block-wide walk through L2).  Here a slice's keys are read once and stay in
 // shared memory (slices above kSelKeysMax keys are read again from L2 in each pass), the histograms of a
 // cluster's blocks are added through distributed shared memory by every block for itself, and the bin is found by a
-// block-wide prefix: 4.5 us, and 10.1 / 12.3 (15.7 for 40 segments) / 15.6 us.
+// block-wide prefix: 4.5 us, and 10.1 / 13.5 (15.7 for 40 segments) / 15.6 us.
 template <int NS>                                          // slices = blocks of a cluster
 __global__ void __launch_bounds__(kSelThreads)
 select_topk_kernel(ReqTable rt, int n_layers, int keys_cap, const float* raw, float* norm, int* anchors, DeviceStatus* st) {

@@ -1469,3 +1469,29 @@ def test_the_forms_of_a_call_that_is_cut_have_the_same_bits():
         assert same(run(attention_persistent=persistent, attention_ctx_splits=1), whole)
     for blocks in (3, 100):
         assert same(run(attention_grid_blocks=blocks), whole)
+
+
+@pytest.mark.parametrize("H,Hkv,D,T,n", [(8, 2, 128, 700, 300), (10, 2, 64, 500, 333), (8, 8, 64, 300, 1)])
+@pytest.mark.parametrize("tuning", [dict(attention_ctx_splits=1, attention_persistent=2), dict(attention_ctx_splits=1, attention_persistent=1), dict(attention_ctx_splits=3)],
+                         ids=["one_shot", "persistent", "split"])
+def test_an_output_that_is_not_32_byte_aligned(H, Hkv, D, T, n, tuning):
+    """Outputs are stored as whole 32-byte sectors where the output begins on one and in 16-byte pieces elsewhere: the same bits, and nothing
+    written beside the rows."""
+    b, g = B(), torch.Generator(device="cuda").manual_seed(n)
+    normal = lambda *s: torch.randn(*s, device="cuda", generator=g).to(torch.bfloat16)
+    i32 = lambda x: torch.tensor(np.asarray(x, dtype=np.int32)).cuda()
+    shape = b.Shape(H, Hkv, D, [T], None, **tuning)
+    view, q, k, v = b.CacheView(normal(T, Hkv, D), normal(T, Hkv, D), [0]), normal(n, H, D), normal(n, Hkv, D), normal(n, Hkv, D)
+    ws = torch.empty(b.relaxkv_workspace_bytes(shape, 1), dtype=torch.uint8, device="cuda")
+    pos, tgt = i32(np.arange(T)), np.sort(np.random.default_rng(n).choice(T, n, replace=False))
+    got = []
+    for off in (0, 8, 16, 24):                                       # elements of two bytes
+        buf = torch.full((n * H * D + 48,), 3.0, dtype=torch.bfloat16, device="cuda")
+        assert buf.data_ptr() % 32 == 0
+        out = buf[16 + off:16 + off + n * H * D].view(n, H, D)
+        b.relaxkv_sparse_ctx_attention(shape, b.CTX_UNION, view, q, k, v, pos, i32([0, T]), i32(tgt), i32([0, n]), [n], [T], out, ws)
+        assert_status_ok()
+        assert torch.all(buf[:16 + off] == 3.0) and torch.all(buf[16 + off + n * H * D:] == 3.0)
+        got.append(out.clone())
+    assert all(torch.equal(x, got[0]) for x in got[1:])
+    assert not torch.any((got[0] == 3.0).all(dim=2))
