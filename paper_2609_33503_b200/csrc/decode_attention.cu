@@ -115,7 +115,7 @@ decode_attention_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
   if (pos < 0 || pos >= rt.ctx_len[b]) {
     if (threadIdx.x == 0) report(st, RELAXKV_ERR_BAD_INDEX, KID_ATTN_SIMT, many ? nr : pos, many ? (int)row : rt.ctx_len[b]);
     if (max_splits > 1 && split == 0 && threadIdx.x < G)             // nor does the merge
-      for (long long r = row; r < min(row + nr, n_target_rows); ++r) part_lse[r * H + hd * G + threadIdx.x] = __uint_as_float(kRefusedLse);
+      for (long long r = max(row, 0ll); r < min(row + nr, n_target_rows); ++r) part_lse[r * H + hd * G + threadIdx.x] = __uint_as_float(kRefusedLse);
     return;
   }
   if (status == RELAXKV_ERR_TIMEOUT) return;                         // drain after a timeout
