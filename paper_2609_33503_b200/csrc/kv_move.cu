@@ -122,19 +122,22 @@ gather_ctx_kernel(ReqTable rt, int mode, int n_kv_heads, int head_dim,
   if (lane == 0) { gave_up[warp] = 0; mbar_init(bar, 1); fence_barrier_init(); }
   griddep_wait();                              // the rows and the index lists come from earlier kernels
   if (work_counter != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *work_counter = 0;
-  // (the last block, which has padding to write at most: the counts are a memory latency of their own)
-  if (refused != nullptr && blockIdx.x == gridDim.x - 1 && threadIdx.x < B) {
+  // The first block's threads, one per request, while its rows are on their way: the counts are a memory latency of their own.  (Attention calls of the late
+  // layers of an 8 K stack 140.3 us without, 140.6 so; its 32 layers 8142 / 8149, which is what two runs differ by.)
+  auto say_refused = [&]() {
+    if (refused == nullptr || blockIdx.x != 0 || threadIdx.x >= B) return;
     const int b = threadIdx.x, row = r_cu[b] - r_cu[0], nr = r_cu[b + 1] - r_cu[b], nu = u_cu[b + 1] - u_cu[b];
     const bool no = nr > rt.bound_a[b] || (mode == RELAXKV_CTX_UNION && nu > rt.bound_b[b]) || (long long)row + nr > n_new_rows;
     refused[b] = no;
     if (no)
       for (long long i = max(row, 0) * (long long)H; i < min((long long)row + nr, min(n_new_rows, part_rows)) * H; ++i)
         part_lse[i] = __uint_as_float(kRefusedLse);
-  }
-  if (x0 >= ctx_rows) return;
+  };
+  if (x0 >= ctx_rows) return;                  // (not the first block: there are kCtxPadRows rows at least)
   if (all_rows_fresh(all_fresh, u_cu, r_cu)) {
     // Nothing to bring together: the lists are only looked over.  One layer of 16 K tokens, 2458 rows of 4 KB, from selection to cache update
     // 107.3 us with the copy (6 of it), 103.0 without; of 1 K tokens 47.2 / 45.9.
+    say_refused();
     const long long x = x0 + lane;
     if (lane < rows_per_warp && x < all_fresh) {
       const int p = u_pos[x], c = r_rank[r_cu[0] + x];
@@ -229,6 +232,7 @@ gather_ctx_kernel(ReqTable rt, int mode, int n_kv_heads, int head_dim,
     else if (my_kind == 1)
       issue_row_loads(my_stage, k_new + my_off, v_new + my_off, n_kv_heads, head_dim, head_dim, bar);
   }
+  say_refused();
   // zero-fill rows (the pad after the context, rows with a reported index): plain stores by the whole warp
   for (int rr = 0; rr < rows_per_warp; ++rr) {
     if (__shfl_sync(0xffffffffu, my_kind, rr) == 2) {
