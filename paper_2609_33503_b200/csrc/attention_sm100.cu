@@ -1376,9 +1376,9 @@ static relaxkv_status launch_attention(const relaxkv_shape* shape, int mode, Att
   if (own_counts) std::copy_n(plan.rt.bound_a, B, pt.bound);
   const long long warps = (own_counts ? plan.sum_targets : pt.slot_cu[B]) * H;
   constexpr int wpb = kCombineThreads / 32;
-  return cuda_ok(launch_chained(own_counts ? combine_splits_kernel<8, LISTS> : combine_splits_kernel<8, PIECES>, (unsigned)((warps + wpb - 1) / wpb), kCombineThreads,
-                                0, stream, plan.split_o, plan.split_lse, own_counts ? (int)n_splits : pt.most, n_target_rows, H, D, r_cu_layer, plan.refused, B,
-                                static_cast<uint16_t*>(out), lse_out, pt, pair_targets, st));
+  auto merge = own_counts ? combine_splits_kernel<8, LISTS> : combine_splits_kernel<8, PIECES>;
+  return cuda_ok(launch_chained(merge, (unsigned)((warps + wpb - 1) / wpb), kCombineThreads, 0, stream, plan.split_o, plan.split_lse,
+                                own_counts ? (int)n_splits : pt.most, n_target_rows, H, D, r_cu_layer, plan.refused, B, static_cast<uint16_t*>(out), lse_out, pt, pair_targets, st));
 }
 
 }  // namespace relaxkv
